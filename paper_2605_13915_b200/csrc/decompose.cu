@@ -14,13 +14,14 @@
 
 namespace msd {
 
-// 256 threads x 64 registers leave room for a CTA of the dependent GEMM (192 threads x ~224 registers) on the same SM,
-// so that GEMM can start prefetching weights everywhere while this kernel still runs.
-constexpr int kDecCache = 4;   // 16-element chunks a thread keeps in registers between the two passes (K <= 16384)
-
-
-template <int kDecThreads>
-__global__ void __launch_bounds__(kDecThreads)
+// Bound by issue slots and latency (4096 rows of 4096: 59 -> 27 us with launch, 67 MB; instructions per value 32 -> 21, of which
+// 5 are the row maximum's reductions and divisions).  The row is read twice: the first pass takes the maximum, the second
+// quantises (its reads hit the L1 cache; a thread's first two units of 8 values stay in registers, which is all there is
+// at decode widths).  The second pass is a loop that is NOT unrolled and keeps two units in flight: with four unrolled
+// copies of the quantisation the kernel spent most of its time waiting for instructions, and with a register limit of 40
+// the spills cost more (38 us) than the warps gained.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads == 1024 ? 1 : 1280 / kThreads)
 decompose_int8_kernel(const uint16_t* __restrict__ x, int64_t ldx, int K, int8_t* __restrict__ q1,
                       int8_t* __restrict__ q2, float* __restrict__ alpha_out, float* __restrict__ beta_out,
                       float c1, float c2) {
@@ -28,56 +29,62 @@ decompose_int8_kernel(const uint16_t* __restrict__ x, int64_t ldx, int K, int8_t
   pdl_launch_dependents();
   const int row = blockIdx.x;
   const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<int64_t>(row) * ldx);
-  const int nchunks = K >> 4;
-  uint4 ca[kDecCache], cb[kDecCache];
+  const int units = K >> 3;
+  const int u0 = threadIdx.x;
+  const uint4 zero = make_uint4(0, 0, 0, 0);
+  uint4 cur = u0 < units ? __ldg(xr + u0) : zero;
+  uint4 next = u0 + kThreads < units ? __ldg(xr + u0 + kThreads) : zero;
   float m = 0.0f;
-#pragma unroll
-  for (int j = 0; j < kDecCache; ++j) {
-    const int c = threadIdx.x + j * kDecThreads;
-    if (c < nchunks) {
-      ca[j] = __ldg(xr + 2 * c);
-      cb[j] = __ldg(xr + 2 * c + 1);
-      m = fmaxf(m, chunk_absmax(ca[j], cb[j]));
-    }
-  }
-  for (int c = threadIdx.x + kDecCache * kDecThreads; c < nchunks; c += kDecThreads)
-    m = fmaxf(m, chunk_absmax(__ldg(xr + 2 * c), __ldg(xr + 2 * c + 1)));
+#pragma unroll 4
+  for (int u = u0 + 2 * kThreads; u < units; u += kThreads) m = fmaxf(m, unit_absmax(__ldg(xr + u)));
+  m = fmaxf(m, fmaxf(unit_absmax(cur), unit_absmax(next)));
 
-  __shared__ float warp_max[kDecThreads / 32];
+  __shared__ float warp_max[kThreads / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
   __syncthreads();
-  m = warp_max[0];
+  m = warp_max[threadIdx.x & (kThreads / 32 - 1)];
 #pragma unroll
-  for (int w = 1; w < kDecThreads / 32; ++w) m = fmaxf(m, warp_max[w]);
+  for (int o = kThreads / 64; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
 
   const float alpha = __fdiv_rn(m, c1);            // Eq. alpha (c1 = 127, or 127.49 with fractional scaling, Sec. 3.3)
   const float beta = __fdiv_rn(alpha, c2);         // Eq. beta  (c2 = 254, or 254.98)
-  // reciprocals only steer the fast path of quant_i8; infinities (tiny scales) simply send every element to the division
+  // reciprocals only steer the fast path of the quantisation
   const float inv_alpha = alpha > 0.0f ? __frcp_rn(alpha) : 0.0f;
   const float inv_beta = beta > 0.0f ? __frcp_rn(beta) : 0.0f;
   if (threadIdx.x == 0) {
     alpha_out[row] = alpha;
     beta_out[row] = beta;
   }
-  uint4* o1 = reinterpret_cast<uint4*>(q1 + static_cast<int64_t>(row) * K);
-  uint4* o2 = reinterpret_cast<uint4*>(q2 + static_cast<int64_t>(row) * K);
-#pragma unroll
-  for (int j = 0; j < kDecCache; ++j) {
-    const int c = threadIdx.x + j * kDecThreads;
-    if (c < nchunks) {
-      uint4 r1, r2;
-      chunk_quantize(ca[j], cb[j], alpha, beta, inv_alpha, inv_beta, r1, r2);
-      o1[c] = r1;
-      o2[c] = r2;
+  if (unit_scales_ok(alpha, beta)) {
+    uint2* o1 = reinterpret_cast<uint2*>(q1 + static_cast<int64_t>(row) * K);
+    uint2* o2 = reinterpret_cast<uint2*>(q2 + static_cast<int64_t>(row) * K);
+#pragma unroll 1
+    for (int u = u0; u < units; u += kThreads) {
+      uint4 after = zero;
+      if (u + 2 * kThreads < units) after = __ldg(xr + u + 2 * kThreads);
+      uint2 r1, r2;
+      unit_quantize(cur, alpha, beta, inv_alpha, inv_beta, r1, r2);
+      o1[u] = r1;
+      o2[u] = r2;
+      cur = next;
+      next = after;
     }
-  }
-  for (int c = threadIdx.x + kDecCache * kDecThreads; c < nchunks; c += kDecThreads) {
-    uint4 r1, r2;
-    chunk_quantize(__ldg(xr + 2 * c), __ldg(xr + 2 * c + 1), alpha, beta, inv_alpha, inv_beta, r1, r2);
-    o1[c] = r1;
-    o2[c] = r2;
+  } else {
+    // a zero row, or scales outside the range the fast path is proven for: value by value, with true divisions
+#pragma unroll 1
+    for (int k = threadIdx.x; k < K; k += kThreads) {
+      const float v = __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const uint16_t*>(xr) + k)) << 16);
+      int a = 0, b = 0;
+      if (alpha > 0.0f) {
+        a = quant_i8(v, alpha, inv_alpha);                               // Eq. x1
+        const float r = __fmaf_rn(-alpha, static_cast<float>(a), v);     // Eq. residual, exact
+        if (beta > 0.0f) b = quant_i8(r, beta, inv_beta);                // Eq. x2
+      }
+      q1[static_cast<int64_t>(row) * K + k] = static_cast<int8_t>(a);
+      q2[static_cast<int64_t>(row) * K + k] = static_cast<int8_t>(b);
+    }
   }
 }
 
@@ -178,18 +185,16 @@ msd_status_t launch_decompose_int8(const void* x_bf16, int64_t M, int64_t K, int
   if (M == 0) return MSD_OK;
   // A plain launch (chaining it to its predecessor as a programmatic dependent measured slower: its loads then queue
   // behind the weight prefetch of the GEMM that follows it).
-  // this kernel sits on the critical path of the GEMM behind it: more threads per row = shorter latency
-  const int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
-  cudaError_t err;
-  if (threads >= 1024)
-    err = launch_pdl(decompose_int8_kernel<1024>, dim3(static_cast<unsigned>(M)), dim3(1024), 0, stream, false,
-                     static_cast<const uint16_t*>(x_bf16), static_cast<int64_t>(ldx), static_cast<int>(K), q1, q2, alpha, beta, c1, c2);
-  else if (threads >= 512)
-    err = launch_pdl(decompose_int8_kernel<512>, dim3(static_cast<unsigned>(M)), dim3(512), 0, stream, false,
-                     static_cast<const uint16_t*>(x_bf16), static_cast<int64_t>(ldx), static_cast<int>(K), q1, q2, alpha, beta, c1, c2);
-  else
-    err = launch_pdl(decompose_int8_kernel<256>, dim3(static_cast<unsigned>(M)), dim3(256), 0, stream, false,
-                     static_cast<const uint16_t*>(x_bf16), static_cast<int64_t>(ldx), static_cast<int>(K), q1, q2, alpha, beta, c1, c2);
+  // Few rows: the kernel sits on the critical path of the GEMM behind it, and more threads per row mean a shorter
+  // latency.  Many rows: throughput counts, so a thread takes several units and many rows share an SM (1000 rows of 4096:
+  // 15 us with 128 threads a row, 20 with 64: too few warps in flight; 1000 rows of 14336: 29 us with 512, 45 before).
+  int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
+  if (M > 128) threads = K <= 4096 ? 128 : (K <= 8192 ? 256 : 512);
+  auto kernel = threads == 1024 ? decompose_int8_kernel<1024>
+              : threads == 512 ? decompose_int8_kernel<512>
+              : threads == 256 ? decompose_int8_kernel<256> : decompose_int8_kernel<128>;
+  const cudaError_t err = launch_pdl(kernel, dim3(static_cast<unsigned>(M)), dim3(static_cast<unsigned>(threads)), 0, stream, false,
+                                     static_cast<const uint16_t*>(x_bf16), ldx, static_cast<int>(K), q1, q2, alpha, beta, c1, c2);
   return err == cudaSuccess ? MSD_OK : MSD_ERR_CUDA;
 }
 

@@ -20,7 +20,6 @@
 #include <type_traits>
 
 #include "host_common.h"
-#include "quant.cuh"
 #include "sm100.cuh"
 
 namespace msd {

@@ -100,3 +100,27 @@ def test_decompose_int8_fractional_scaling_bit_exact(M, K):
                                                None)
     assert code == 4                                       # MSD_ERR_UNSUPPORTED
     binding.last_device_status()
+
+
+@pytest.mark.parametrize("M,K", [(128, 2832), (129, 2832), (256, 4112), (130, 8208), (3, 16400)])
+@pytest.mark.parametrize("fractional", [False, True])
+def test_decompose_int8_ties_bit_exact(M, K, fractional):
+    """Quotients on and next to half-integers: every BF16 mantissa at 11 exponents below row maxima that run over all
+    mantissas (short integers divide evenly far more often than random reals), at every thread count of the kernel and
+    across the limit of the range that avoids the division.  Codes equal the true division's, bit for bit."""
+    rng = np.random.default_rng(M + K)
+    top = 140                                                            # exponent field of the row maxima
+    xb = np.zeros((M, K), np.uint16)
+    for i in range(M):
+        mant, expo = np.meshgrid(np.arange(128), top - 1 - np.arange(11))
+        vals = ((expo << 7) | mant).astype(np.uint16).reshape(-1)        # all below the maximum's binade
+        vals |= (rng.integers(0, 2, vals.size) << 15).astype(np.uint16)
+        row = np.resize(vals, K)
+        row[rng.integers(0, K)] = (top << 7) | (i % 128)                 # the maximum: mantissa i
+        shift = [0, 0, 40, 90, 120, 130, 138][i % 7]                     # down to scales in the denormal range
+        e = ((row >> 7) & 255).astype(np.int32) - shift
+        xb[i] = np.where(e > 0, (row & 0x807F) | (np.maximum(e, 0) << 7), 0)
+    q1, q2, a, b = binding.decompose_int8(bf16_dev(xb), fractional=fractional)
+    o1, o2, oa, ob = oracle.decompose_int8(xb, fractional=fractional)
+    assert np.array_equal(a.cpu().numpy(), oa) and np.array_equal(b.cpu().numpy(), ob)
+    assert np.array_equal(q1.cpu().numpy(), o1) and np.array_equal(q2.cpu().numpy(), o2)
