@@ -1,7 +1,8 @@
-"""Thin ctypes binding of the C ABI in ``include/msd.h``: argument marshalling only.
+"""Thin binding of the C ABI in ``include/msd.h``: argument marshalling only.
 
 Tensors are torch CUDA tensors (torch is used for device memory and streams); every step of the path runs in
-the library's kernels.  There is no fallback: a missing library or a non-zero status raises.
+the library's kernels.  There is no fallback: a missing library or a non-zero status raises.  The linear layers and the
+decode attention go through the native call module (``_native.so``); everything else through ctypes.
 """
 from __future__ import annotations
 
@@ -25,6 +26,7 @@ class MsdError(RuntimeError):
 
 
 _lib = None
+_native = None
 _vp, _i64, _i32, _sz, _f32 = C.c_void_p, C.c_int64, C.c_int32, C.c_size_t, C.c_float
 
 _SIGS = {
@@ -81,20 +83,29 @@ _SIGS = {
 
 def lib():
     """Loads ``libmsd.so`` (building it when the sources are newer); raises when that is impossible."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         path = _build.LIB_PATH
         if _build.needs_build():
             path = _build.build()
         if not os.path.exists(path):
             raise RuntimeError("libmsd.so is missing and could not be built; there is no fallback path")
-        h = C.CDLL(path)
+        h = C.CDLL(path, mode=C.RTLD_GLOBAL)
         for name, (res, args) in _SIGS.items():
             fn = getattr(h, name)
             fn.restype = res
             fn.argtypes = args
+        from . import _native as native      # links against the library just loaded
+        _native = native
         _lib = h
     return _lib
+
+
+def _calls():
+    """The native call module (loads the library first)."""
+    if _native is None:
+        lib()
+    return _native
 
 
 def _ptr(t):
@@ -102,7 +113,7 @@ def _ptr(t):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _check(code, where):
@@ -184,64 +195,53 @@ def gemm_w8a16_workspace_bytes(M, N, K):
 
 def gemm_w8a16(x, w, w_scale, out_dtype=torch.bfloat16, ws=None, want_acc=False, out=None, fractional=False):
     """x [M,K] bf16, w [N,K] int8, w_scale [N] f32 -> y [M,N] (bf16 or f32); optional INT32 accumulators [2,M,N]."""
-    _need_cuda(x, w, w_scale)
-    M, K = x.shape
-    N = w.shape[0]
-    if ws is None:
-        ws = workspace(gemm_w8a16_workspace_bytes(M, N, K), x.device)
-    y = out if out is not None else _empty((M, N), out_dtype, x.device)
+    if ws is None or out is None or want_acc:
+        _need_cuda(x, w, w_scale)
+        M, K = x.shape
+        N = w.shape[0]
+        if ws is None:
+            ws = workspace(gemm_w8a16_workspace_bytes(M, N, K), x.device)
+        if out is None:
+            out = _empty((M, N), out_dtype, x.device)
     acc = _empty((2, M, N), torch.int32, x.device) if want_acc else None
-    wp, wb = _ws_ptr(ws)
-    yt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_FP32
-    if fractional:
-        code = lib().msd_gemm_w8a16_ex(_ptr(x), _ptr(w), _ptr(w_scale), M, N, K, _ptr(y), yt, _ptr(acc), SCALING_FRACTIONAL, wp, wb,
-                                       _stream())
-    else:
-        code = lib().msd_gemm_w8a16(_ptr(x), _ptr(w), _ptr(w_scale), M, N, K, _ptr(y), yt, _ptr(acc), wp, wb, _stream())
-    _check(code, "msd_gemm_w8a16")
-    return (y, acc) if want_acc else y
+    code = _calls().gemm_w8a16(x, w, w_scale, ws, out, acc, SCALING_FRACTIONAL if fractional else SCALING_DEFAULT)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_gemm_w8a16")
+    return (out, acc) if want_acc else out
 
 
 def grouped_gemm_w8a16(x, w, w_scale, group_sizes, out_dtype=torch.bfloat16, ws=None, out=None):
     """MoE experts: x [M_total,K] bf16 with rows sorted by expert, w [E,N,K] int8, w_scale [E,N] f32, group_sizes: E host ints
     (rows per expert, each <= 128) -> y [M_total,N]."""
-    _need_cuda(x, w, w_scale)
-    E, N, K = w.shape
-    sizes = (C.c_int32 * E)(*[int(v) for v in group_sizes])
-    M_total = int(sum(int(v) for v in group_sizes))
-    assert x.shape[0] == M_total and x.shape[1] == K
-    if ws is None:
-        ws = workspace(int(lib().msd_grouped_gemm_w8a16_workspace_bytes(M_total, max(int(v) for v in group_sizes), E, N, K)), x.device)
-    y = out if out is not None else _empty((M_total, N), out_dtype, x.device)
-    wp, wb = _ws_ptr(ws)
-    code = lib().msd_grouped_gemm_w8a16(_ptr(x), _ptr(w), _ptr(w_scale), C.cast(sizes, C.c_void_p), E, N, K, _ptr(y),
-                                        OUT_BF16 if y.dtype == torch.bfloat16 else OUT_FP32, wp, wb, _stream())
-    _check(code, "msd_grouped_gemm_w8a16")
-    return y
+    if ws is None or out is None:
+        _need_cuda(x, w, w_scale)
+        E, N, K = w.shape
+        if ws is None:
+            ws = workspace(int(lib().msd_grouped_gemm_w8a16_workspace_bytes(x.shape[0], max(int(v) for v in group_sizes), E, N, K)), x.device)
+        if out is None:
+            out = _empty((x.shape[0], N), out_dtype, x.device)
+    code = _calls().grouped_gemm_w8a16(x, w, w_scale, group_sizes, ws, out)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_grouped_gemm_w8a16")
+    return out
 
 
 def grouped_gemm_w4a16(x, w_fp4, w_e8m0, group_sizes, out_dtype=torch.bfloat16, ws=None, out=None, prepared=None):
     """MoE experts with MXFP4 weights: x [M_total,K] bf16 with rows sorted by expert, w_fp4 [E,N,K/2] u8, w_e8m0 [E,N,K/32] u8,
     group_sizes: E host ints (rows per expert, each <= 128) -> y [M_total,N].
     prepared: the result of prepare_w4a16_scales(w_e8m0); w_e8m0 may then be None."""
-    _need_cuda(x, w_fp4, prepared if prepared is not None else w_e8m0)
-    E, N, K2 = w_fp4.shape
-    K = 2 * K2
-    sizes = (C.c_int32 * E)(*[int(v) for v in group_sizes])
-    M_total = int(sum(int(v) for v in group_sizes))
-    assert x.shape[0] == M_total and x.shape[1] == K
-    if ws is None:
-        ws = workspace(int(lib().msd_grouped_gemm_w4a16_workspace_bytes(E, N, K)), x.device)
-    y = out if out is not None else _empty((M_total, N), out_dtype, x.device)
-    wp, wb = _ws_ptr(ws)
-    if prepared is not None:
-        code = lib().msd_grouped_gemm_w4a16_prepared(_ptr(x), _ptr(w_fp4), _ptr(prepared), sizes, E, N, K, _ptr(y),
-                                                     OUT_BF16 if y.dtype == torch.bfloat16 else OUT_FP32, wp, wb, _stream())
-    else:
-        code = lib().msd_grouped_gemm_w4a16(_ptr(x), _ptr(w_fp4), _ptr(w_e8m0), sizes, E, N, K, _ptr(y),
-                                            OUT_BF16 if y.dtype == torch.bfloat16 else OUT_FP32, wp, wb, _stream())
-    _check(code, "msd_grouped_gemm_w4a16")
-    return y
+    scales = w_e8m0 if prepared is None else prepared
+    if ws is None or out is None:
+        _need_cuda(x, w_fp4, scales)
+        E, N, K2 = w_fp4.shape
+        if ws is None:
+            ws = workspace(int(lib().msd_grouped_gemm_w4a16_workspace_bytes(E, N, 2 * K2)), x.device)
+        if out is None:
+            out = _empty((x.shape[0], N), out_dtype, x.device)
+    code = _calls().grouped_gemm_w4a16(x, w_fp4, scales, group_sizes, prepared is not None, ws, out)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_grouped_gemm_w4a16")
+    return out
 
 
 def gemm_w8a16_noalloc(x, w, w_scale, out):
@@ -325,20 +325,19 @@ def prepare_w4a16_scales(w_e8m0):
 
 def gemm_w4a16(x, w_fp4, w_e8m0, out_dtype=torch.bfloat16, ws=None, out=None, prepared=None):
     """prepared: the result of prepare_w4a16_scales(w_e8m0); w_e8m0 may then be None."""
-    _need_cuda(x, w_fp4, prepared if prepared is not None else w_e8m0)
-    M, K = x.shape
-    N = w_fp4.shape[0]
-    if ws is None:
-        ws = workspace(gemm_w4a16_workspace_bytes(M, N, K), x.device)
-    y = out if out is not None else _empty((M, N), out_dtype, x.device)
-    wp, wb = _ws_ptr(ws)
-    yt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_FP32
-    if prepared is not None:
-        _check(lib().msd_gemm_w4a16_prepared(_ptr(x), _ptr(w_fp4), _ptr(prepared), M, N, K, _ptr(y), yt, wp, wb, _stream()),
-               "msd_gemm_w4a16_prepared")
-    else:
-        _check(lib().msd_gemm_w4a16(_ptr(x), _ptr(w_fp4), _ptr(w_e8m0), M, N, K, _ptr(y), yt, wp, wb, _stream()), "msd_gemm_w4a16")
-    return y
+    scales = w_e8m0 if prepared is None else prepared
+    if ws is None or out is None:
+        _need_cuda(x, w_fp4, scales)
+        M, K = x.shape
+        N = w_fp4.shape[0]
+        if ws is None:
+            ws = workspace(gemm_w4a16_workspace_bytes(M, N, K), x.device)
+        if out is None:
+            out = _empty((M, N), out_dtype, x.device)
+    code = _calls().gemm_w4a16(x, w_fp4, scales, prepared is not None, ws, out)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_gemm_w4a16")
+    return out
 
 
 def attn_decode_schedule(B, Hq, Hkv, D, Dv, max_seqlen):
@@ -420,18 +419,16 @@ def gemm_w4a16_e1m2(x, w_fp4, w_e8m0, out_dtype=torch.bfloat16, ws=None, out=Non
 
 def attn_decode_int8kv_spec(q, k, v, k_scale, v_scale, cu_seqlens, max_seqlen, softmax_scale, dv=None, ws=None, want_lse=False):
     """q [B,Sq,Hq,D] bf16: the last Sq tokens of every sequence query its cache causally -> out [B,Sq,Hq,Dv]."""
-    _need_cuda(q, k, v, k_scale, v_scale, cu_seqlens)
     B, Sq, Hq, D = q.shape
-    Hkv = k.shape[1]
     Dv = v.shape[2] if v is not None else int(dv)
     if ws is None:
-        ws = workspace(attn_decode_int8kv_workspace_bytes(B, Hq * Sq, Hkv, D, Dv, max_seqlen), q.device)
+        _need_cuda(q, k)
+        ws = workspace(attn_decode_int8kv_workspace_bytes(B, Hq * Sq, k.shape[1], D, Dv, max_seqlen), q.device)
     o = _empty((B, Sq, Hq, Dv), torch.bfloat16, q.device)
     lse = _empty((B, Sq, Hq), torch.float32, q.device) if want_lse else None
-    wp, wb = _ws_ptr(ws)
-    code = lib().msd_attn_decode_int8kv_spec(_ptr(q), _ptr(k), _ptr(v), _ptr(k_scale), _ptr(v_scale), _ptr(cu_seqlens), int(k.shape[0]),
-                                             max_seqlen, B, Sq, Hq, Hkv, D, Dv, softmax_scale, _ptr(o), _ptr(lse), wp, wb, _stream())
-    _check(code, "msd_attn_decode_int8kv_spec")
+    code = _calls().attn_decode_int8kv_spec(q, k, v, k_scale, v_scale, cu_seqlens, max_seqlen, softmax_scale, Dv, ws, o, lse)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_attn_decode_int8kv_spec")
     return (o, lse) if want_lse else o
 
 
@@ -439,21 +436,22 @@ def attn_decode_int8kv_paged(q, k, v, k_scale, v_scale, block_table, seqlens, pa
                              ws=None, want_lse=False, out=None):
     """Paged cache: k [num_blocks*page, Hkv, D] int8, v likewise or None, scales [num_blocks*page, Hkv] f32,
     block_table [B, max_blocks] int32, seqlens [B] int32."""
-    _need_cuda(q, k, v, k_scale, v_scale, block_table, seqlens)
-    B, Hq, D = q.shape
-    Hkv = k.shape[1]
-    Dv = v.shape[2] if v is not None else dv
-    nblk = k.shape[0] // page_size
-    if ws is None:
-        ws = workspace(attn_decode_int8kv_workspace_bytes(B, Hq, Hkv, D, Dv, max_seqlen), q.device)
-    o = out if out is not None else _empty((B, Hq, Dv), torch.bfloat16, q.device)
-    lse = _empty((B, Hq), torch.float32, q.device) if want_lse else None
-    wp, wb = _ws_ptr(ws)
-    code = lib().msd_attn_decode_int8kv_paged(_ptr(q), _ptr(k), _ptr(v), _ptr(k_scale), _ptr(v_scale), _ptr(block_table), _ptr(seqlens),
-                                              nblk, page_size, block_table.shape[1], max_seqlen, B, Hq, Hkv, D, Dv, softmax_scale,
-                                              _ptr(o), _ptr(lse), wp, wb, _stream())
-    _check(code, "msd_attn_decode_int8kv_paged")
-    return (o, lse) if want_lse else o
+    Dv = v.shape[2] if v is not None else int(dv)
+    lse = None
+    if ws is None or out is None or want_lse:
+        _need_cuda(q, k)
+        B, Hq, D = q.shape
+        if ws is None:
+            ws = workspace(attn_decode_int8kv_workspace_bytes(B, Hq, k.shape[1], D, Dv, max_seqlen), q.device)
+        if out is None:
+            out = _empty((B, Hq, Dv), torch.bfloat16, q.device)
+        if want_lse:
+            lse = _empty((B, Hq), torch.float32, q.device)
+    code = _calls().attn_decode_int8kv_paged(q, k, v, k_scale, v_scale, block_table, seqlens, page_size, max_seqlen, softmax_scale, Dv, ws,
+                                             out, lse)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_attn_decode_int8kv_paged")
+    return (out, lse) if want_lse else out
 
 
 def kv_dequant_bf16(cache, scale, out=None):
@@ -491,16 +489,18 @@ def attn_decode_int8kv_workspace_bytes(B, Hq, Hkv, D, Dv, max_seqlen):
 def attn_decode_int8kv(q, k, v, k_scale, v_scale, cu_seqlens, max_seqlen, softmax_scale, dv=None, ws=None, want_lse=False,
                        out=None):
     """q [B,Hq,D] bf16; k [T,Hkv,D] int8; v [T,Hkv,Dv] int8 or None; scales [T,Hkv] f32; cu_seqlens [B+1] int32."""
-    _need_cuda(q, k, v, k_scale, v_scale, cu_seqlens)
-    B, Hq, D = q.shape
-    Hkv = k.shape[1]
     Dv = v.shape[2] if v is not None else int(dv)
-    if ws is None:
-        ws = workspace(attn_decode_int8kv_workspace_bytes(B, Hq, Hkv, D, Dv, max_seqlen), q.device)
-    o = out if out is not None else _empty((B, Hq, Dv), torch.bfloat16, q.device)
-    lse = _empty((B, Hq), torch.float32, q.device) if want_lse else None
-    wp, wb = _ws_ptr(ws)
-    code = lib().msd_attn_decode_int8kv(_ptr(q), _ptr(k), _ptr(v), _ptr(k_scale), _ptr(v_scale), _ptr(cu_seqlens), int(k.shape[0]),
-                                        max_seqlen, B, Hq, Hkv, D, Dv, softmax_scale, _ptr(o), _ptr(lse), wp, wb, _stream())
-    _check(code, "msd_attn_decode_int8kv")
-    return (o, lse) if want_lse else o
+    lse = None
+    if ws is None or out is None or want_lse:
+        _need_cuda(q, k)
+        B, Hq, D = q.shape
+        if ws is None:
+            ws = workspace(attn_decode_int8kv_workspace_bytes(B, Hq, k.shape[1], D, Dv, max_seqlen), q.device)
+        if out is None:
+            out = _empty((B, Hq, Dv), torch.bfloat16, q.device)
+        if want_lse:
+            lse = _empty((B, Hq), torch.float32, q.device)
+    code = _calls().attn_decode_int8kv(q, k, v, k_scale, v_scale, cu_seqlens, max_seqlen, softmax_scale, Dv, ws, out, lse)
+    if code != MSD_OK:
+        raise MsdError(code, "msd_attn_decode_int8kv")
+    return (out, lse) if want_lse else out

@@ -1,7 +1,8 @@
-"""Builds the CUDA library in-tree: ``libmsd.so`` next to this file, for sm_100a only.
+"""Builds the native code in-tree: the CUDA library ``libmsd.so`` (sm_100a only) and the call module ``_native.so`` next
+to this file.
 
 Every ``csrc/*.cu`` is compiled to an object of its own (in parallel, and only when it or a header changed), then the
-objects are linked into one shared library.
+objects are linked into one shared library; ``csrc/native_call.cpp`` marshals torch tensors into its calls.
 """
 from __future__ import annotations
 
@@ -14,6 +15,8 @@ from concurrent.futures import ThreadPoolExecutor
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libmsd.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
+NATIVE_SRC = os.path.join(_HERE, "csrc", "native_call.cpp")
 OBJ_DIR = os.path.join(_HERE, "build")
 
 NVCC_FLAGS = [
@@ -35,7 +38,32 @@ def needs_build() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(d) > t for d in sources() + _headers())
+    return any(os.path.getmtime(d) > t for d in sources() + _headers()) or _native_stale()
+
+
+def _native_stale() -> bool:
+    if not os.path.exists(NATIVE_PATH):
+        return True
+    t = os.path.getmtime(NATIVE_PATH)
+    return any(os.path.getmtime(d) > t for d in (NATIVE_SRC, os.path.join(_ROOT, "include", "msd.h")))
+
+
+def _build_native():
+    """The call module: a CPython extension against torch's headers, linked to libmsd.so beside it."""
+    import sysconfig
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++20", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), NATIVE_SRC, "-o", NATIVE_PATH,
+           "-I", os.path.join(_ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+           "-isystem", os.path.join(troot, "include"), "-isystem", os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+           "-isystem", os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include"),
+           "-L", _HERE, "-l:libmsd.so", "-Wl,-rpath,$ORIGIN",
+           "-L", os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("building _native.so failed")
 
 
 def _obj(src):
@@ -70,12 +98,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
         failed = failed or rc != 0
     if failed:
         raise RuntimeError("nvcc failed")
-    link = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-cudart", "static", "-o", LIB_PATH] + \
-        [_obj(s) for s in srcs]
+    link = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-cudart", "static", "-o", LIB_PATH,
+            "-Xlinker", "-soname=libmsd.so"] + [_obj(s) for s in srcs]
     res = subprocess.run(link, capture_output=True, text=True)
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("nvcc link failed")
+    if force or _native_stale():
+        _build_native()
     return LIB_PATH
 
 

@@ -1,0 +1,242 @@
+// Argument marshalling of the hot entry points in native code (the module paper_2605_13915_b200._native): a call takes torch
+// tensors, checks them, and passes their addresses, sizes and the current CUDA stream to the C ABI of msd.h.
+//
+// Why: through ctypes a decode-sized linear layer cost 18 us of host time, of which the library itself (argument checks,
+// tensor maps, two kernel launches) is 5; looking up the stream alone took 3.4 us.  The kernels of such a layer run for
+// 12 to 20 us, so it was the host that set the pace.  Only marshalling lives here: every call returns the status code of
+// the C function and binding.py turns it into an exception, allocates outputs and workspaces, and documents the arguments.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <vector>
+
+#include "msd.h"
+
+namespace {
+
+// One call's arguments, taken off the array in order; the first problem sets a Python exception and every later take
+// returns an empty value.
+class Args {
+ public:
+  Args(PyObject* const* a, Py_ssize_t n) : a_(a), n_(n) {}
+  bool ok() const { return ok_; }
+
+  const at::Tensor* tensor(bool nullable = false, bool device = true) {
+    PyObject* o = next();
+    if (!o) return nullptr;
+    if (o == Py_None && nullable) return nullptr;
+    if (!THPVariable_Check(o)) {
+      fail(PyExc_TypeError, "expected a tensor");
+      return nullptr;
+    }
+    const at::Tensor& t = THPVariable_Unpack(o);
+    if (device && (!t.is_cuda() || !t.is_contiguous())) {
+      fail(PyExc_ValueError, "expected contiguous CUDA tensors");
+      return nullptr;
+    }
+    return &t;
+  }
+  int64_t integer() {
+    PyObject* o = next();
+    if (!o) return 0;
+    const long long v = PyLong_AsLongLong(o);
+    if (v == -1 && PyErr_Occurred()) ok_ = false;
+    return v;
+  }
+  double number() {
+    PyObject* o = next();
+    if (!o) return 0.0;
+    const double v = PyFloat_AsDouble(o);
+    if (v == -1.0 && PyErr_Occurred()) ok_ = false;
+    return v;
+  }
+  void fail(PyObject* type, const char* what) {
+    if (ok_) PyErr_SetString(type, what);
+    ok_ = false;
+  }
+
+ private:
+  PyObject* next() {
+    if (!ok_) return nullptr;
+    if (i_ >= n_) {
+      fail(PyExc_TypeError, "too few arguments");
+      return nullptr;
+    }
+    return a_[i_++];
+  }
+  PyObject* const* a_;
+  Py_ssize_t n_, i_ = 0;
+  bool ok_ = true;
+};
+
+void* addr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
+template <typename T>
+T* addr_as(const at::Tensor* t) { return static_cast<T*>(addr(t)); }
+msd_out_t out_type(const at::Tensor* y) { return y->scalar_type() == at::kBFloat16 ? MSD_OUT_BF16 : MSD_OUT_FP32; }
+void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+
+// The workspace a tensor of bytes offers: from its first 1024-byte boundary on.
+struct Workspace {
+  void* p;
+  size_t bytes;
+  explicit Workspace(const at::Tensor* t) {
+    const uintptr_t base = reinterpret_cast<uintptr_t>(t->data_ptr()), al = (base + 1023) / 1024 * 1024;
+    p = reinterpret_cast<void*>(al);
+    bytes = static_cast<size_t>(t->numel()) - (al - base);
+  }
+};
+
+PyObject* status(msd_status_t s) { return PyLong_FromLong(static_cast<long>(s)); }
+
+bool dims(Args& a, std::initializer_list<std::pair<const at::Tensor*, int>> want) {
+  if (!a.ok()) return false;
+  for (const auto& w : want)
+    if (w.first->dim() != w.second) {
+      a.fail(PyExc_ValueError, "a tensor has the wrong number of dimensions");
+      return false;
+    }
+  return true;
+}
+
+// (x, w, w_scale, ws, y, acc or None, scaling)
+PyObject* gemm_w8a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  Args a(args, n);
+  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(), *ws = a.tensor(false, false), *y = a.tensor(false, false),
+                   *acc = a.tensor(true, false);
+  const int64_t scaling = a.integer();
+  if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
+  const Workspace k(ws);
+  return status(msd_gemm_w8a16_ex(addr(x), addr_as<int8_t>(w), addr_as<float>(s), x->size(0), w->size(0), x->size(1), addr(y), out_type(y),
+                                  addr_as<int32_t>(acc), static_cast<msd_scaling_t>(scaling), k.p, k.bytes, stream()));
+}
+
+// (x, w_fp4, scales, prepared, ws, y)
+PyObject* gemm_w4a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  Args a(args, n);
+  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor();
+  const bool prepared = a.integer() != 0;
+  const at::Tensor *ws = a.tensor(false, false), *y = a.tensor(false, false);
+  if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
+  const Workspace k(ws);
+  const auto fn = prepared ? msd_gemm_w4a16_prepared : msd_gemm_w4a16;
+  return status(fn(addr(x), addr_as<uint8_t>(w), addr_as<uint8_t>(s), x->size(0), w->size(0), x->size(1), addr(y), out_type(y), k.p, k.bytes,
+                   stream()));
+}
+
+// Rows per expert from a Python sequence; their sum must be the number of rows of x.
+bool group_sizes(Args& a, PyObject* seq, int64_t E, int64_t rows, std::vector<int32_t>& out) {
+  PyObject* fast = PySequence_Fast(seq, "group_sizes: expected a sequence");
+  if (!fast) return false;
+  int64_t sum = 0;
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast);
+  out.reserve(static_cast<size_t>(E));
+  for (Py_ssize_t i = 0; i < n; ++i) {
+    const long v = PyLong_AsLong(PySequence_Fast_GET_ITEM(fast, i));
+    if (v == -1 && PyErr_Occurred()) {
+      Py_DECREF(fast);
+      return false;
+    }
+    out.push_back(static_cast<int32_t>(v));
+    sum += v;
+  }
+  Py_DECREF(fast);
+  if (n != E || sum != rows) {
+    a.fail(PyExc_AssertionError, "group_sizes: one per expert, adding up to the rows of x");
+    return false;
+  }
+  return true;
+}
+
+// (x, w, w_scale, group_sizes, ws, y)
+PyObject* grouped_gemm_w8a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  if (n != 6) return PyErr_Format(PyExc_TypeError, "expected 6 arguments");
+  Args t(args, 3), u(args + 4, 2);
+  const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
+  if (!dims(t, {{x, 2}, {w, 3}})) return nullptr;
+  const at::Tensor *ws = u.tensor(false, false), *y = u.tensor(false, false);
+  std::vector<int32_t> sizes;
+  if (!u.ok() || !group_sizes(u, args[3], w->size(0), x->size(0), sizes)) return nullptr;
+  if (x->size(1) != w->size(2)) return PyErr_Format(PyExc_AssertionError, "x and w differ in K");
+  const Workspace k(ws);
+  return status(msd_grouped_gemm_w8a16(addr(x), addr_as<int8_t>(w), addr_as<float>(s), sizes.data(), static_cast<int32_t>(w->size(0)),
+                                       w->size(1), w->size(2), addr(y), out_type(y), k.p, k.bytes, stream()));
+}
+
+// (x, w_fp4, scales, group_sizes, prepared, ws, y)
+PyObject* grouped_gemm_w4a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  if (n != 7) return PyErr_Format(PyExc_TypeError, "expected 7 arguments");
+  Args t(args, 3), u(args + 4, 3);
+  const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
+  if (!dims(t, {{x, 2}, {w, 3}})) return nullptr;
+  const bool prepared = u.integer() != 0;
+  const at::Tensor *ws = u.tensor(false, false), *y = u.tensor(false, false);
+  std::vector<int32_t> sizes;
+  if (!u.ok() || !group_sizes(u, args[3], w->size(0), x->size(0), sizes)) return nullptr;
+  if (x->size(1) != 2 * w->size(2)) return PyErr_Format(PyExc_AssertionError, "x and w_fp4 differ in K");
+  const Workspace k(ws);
+  const auto fn = prepared ? msd_grouped_gemm_w4a16_prepared : msd_grouped_gemm_w4a16;
+  return status(fn(addr(x), addr_as<uint8_t>(w), addr_as<uint8_t>(s), sizes.data(), static_cast<int32_t>(w->size(0)), w->size(1),
+                   2 * w->size(2), addr(y), out_type(y), k.p, k.bytes, stream()));
+}
+
+// (q, k, v or None, k_scale, v_scale or None, cu_seqlens, max_seqlen, softmax_scale, Dv, ws, out, lse or None);
+// q is [B, Hq, D], or with `spec` (several query tokens) [B, q_len, Hq, D]
+template <bool spec>
+PyObject* attn_decode(PyObject* const* args, Py_ssize_t n) {
+  Args a(args, n);
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(), *vs = a.tensor(true), *cu = a.tensor();
+  const int32_t max_seqlen = static_cast<int32_t>(a.integer());
+  const float scale = static_cast<float>(a.number());
+  const int32_t Dv = static_cast<int32_t>(a.integer());
+  const at::Tensor *ws = a.tensor(false, false), *out = a.tensor(false, false), *lse = a.tensor(true, false);
+  constexpr int rank = spec ? 4 : 3;
+  if (!dims(a, {{q, rank}, {k, 3}})) return nullptr;
+  const Workspace w(ws);
+  const int32_t B = static_cast<int32_t>(q->size(0)), Hq = static_cast<int32_t>(q->size(rank - 2)), D = static_cast<int32_t>(q->size(rank - 1));
+  const int32_t Hkv = static_cast<int32_t>(k->size(1));
+  if constexpr (!spec)
+    return status(msd_attn_decode_int8kv(addr(q), addr_as<int8_t>(k), addr_as<int8_t>(v), addr_as<float>(ks), addr_as<float>(vs),
+                                         addr_as<int32_t>(cu), k->size(0), max_seqlen, B, Hq, Hkv, D, Dv, scale, addr(out),
+                                         addr_as<float>(lse), w.p, w.bytes, stream()));
+  return status(msd_attn_decode_int8kv_spec(addr(q), addr_as<int8_t>(k), addr_as<int8_t>(v), addr_as<float>(ks), addr_as<float>(vs),
+                                            addr_as<int32_t>(cu), k->size(0), max_seqlen, B, static_cast<int32_t>(q->size(1)), Hq, Hkv, D,
+                                            Dv, scale, addr(out), addr_as<float>(lse), w.p, w.bytes, stream()));
+}
+
+PyObject* attn_decode_int8kv(PyObject*, PyObject* const* args, Py_ssize_t n) { return attn_decode<false>(args, n); }
+PyObject* attn_decode_int8kv_spec(PyObject*, PyObject* const* args, Py_ssize_t n) { return attn_decode<true>(args, n); }
+
+// (q, k, v or None, k_scale, v_scale or None, block_table, seqlens, page_size, max_seqlen, softmax_scale, Dv, ws, out, lse or None)
+PyObject* attn_decode_int8kv_paged(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  Args a(args, n);
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(), *vs = a.tensor(true), *table = a.tensor(),
+                   *len = a.tensor();
+  const int32_t page = static_cast<int32_t>(a.integer()), max_seqlen = static_cast<int32_t>(a.integer());
+  const float scale = static_cast<float>(a.number());
+  const int32_t Dv = static_cast<int32_t>(a.integer());
+  const at::Tensor *ws = a.tensor(false, false), *out = a.tensor(false, false), *lse = a.tensor(true, false);
+  if (!dims(a, {{q, 3}, {k, 3}, {table, 2}})) return nullptr;
+  if (page < 1) return PyErr_Format(PyExc_ValueError, "page_size must be positive");
+  const Workspace w(ws);
+  return status(msd_attn_decode_int8kv_paged(
+      addr(q), addr_as<int8_t>(k), addr_as<int8_t>(v), addr_as<float>(ks), addr_as<float>(vs), addr_as<int32_t>(table), addr_as<int32_t>(len),
+      k->size(0) / page, page, static_cast<int32_t>(table->size(1)), max_seqlen, static_cast<int32_t>(q->size(0)),
+      static_cast<int32_t>(q->size(1)), static_cast<int32_t>(k->size(1)), static_cast<int32_t>(q->size(2)), Dv, scale, addr(out),
+      addr_as<float>(lse), w.p, w.bytes, stream()));
+}
+
+PyMethodDef methods[] = {
+#define MSD_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(name)), METH_FASTCALL, nullptr}
+    MSD_METHOD(gemm_w8a16), MSD_METHOD(gemm_w4a16), MSD_METHOD(grouped_gemm_w8a16), MSD_METHOD(grouped_gemm_w4a16),
+    MSD_METHOD(attn_decode_int8kv), MSD_METHOD(attn_decode_int8kv_spec), MSD_METHOD(attn_decode_int8kv_paged),
+#undef MSD_METHOD
+    {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }
