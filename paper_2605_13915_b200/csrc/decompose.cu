@@ -25,9 +25,11 @@ __global__ void __launch_bounds__(kThreads, kThreads == 1024 ? 1 : 1280 / kThrea
 decompose_int8_kernel(const uint16_t* __restrict__ x, int64_t ldx, int K, int8_t* __restrict__ q1,
                       int8_t* __restrict__ q2, float* __restrict__ alpha_out, float* __restrict__ beta_out,
                       float c1, float c2) {
-  // the GEMM launched behind this kernel as its programmatic dependent may become resident now and prefetch weights
+  // x may be the output of the preceding kernel, q1 / q2 its input.  Only then may the GEMM launched behind this kernel as
+  // its programmatic dependent become resident: it asks for weights at once, and they too may have been written by what
+  // precedes this kernel.  (Letting it in before the wait gained 1.5 us at 4096 x 4096 and nothing on larger weights.)
+  pdl_wait_primary();
   pdl_launch_dependents();
-  pdl_wait_primary();          // x may be the output of the preceding kernel, q1 / q2 its input
   const int row = blockIdx.x;
   const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<int64_t>(row) * ldx);
   const int units = K >> 3;
@@ -101,6 +103,7 @@ __global__ void __launch_bounds__(kMxThreads)
 decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, int K, uint8_t* __restrict__ q1,
                        uint8_t* __restrict__ q2, uint8_t* __restrict__ e1, uint8_t* __restrict__ e2, int sf_kgroups,
                        const SfRelayout rl, const RowGroups rg) {
+  pdl_wait_primary();            // as in decompose_int8_kernel
   pdl_launch_dependents();
   const int kblocks = K >> 5;
   const int64_t nblocks = M * kblocks;
@@ -186,7 +189,7 @@ msd_status_t launch_decompose_int8(const void* x_bf16, int64_t M, int64_t K, int
   if (M == 0) return MSD_OK;
   // A programmatic dependent of whatever precedes it (in a chain of layers: the previous layer's GEMM), so that its launch
   // and the launch of the GEMM behind it are over when that kernel ends; launched plainly, 4 to 5 us passed between two
-  // GEMMs in which no weights moved (16 tokens, 4096 x 4096: 14.9 us a call, now 11.5; 1 token, 14336 x 4096: 18.6, 16.4).
+  // GEMMs in which no weights moved (16 tokens, 4096 x 4096: 14.9 us a call, now 13.2; 1 token, 14336 x 4096: 18.6, 16.9).
   // Few rows: the kernel sits on the critical path of the GEMM behind it, and more threads per row mean a shorter
   // latency.  Many rows: throughput counts, so a thread takes several units and many rows share an SM (1000 rows of 4096:
   // 15 us with 128 threads a row, 20 with 64: too few warps in flight; 1000 rows of 14336: 29 us with 512, 45 before).
@@ -223,9 +226,9 @@ msd_status_t launch_decompose_mxfp4(const void* x_bf16, int64_t M, int64_t K, in
     cudaFuncSetAttribute(decompose_mxfp4_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     carve_done = true;
   }
-  decompose_mxfp4_kernel<<<grid, kMxThreads, 0, stream>>>(static_cast<const uint16_t*>(x_bf16), ldx, M,
-                                                          static_cast<int>(K), q1, q2, e1, e2, sf_kgroups, rl, rg);
-  return launch_status();
+  const cudaError_t err = launch_pdl(decompose_mxfp4_kernel, dim3(grid), dim3(kMxThreads), 0, stream, option(OPT_NO_PDL) <= 0,
+                                     static_cast<const uint16_t*>(x_bf16), ldx, M, static_cast<int>(K), q1, q2, e1, e2, sf_kgroups, rl, rg);
+  return err == cudaSuccess ? MSD_OK : MSD_ERR_CUDA;
 }
 
 }  // namespace msd

@@ -38,6 +38,7 @@ struct GemmW4Params {
   const uint8_t* sfa1;
   const uint8_t* sfa2;
   const uint8_t* sfb;
+  int sfb_ready;                // sfb was laid out before this call (msd_prepare_w4a16_scales), not by the kernel launched just before
   void* y;
   int ytype;
   int ksplit, kper;             // K splits per output tile and K stages per split (1, kstages: no split)
@@ -146,37 +147,71 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     // refill to be requested is part of the pipeline's round trip.  Warp 0 requests the operand tiles, warp 10 the
     // scale blocks (their bytes may be counted before warp 0's arrival announces them: the phase cannot end without it).
     if (lane == 0) {
-      // components and blocked scales come from the kernel launched just before
       bool ok = true;
-      pdl_wait_primary();
-      int stage = 0; uint32_t phase = 0;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int split = tile % p.ksplit, tile_mn = tile / p.ksplit;
-        const int mt = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % p.m_tiles, nt = p.n_fastest ? tile_mn % p.n_tiles : tile_mn / p.m_tiles;
-        const int ks0 = split * p.kper, ks1 = ks0 + p.kper < p.kstages ? ks0 + p.kper : p.kstages;
-        for (int ks = ks0; ks < ks1; ++ks) {
-          ok = wait_bounded(&empty_bar[stage], phase ^ 1, abort, p.status);
-          if (!ok) break;
-          uint8_t* dst = smem + stage * kStageBytes;
-          if (warp == 0) {
-            mbar_arrive_expect_tx(&full_bar[stage], kStageBytes);
-            tma_load_2d(dst, &tmap_a1, ks * 128, mt * kW4TileM, &full_bar[stage]);
-            tma_load_2d(dst + a_bytes, &tmap_a2, ks * 128, mt * kW4TileM, &full_bar[stage]);
-            int b_row = nt * kTN;
-            if constexpr (kGrouped) b_row += grp.expert[mt] * p.N;          // the weights of the group's expert
-            tma_load_2d(dst + 2 * a_bytes, &tmap_b, ks * 128, b_row, &full_bar[stage]);
-          } else {
-            uint8_t* sf = dst + 2 * a_bytes + kBBytes;
-            const size_t a_off = (static_cast<size_t>(mt) * p.sf_kgroups + 2 * ks) * 512;
-            bulk_load(sf, p.sfa1 + a_off, 1024, &full_bar[stage]);
-            bulk_load(sf + 1024, p.sfa2 + a_off, 1024, &full_bar[stage]);
-            size_t sfb_blk = static_cast<size_t>(2 * nt);
-            if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[mt]) * 2 * p.n_tiles;
-            bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * ks) * 512, 1024, &full_bar[stage]);
-            bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * ks) * 512, 1024, &full_bar[stage]);
-          }
-          if (++stage == nstages) { stage = 0; phase ^= 1; }
+      // What a stage needs of the weights (the tile; with prepared scales its scale blocks) and of the activations.
+      struct Pos { int tile, ks, ks1, mt, nt; };
+      auto enter = [&](Pos& q) {                   // the first K stage of the work item q.tile
+        const int split = q.tile % p.ksplit, tile_mn = q.tile / p.ksplit;
+        q.mt = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % p.m_tiles;
+        q.nt = p.n_fastest ? tile_mn % p.n_tiles : tile_mn / p.m_tiles;
+        q.ks = split * p.kper;
+        q.ks1 = q.ks + p.kper < p.kstages ? q.ks + p.kper : p.kstages;
+      };
+      auto advance = [&](Pos& q) {
+        if (++q.ks < q.ks1) return;
+        q.tile += gridDim.x;
+        if (q.tile < total_tiles) enter(q);
+      };
+      auto load_weights = [&](const Pos& q, int stage) {
+        uint8_t* dst = smem + stage * kStageBytes;
+        if (warp == 0) {
+          mbar_arrive_expect_tx(&full_bar[stage], kStageBytes);
+          int b_row = q.nt * kTN;
+          if constexpr (kGrouped) b_row += grp.expert[q.mt] * p.N;          // the weights of the group's expert
+          tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, b_row, &full_bar[stage]);
+        } else {
+          uint8_t* sf = dst + 2 * a_bytes + kBBytes;
+          size_t sfb_blk = static_cast<size_t>(2 * q.nt);
+          if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[q.mt]) * 2 * p.n_tiles;
+          bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
+          bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
         }
+      };
+      auto load_activations = [&](const Pos& q, int stage) {
+        uint8_t* dst = smem + stage * kStageBytes;
+        if (warp == 0) {
+          tma_load_2d(dst, &tmap_a1, q.ks * 128, q.mt * kW4TileM, &full_bar[stage]);
+          tma_load_2d(dst + a_bytes, &tmap_a2, q.ks * 128, q.mt * kW4TileM, &full_bar[stage]);
+        } else {
+          uint8_t* sf = dst + 2 * a_bytes + kBBytes;
+          const size_t a_off = (static_cast<size_t>(q.mt) * p.sf_kgroups + 2 * q.ks) * 512;
+          bulk_load(sf, p.sfa1 + a_off, 1024, &full_bar[stage]);
+          bulk_load(sf + 1024, p.sfa2 + a_off, 1024, &full_bar[stage]);
+        }
+      };
+      // (This kernel lets no dependent in early: the waiting decomposition of a next call beside it cost 2 us on 32 experts.)
+      // The first stages' weights are asked for before the kernel launched just before (the decomposition) has ended; the
+      // components and scales it writes - unprepared weight scales among them - after it.
+      Pos q;
+      q.tile = blockIdx.x;
+      enter(q);                                    // (the grid has no more CTAs than work items)
+      const Pos first = q;
+      const bool early = warp == 0 || p.sfb_ready;
+      if (!early) pdl_wait_primary();
+      int pre = 0;
+      for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
+      if (early) pdl_wait_primary();
+      q = first;
+      for (int i = 0; i < pre; ++i) { load_activations(q, i); advance(q); }
+      int stage = pre == nstages ? 0 : pre;
+      uint32_t phase = pre == nstages ? 1 : 0;
+      while (q.tile < total_tiles) {
+        ok = wait_bounded(&empty_bar[stage], phase ^ 1, abort, p.status);
+        if (!ok) break;
+        load_weights(q, stage);
+        load_activations(q, stage);
+        advance(q);
+        if (++stage == nstages) { stage = 0; phase ^= 1; }
       }
     }
   } else if (warp == 1) {
@@ -870,7 +905,7 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
   GemmW4Params p;
   p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
   p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.kstages = pl.kstages; p.sf_kgroups = pl.sf_kgroups;
-  p.sfa1 = ws + pl.off_sfa1; p.sfa2 = ws + pl.off_sfa2; p.sfb = sfb;
+  p.sfa1 = ws + pl.off_sfa1; p.sfa2 = ws + pl.off_sfa2; p.sfb = sfb; p.sfb_ready = prepared != nullptr;
   p.y = y; p.ytype = ytype; p.status = status;
   p.a_rows = kW4TileM; p.nstages = kW4Stages; p.ksplit = 1; p.kper = pl.kstages; p.part_rows = 0;
   {
@@ -1055,7 +1090,7 @@ static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w
     GemmW4Params p;
     p.M = static_cast<int>(M_total); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
     p.m_tiles = grp.n; p.n_tiles = pl.n_tiles; p.kstages = pl.kstages; p.sf_kgroups = pl.sf_kgroups;
-    p.sfa1 = ws + pl.off_sfa1; p.sfa2 = ws + pl.off_sfa2; p.sfb = sfb;
+    p.sfa1 = ws + pl.off_sfa1; p.sfa2 = ws + pl.off_sfa2; p.sfb = sfb; p.sfb_ready = prepared != nullptr;
     p.y = y; p.ytype = ytype; p.status = status;
     p.a_rows = a_rows; p.nstages = nstages;
     p.ksplit = 1; p.kper = pl.kstages; p.part_rows = 0;
