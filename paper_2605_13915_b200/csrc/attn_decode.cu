@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 #include <cstdlib>
 
 #include "host_common.h"
@@ -471,63 +472,101 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 
   if (warp == 0) {
     // ------------------------------ TMA producer: K (and V) tiles ------------------------------
-    if (lane == 0) {
-      // K tiles and (when V is a separate cache) V tiles travel in rings of their own: a K buffer is free again as
-      // soon as QK^T has read it, long before the PV product of the same tile releases the V buffer, so the next K
-      // tile can be fetched that much earlier.  With V aliased to the K rows there is only the K ring.
-      const int k_bytes = p.DC * kChunkBytes, v_bytes = p.DVT * kChunkBytes;
+    // K tiles and (when V is a separate cache) V tiles travel in rings of their own: a K buffer is free again as
+    // soon as QK^T has read it, long before the PV product of the same tile releases the V buffer, so the next K
+    // tile can be fetched that much earlier.  With V aliased to the K rows there is only the K ring.
+    //
+    // Paged, with pages of fewer than 64 tokens, the whole warp takes part: lane g looks after page g of a tile (at most
+    // 16), and reads its table entry for the next tile as soon as it has used the one in hand.  One thread that
+    // issued the boxes one by one, each after a look-up, was what paced small pages (16 tokens, 32 sequences of 2048 to
+    // 4096: 68.4 -> 56.5 us).  From 64 tokens on there are one or two boxes and the lone thread is 3 % faster (54.8 against
+    // 56.4 us at 128), as it is on a contiguous cache.
+    auto produce = [&](auto whole_warp) {
+      constexpr bool kWarp = decltype(whole_warp)::value;
       AttnWalk wk = w0, wv = w0;                 // where the next K / V tile comes from
       int kq = 0, vq = p.v_alias ? total_tiles : 0;
-      // the tile at walk position w: chunks [0, nchunks) of the rows of KV head hk into dst
       const int hk = w0.u / p.groups;
-      auto load_tile = [&](const AttnWalk& w, const CUtensorMap* tmap, int nchunks, uint8_t* dst, uint64_t* bar) {
-        const int u0 = w.t * kTok;
+      auto pages_of = [&](const AttnWalk& w) {   // pages of the tile at w that hold tokens of the sequence
+        return min(kTok >> p.page_shift, (w.L - w.t * kTok + p.page - 1) >> p.page_shift);
+      };
+      auto table_of = [&](const AttnWalk& w) {   // the tile's first entry of the block table
+        return p.block_table + static_cast<long long>(w.b) * p.max_blocks + ((w.t * kTok) >> p.page_shift);
+      };
+      auto entry_of = [&](const AttnWalk& w, int left) -> int {      // kWarp: this lane's page of that tile (left: tiles to go)
+        return (left <= 0 || lane >= pages_of(w)) ? 0 : __ldg(table_of(w) + lane);
+      };
+      // the tile at walk position w: chunks [0, nchunks) of the rows of KV head hk into dst
+      auto load_tile = [&](const AttnWalk& w, int entry, const CUtensorMap* tmap, int nchunks, uint8_t* dst, uint64_t* bar) {
         if constexpr (!kPaged) {
           mbar_arrive_expect_tx(bar, nchunks * kChunkBytes);
-          for (int c = 0; c < nchunks; ++c) tma_load_3d(dst + c * kChunkBytes, tmap, c * kChunk, hk, w.seq0 + u0, bar);
+          for (int c = 0; c < nchunks; ++c) tma_load_3d(dst + c * kChunkBytes, tmap, c * kChunk, hk, w.seq0 + w.t * kTok, bar);
         } else {
           // one box per page that holds tokens of the sequence; rows of the tile past them keep stale (finite) codes
           // and are masked like every token past the end
-          const int32_t* bt = p.block_table + static_cast<long long>(w.b) * p.max_blocks;
-          const int npg = min(kTok >> p.page_shift, (w.L - u0 + p.page - 1) >> p.page_shift);
-          mbar_arrive_expect_tx(bar, nchunks * kChunk * p.page * npg);
-          for (int pg = 0; pg < npg; ++pg) {
-            const int tok = __ldg(bt + (u0 >> p.page_shift) + pg) * p.page;
-            for (int c = 0; c < nchunks; ++c)
-              tma_load_3d(dst + c * kChunkBytes + pg * p.page * kChunk, tmap, c * kChunk, hk, tok, bar);
+          const int npg = pages_of(w);
+          if (!kWarp || lane == 0) mbar_arrive_expect_tx(bar, nchunks * kChunk * p.page * npg);
+          if constexpr (kWarp) {
+            __syncwarp();
+            if (lane < npg)
+              for (int c = 0; c < nchunks; ++c)
+                tma_load_3d(dst + c * kChunkBytes + lane * p.page * kChunk, tmap, c * kChunk, hk, entry * p.page, bar);
+          } else {
+            for (int pg = 0; pg < npg; ++pg) {
+              const int tok = __ldg(table_of(w) + pg) * p.page;
+              for (int c = 0; c < nchunks; ++c) tma_load_3d(dst + c * kChunkBytes + pg * p.page * kChunk, tmap, c * kChunk, hk, tok, bar);
+            }
           }
         }
       };
+      auto ready = [&](uint64_t* bar, uint32_t parity) -> bool {
+        if constexpr (kWarp) {
+          bool r = false;
+          if (lane == 0) r = mbar_test_wait(bar, parity);
+          return __shfl_sync(0xffffffffu, r ? 1 : 0, 0) != 0;
+        } else {
+          return mbar_test_wait(bar, parity);
+        }
+      };
+      int ek = 0, ev = 0;
+      if constexpr (kWarp) {
+        ek = entry_of(wk, total_tiles);
+        ev = entry_of(wv, total_tiles - vq);
+      }
       long long t_idle = clock64();
       while (kq < total_tiles || vq < total_tiles) {
         bool progressed = false;
-        if (kq < total_tiles && mbar_test_wait(&kv_empty[kq % p.stages], ((kq / p.stages) & 1) ^ 1)) {
+        if (kq < total_tiles && ready(&kv_empty[kq % p.stages], ((kq / p.stages) & 1) ^ 1)) {
           const int st = kq % p.stages;
-          load_tile(wk, &tmap_k, p.DC, smem + st * kv_stage_bytes, &kv_full[st]);
+          load_tile(wk, ek, &tmap_k, p.DC, smem + st * kv_stage_bytes, &kv_full[st]);
           attn_walk_advance<kBalanced>(p, wk, 1);
           ++kq;
+          if constexpr (kWarp) ek = entry_of(wk, total_tiles - kq);
           progressed = true;
         }
-        if (vq < total_tiles && mbar_test_wait(&v_empty[vq % p.stages], ((vq / p.stages) & 1) ^ 1)) {
+        if (vq < total_tiles && ready(&v_empty[vq % p.stages], ((vq / p.stages) & 1) ^ 1)) {
           const int st = vq % p.stages;
-          load_tile(wv, &tmap_v, p.DVT, smem + st * kv_stage_bytes + k_bytes, &v_full[st]);
+          load_tile(wv, ev, &tmap_v, p.DVT, smem + st * kv_stage_bytes + p.DC * kChunkBytes, &v_full[st]);
           attn_walk_advance<kBalanced>(p, wv, 1);
           ++vq;
+          if constexpr (kWarp) ev = entry_of(wv, total_tiles - vq);
           progressed = true;
         }
         if (progressed) {
           t_idle = clock64();
         } else {
-          if (*abort) break;
-          if (clock64() - t_idle > kWaitBudgetCycles) {
+          bool give_up = *abort != 0;
+          if (!give_up && clock64() - t_idle > kWaitBudgetCycles) {
             *abort = 1;
             atomicMax(p.status, kStatusTimeout);
-            break;
+            give_up = true;
           }
+          if constexpr (kWarp) give_up = __any_sync(0xffffffffu, give_up);
+          if (give_up) break;
         }
       }
-      (void)v_bytes;
-    }
+    };
+    if (kPaged && p.page < 64) produce(std::true_type{});
+    else if (lane == 0) produce(std::false_type{});
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     if (lane == 0) {

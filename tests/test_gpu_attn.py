@@ -301,6 +301,24 @@ def test_paged_cache_gqa(page):
     assert torch.equal(o[torch.from_numpy(live).cuda()], o2[torch.from_numpy(live).cuda()])
 
 
+@pytest.mark.parametrize("page", [8, 32, -8, -16])
+@pytest.mark.parametrize("Hq", [8, 32])
+def test_paged_cache_small_pages_equal_contiguous(page, Hq):
+    """Pages whose boxes are spread over the producer warp's lanes, at the edges: one token, a page less one, a page, a
+    tile less one page, a tile and one token, no token at all.  Bit for bit what the contiguous cache gives."""
+    if page < 0:
+        binding.debug_set_option("MSD_ATTN_BALANCED", 1)
+        page = -page
+    seqlens = [1, page - 1, page, page + 1, 0, 128 - page, 127, 129, 1024]
+    c = inputs.gqa_case(B=len(seqlens), Hq=Hq, Hkv=4, D=128, seqlens=seqlens, seed=page)
+    k, v, ks, vs, table, sl = inputs.paginate(c, page, seed=page)
+    o = binding.attn_decode_int8kv_paged(bf16_dev(c.q), dev(k), dev(v), dev(ks), dev(vs), dev(table), dev(sl), page, c.max_seqlen,
+                                         c.softmax_scale)
+    ref, _ = _run_gpu(c)
+    binding.last_device_status()
+    assert torch.equal(o, ref)
+
+
 def test_paged_cache_mla_and_bad_page_size():
     c = inputs.mla_case(B=3, Hq=64, D=576, Dv=512, seqlens=[300, 129, 1000], seed=62)
     k, v, ks, vs, table, sl = inputs.paginate(c, 32, seed=5)
