@@ -921,8 +921,8 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 
 
 // ------------------------------------------------------------------------------------------------------------------
-// Wide head groups (more than 16 query rows per KV head, e.g. an MLA latent cache shared by 64 heads): 32 head slots per
-// CTA, sixteen softmax warps (four groups of four; a group owns 8 head slots, a thread one token lane of them).
+// Wide head groups (more than 8 query rows per KV head, e.g. an MLA latent cache shared by 64 heads): 32 head slots per
+// CTA, sixteen softmax warps (four groups of four; a group owns 8 head slots, a thread one token lane of them), or half of that.
 //
 // The PV products of consecutive tiles accumulate in the SAME INT32 tensor-memory accumulators (Alg. 3 lines 10-12
 // applied once per run of tiles): that needs the reference maximum of every head and the probability scale alpha_P to
@@ -938,7 +938,6 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 // that fit shared memory for a 576-byte row bound the pipeline, not the latency of L2 misses.)
 constexpr float kHoldMarginLog2 = 3.0f;
 constexpr float kHoldScaleGrowth = 1.25f;
-constexpr int kWideSlots = 32;                      // head slots per CTA, Rp = 64 stacked rows
 template <int W> __device__ __forceinline__ void tmem_stw(uint32_t taddr, const uint32_t (&v)[W]) {
   static_assert(W == 8 || W == 16, "8 or 16 columns per store");
   if constexpr (W == 8) tmem_st8(taddr, v);
@@ -946,21 +945,26 @@ template <int W> __device__ __forceinline__ void tmem_stw(uint32_t taddr, const 
 }
 
 
-// kWideHS: head slots per softmax thread (8 or 16); the 32 slots of the CTA are shared out over 32 / kWideHS groups of
+// kSlots: head slots per CTA (2 kSlots stacked rows).  32 for latent caches and for more than 16 rows per KV head: one CTA
+// per SM, all 512 tensor-memory columns.  16 for 9 to 16 rows at D, Dv <= 128: 128 columns, 78 KB of shared memory and 80
+// registers (the block is bounded as 12 warps: the register file is four banks, one per scheduler, and two CTAs of 11 warps put
+// six on one of them), so two CTAs share an SM and one's softmax runs while the other waits for its products.
+// kWideHS: head slots per softmax thread (8 or 16); the slots are shared out over kSlots / kWideHS groups of
 // four softmax warps.  kFixDC / kFixDVT: the chunk counts of D and Dv when known at compile time (0: taken from the
 // plan) - the MMA thread shares its scheduler with four busy softmax warps, so every instruction it spends per MMA on
 // loop control and address arithmetic delays the tensor pipe; with fixed counts its loops unroll to an add per operand.
-template <int kWideHS, bool kPaged, int kFixDC, int kFixDVT>
-__global__ void __launch_bounds__(((kFixDC == 5 && kFixDVT == 4 && !kPaged) ? 64 : 96) + 128 * (kWideSlots / kWideHS), 1)
+template <int kSlots, int kWideHS, bool kPaged, int kFixDC, int kFixDVT>
+__global__ void __launch_bounds__(kSlots == 16 ? 384 : ((kFixDC == 5 && kFixDVT == 4 && !kPaged) ? 64 : 96) + 128 * (kSlots / kWideHS),
+                                  kSlots == 16 ? 2 : 1)
 attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v, const AttnParams p) {
   extern __shared__ uint8_t smem_dyn[];
   __shared__ __align__(8) uint64_t kv_full[4], kv_empty[4], v_full[4], v_empty[4], s_full[2], p_full[2], q_ready, pv_done[2], p_redo;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   __shared__ int flush_stamp[2];                    // tile number + 1 of the last tile whose references had to move, per P buffer
-  __shared__ float s_aq[kWideSlots];
-  __shared__ float red[kWideSlots / kWideHS][4][kWideHS + 1];    // per-warp tile maxima (slow path only)
-  constexpr int kWideWG = kWideSlots / kWideHS;
+  __shared__ float s_aq[kSlots];
+  __shared__ float red[kSlots / kWideHS][4][kWideHS + 1];    // per-warp tile maxima (slow path only)
+  constexpr int kWideWG = kSlots / kWideHS;
   constexpr int kNSW = 4 * kWideWG;
   // Latent cache of 576 bytes per token with V aliased to its first 512 (the launcher picks this instantiation only
   // then): the two KV stages are given back chunk by chunk (five 128-byte-wide chunks of 16 KB): every chunk is
@@ -971,7 +975,12 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   // the thread has nothing else to do and the scores are ready 0.2-0.5 us earlier.)
   constexpr bool kChunked = kFixDC == 5 && kFixDVT == 4 && !kPaged;
   __shared__ __align__(8) uint64_t ck_empty[2][5], ck_full[2][5];      // per stage and chunk: free again / landed
-  constexpr int kDVT = 4;
+  constexpr int kDVT = kSlots == 16 ? kFixDVT : 4;
+  // P lies token-major, [128 tokens][2 kSlots bytes], swizzled over its row width (64 or 32 bytes): an MN-major B operand
+  // whose groups of 8 tokens follow one another (a softmax thread then stores its token's codes as whole words)
+  static_assert(kSlots == 32 || (kSlots == 16 && kFixDC > 0 && kFixDVT > 0), "16 slots: chunk counts known");
+  constexpr int kPRow = 2 * kSlots;
+  constexpr auto kPSwizzle = kSlots == 32 ? kSwizzle64B : kSwizzle32B;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // splits along x, units along y (the two head groups of a sequence split, which read the same tiles, a few CTAs apart:
@@ -1140,9 +1149,6 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);         // K-major tiles: K, stacked Q
       const uint64_t dvt = smem_desc(0, 16384, 1024, kSwizzle128B);     // V^T read MN-major from the token-major tile
       const uint64_t q_enc = dk + (smem_u32(sm_q) >> 4);
-      // P lies token-major, [128 tokens][64 bytes = 2 x 32 head slots], 64-byte swizzle: an MN-major B operand whose
-      // groups of 8 tokens are 512 bytes apart (a softmax thread then stores its token's codes as whole words)
-      const uint64_t p_enc = smem_desc(0, 512, 512, kSwizzle64B) + (smem_u32(sm_p) >> 4);
       const uint32_t smem_enc = smem_u32(smem) >> 4;
       const uint32_t q_step = static_cast<uint32_t>(p.Rp * kChunk) >> 4;
       const int nDC = kFixDC ? kFixDC : p.DC;
@@ -1163,7 +1169,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
             for (int k = 0; k < 4; ++k)
               if (c + 1 < kFixDC || k < last_steps) {
                 if (c > 0 || k > 0)
-                  mma_i8_lohi<true>(d, ka_lo + (c * (kChunkBytes >> 4) + 2 * k), k_hi, qa_lo + (c * ((kWideSlots * 2 * kChunk) >> 4) + 2 * k), q_hi, idesc_qk);
+                  mma_i8_lohi<true>(d, ka_lo + (c * (kChunkBytes >> 4) + 2 * k), k_hi, qa_lo + (c * ((kSlots * 2 * kChunk) >> 4) + 2 * k), q_hi, idesc_qk);
                 else
                   mma_i8_lohi<false>(d, ka_lo, k_hi, qa_lo, q_hi, idesc_qk);
               }
@@ -1210,7 +1216,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
 #pragma unroll
             for (int k = 0; k < 4; ++k)
               if (c < 4 || k < last_steps) {
-                const uint32_t ka = k_lo + (c * (kChunkBytes >> 4) + 2 * k), qa = q_lo0 + (c * ((kWideSlots * 2 * kChunk) >> 4) + 2 * k);
+                const uint32_t ka = k_lo + (c * (kChunkBytes >> 4) + 2 * k), qa = q_lo0 + (c * ((kSlots * 2 * kChunk) >> 4) + 2 * k);
                 if (i == 0 && k == 0) mma_i8_lohi<false>(d, ka, k_hi, qa, q_hi, idesc_qk);
                 else mma_i8_lohi<true>(d, ka, k_hi, qa, q_hi, idesc_qk);
               }
@@ -1241,7 +1247,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     if constexpr (!kChunked) {
       if (lane == 0) {
         const uint64_t vdesc = smem_desc(0, 16384, 1024, kSwizzle128B) + (smem_u32(smem) >> 4);       // V^T, MN-major from the token-major tile
-        const uint64_t pdesc = smem_desc(0, 512, 512, kSwizzle64B) + (smem_u32(sm_p) >> 4);           // P, token-major
+        const uint64_t pdesc = smem_desc(0, 8 * kPRow, 8 * kPRow, kPSwizzle) + (smem_u32(sm_p) >> 4);           // P, token-major
         const uint32_t va0 = static_cast<uint32_t>(vdesc), v_hi = static_cast<uint32_t>(vdesc >> 32);
         const uint32_t pa0 = static_cast<uint32_t>(pdesc), p_hi = static_cast<uint32_t>(pdesc >> 32);
         const uint32_t p_step = static_cast<uint32_t>(p.Rp * kChunk) >> 4;
@@ -1266,12 +1272,12 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
           const uint32_t va = va0 + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + (p.v_alias ? 0u : static_cast<uint32_t>(p.DC * (kChunkBytes >> 4)));
           const uint32_t pa = pa0 + (t & 1) * p_step;
           for (int j = 0; j < n_dvt; ++j) {
-            const uint32_t acc = tmem_o + j * (2 * kWideSlots);
+            const uint32_t acc = tmem_o + j * (2 * kSlots);
             if (fresh) mma_i8_lohi<false>(acc, va + j * (kChunkBytes >> 4), v_hi, pa, p_hi, idesc);
             else mma_i8_lohi<true>(acc, va + j * (kChunkBytes >> 4), v_hi, pa, p_hi, idesc);
 #pragma unroll
             for (int k = 1; k < 4; ++k)      // 32 tokens per MMA: four 8-token groups of 1024 bytes
-              mma_i8_lohi<true>(acc, va + j * (kChunkBytes >> 4) + k * (4096 >> 4), v_hi, pa + k * (2048 >> 4), p_hi, idesc);
+              mma_i8_lohi<true>(acc, va + j * (kChunkBytes >> 4) + k * (4096 >> 4), v_hi, pa + k * (32 * kPRow >> 4), p_hi, idesc);
           }
           tc_commit(&pv_done[t & 1]);
           tc_commit(p.v_alias ? &kv_empty[st] : &v_empty[st]);
@@ -1293,7 +1299,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       pdl_wait_primary();
       const int i = threadIdx.x - 64;
       const float* sc = p.q_scales + static_cast<size_t>(blockIdx.y) * 2 * p.HG;
-      if (i < kWideSlots) s_aq[i] = __ldg(sc + i);
+      if (i < kSlots) s_aq[i] = __ldg(sc + i);
     }
     named_bar_sync(8, 128 * kWideWG);
     if (threadIdx.x == 64) attn_mark(p, 3);
@@ -1318,7 +1324,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
 #pragma unroll
       for (int h = 0; h < kWideHS; ++h) z[h] = 0u;
 #pragma unroll
-      for (int j = 0; j < kDVT; ++j) tmem_stw<kWideHS>(orun_row + j * kWideSlots, z);
+      for (int j = 0; j < kDVT; ++j) tmem_stw<kWideHS>(orun_row + j * kSlots, z);
       tmem_st_wait();
     }
     float a_ref = 0.0f, alpha_p = 0.0f, inv_a = 0.0f, inv_b = 0.0f;
@@ -1348,7 +1354,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       const uint32_t srow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + (t & 1) * p.Rp;
       uint32_t v1[kWideHS], v2[kWideHS];
       tmem_ldw<kWideHS>(srow + hs0, v1);
-      tmem_ldw<kWideHS>(srow + kWideSlots + hs0, v2);
+      tmem_ldw<kWideHS>(srow + kSlots + hs0, v2);
       tmem_ld_wait();
       if (p.s_dbg && valid) {
         long long tok_row = seq0 + tok_rel;
@@ -1366,9 +1372,10 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     // c4-c5: P = 2^(s - reference), value scale folded in, two-pass INT8 with the scale in force, into P buffer t&1.
     // Returns the largest s - reference of this thread (> 0: the reference must move).
     auto write_p = [&](int t, const float (&s)[kWideHS], float vs, float (&pl)[kWideHS]) -> float {
-      // this token's row of the P buffer: 64 bytes, the 16-byte pieces XORed with (token / 2) % 4 (64-byte swizzle)
-      uint8_t* prow = sm_p + (t & 1) * p.Rp * kChunk + tl * 64;
-      const int sw = (tl >> 1) & 3;
+      // this token's row of the P buffer: 64 (32) bytes, the 16-byte pieces XORed with address bits 7 and 8 (bit 7)
+      uint8_t* prow = sm_p + (t & 1) * p.Rp * kChunk + tl * kPRow;
+      constexpr int kPieces = kPRow / 16;
+      const int sw = (tl * kPRow >> 7) & (kPieces - 1);
       uint32_t c1[kWideHS], c2[kWideHS];
       float xm = -INFINITY;
 #pragma unroll
@@ -1392,8 +1399,8 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         w1[g] = __byte_perm(__byte_perm(c1[4 * g], c1[4 * g + 1], 0x0040), __byte_perm(c1[4 * g + 2], c1[4 * g + 3], 0x0040), 0x5410);
         w2[g] = __byte_perm(__byte_perm(c2[4 * g], c2[4 * g + 1], 0x0040), __byte_perm(c2[4 * g + 2], c2[4 * g + 3], 0x0040), 0x5410);
       }
-      uint8_t* d1 = prow + ((((hs0 >> 4) ^ sw) & 3) << 4) + (hs0 & 15);
-      uint8_t* d2 = prow + (((((kWideSlots + hs0) >> 4) ^ sw) & 3) << 4) + (hs0 & 15);
+      uint8_t* d1 = prow + ((((hs0 >> 4) ^ sw) & (kPieces - 1)) << 4) + (hs0 & 15);
+      uint8_t* d2 = prow + (((((kSlots + hs0) >> 4) ^ sw) & (kPieces - 1)) << 4) + (hs0 & 15);
       if constexpr (kWideHS == 8) {
         *reinterpret_cast<uint2*>(d1) = make_uint2(w1[0], w1[1]);
         *reinterpret_cast<uint2*>(d2) = make_uint2(w2[0], w2[1]);
@@ -1411,8 +1418,8 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
           const uint32_t orow = tmem_o + (static_cast<uint32_t>(quad * 32) << 16) + j * p.Rp;
           uint32_t v1[kWideHS], v2[kWideHS], o[kWideHS];
           tmem_ldw<kWideHS>(orow + hs0, v1);
-          tmem_ldw<kWideHS>(orow + kWideSlots + hs0, v2);
-          tmem_ldw<kWideHS>(orun_row + j * kWideSlots, o);
+          tmem_ldw<kWideHS>(orow + kSlots + hs0, v2);
+          tmem_ldw<kWideHS>(orun_row + j * kSlots, o);
           tmem_ld_wait();
 #pragma unroll
           for (int h = 0; h < kWideHS; ++h) {
@@ -1420,16 +1427,16 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
             // the drained sums belong to the OLD reference: add them, then rescale
             o[h] = __float_as_uint(__fmaf_rn(alpha_old, acc, __uint_as_float(o[h])) * resc[h]);
           }
-          tmem_stw<kWideHS>(orun_row + j * kWideSlots, o);
+          tmem_stw<kWideHS>(orun_row + j * kSlots, o);
         }
       }
       tmem_st_wait();
     };
 
     // operand descriptors of PV as lower / upper words (see mma_i8_lohi): V^T read MN-major from the token-major KV tile,
-    // P an MN-major operand too (token-major, 64-byte swizzle, groups of 8 tokens 512 bytes apart)
+    // P an MN-major operand too
     const uint64_t pv_vdesc = smem_desc(0, 16384, 1024, kSwizzle128B) + (smem_u32(smem) >> 4);
-    const uint64_t pv_pdesc = smem_desc(0, 512, 512, kSwizzle64B) + (smem_u32(sm_p) >> 4);
+    const uint64_t pv_pdesc = smem_desc(0, 8 * kPRow, 8 * kPRow, kPSwizzle) + (smem_u32(sm_p) >> 4);
     const uint32_t pv_va_lo = static_cast<uint32_t>(pv_vdesc), pv_v_hi = static_cast<uint32_t>(pv_vdesc >> 32);
     const uint32_t pv_pa_lo = static_cast<uint32_t>(pv_pdesc), pv_p_hi = static_cast<uint32_t>(pv_pdesc >> 32);
     const uint32_t pv_p_step = static_cast<uint32_t>(p.Rp * kChunk) >> 4;
@@ -1551,12 +1558,12 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
             if (wq == 0 && t >= 2 && t < 5) attn_mark(p, 8 + 6 * (t - 2));
             const uint32_t va_lo = pv_va_lo + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + wq * (kChunkBytes >> 4);
             const uint32_t pa_lo = pv_pa_lo + (t & 1) * pv_p_step;
-            const uint32_t acc = tmem_o + wq * (2 * kWideSlots);
+            const uint32_t acc = tmem_o + wq * (2 * kSlots);
             if (slow) mma_i8_lohi<false>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
             else mma_i8_lohi<true>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
 #pragma unroll
             for (int k = 1; k < 4; ++k)      // 32 tokens per MMA: four 8-token groups of 1024 bytes
-              mma_i8_lohi<true>(acc, va_lo + k * (4096 >> 4), pv_v_hi, pa_lo + k * (2048 >> 4), pv_p_hi, pv_idesc);
+              mma_i8_lohi<true>(acc, va_lo + k * (4096 >> 4), pv_v_hi, pa_lo + k * (32 * kPRow >> 4), pv_p_hi, pv_idesc);
             tc_commit(&ck_empty[st][wq]);      // value chunk wq may be requested again; also "this dv tile of PV(t) is complete"
             if (wq == 0 && t >= 2 && t < 5) attn_mark(p, 20 + t);
           }
@@ -1608,7 +1615,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       for (int j = 0; j < kDVT; ++j) {
         if (j < p.DVT) {            // (warp-uniform: the tensor-memory load is a whole-warp instruction)
           uint32_t o[kWideHS];
-          tmem_ldw<kWideHS>(orun_row + j * kWideSlots, o);
+          tmem_ldw<kWideHS>(orun_row + j * kSlots, o);
           tmem_ld_wait();
 #pragma unroll
           for (int h = 0; h < kWideHS; ++h)
@@ -1721,9 +1728,9 @@ struct AttnPlan {
 static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, bool v_alias, AttnPlan* pl) {
   if (B < 1 || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || D < 16 || D % 16 != 0 || Dv < 16 || Dv % 16 != 0) return false;
   const int G = Hq / Hkv;
-  // up to 8 rows per KV head: the narrow kernel (three CTAs per SM); more: the wide kernel's 32 head slots (a 16-slot
-  // narrow kernel needs 166 registers, runs one or two CTAs per SM and measured 5-12 % slower than the wide one half full)
-  pl->HG = (G <= 8) ? 8 : 32;
+  // up to 8 rows per KV head: the narrow kernel (three CTAs per SM); 9 to 16 at D, Dv <= 128: the wide kernel with 16 head
+  // slots (two CTAs per SM); everything else: with 32.
+  pl->HG = (G <= 8) ? 8 : (G <= 16 && D <= kChunk && Dv <= kChunk ? 16 : 32);
   pl->Rp = 2 * pl->HG;
   pl->groups = (G + pl->HG - 1) / pl->HG;
   pl->DC = (D + kChunk - 1) / kChunk;
@@ -1774,8 +1781,9 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   }
   pl->smem_bytes = static_cast<size_t>(pl->stages) * kv_stage + fixed;
   int cols = 32;
-  // wide head groups keep the FP32 running output (4 x 32 columns) behind the two score buffers and the accumulators
-  const int cols_needed = pl->HG > 16 ? 2 * pl->Rp + 4 * pl->Rp + 4 * 32 : 2 * pl->Rp + pl->DVT * pl->Rp;
+  // wide head groups keep the FP32 running output (a column per slot and dv tile) behind the two score buffers and the accumulators
+  const int dv_tiles = pl->HG == 16 ? 1 : 4;
+  const int cols_needed = pl->HG > 8 ? 2 * pl->Rp + dv_tiles * (pl->Rp + pl->HG) : 2 * pl->Rp + pl->DVT * pl->Rp;
   while (cols < cols_needed) cols <<= 1;
   pl->tmem_cols = cols;
   pl->ws_partial_bytes = round_up(static_cast<size_t>(B) * Hq * ns * (Dv + kPartHdr) * sizeof(float), 1024);
@@ -1810,11 +1818,17 @@ static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* b
   } else if (pl.HG == 8) {
     if (G <= 4) { MSD_ATTN_PICK(8, 4); } else { MSD_ATTN_PICK(8, 8); }
   } else {
-    // wide head groups: 32 head slots per CTA, sixteen softmax warps, held references (attn_decode_wide_kernel)
+    // wide head groups: 32 or 16 head slots per CTA, held references (attn_decode_wide_kernel)
     const bool mla = pl.DC == 5 && pl.DVT == 4 && pl.v_alias && pl.stages == 2;     // a 513..640-byte latent row whose first 512 bytes are V
-    if (paged) kernel = mla ? attn_decode_wide_kernel<8, true, 5, 4> : attn_decode_wide_kernel<8, true, 0, 0>;
-    else kernel = mla ? attn_decode_wide_kernel<8, false, 5, 4> : attn_decode_wide_kernel<8, false, 0, 0>;
     *block_threads = ((mla && !paged) ? 64 : 96) + 128 * 4;      // producer, QK^T issuer, 16 softmax warps and, except for the chunk-wise kernel, a PV issuer
+    if (pl.HG == 16) {
+      kernel = paged ? attn_decode_wide_kernel<16, 8, true, 1, 1> : attn_decode_wide_kernel<16, 8, false, 1, 1>;
+      *block_threads = 96 + 128 * 2;
+    } else if (paged) {
+      kernel = mla ? attn_decode_wide_kernel<32, 8, true, 5, 4> : attn_decode_wide_kernel<32, 8, true, 0, 0>;
+    } else {
+      kernel = mla ? attn_decode_wide_kernel<32, 8, false, 5, 4> : attn_decode_wide_kernel<32, 8, false, 0, 0>;
+    }
   }
 #undef MSD_ATTN_PICK
 #undef MSD_ATTN_PICK_B
@@ -1887,7 +1901,7 @@ msd_status_t msd_attn_decode_softmax_rule(int32_t B, int32_t Hq, int32_t Hkv, in
   msd::AttnPlan pl;
   if (!m_margin || !sv_growth) return MSD_ERR_NULL_POINTER;
   if (!msd::plan_attn(B, Hq, Hkv, D, Dv, max_seqlen, false, &pl)) return MSD_ERR_BAD_SHAPE;
-  const bool held = pl.HG > 16;
+  const bool held = pl.HG > 8;
   *m_margin = held ? msd::kHoldMarginLog2 * 0.6931471805599453f : 0.0f;
   *sv_growth = held ? msd::kHoldScaleGrowth : 0.0f;
   return MSD_OK;

@@ -245,6 +245,7 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 // bits 61-63 (0 none, 2 = 128-byte, 4 = 64-byte, 6 = 32-byte).
 constexpr uint64_t kSwizzle128B = 2;
 constexpr uint64_t kSwizzle64B = 4;
+constexpr uint64_t kSwizzle32B = 6;
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes, uint64_t swizzle) {
   uint64_t d = 0;
   d |= static_cast<uint64_t>((saddr & 0x3FFFF) >> 4);
