@@ -371,6 +371,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
   // scales, and the rescale factors a tile's softmax hands to its merge - stays in shared memory (per warp, by tile
   // parity), or the kernel does not fit the 96 registers that three CTAs per SM allow.
   constexpr bool kSmemState = kNH > 4;
+  constexpr bool kIntCombine = kMaxDVT == 1;       // D <= 512 (pick_attn_kernel)
   __shared__ float s_resc[kSmemState ? 2 : 1][4][kNH];
   __shared__ int s_scan[kAttnThreads];
   __shared__ AttnWalk s_walk;                      // the softmax warps' walk (kept here, not in registers, between segments)
@@ -757,10 +758,24 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 #pragma unroll
           for (int h = 0; h < kNH; ++h)
           {
-            const float a_q = kSmemState ? s_aq[hs0 + h] : aq[h], b_q = kSmemState ? s_bq[hs0 + h] : bq[h];
-            bool vh = valid;
-            if (p.Sq > 1) vh = valid && tok_rel < L - p.Sq + 1 + (grp * p.HG + hs0 + h) / p.Gr;    // causal among the new tokens
-            s[h] = vh ? __fmaf_rn(a_q, static_cast<float>(static_cast<int32_t>(v1[h])), b_q * static_cast<float>(static_cast<int32_t>(v2[h]))) * ks : -INFINITY;
+            const float b_q = kSmemState ? s_bq[hs0 + h] : bq[h];
+            float sum;
+            if constexpr (kIntCombine) {
+              // alpha_Q S1 + beta_Q S2 with beta_Q = alpha_Q / 254: one integer multiply-add and one conversion
+              // (|254 S1 + S2| <= 255 * 127 * 128 * D < 2^31)
+              sum = b_q * static_cast<float>(254 * static_cast<int32_t>(v1[h]) + static_cast<int32_t>(v2[h]));
+            } else {
+              const float a_q = kSmemState ? s_aq[hs0 + h] : aq[h];
+              sum = __fmaf_rn(a_q, static_cast<float>(static_cast<int32_t>(v1[h])), b_q * static_cast<float>(static_cast<int32_t>(v2[h])));
+            }
+            s[h] = valid ? sum * ks : -INFINITY;
+          }
+          // several query tokens: the rows of a tile that reaches the new tokens are masked one by one (in a block of its
+          // own: as a condition on every score it cost all other calls 3 to 6 %)
+          if (p.Sq > 1 && t_begin + (t + 1) * kTok > L - p.Sq + 1) {
+#pragma unroll
+            for (int h = 0; h < kNH; ++h)
+              if (tok_rel >= L - p.Sq + 1 + (grp * p.HG + hs0 + h) / p.Gr) s[h] = -INFINITY;
           }
         }
         // c4: tile maxima per head (and of the value scales) over the 128 token lanes
@@ -980,6 +995,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   // whose groups of 8 tokens follow one another (a softmax thread then stores its token's codes as whole words)
   static_assert(kSlots == 32 || (kSlots == 16 && kFixDC > 0 && kFixDVT > 0), "16 slots: chunk counts known");
   constexpr int kPRow = 2 * kSlots;
+  constexpr bool kIntCombine = kFixDC >= 1 && kFixDC <= 4;      // D <= 512
   constexpr auto kPSwizzle = kSlots == 32 ? kSwizzle64B : kSwizzle32B;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1315,7 +1331,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
 #pragma unroll
     for (int h = 0; h < kWideHS; ++h) {
       const bool present = hs0 + h < nh;
-      aq[h] = present ? s_aq[hs0 + h] : 0.0f;
+      aq[h] = present ? (kIntCombine ? s_aq[hs0 + h] * (1.0f / 254.0f) : s_aq[hs0 + h]) : 0.0f;
       nm[h] = present ? 1e30f : -1e30f;
       l_part[h] = 0.0f;
     }
@@ -1363,10 +1379,18 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       }
 #pragma unroll
       for (int h = 0; h < kWideHS; ++h) {
-        bool vh = valid;
-        if (p.Sq > 1) vh = valid && tok_rel < L - p.Sq + 1 + (grp * p.HG + hs0 + h) / p.Gr;    // causal among the new tokens
-        const float tsum = __fmaf_rn(static_cast<float>(static_cast<int32_t>(v2[h])), kInv254, static_cast<float>(static_cast<int32_t>(v1[h])));
-        s[h] = vh ? (aq[h] * ks) * tsum : -INFINITY;
+        // S1 + S2 / 254; with D <= 512 as (254 S1 + S2) / 254 (|254 S1 + S2| <= 255 * 127 * 128 * D < 2^31): one conversion
+        // instead of two on a pipe that takes a warp every eighth cycle (the factor is in aq)
+        const float tsum = kIntCombine ? static_cast<float>(254 * static_cast<int32_t>(v1[h]) + static_cast<int32_t>(v2[h]))
+                                       : __fmaf_rn(static_cast<float>(static_cast<int32_t>(v2[h])), kInv254, static_cast<float>(static_cast<int32_t>(v1[h])));
+        s[h] = valid ? (aq[h] * ks) * tsum : -INFINITY;
+      }
+      // causal among the new tokens: only the tiles that reach them are masked row by row (a division per row and tile
+      // took 0.8 of 2.5 us a tile when every tile was; as a condition on every score it cost all other calls 3 to 6 %)
+      if (p.Sq > 1 && t_begin + (t + 1) * kTok > L - p.Sq + 1) {
+#pragma unroll
+        for (int h = 0; h < kWideHS; ++h)
+          if (tok_rel >= L - p.Sq + 1 + (grp * p.HG + hs0 + h) / p.Gr) s[h] = -INFINITY;
       }
     };
     // c4-c5: P = 2^(s - reference), value scale folded in, two-pass INT8 with the scale in force, into P buffer t&1.
@@ -1729,7 +1753,8 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   if (B < 1 || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || D < 16 || D % 16 != 0 || Dv < 16 || Dv % 16 != 0) return false;
   const int G = Hq / Hkv;
   // up to 8 rows per KV head: the narrow kernel (three CTAs per SM); 9 to 16 at D, Dv <= 128: the wide kernel with 16 head
-  // slots (two CTAs per SM); everything else: with 32.
+  // slots (two CTAs per SM; 16 rows, 32 x 4096 tokens: 130 us with 32 slots half empty and one CTA per SM, 85 now; 8 x 32768:
+  // 199 and 135); everything else: with 32.  (A 16-slot narrow kernel needs 166 registers and was slower than either.)
   pl->HG = (G <= 8) ? 8 : (G <= 16 && D <= kChunk && Dv <= kChunk ? 16 : 32);
   pl->Rp = 2 * pl->HG;
   pl->groups = (G + pl->HG - 1) / pl->HG;
@@ -1807,7 +1832,7 @@ using AttnKernel = void (*)(CUtensorMap, CUtensorMap, AttnParams);
 static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* block_threads) {
   AttnKernel kernel = nullptr;
 #define MSD_ATTN_PICK_B(HG_, NH_, P_, B_) \
-  kernel = (pl.DVT == 1) ? attn_decode_kernel<HG_, NH_, 1, P_, B_> : (pl.DVT == 2) ? attn_decode_kernel<HG_, NH_, 2, P_, B_> \
+  kernel = (pl.DVT == 1 && pl.DC <= 4) ? attn_decode_kernel<HG_, NH_, 1, P_, B_> : (pl.DVT == 2) ? attn_decode_kernel<HG_, NH_, 2, P_, B_> \
                                                                                    : attn_decode_kernel<HG_, NH_, 4, P_, B_>
 #define MSD_ATTN_PICK(HG_, NH_) \
   do { if (paged) { MSD_ATTN_PICK_B(HG_, NH_, true, false); } else { MSD_ATTN_PICK_B(HG_, NH_, false, false); } } while (0)

@@ -91,6 +91,26 @@ def test_mla_parity(seqlens):
     _check(inputs.mla_case(len(seqlens), 64, 576, 512, seqlens, seed=11))
 
 
+@pytest.mark.parametrize("rows,D", [(9, 128), (12, 64), (15, 128), (16, 128), (17, 128)])
+def test_wide_groups_at_the_edges_of_the_slot_counts(rows, D):
+    """9 to 16 rows per KV head (16 head slots) and the first count past them (32): one token, the edges of a tile, an
+    empty sequence, one that the context splits cut."""
+    _check(inputs.gqa_case(6, 2 * rows, 2, D, [1, 127, 0, 128, 129, 2500], seed=rows + D))
+
+
+@pytest.mark.parametrize("rows,D", [(4, 512), (8, 512), (4, 640), (16, 128)])
+def test_scores_at_the_largest_codes(rows, D):
+    """Every code of the keys and of the queries' first components at its limit: the integer sums of both components, and
+    what they are combined into, stay exact (D <= 512 in one 32-bit integer, 255 * 127 * 128 * 512 < 2^31)."""
+    c = inputs.gqa_case(1, rows, 1, 128, [200], seed=rows + D)
+    T = c.k.shape[0]
+    sign = np.where(np.arange(D) % 2 == 0, 1, -1)
+    k = np.where(np.arange(T)[:, None] % 3 == 0, -127 * sign, 127 * sign).astype(np.int8)[:, None, :]
+    q = inputs.f32_to_bf16_bits(np.tile(sign * 3.0, (1, rows, 1)).astype(np.float32))
+    ks = np.full((T, 1), 2.0 ** -14, np.float32) * (1 + np.arange(T, dtype=np.float32)[:, None] / T)
+    _check(inputs.AttnCase(q, k, c.v, ks, c.v_scale, c.cu_seqlens, 128, float(D) ** -0.5))
+
+
 def test_other_head_dims():
     c = inputs.gqa_case(2, 8, 2, 64, [400, 77], seed=5)          # D = Dv = 64: half-filled chunk
     _check(c)
