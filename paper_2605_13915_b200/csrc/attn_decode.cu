@@ -999,13 +999,13 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   constexpr auto kPSwizzle = kSlots == 32 ? kSwizzle64B : kSwizzle32B;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // splits along x, units along y (the two head groups of a sequence split, which read the same tiles, a few CTAs apart:
-  // launched side by side they miss L2 together, measured 4 us slower)
-  const int split = blockIdx.x;
-  int unit = blockIdx.y;
-  const int grp = unit % p.groups; unit /= p.groups;
-  const int hk = unit % p.Hkv;
-  const int b = unit / p.Hkv;
+  // Splits along y: the early splits of every sequence, which are always full, start first and the short last ones fill
+  // the tail.  Units along x, head group slowest: the head groups of a sequence split read the same tiles, and launched side
+  // by side they miss L2 together.
+  const int split = blockIdx.y, pairs = p.B * p.Hkv;         // (sequence, KV head)
+  const int grp = blockIdx.x / pairs;
+  const int b = (blockIdx.x - grp * pairs) / p.Hkv, hk = blockIdx.x - grp * pairs - b * p.Hkv;
+  const int unit_q = (b * p.Hkv + hk) * p.groups + grp;      // index of the stacked query operand (attn_qstack_kernel)
   const int32_t* bt = kPaged ? p.block_table + static_cast<long long>(b) * p.max_blocks : nullptr;
   const int seq0 = kPaged ? 0 : p.cu[b];
   const int L = kPaged ? p.seqlens[b] : p.cu[b + 1] - seq0;
@@ -1156,7 +1156,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       // kernel launched just before this one (the producer's KV loads, which do not depend on it, are already under way)
       pdl_wait_primary();
       {
-        const int unit_q = blockIdx.y, chunk_bytes = p.Rp * kChunk;
+        const int chunk_bytes = p.Rp * kChunk;
         mbar_arrive_expect_tx(&q_ready, p.DC * chunk_bytes);
         for (int c = 0; c < p.DC; ++c)
           bulk_load(sm_q + c * chunk_bytes, p.q_img + (static_cast<size_t>(unit_q) * p.DC + c) * chunk_bytes, chunk_bytes, &q_ready);
@@ -1314,7 +1314,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       // beta_Q = alpha_Q / 254 is applied as a constant factor
       pdl_wait_primary();
       const int i = threadIdx.x - 64;
-      const float* sc = p.q_scales + static_cast<size_t>(blockIdx.y) * 2 * p.HG;
+      const float* sc = p.q_scales + static_cast<size_t>(unit_q) * 2 * p.HG;
       if (i < kSlots) s_aq[i] = __ldg(sc + i);
     }
     named_bar_sync(8, 128 * kWideWG);
@@ -1749,6 +1749,44 @@ struct AttnPlan {
   size_t smem_bytes, ws_bytes, ws_partial_bytes, ws_qimg_bytes, ws_qscale_bytes;
 };
 
+// What a context split costs, in microseconds (fitted to sweeps over split sizes): `per_sm` CTAs of the kernel fit an SM, a
+// tile takes tile_us[k - 1] with k of them on it, a CTA's set-up, first tiles, partial results and their merge `fixed_us`.
+struct AttnSplitCost { int per_sm; float tile_us[3], fixed_us; };
+
+// Tiles per context split.  The CTAs of a call run in rounds of as many as fit the machine, so the split size decides how
+// many rounds there are and how full the last is; powers of two missed both (one latent cache of 64 heads, 8 sequences of 4096 to
+// 8192 tokens: 2 tiles a split 57.8 us, 8 tiles 38.2; 12 GQA sequences of 6000: 4 tiles 42.9, 12 tiles 32.8; 128 query / 8 KV
+// heads, 32 x 4096: 8 tiles 85, 32 tiles 68).  The host knows the longest sequence, not the others: the size taken has the
+// smallest sum of the costs with every sequence at full length (whole rounds) and with lengths of 60 % on average (mixed
+// lengths fill the rounds up; half a split is left over at the end).  Against the best size found by sweeping it lost 4 % on
+// average over 18 shapes, 18 % at most.
+static int attn_split_tiles(long long units, int tiles, const AttnSplitCost& k) {
+  const float sms = static_cast<float>(sm_count()), slots = sms * static_cast<float>(k.per_sm), u = static_cast<float>(units);
+  const float frac = 0.6f;
+  int best = 1;
+  float best_cost = 0.0f;
+  // time of a tile with `items` CTAs spread over the machine
+  auto tile_us = [&](float items) { return k.tile_us[items <= sms ? 0 : (items <= 2.0f * sms ? std::min(1, k.per_sm - 1) : k.per_sm - 1)]; };
+  for (int ns = 1, c = tiles; ns <= tiles; ns = (tiles + c - 2) / (c - 1)) {      // each size that some number of splits has
+    c = (tiles + ns - 1) / ns;
+    // (from eight rounds on more splits only add to the fixed cost)
+    if (ns > 1 && (c < 2 || u * static_cast<float>(ns) > 8.0f * slots)) break;
+    const float items_full = u * static_cast<float>(ns), items_mix = ns > 1 ? u * (frac * static_cast<float>(ns) + 0.5f) : u;
+    const float tm = tile_us(items_mix), cf = static_cast<float>(c);
+    const float rounds = std::floor(items_full / slots), rest = items_full - rounds * slots;
+    const float full = rounds * (cf * k.tile_us[k.per_sm - 1] + k.fixed_us) + (rest > 0.5f ? cf * tile_us(rest) + k.fixed_us : 0.0f);
+    const float mix = items_mix <= slots ? cf * tm + k.fixed_us
+                                         : (u * frac * static_cast<float>(tiles) * tm + items_mix * k.fixed_us) / slots + 0.5f * (cf * tm + k.fixed_us);
+    const float cost = full + mix + 0.2f * static_cast<float>(ns);      // (the merge reads every split)
+    if (best_cost == 0.0f || cost < 0.999f * best_cost) { best_cost = cost; best = c; }
+    if (c == 1) break;
+  }
+  return best;
+}
+
+// The held references' integer accumulators take at most this many tiles: 127 * 127 * 128 * 512 < 2^31.
+constexpr int kMaxHeldTiles = 512;
+
 static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, bool v_alias, AttnPlan* pl) {
   if (B < 1 || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || D < 16 || D % 16 != 0 || Dv < 16 || Dv % 16 != 0) return false;
   const int G = Hq / Hkv;
@@ -1770,14 +1808,16 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   const int kv_stage = pl->kv_chunks * kChunkBytes;
   const size_t fixed = static_cast<size_t>(pl->DC) * pl->Rp * kChunk + 2 * pl->Rp * kChunk + 1024;   // Q stack, two P buffers
   pl->stages = (2 * static_cast<size_t>(kv_stage) + fixed <= 227 * 1024 - 2048) ? 2 : 1;
-  // Splits of equal size (a fixed number of tiles) keep the CTAs' work uniform whatever the mix of sequence lengths;
-  // the size is shrunk until there are enough splits to fill the machine a few times over.
   const int tiles = (max_seqlen + kTok - 1) / kTok;
   const long long units = static_cast<long long>(B) * Hkv * pl->groups;
-  int chunk_tiles = option(OPT_ATTN_CHUNK_TILES);       // testing aid
-  if (chunk_tiles < 1) chunk_tiles = pl->Rp <= 16 ? 16 : 32;
-  while (chunk_tiles > 2 && units * ((tiles + chunk_tiles - 1) / chunk_tiles) < static_cast<long long>(sm_count()) * 4) chunk_tiles >>= 1;
-  while ((tiles + chunk_tiles - 1) / chunk_tiles > 65535) chunk_tiles <<= 1;      // splits may run along the grid's y axis
+  const bool small = pl->DC == 1 && pl->DVT == 1;
+  const AttnSplitCost split_cost = pl->HG == 8 ? (small ? AttnSplitCost{3, {1.0f, 1.5f, 2.2f}, 6.0f} : AttnSplitCost{1, {2.0f, 2.0f, 2.0f}, 8.0f})
+                                 : pl->HG == 16 ? AttnSplitCost{2, {1.3f, 1.75f, 1.75f}, 7.0f}
+                                                : AttnSplitCost{1, {small ? 1.3f : 2.0f, 2.0f, 2.0f}, small ? 7.0f : 11.0f};
+  int chunk_tiles = option(OPT_ATTN_CHUNK_TILES);       // testing aid: a given split size
+  if (chunk_tiles < 1) chunk_tiles = attn_split_tiles(units, tiles, split_cost);
+  if (pl->HG > 8 && chunk_tiles > kMaxHeldTiles) chunk_tiles = kMaxHeldTiles;
+  while ((tiles + chunk_tiles - 1) / chunk_tiles > 65535) chunk_tiles <<= 1;      // splits run along the grid's y axis
   int ns = (tiles + chunk_tiles - 1) / chunk_tiles;
   if (ns < 1) ns = 1;
   if (const int forced = option(OPT_ATTN_SPLITS); forced >= 1) {      // testing aid: a given number of splits
@@ -1799,7 +1839,9 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   const long long items16 = units * ((tiles + 15) / 16), resident = 3LL * sm_count();
   const int want = option(OPT_ATTN_BALANCED);
   pl->balanced = (can_balance && (want >= 0 ? want > 0 : (tiles >= 32 && items16 >= resident && items16 <= 3 * resident))) ? 1 : 0;
-  pl->q_min = chunk_tiles >= 4 ? chunk_tiles / 2 : 2;
+  int q_chunk = 16;        // half of the split size, a power of two, that gives four items per SM
+  while (q_chunk > 2 && units * ((tiles + q_chunk - 1) / q_chunk) < 4LL * sm_count()) q_chunk >>= 1;
+  pl->q_min = q_chunk >= 4 ? q_chunk / 2 : 2;
   if (pl->balanced) {
     pl->n_splits = (tiles + pl->q_min - 1) / pl->q_min + 1;
     ns = pl->n_splits;
@@ -2082,9 +2124,7 @@ static msd_status_t attn_launch(const void* q_bf16, const int8_t* k_cache, const
   p.n_slots = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + pl.ws_partial_bytes);
   int balanced_ctas = 0;
   if (pl.balanced && (balanced_ctas = attn_balanced_ctas(kernel, block_threads, pl.smem_bytes, pl.tmem_cols, Hkv * pl.groups)) < 1) return MSD_ERR_CUDA;
-  // narrow groups: units along x; wide groups: splits along x (see the kernels)
-  dim3 grid(B * Hkv * pl.groups, pl.n_splits);
-  if (block_threads > kAttnThreads) grid = dim3(pl.n_splits, B * Hkv * pl.groups);
+  dim3 grid(B * Hkv * pl.groups, pl.n_splits);          // (units, splits: see the kernels)
   if (pl.balanced) grid = dim3(balanced_ctas);
   const bool pdl = option(OPT_NO_PDL) <= 0;
   if (block_threads > kAttnThreads) {
