@@ -122,14 +122,7 @@ __device__ __forceinline__ void attn_decompose_q_row(const AttnParams& p, int b,
     qv[j] = (i < nvec) ? __ldg(qrow + i) : make_uint4(0, 0, 0, 0);
   }
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    const uint32_t w[4] = {qv[j].x, qv[j].y, qv[j].z, qv[j].w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      m = fmaxf(m, fabsf(__uint_as_float(w[k] << 16)));
-      m = fmaxf(m, fabsf(__uint_as_float(w[k] & 0xFFFF0000u)));
-    }
-  }
+  for (int j = 0; j < 3; ++j) m = fmaxf(m, unit_absmax(qv[j]));
   m = warp_max(m);
   const float alpha = __fdiv_rn(m, 127.0f), beta = __fdiv_rn(alpha, 254.0f);
   const float inv_alpha = alpha > 0.0f ? __frcp_rn(alpha) : 0.0f, inv_beta = beta > 0.0f ? __frcp_rn(beta) : 0.0f;
@@ -144,27 +137,15 @@ __device__ __forceinline__ void attn_decompose_q_row(const AttnParams& p, int b,
   for (int j = 0; j < 3; ++j) {
     const int i = lane + 32 * j;
     if (i >= nvec) continue;
-    const uint32_t w[4] = {qv[j].x, qv[j].y, qv[j].z, qv[j].w};
-    uint32_t o1[2] = {0, 0}, o2[2] = {0, 0};
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float x = (e & 1) ? __uint_as_float(w[e >> 1] & 0xFFFF0000u) : __uint_as_float(w[e >> 1] << 16);
-      int c1 = 0, c2 = 0;
-      if (alpha > 0.0f) {
-        c1 = quant_i8(x, alpha, inv_alpha);
-        const float r = __fmaf_rn(-alpha, static_cast<float>(c1), x);
-        if (beta > 0.0f) c2 = quant_i8(r, beta, inv_beta);
-      }
-      o1[e >> 2] |= static_cast<uint32_t>(c1 & 0xFF) << (8 * (e & 3));
-      o2[e >> 2] |= static_cast<uint32_t>(c2 & 0xFF) << (8 * (e & 3));
-    }
+    uint2 o1, o2;
+    unit_quantize_any(qv[j], alpha, beta, inv_alpha, inv_beta, o1, o2);
     const int d = i << 3;                       // eight consecutive bytes stay inside one 16-byte swizzle chunk
     uint8_t* chunk = img + (d >> 7) * p.Rp * kChunk;
-    *reinterpret_cast<uint2*>(chunk + swz_off(h, d & 127)) = make_uint2(o1[0], o1[1]);
-    *reinterpret_cast<uint2*>(chunk + swz_off(p.HG + h, d & 127)) = make_uint2(o2[0], o2[1]);
+    *reinterpret_cast<uint2*>(chunk + swz_off(h, d & 127)) = o1;
+    *reinterpret_cast<uint2*>(chunk + swz_off(p.HG + h, d & 127)) = o2;
     if (p.q_dbg) {
-      *reinterpret_cast<uint2*>(p.q_dbg + q_row * p.D + d) = make_uint2(o1[0], o1[1]);
-      *reinterpret_cast<uint2*>(p.q_dbg + (static_cast<long long>(p.B) * p.Hq + q_row) * p.D + d) = make_uint2(o2[0], o2[1]);
+      *reinterpret_cast<uint2*>(p.q_dbg + q_row * p.D + d) = o1;
+      *reinterpret_cast<uint2*>(p.q_dbg + (static_cast<long long>(p.B) * p.Hq + q_row) * p.D + d) = o2;
     }
   }
 }
@@ -180,13 +161,7 @@ __device__ __forceinline__ void attn_decompose_q_pair(const AttnParams& p, int b
   const long long q_row = row ? attn_q_row_index(p, b, hk, grp, h) : 0;
   uint4 qv = make_uint4(0, 0, 0, 0);
   if (live) qv = __ldg(reinterpret_cast<const uint4*>(p.q + q_row * p.D) + i);
-  const uint32_t w[4] = {qv.x, qv.y, qv.z, qv.w};
-  float m = 0.0f;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    m = fmaxf(m, fabsf(__uint_as_float(w[k] << 16)));
-    m = fmaxf(m, fabsf(__uint_as_float(w[k] & 0xFFFF0000u)));
-  }
+  float m = unit_absmax(qv);
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));      // stays inside the 16 lanes
   const float alpha = __fdiv_rn(m, 127.0f), beta = __fdiv_rn(alpha, 254.0f);
@@ -199,25 +174,14 @@ __device__ __forceinline__ void attn_decompose_q_pair(const AttnParams& p, int b
     }
   }
   if (!live) return;
-  uint32_t o1[2] = {0, 0}, o2[2] = {0, 0};
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const float x = (e & 1) ? __uint_as_float(w[e >> 1] & 0xFFFF0000u) : __uint_as_float(w[e >> 1] << 16);
-    int c1 = 0, c2 = 0;
-    if (alpha > 0.0f) {
-      c1 = quant_i8(x, alpha, inv_alpha);
-      const float r = __fmaf_rn(-alpha, static_cast<float>(c1), x);
-      if (beta > 0.0f) c2 = quant_i8(r, beta, inv_beta);
-    }
-    o1[e >> 2] |= static_cast<uint32_t>(c1 & 0xFF) << (8 * (e & 3));
-    o2[e >> 2] |= static_cast<uint32_t>(c2 & 0xFF) << (8 * (e & 3));
-  }
+  uint2 o1, o2;
+  unit_quantize_any(qv, alpha, beta, inv_alpha, inv_beta, o1, o2);
   const int d = i << 3;                         // < 128: the row's single chunk
-  *reinterpret_cast<uint2*>(img + swz_off(h, d)) = make_uint2(o1[0], o1[1]);
-  *reinterpret_cast<uint2*>(img + swz_off(p.HG + h, d)) = make_uint2(o2[0], o2[1]);
+  *reinterpret_cast<uint2*>(img + swz_off(h, d)) = o1;
+  *reinterpret_cast<uint2*>(img + swz_off(p.HG + h, d)) = o2;
   if (p.q_dbg) {
-    *reinterpret_cast<uint2*>(p.q_dbg + q_row * p.D + d) = make_uint2(o1[0], o1[1]);
-    *reinterpret_cast<uint2*>(p.q_dbg + (static_cast<long long>(p.B) * p.Hq + q_row) * p.D + d) = make_uint2(o2[0], o2[1]);
+    *reinterpret_cast<uint2*>(p.q_dbg + q_row * p.D + d) = o1;
+    *reinterpret_cast<uint2*>(p.q_dbg + (static_cast<long long>(p.B) * p.Hq + q_row) * p.D + d) = o2;
   }
 }
 

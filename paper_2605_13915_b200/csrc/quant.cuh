@@ -130,4 +130,31 @@ __device__ __forceinline__ void unit_quantize(const uint4& a, float alpha, float
   quad_quantize(a.z, a.w, alpha, beta, inv_alpha, inv_beta, o1.y, o2.y);
 }
 
+// The same for any scales, a zero row included: what does not fit the fast path goes value by value with true divisions.
+__device__ __forceinline__ void unit_quantize_any(const uint4& a, float alpha, float beta, float inv_alpha, float inv_beta, uint2& o1,
+                                                  uint2& o2) {
+  if (unit_scales_ok(alpha, beta)) {
+    unit_quantize(a, alpha, beta, inv_alpha, inv_beta, o1, o2);
+    return;
+  }
+  uint32_t w[4] = {a.x, a.y, a.z, a.w};
+  unsigned long long p1 = 0, p2 = 0;
+#pragma unroll 1
+  for (int e = 0; e < 8; ++e) {
+    const float v = bf16lo(w[0]);
+    int c1 = 0, c2 = 0;
+    if (alpha > 0.0f) {
+      c1 = quant_i8(v, alpha, inv_alpha);
+      const float r = __fmaf_rn(-alpha, static_cast<float>(c1), v);
+      if (beta > 0.0f) c2 = quant_i8(r, beta, inv_beta);
+    }
+    p1 |= static_cast<unsigned long long>(c1 & 0xFF) << (8 * e);
+    p2 |= static_cast<unsigned long long>(c2 & 0xFF) << (8 * e);
+    // the next value moves into the low half of w[0]
+    w[0] = __funnelshift_r(w[0], w[1], 16); w[1] = __funnelshift_r(w[1], w[2], 16); w[2] = __funnelshift_r(w[2], w[3], 16); w[3] >>= 16;
+  }
+  o1 = make_uint2(static_cast<uint32_t>(p1), static_cast<uint32_t>(p1 >> 32));
+  o2 = make_uint2(static_cast<uint32_t>(p2), static_cast<uint32_t>(p2 >> 32));
+}
+
 }  // namespace msd
