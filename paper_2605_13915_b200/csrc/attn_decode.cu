@@ -1792,17 +1792,18 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   pl->n_splits = ns;
   pl->chunk = chunk_tiles * kTok;
   // Balanced schedule: every CTA of a grid that just fills the machine gets the same number of tiles, at least q_min
-  // (a unit of n tiles then meets at most ceil(n / q_min) + 1 CTAs).  It pays where full-size fixed splits (16 tiles)
-  // would leave the resident CTAs between one and three items each to share out - there the SMs that get one more
-  // finish a whole split later - and the sequences are long enough (32 tiles) for a run to stay inside one or two of
-  // them; elsewhere it costs a few percent (every CTA starts at once and cuts its own run first; every sequence a run
-  // enters is a new set-up).  Built for the kernels that keep three CTAs per SM (up to 8 rows per KV head, D and
-  // Dv <= 128).
+  // (a unit of n tiles then meets at most ceil(n / q_min) + 1 CTAs).  It costs a few percent (every CTA starts at once and
+  // cuts its own run first; every sequence a run enters is a new set-up), and pays where fixed splits fit badly: sequences
+  // of 32 tiles or more, up to three 16-tile splits per resident CTA, and more units than half the resident CTAs.  Against
+  // fixed splits of the size chosen above (32 query / 8 KV heads, lengths up to 8192 / all 8192): 32 sequences 65 to 67 us
+  // mixed, 100 to 97 uniform; 36: 72 to 78, 110 to 108; 44: 85 to 93, 132 to 130.  With at least two CTAs per unit in one round
+  // the fixed splits of mixed lengths fill it: 24 sequences 53 to 46, 79 to 83; 20 of up to 7000, 5 rows per KV head, 53 to 44.
+  // Built for the kernels that keep three CTAs per SM (up to 8 rows per KV head, D and Dv <= 128).
   const bool can_balance = pl->HG == 8 && pl->DC == 1 && pl->DVT == 1 && option(OPT_ATTN_SPLITS) < 1 &&
                            option(OPT_ATTN_CHUNK_TILES) < 1;
   const long long items16 = units * ((tiles + 15) / 16), resident = 3LL * sm_count();
   const int want = option(OPT_ATTN_BALANCED);
-  pl->balanced = (can_balance && (want >= 0 ? want > 0 : (tiles >= 32 && items16 >= resident && items16 <= 3 * resident))) ? 1 : 0;
+  pl->balanced = (can_balance && (want >= 0 ? want > 0 : (tiles >= 32 && 2 * units > resident && items16 >= resident && items16 <= 3 * resident))) ? 1 : 0;
   int q_chunk = 16;        // half of the split size, a power of two, that gives four items per SM
   while (q_chunk > 2 && units * ((tiles + q_chunk - 1) / q_chunk) < 4LL * sm_count()) q_chunk >>= 1;
   pl->q_min = q_chunk >= 4 ? q_chunk / 2 : 2;
