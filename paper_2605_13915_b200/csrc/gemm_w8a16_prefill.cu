@@ -18,6 +18,7 @@
 // default (CTA-scope) semantics: what is handed over is tensor memory, ordered by the tcgen05 fences.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdlib>
 
 #include "host_common.h"
@@ -44,6 +45,9 @@ struct GemmP8Params {
   int ksplit, kper;             // K splits per output tile and K stages per split (1, kstages: no split)
   int part_rows;                // ksplit > 1: rows per split of the FP32 partial-result buffer the tiles are written to
   int n_fastest;                // tile index -> (token tile, weight tile): weight tile fastest (1) or token tile fastest (0)
+  // The tiles of a last round that would leave most units idle are cut along K instead (plan_p8): tiles [0, tail0) are
+  // whole items, tile tail0 + r (r < tail_n) is tail_s items of tail_k stages that write FP32 partial tiles.
+  int tail0, tail_n, tail_s, tail_k;
   const float* alpha;           // [M]
   const float* beta;            // [M]
   const float* w_scale;         // [N]
@@ -59,7 +63,7 @@ template <bool kPair, bool kBase = false>
 __global__ void __launch_bounds__(kP8Threads, 1)
 gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_a2,
                           const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_y,
-                          const GemmP8Params p) {
+                          const __grid_constant__ CUtensorMap tmap_part, const GemmP8Params p) {
   constexpr int kStages = kPair ? kP8PairStages : kP8Stages;
   constexpr int kStageBytes = kPair ? kP8PairStageBytes : kP8StageBytes;
   extern __shared__ uint8_t smem_dyn[];
@@ -101,7 +105,25 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
   // splits in a fixed order.
   // A pair takes two token tiles at once (no K split there); its CTAs stride over the pair tiles together.
   const int m_units = kPair ? (p.m_tiles + 1) >> 1 : p.m_tiles;
-  const int total_tiles = m_units * p.n_tiles * p.ksplit;
+  const int total_tiles = p.tail_n > 0 ? p.tail0 + p.tail_n * p.tail_s : m_units * p.n_tiles * p.ksplit;
+  // item -> output tile, its range of K stages, the split of a K-split plan (row block of its partial results) and, for
+  // the tail, the number of its partial tile (-1: none)
+  auto item_of = [&](int item, int& tile_mn, int& ks0, int& ks1, int& split, int& part_tile) {
+    split = 0;
+    part_tile = -1;
+    if (p.tail_n > 0) {
+      const int t = item - p.tail0, r = t / p.tail_s, sp = t - r * p.tail_s;
+      tile_mn = t < 0 ? item : p.tail0 + r;
+      ks0 = t < 0 ? 0 : sp * p.tail_k;
+      ks1 = t < 0 ? p.kstages : min(ks0 + p.tail_k, p.kstages);
+      if (t >= 0) part_tile = sp * p.tail_n + r;
+    } else {
+      tile_mn = item / p.ksplit;
+      split = item - tile_mn * p.ksplit;
+      ks0 = split * p.kper;
+      ks1 = min(ks0 + p.kper, p.kstages);
+    }
+  };
   const int first = kPair ? blockIdx.x >> 1 : blockIdx.x, step = kPair ? gridDim.x >> 1 : gridDim.x;
   auto tile_of = [&](int tile_mn, int& mt, int& nt) {
     const int mu = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % m_units;
@@ -115,10 +137,9 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       for (int tile = first; tile < total_tiles && ok; tile += step) {
-        const int split = tile % p.ksplit, tile_mn = tile / p.ksplit;
-        int mt, nt;
+        int mt, nt, tile_mn, ks0, ks1, split, part_tile;
+        item_of(tile, tile_mn, ks0, ks1, split, part_tile);
         tile_of(tile_mn, mt, nt);
-        const int ks0 = split * p.kper, ks1 = ks0 + p.kper < p.kstages ? ks0 + p.kper : p.kstages;
         for (int ks = ks0; ks < ks1; ++ks) {
           ok = wait_bounded(&empty_bar[stage], phase ^ 1, abort, p.status);
           if (!ok) break;
@@ -152,7 +173,8 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
         ok = wait_bounded(&tempty_bar, (it & 1) ^ 1, abort, p.status);        // the epilogue has drained both accumulators
         if (!ok) break;
         tc_fence_after();
-        const int ks0 = (tile % p.ksplit) * p.kper, ks1 = ks0 + p.kper < p.kstages ? ks0 + p.kper : p.kstages;
+        int tile_mn, ks0, ks1, split, part_tile;
+        item_of(tile, tile_mn, ks0, ks1, split, part_tile);
         for (int ks = ks0; ks < ks1; ++ks) {
           ok = wait_bounded(&full_bar[stage], phase, abort, p.status);
           if (!ok) break;
@@ -196,7 +218,6 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
         if (kPair) mbar_arrive_remote(leader_tempty); else mbar_arrive(&tempty_bar);
       }
     };
-    const int ccols = (p.ytype == MSD_OUT_BF16) ? 32 : 16;
     const uint32_t swz = static_cast<uint32_t>((lane >> 1) & 3);
     int it = 0;
     bool ok = true;
@@ -204,9 +225,11 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
     // Column scales: every lane needs the same scales of a chunk.  Lane l loads the scale of the chunk's l-th column
     // one chunk ahead and the lanes fetch them from one another by shuffles.
     for (int tile = first; tile < total_tiles && ok; tile += step, ++it) {
-      const int split = tile % p.ksplit, tile_mn = tile / p.ksplit;
-      int mt, nt;
+      int mt, nt, tile_mn, ks0, ks1, split, part_tile;
+      item_of(tile, tile_mn, ks0, ks1, split, part_tile);
       tile_of(tile_mn, mt, nt);
+      const bool bf = p.ytype == MSD_OUT_BF16 && part_tile < 0;
+      const int ccols = bf ? 32 : 16;
       const int row0 = mt * kP8TileM + quad * 32, row = row0 + lane;
       float a_i = 0.0f, b_i = 0.0f;
       if constexpr (!kBase) {
@@ -230,14 +253,14 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
         sw_next = (!kBase && lane < ccols && c0 + ccols < cend && col_w + c0 + ccols < p.N) ? __ldg(p.w_scale + col_w + c0 + ccols) : 0.0f;
 #pragma unroll
         for (int hsub = 0; hsub < 2; ++hsub) {       // 16 accumulator columns per load
-          if (hsub == 1 && p.ytype != MSD_OUT_BF16) break;
+          if (hsub == 1 && !bf) break;
           uint32_t v1[16], v2[16];
           tmem_ld16(trow + c0 + 16 * hsub, v1);
           if constexpr (!kBase) tmem_ld16(trow + kP8TileN + c0 + 16 * hsub, v2);
           tmem_ld_wait();
           if constexpr (kBase) {
             // the FP32 sums as they are, rounded once to the output type
-            if (p.ytype == MSD_OUT_BF16) {
+            if (bf) {
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v1[2 * j]), __uint_as_float(v1[2 * j + 1]));
@@ -255,7 +278,7 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
               p.acc_dbg[(static_cast<long long>(p.M) + row) * p.N + col + 16 * hsub + j] = static_cast<int32_t>(v2[j]);
             }
           }
-          if (p.ytype == MSD_OUT_BF16) {
+          if (bf) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const int cj = 16 * hsub + 4 * j;
@@ -291,7 +314,8 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-          tma_store_2d(&tmap_y, col, row0 + split * p.part_rows, sb);
+          if (part_tile < 0) tma_store_2d(&tmap_y, col, row0 + split * p.part_rows, sb);
+          else tma_store_2d(&tmap_part, part * 64 + c0, part_tile * ((kPair ? 2 : 1) * kP8TileM) + (kPair ? static_cast<int>(rank) * kP8TileM : 0) + quad * 32, sb);
           bulk_commit_group();
         }
       }
@@ -311,10 +335,64 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
   }
 }
 
+// Sums of the tail's partial tiles part[split][tile r][rows][256], split 0 first (fixed order), rounded once to y.
+__global__ void __launch_bounds__(256)
+p8_tail_reduce_kernel(const float* __restrict__ part, const GemmP8Params p, int unit_rows, void* __restrict__ y, int ytype) {
+  pdl_wait_primary();
+  const int m_units = (p.m_tiles * kP8TileM + unit_rows - 1) / unit_rows;
+  const int quads = p.tail_n * unit_rows * (kP8TileN / 4);
+  const long long stride = static_cast<long long>(quads) * 4;              // floats per split
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += gridDim.x * blockDim.x) {
+    const int c = (i & (kP8TileN / 4 - 1)) * 4, rr = i / (kP8TileN / 4), r = rr / unit_rows;
+    const int tile = p.tail0 + r;
+    const int mu = p.n_fastest ? tile / p.n_tiles : tile % m_units, nt = p.n_fastest ? tile % p.n_tiles : tile / m_units;
+    const int row = mu * unit_rows + (rr - r * unit_rows), col = nt * kP8TileN + c;
+    if (row >= p.M || col >= p.N) continue;                                // (N is a multiple of 4)
+    const float* src = part + static_cast<long long>(i) * 4;
+    float4 acc = __ldg(reinterpret_cast<const float4*>(src));
+    for (int sp = 1; sp < p.tail_s; ++sp) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(src + sp * stride));
+      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+    const long long o = static_cast<long long>(row) * p.N + col;
+    if (ytype == MSD_OUT_BF16) {
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x, acc.y), h1 = __floats2bfloat162_rn(acc.z, acc.w);
+      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(y) + o) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+    } else {
+      *reinterpret_cast<float4*>(static_cast<float*>(y) + o) = acc;
+    }
+  }
+}
+
 struct GemmP8Plan {
-  int m_tiles, n_tiles, kstages, grid, ksplit, kper;
+  int m_tiles, n_tiles, kstages, ksplit, kper;
+  bool pair;                               // CTA pairs: 256 tokens x 256 weight rows on 74 pairs, otherwise 128 x 256 on 148 CTAs
+  int tail0, tail_n, tail_s, tail_k;       // see GemmP8Params (tail_n = 0: no tail)
   size_t off_q1, off_q2, off_alpha, off_beta, off_part, bytes;
 };
+
+// The round structure of `tiles` output tiles on `units` pairs or CTAs; returns its length in rounds.
+// A last round of at most half the units is cut along K (stages of 128) so that all of them share it: 1000 tokens on 14336
+// weight rows are 224 pair tiles on 74 pairs, 3.03 rounds that took four (an MLP of 4096 x 14336, both layers: 188 -> 179 us;
+// 1100 tokens, 5120 x 10240: 206 -> 186).  Pieces keep at least four
+// stages (a shorter one is all pipeline fill), and the partial tiles and their sum cost about 8 us, eleven stages.
+static double p8_rounds(long long tiles, long long units, int kstages, int* tail0, int* tail_n, int* tail_s, int* tail_k) {
+  const long long full = tiles / units * units, rest = tiles - full;
+  *tail0 = static_cast<int>(full); *tail_n = 0; *tail_s = 1; *tail_k = kstages;
+  if (rest == 0) return static_cast<double>(full / units);
+  long long sp = units / rest;
+  if (sp > kstages / 4) sp = kstages / 4;
+  if (full > 0 && sp >= 2) {
+    const int per = static_cast<int>((kstages + sp - 1) / sp);
+    if (kstages - per > 11) {
+      *tail_n = static_cast<int>(rest);
+      *tail_k = per;
+      *tail_s = (kstages + per - 1) / per;
+      return static_cast<double>(full / units) + static_cast<double>(per + 11) / kstages;
+    }
+  }
+  return static_cast<double>(full / units + 1);
+}
 
 // base: the dequantize-to-BF16 comparison path (K counted in bytes of BF16; off_q1 holds the BF16 weights)
 static GemmP8Plan plan_p8(int64_t M, int64_t N, int64_t K, bool base = false) {
@@ -327,17 +405,26 @@ static GemmP8Plan plan_p8(int64_t M, int64_t N, int64_t K, bool base = false) {
   // per SM, each at least eight stages long; the FP32 partial results are added by a second kernel.
   pl.ksplit = 1;
   pl.kper = pl.kstages;
+  const int forced_split = option(OPT_P8_KSPLIT);     // testing aid
   {
-    const int forced = option(OPT_P8_KSPLIT);     // testing aid
-    long long want = forced >= 0 ? forced : (2 * tiles <= sm_count() ? sm_count() / tiles : 1);
+    long long want = forced_split >= 0 ? forced_split : (2 * tiles <= sm_count() ? sm_count() / tiles : 1);
     if (want > pl.kstages / 8) want = pl.kstages / 8;
     if (want > 1) {
       pl.kper = static_cast<int>((pl.kstages + want - 1) / want);
       pl.ksplit = (pl.kstages + pl.kper - 1) / pl.kper;
     }
   }
-  const long long items = tiles * pl.ksplit;
-  pl.grid = static_cast<int>(items < sm_count() ? items : sm_count());
+  // CTA pairs where there is no K split and their tiles need no more rounds (an odd number of token tiles leaves a CTA
+  // idle); the option MSD_P8_PAIR forces the choice.
+  const long long pair_tiles = static_cast<long long>((pl.m_tiles + 1) / 2) * pl.n_tiles;
+  int t1[4], t2[4];
+  const double r1 = p8_rounds(tiles, sm_count(), pl.kstages, &t1[0], &t1[1], &t1[2], &t1[3]);
+  const double r2 = p8_rounds(pair_tiles, sm_count() / 2, pl.kstages, &t2[0], &t2[1], &t2[2], &t2[3]);
+  const int forced_pair = option(OPT_P8_PAIR);       // testing aid
+  pl.pair = pl.ksplit == 1 && pl.m_tiles >= 2 && (forced_pair >= 0 ? forced_pair != 0 : r2 <= 1.01 * r1);
+  const int* t = pl.pair ? t2 : t1;
+  const bool tail = pl.ksplit == 1 && forced_split < 0;
+  pl.tail0 = t[0]; pl.tail_n = tail ? t[1] : 0; pl.tail_s = t[2]; pl.tail_k = t[3];
   size_t off = 0;
   pl.off_q1 = off;    off = round_up(off + (base ? static_cast<size_t>(N) * K * 2 : static_cast<size_t>(M) * K), 1024);
   pl.off_q2 = off;    off = round_up(off + (base ? 0 : static_cast<size_t>(M) * K), 1024);
@@ -345,6 +432,7 @@ static GemmP8Plan plan_p8(int64_t M, int64_t N, int64_t K, bool base = false) {
   pl.off_beta = off;  off = round_up(off + static_cast<size_t>(M) * sizeof(float), 1024);
   pl.off_part = off;
   if (pl.ksplit > 1) off = round_up(off + static_cast<size_t>(pl.ksplit) * pl.m_tiles * kP8TileM * N * sizeof(float), 1024);
+  if (pl.tail_n > 0) off = round_up(off + static_cast<size_t>(pl.tail_s) * pl.tail_n * (pl.pair ? 2 : 1) * kP8TileM * kP8TileN * sizeof(float), 1024);
   pl.bytes = off;
   return pl;
 }
@@ -399,18 +487,10 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
   const uint64_t part_rows = static_cast<uint64_t>(pl.m_tiles) * kP8TileM;
   CUtensorMap tmap_a1, tmap_a2, tmap_b, tmap_y;
   const bool ybf = !split && ytype == MSD_OUT_BF16;
-  // CTA pairs (256 tokens x 256 weight rows per pair, half of the weight tile loaded by each CTA) where there is no K
-  // split (the option MSD_P8_PAIR forces the choice).
-  bool use_pair = false;
-  {
-    const int forced = option(OPT_P8_PAIR);       // testing aid
-    const bool can = pl.ksplit == 1 && pl.m_tiles >= 2;
-    // where the pair tiles need no more rounds on half as many units (an odd number of token tiles leaves a CTA idle)
-    const long long tiles = static_cast<long long>(pl.m_tiles) * pl.n_tiles, pair_tiles = static_cast<long long>((pl.m_tiles + 1) / 2) * pl.n_tiles;
-    const long long clusters = sm_count() / 2;
-    const bool want = (pair_tiles + clusters - 1) / clusters <= (tiles + sm_count() - 1) / sm_count();
-    use_pair = can && (forced >= 0 ? forced != 0 : want);
-  }
+  const bool use_pair = pl.pair;
+  // (the INT32 accumulators exist only for whole tiles)
+  const int tail_n = acc_dbg == nullptr ? pl.tail_n : 0;
+  const uint64_t unit_rows = (use_pair ? 2 : 1) * kP8TileM;
   if (!encode_tmap_2d(&tmap_a1, CU_TENSOR_MAP_DATA_TYPE_UINT8, a1_ptr, kb, M, kb, kP8BlockK, kP8TileM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_tmap_2d(&tmap_a2, CU_TENSOR_MAP_DATA_TYPE_UINT8, base ? a1_ptr : static_cast<const void*>(q2), kb, M, kb, kP8BlockK, kP8TileM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_tmap_2d(&tmap_b, CU_TENSOR_MAP_DATA_TYPE_UINT8, b_ptr, kb, N, kb, kP8BlockK, use_pair ? kP8TileN / 2 : kP8TileN, CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -418,12 +498,17 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
                       static_cast<uint64_t>(N), split ? part_rows * ksplit : static_cast<uint64_t>(M),
                       static_cast<uint64_t>(N) * (ybf ? 2 : 4), ybf ? 32 : 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
     return MSD_ERR_CUDA;
+  CUtensorMap tmap_part = tmap_y;
+  if (tail_n > 0 && !encode_tmap_2d(&tmap_part, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, part, kP8TileN, unit_rows * tail_n * pl.tail_s,
+                                    kP8TileN * sizeof(float), 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
+    return MSD_ERR_CUDA;
 
   GemmP8Params p;
   p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
   p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.kstages = pl.kstages;
   p.alpha = alpha; p.beta = beta; p.w_scale = w_scale; p.acc_dbg = acc_dbg; p.ytype = split ? MSD_OUT_FP32 : ytype; p.status = status;
   p.ksplit = ksplit; p.kper = kper; p.part_rows = static_cast<int>(part_rows);
+  p.tail0 = pl.tail0; p.tail_n = tail_n; p.tail_s = pl.tail_s; p.tail_k = pl.tail_k;
   {
     // A wave of CTAs either shares a few weight tiles and sweeps the token tiles (token tile fastest) or the other way
     // round; the operand that is swept should be the one that stays in L2 (40 MB assumed usable for it).
@@ -443,22 +528,25 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
     attr_done = true;
   }
   const bool pdl = option(OPT_NO_PDL) <= 0;
-  if (use_pair) {
-    const long long pair_tiles = static_cast<long long>((pl.m_tiles + 1) / 2) * pl.n_tiles;
-    const int clusters = static_cast<int>(pair_tiles < sm_count() / 2 ? pair_tiles : sm_count() / 2);
-    const cudaError_t pe = base
-        ? launch_pdl_cluster(gemm_w8a16_prefill_kernel<true, true>, dim3(2 * clusters), dim3(kP8Threads), smem_pair, s, pdl, 2u, tmap_a1, tmap_a2, tmap_b, tmap_y, p)
-        : launch_pdl_cluster(gemm_w8a16_prefill_kernel<true>, dim3(2 * clusters), dim3(kP8Threads), smem_pair, s, pdl, 2u, tmap_a1, tmap_a2, tmap_b, tmap_y, p);
-    if (pe != cudaSuccess) return MSD_ERR_CUDA;
-    return MSD_OK;
-  }
-  const long long items = static_cast<long long>(pl.m_tiles) * pl.n_tiles * ksplit;
-  const int grid = static_cast<int>(items < sm_count() ? items : sm_count());
-  const cudaError_t le = base
-      ? launch_pdl(gemm_w8a16_prefill_kernel<false, true>, dim3(grid), dim3(kP8Threads), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p)
-      : launch_pdl(gemm_w8a16_prefill_kernel<false>, dim3(grid), dim3(kP8Threads), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p);
-  if (le != cudaSuccess) return MSD_ERR_CUDA;
+  const long long units = use_pair ? sm_count() / 2 : sm_count();
+  const long long tiles = static_cast<long long>(use_pair ? (pl.m_tiles + 1) / 2 : pl.m_tiles) * pl.n_tiles;
+  const long long items = tail_n > 0 ? pl.tail0 + static_cast<long long>(tail_n) * pl.tail_s : tiles * ksplit;
+  const unsigned grid = static_cast<unsigned>(items < units ? items : units);
+  cudaError_t e;
+  if (use_pair)
+    e = base ? launch_pdl_cluster(gemm_w8a16_prefill_kernel<true, true>, dim3(2 * grid), dim3(kP8Threads), smem_pair, s, pdl, 2u, tmap_a1, tmap_a2, tmap_b, tmap_y, tmap_part, p)
+             : launch_pdl_cluster(gemm_w8a16_prefill_kernel<true>, dim3(2 * grid), dim3(kP8Threads), smem_pair, s, pdl, 2u, tmap_a1, tmap_a2, tmap_b, tmap_y, tmap_part, p);
+  else
+    e = base ? launch_pdl(gemm_w8a16_prefill_kernel<false, true>, dim3(grid), dim3(kP8Threads), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, tmap_part, p)
+             : launch_pdl(gemm_w8a16_prefill_kernel<false>, dim3(grid), dim3(kP8Threads), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, tmap_part, p);
+  if (e != cudaSuccess) return MSD_ERR_CUDA;
   if (split) return launch_ksplit_reduce(part, ksplit, static_cast<int64_t>(part_rows) * N, M, N, y, ytype, s, pdl);
+  if (tail_n > 0) {
+    const long long quads = static_cast<long long>(tail_n) * unit_rows * (kP8TileN / 4);
+    const unsigned blocks = static_cast<unsigned>(std::min<long long>((quads + 255) / 256, 4LL * sm_count()));
+    if (launch_pdl(p8_tail_reduce_kernel, dim3(blocks), dim3(256), 0, s, pdl, static_cast<const float*>(part), p, static_cast<int>(unit_rows), y, ytype) != cudaSuccess)
+      return MSD_ERR_CUDA;
+  }
   return MSD_OK;
 }
 
