@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdlib>
+#include <mutex>
 
 #include "host_common.h"
 #include "sm100.cuh"
@@ -94,8 +95,13 @@ msd_status_t launch_ksplit_reduce(const float* part, int ksplit, int64_t part_st
 
 
 // kTN = weight rows per tile: 256 (one accumulator) or 224 (two accumulators of 224 columns + the two sets of scale
-// columns fill the 512 TMEM columns exactly, so the epilogue of a tile overlaps the MMAs of the next).
-template <int kTN, bool kGrouped = false>
+// columns fill the 512 TMEM columns exactly, so the epilogue of a tile overlaps the MMAs of the next); 128 for decode
+// shapes on narrow layers (kCluster only).
+// kCluster: one token tile of at most 128 rows, one work item per CTA, and the K splits of a weight tile are the CTAs of a
+// thread-block cluster: when all of them are done every CTA writes the columns that a peer finishes into that peer's
+// shared memory (the drained pipeline), and after a second cluster barrier sums its own columns, split 0 first.  Without it
+// the FP32 partial tiles went through memory and a reduce kernel of their own (see w4_decode_shape).
+template <int kTN, bool kGrouped = false, bool kCluster = false>
 __global__ void __launch_bounds__(kW4ThreadsSf, 1)
 gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_a2,
                   const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_y,
@@ -107,7 +113,8 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   // reads 128 rows from where a component tile starts: whatever follows it there, results never stored.
   constexpr int kMaxStages = 8;
   const int a_bytes = p.a_rows * 128;
-  const int kStageBytes = 2 * a_bytes + kBBytes + kW4SfBytes;
+  constexpr int kSfbBlocks = kTN > 128 ? 2 : 1;                     // 128-row scale blocks of a weight tile
+  const int kStageBytes = 2 * a_bytes + kBBytes + 2048 + kSfbBlocks * 1024;
   const int nstages = p.nstages;
   constexpr int kAcc = (2 * kTN + 64 <= kW4TmemCols) ? 2 : 1;       // accumulators that fit beside 2 x 32 scale columns
   constexpr int kSfCol = kAcc * kTN;
@@ -141,6 +148,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   // covers kper K stages and its FP32 partial tile goes to rows [split * part_rows, ...) of a partial-sum buffer that a
   // second kernel adds up in a fixed order.
   const int total_tiles = p.m_tiles * p.n_tiles * p.ksplit;
+  bool ok_tile = true;           // kCluster: this warp's accumulator is complete
 
   if (warp == 0 || warp == 10) {
     // Two producer threads: issuing a bulk copy costs its thread 50-100 ns, and the time a freed stage waits for its
@@ -171,10 +179,10 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, b_row, &full_bar[stage]);
         } else {
           uint8_t* sf = dst + 2 * a_bytes + kBBytes;
-          size_t sfb_blk = static_cast<size_t>(2 * q.nt);
+          size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
           if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[q.mt]) * 2 * p.n_tiles;
           bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
-          bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
+          if constexpr (kSfbBlocks == 2) bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
         }
       };
       auto load_activations = [&](const Pos& q, int stage) {
@@ -289,7 +297,8 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
         const uint4* sf = reinterpret_cast<const uint4*>(smem + stage * kStageBytes + 2 * a_bytes + kBBytes) + lane;
         uint32_t v[32];
         // column order of a set: sfa1 (g0, g1), sfa2 (g0, g1), then per K group the two halves of the weight tile
-        constexpr int kBlk[8] = {0, 1, 2, 3, 4, 6, 5, 7};
+        // (a tile of 128 weight rows has one half; the columns of the other are never read)
+        constexpr int kBlk[8] = {0, 1, 2, 3, 4, kSfbBlocks == 2 ? 6 : 4, 5, kSfbBlocks == 2 ? 7 : 5};
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const uint4 q = sf[kBlk[j] * 32];
@@ -303,6 +312,9 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
         if (++stage == nstages) { stage = 0; phase ^= 1; }
       }
     }
+  } else if constexpr (kCluster) {
+    ok_tile = wait_bounded(&tfull_bar[0], 0, abort, p.status);      // the sums of this split are complete, its pipeline is drained
+    tc_fence_after();
   } else {
     // Epilogue: TMEM -> registers -> (BF16) -> this warp's staging buffer in shared memory -> TMA store.  A chunk is
     // 64 bytes of every row of the warp's 32 rows (32 BF16 or 16 FP32 columns), laid out with the 64-byte swizzle of
@@ -395,6 +407,89 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       }
     }
     if (lane == 0) bulk_wait_group<0>();            // every store has been written before the CTA goes away
+  }
+
+  if constexpr (kCluster) {
+    // Columns in chunks of 16: rank f finishes the chunks [f C / S, (f + 1) C / S).  Slot s of a CTA's buffer holds what rank s
+    // sent: [chunk][4 columns][row] pieces of 16 bytes, a warp's stores and loads (a row per lane) contiguous.
+    const int S = p.ksplit, rank = static_cast<int>(blockIdx.x) % S, nt = static_cast<int>(blockIdx.x) / S;
+    constexpr int C = kTN / 16;
+    const int per = (C + S - 1) / S;                            // most chunks a rank finishes
+    const int rows = p.a_rows, slot_bytes = per * 4 * rows * 16;
+    const int quad = warp & 3, row = quad * 32 + lane;
+    const bool epi = warp >= 2 && warp < 6 && quad * 32 < p.M;
+    const bool live = row < p.M;
+    const uint32_t trow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+    __syncwarp();
+    cluster_arrive_all();                                       // every CTA's pipeline is drained
+    cluster_wait_all();
+    if (epi && ok_tile) {
+      for (int f = 0; f < S; ++f) {
+        if (f == rank) continue;
+        const int c_begin = f * C / S, c_end = (f + 1) * C / S;
+        const uint32_t dst0 = mapa_shared(smem_u32(smem) + static_cast<uint32_t>(rank * slot_bytes + row * 16), f);
+        for (int c = c_begin; c < c_end; c += 2) {              // two chunks' tensor-memory loads in flight
+          uint32_t v[2][16];
+          __syncwarp();
+          tmem_ld16(trow + c * 16, v[0]);
+          if (c + 1 < c_end) tmem_ld16(trow + (c + 1) * 16, v[1]);
+          tmem_ld_wait();
+          if (live) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              if (c + h < c_end)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                  st_cluster_v4(dst0 + static_cast<uint32_t>(((c + h - c_begin) * 4 + j) * rows * 16), v[h][4 * j], v[h][4 * j + 1], v[h][4 * j + 2], v[h][4 * j + 3]);
+          }
+        }
+      }
+    }
+    __syncwarp();
+    cluster_arrive_all();                                       // everything has been delivered
+    cluster_wait_all();
+    if (epi && ok_tile) {
+      const int c_begin = rank * C / S, c_end = (rank + 1) * C / S;
+      for (int c = c_begin; c < c_end; ++c) {
+        uint32_t own[16];
+        __syncwarp();                                           // the load is the whole warp's
+        tmem_ld16(trow + c * 16, own);
+        tmem_ld_wait();
+        const int col = nt * kTN + c * 16;
+        if (!live || col >= p.N) continue;
+        float acc[16];
+        for (int s = 0; s < S; ++s) {
+          const uint8_t* src = smem + s * slot_bytes + (c - c_begin) * 4 * rows * 16 + row * 16;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 v = s == rank ? make_float4(__uint_as_float(own[4 * j]), __uint_as_float(own[4 * j + 1]), __uint_as_float(own[4 * j + 2]), __uint_as_float(own[4 * j + 3]))
+                                       : *reinterpret_cast<const float4*>(src + j * rows * 16);
+            acc[4 * j] = s == 0 ? v.x : acc[4 * j] + v.x;
+            acc[4 * j + 1] = s == 0 ? v.y : acc[4 * j + 1] + v.y;
+            acc[4 * j + 2] = s == 0 ? v.z : acc[4 * j + 2] + v.z;
+            acc[4 * j + 3] = s == 0 ? v.w : acc[4 * j + 3] + v.w;
+          }
+        }
+        const size_t at = static_cast<size_t>(row) * p.N + col;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {                           // N is a multiple of 8
+          if (col + 8 * h >= p.N) break;
+          if (p.ytype == MSD_OUT_BF16) {
+            uint32_t o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const __nv_bfloat162 b2 = __floats2bfloat162_rn(acc[8 * h + 2 * j], acc[8 * h + 2 * j + 1]);
+              o[j] = *reinterpret_cast<const uint32_t*>(&b2);
+            }
+            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.y) + at + 8 * h) = make_uint4(o[0], o[1], o[2], o[3]);
+          } else {
+            float* y = static_cast<float*>(p.y) + at + 8 * h;
+            *reinterpret_cast<float4*>(y) = make_float4(acc[8 * h], acc[8 * h + 1], acc[8 * h + 2], acc[8 * h + 3]);
+            *reinterpret_cast<float4*>(y + 4) = make_float4(acc[8 * h + 4], acc[8 * h + 5], acc[8 * h + 6], acc[8 * h + 7]);
+          }
+        }
+      }
+    }
   }
 
   tc_fence_before();
@@ -671,6 +766,8 @@ gemm_w4a16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid
 
 struct GemmW4Plan {
   int m_tiles, n_tiles, kstages, sf_kgroups, grid, tile_n;
+  int cluster;                  // > 1: K splits of a weight tile = CTAs of a cluster (kCluster)
+  int sf_tile_rows;             // weight rows per tile of the blocked scale layout (224 or 256; 128-row tiles use 256)
   int ksplit, kper, a_rows, nstages;
   size_t off_q1, off_q2, off_sfa1, off_sfa2, off_sfb, off_part, bytes;
 };
@@ -699,9 +796,84 @@ static int w4_tile_n(bool pair = false) {
   return pair ? 256 : 224;
 }
 
+using W4Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmW4Params, GemmW4NoGroups);
+static W4Kernel w4_cluster_kernel(int tile_n) {
+  return tile_n == 128 ? gemm_w4a16_kernel<128, false, true> : tile_n == 224 ? gemm_w4a16_kernel<224, false, true> : gemm_w4a16_kernel<256, false, true>;
+}
+
+// How many clusters of S CTAs of that kernel the device holds at once (0 on error).
+static int w4_resident_clusters(int tile_n, int S) {
+  struct Entry { int tile_n, S, n; };
+  static std::mutex mu;
+  static Entry cache[32];
+  static int used = 0;
+  std::lock_guard<std::mutex> lock(mu);
+  for (int i = 0; i < used; ++i)
+    if (cache[i].tile_n == tile_n && cache[i].S == S) return cache[i].n;
+  const W4Kernel kernel = w4_cluster_kernel(tile_n);
+  int n = 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(S) * 64);
+  cfg.blockDim = dim3(kW4ThreadsSf);
+  cfg.dynamicSmemBytes = 227 * 1024 - 2048;          // (one CTA per SM whatever the stages)
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(S);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+  if (used < 32) cache[used++] = Entry{tile_n, S, n};
+  return n;
+}
+
+// Pipeline of a launch that loads a_rows rows per component tile: stages that fit and bytes of a stage.
+static void w4_stages(int a_rows, int tile_n, size_t extra_bytes, int* nstages, size_t* stage_bytes) {
+  *stage_bytes = static_cast<size_t>(2 * a_rows * 128 + tile_n * 128 + 2048 + (tile_n > 128 ? 2048 : 1024));
+  const int ns = static_cast<int>((227 * 1024 - 2048 - extra_bytes - 1024) / *stage_bytes);
+  *nstages = ns > 8 ? 8 : ns;
+}
+
+// Decode shapes (one token tile): tile width and K splits as a cluster.  Every CTA has one item, so the call takes as long as
+// the longest item, width x stages: the smallest wins, of equal ones the smaller cluster.  At most 8 CTAs a cluster, items
+// of at least two stages, all clusters resident at once.  cluster = 1: no split gains anything, or none fits.
+static void w4_decode_shape(int64_t M, int64_t N, int kstages, int* tile_n, int* cluster) {
+  const int a_rows = static_cast<int>((M + 7) / 8 * 8);
+  *cluster = 1;
+  long long best = 0;
+  for (const int w : {128, 224, 256}) {
+    const long long tiles = (N + w - 1) / w;
+    long long S = sm_count() / tiles;
+    if (S > 8) S = 8;
+    if (S > kstages / 2) S = kstages / 2;
+    for (; S >= 2; --S) {
+      const int per = static_cast<int>((kstages + S - 1) / S);
+      if ((kstages + per - 1) / per != S) continue;                     // a split without stages
+      const long long cost = static_cast<long long>(w) * per * 16 + S;
+      if (best != 0 && cost >= best) break;
+      int nstages;
+      size_t stage_bytes;
+      w4_stages(a_rows, w, 0, &nstages, &stage_bytes);
+      const size_t slots = static_cast<size_t>(S) * ((w / 16 + S - 1) / S) * 64 * a_rows;        // what the peers send, in the drained pipeline
+      if (slots > nstages * stage_bytes || w4_resident_clusters(w, static_cast<int>(S)) < tiles) continue;
+      best = cost; *tile_n = w; *cluster = static_cast<int>(S);
+      break;
+    }
+  }
+}
+
 static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   GemmW4Plan pl;
-  const int tile_n = w4_tile_n(w4_use_pair(M, N, K));
+  int tile_n = w4_tile_n(w4_use_pair(M, N, K));
+  pl.cluster = 1;
+  if (M <= kW4TileM && option(OPT_W4_TILEN) < 0 && option(OPT_W4_KSPLIT) < 0 && option(OPT_W4_PAIR) < 0)
+    w4_decode_shape(M, N, static_cast<int>((K + kW4BlockK - 1) / kW4BlockK), &tile_n, &pl.cluster);
+  pl.sf_tile_rows = tile_n == 224 ? 224 : 256;
   pl.tile_n = tile_n;
   pl.m_tiles = static_cast<int>((M + kW4TileM - 1) / kW4TileM);
   pl.n_tiles = static_cast<int>((N + tile_n - 1) / tile_n);
@@ -720,6 +892,10 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
       pl.kper = (pl.kstages + want - 1) / want;
       pl.ksplit = (pl.kstages + pl.kper - 1) / pl.kper;
     }
+    if (pl.cluster > 1) {
+      pl.ksplit = pl.cluster;
+      pl.kper = (pl.kstages + pl.ksplit - 1) / pl.ksplit;
+    }
   }
   const int items = tiles * pl.ksplit;
   int grid = sm_count();
@@ -727,19 +903,16 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   pl.grid = grid;
   // one token tile of fewer than 128 rows: only those rows are loaded and the stages are packed (more of them fit)
   pl.a_rows = pl.m_tiles == 1 ? static_cast<int>((M + 7) / 8 * 8) : kW4TileM;
-  {
-    const size_t stage_bytes = static_cast<size_t>(2 * pl.a_rows * 128 + tile_n * 128 + kW4SfBytes);
-    int ns = static_cast<int>((227 * 1024 - 2048 - 8 * kW4StoreBytes - 1024) / stage_bytes);
-    pl.nstages = ns > 8 ? 8 : ns;
-  }
+  size_t stage_bytes;
+  w4_stages(pl.a_rows, tile_n, pl.cluster > 1 ? 0 : 8 * kW4StoreBytes, &pl.nstages, &stage_bytes);
   size_t off = 0;
   pl.off_q1 = off;   off = round_up(off + static_cast<size_t>(M) * (K / 2), 1024);
   pl.off_q2 = off;   off = round_up(off + static_cast<size_t>(M) * (K / 2), 1024);
   pl.off_sfa1 = off; off = round_up(off + static_cast<size_t>(pl.m_tiles) * pl.sf_kgroups * 512, 1024);
   pl.off_sfa2 = off; off = round_up(off + static_cast<size_t>(pl.m_tiles) * pl.sf_kgroups * 512, 1024);
-  pl.off_sfb = off;  off = round_up(off + static_cast<size_t>(2 * pl.n_tiles) * pl.sf_kgroups * 512, 1024);
+  pl.off_sfb = off;  off = round_up(off + static_cast<size_t>(2 * ((N + pl.sf_tile_rows - 1) / pl.sf_tile_rows)) * pl.sf_kgroups * 512, 1024);
   pl.off_part = off;
-  if (pl.ksplit > 1) off = round_up(off + static_cast<size_t>(pl.ksplit) * pl.m_tiles * kW4TileM * N * sizeof(float), 1024);
+  if (pl.ksplit > 1 && pl.cluster == 1) off = round_up(off + static_cast<size_t>(pl.ksplit) * pl.m_tiles * kW4TileM * N * sizeof(float), 1024);
   pl.bytes = off;
   return pl;
 }
@@ -884,12 +1057,13 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
   const bool pdl = option(OPT_NO_PDL) <= 0;
   SfRelayout rl = {};
   rl.src = w_e8m0; rl.dst = ws + pl.off_sfb; rl.rows = N; rl.kblocks = static_cast<int>(K / 32);
-  rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = pl.tile_n; rl.row_blocks = 2 * pl.n_tiles;
+  rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = pl.sf_tile_rows;
+  rl.row_blocks = 2 * static_cast<int>((N + pl.sf_tile_rows - 1) / pl.sf_tile_rows);
   // (scales prepared once by msd_prepare_w4a16_scales: nothing to bring into the blocked layout here)
   const uint8_t* sfb = ws + pl.off_sfb;
   if (prepared) {
     const PreparedScales ps = prepared_scales_layout(1, N, K);
-    sfb = prepared + (pl.tile_n == 224 ? ps.off224 : ps.off256);
+    sfb = prepared + (pl.sf_tile_rows == 224 ? ps.off224 : ps.off256);
   }
   msd_status_t st = launch_decompose_mxfp4(x_bf16, M, K, K, q1, q2, ws + pl.off_sfa1, ws + pl.off_sfa2, pl.sf_kgroups, s,
                                            prepared ? nullptr : &rl);
@@ -918,7 +1092,7 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
 
   // With a K split the kernel writes FP32 partial tiles (split s at rows s * part_rows ...) and a second kernel adds them.
   CUtensorMap tmap_y;
-  const bool split = pl.ksplit > 1 && !use_pair;        // the CTA-pair kernel does not split K
+  const bool split = pl.ksplit > 1 && pl.cluster == 1 && !use_pair;        // the CTA-pair kernel does not split K
   const bool ybf = !split && ytype == MSD_OUT_BF16;
   float* part = reinterpret_cast<float*>(ws + pl.off_part);
   const uint64_t part_rows = static_cast<uint64_t>(pl.m_tiles) * kW4TileM;
@@ -952,6 +1126,15 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
   if (split) p.ytype = MSD_OUT_FP32;
   p.ksplit = pl.ksplit; p.kper = pl.kper; p.part_rows = static_cast<int>(part_rows);
   p.a_rows = pl.a_rows; p.nstages = pl.nstages;
+  if (pl.cluster > 1) {          // (its shared-memory limit was raised when the plan asked how many clusters fit)
+    int nstages;
+    size_t stage_bytes;
+    w4_stages(pl.a_rows, pl.tile_n, 0, &nstages, &stage_bytes);
+    if (launch_pdl_cluster(w4_cluster_kernel(pl.tile_n), dim3(pl.grid), dim3(kW4ThreadsSf), nstages * stage_bytes + 1024, s, pdl,
+                           static_cast<unsigned>(pl.cluster), tmap_a1, tmap_a2, tmap_b, tmap_y, p, GemmW4NoGroups()) != cudaSuccess)
+      return MSD_ERR_CUDA;
+    return MSD_OK;
+  }
   const size_t smem_bytes = static_cast<size_t>(pl.nstages) * (2 * pl.a_rows * 128 + pl.tile_n * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
   static bool attr_done = false;
   if (!attr_done) {

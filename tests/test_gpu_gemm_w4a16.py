@@ -128,3 +128,21 @@ def test_prepared_weight_scales(M, N, K, pair, tile):
         assert torch.equal(y, plain)
     yb = binding.gemm_w4a16(xd, qd, None, out_dtype=torch.bfloat16, prepared=prepared)
     assert torch.equal(yb, binding.gemm_w4a16(xd, qd, ed, out_dtype=torch.bfloat16))
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 4096, 2048), (16, 4088, 14336), (33, 1000, 1280), (61, 14336, 1024), (128, 2056, 4096),
+                                   (8, 8, 4096), (100, 136, 8192), (17, 16776, 1152)])
+def test_decode_k_split_as_a_cluster(M, N, K):
+    """One token tile with the K splits of a weight tile as the CTAs of a cluster: every tile width, ragged last tiles (one 8-column
+    piece among them), uneven last splits, one row to a full tile; row-major and prepared scales give the same bits, FP32
+    against the oracle, BF16 the FP32 result rounded once."""
+    c = inputs.gemm_w4_case(M, N, K, seed=M + N)
+    x, w, e = bf16_dev(c.x), dev(c.w_fp4), dev(c.w_e8m0)
+    y = binding.gemm_w4a16(x, w, e, out_dtype=torch.float32)
+    prep = binding.prepare_w4a16_scales(e)
+    y2 = binding.gemm_w4a16(x, w, None, out_dtype=torch.float32, prepared=prep)
+    yb = binding.gemm_w4a16(x, w, None, out_dtype=torch.bfloat16, prepared=prep)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
+    _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)
