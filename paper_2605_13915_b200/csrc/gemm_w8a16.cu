@@ -264,8 +264,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
   __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
   __shared__ __align__(8) uint64_t tfull_bar[2];
   __shared__ __align__(8) uint64_t tempty_bar[2];
-  __shared__ __align__(8) uint64_t cfree_bar, crecv_bar, cdone_bar;
-  __shared__ float s_red[4];      // mode 2: "pipelines of the cluster drained", "partials delivered"
+  __shared__ __align__(8) uint64_t cfree_bar, crecv_bar;      // mode 2: "pipelines of the cluster drained", "partials delivered"
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   __shared__ int is_last_flag;
@@ -334,14 +333,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     }
     if (p.mode == 2) {
       mbar_init(&cfree_bar, p.csplit);               // one arrival per CTA of the cluster
-      mbar_init(&crecv_bar, 1);                      // this CTA's own arrival; the peers' copies count in bytes
-      {
-        // finishing CTAs this one sends to: each lets it know when its copy has landed
-        const int G8i = p.Mp >> 3, Fi = p.csplit < G8i ? p.csplit : G8i;
-        const int ranki = static_cast<int>(blockIdx.x) % p.csplit;
-        const int n_to = Fi - (ranki < Fi ? 1 : 0);
-        mbar_init(&cdone_bar, n_to > 0 ? n_to : 1);
-      }
+      mbar_init(&crecv_bar, 4 * (p.csplit - 1));     // one arrival per epilogue warp of every peer
     }
     abort_flag = 0;
   }
@@ -523,7 +515,6 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     }
     named_bar_sync(1, 128);
     int seg = 0;
-    int sent_to = 0;           // mode 2: finishing CTAs whose acknowledgement is outstanding
     bool ok = true;
     long long blk = blk_begin;
     while (blk < blk_end && ok) {
@@ -564,18 +555,24 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
         const int tmax = 8 * ((G8 + F - 1) / F);
         const int passes = kBase ? 1 : 2;
         const int slot_words = passes * tmax * kTileN;
-        // shared memory of the drained pipeline: S-1 incoming slots (one per peer), then the outgoing staging slots
-        uint8_t* stage_out = smem + static_cast<size_t>(S - 1) * slot_words * 4;
-        // 1. this CTA's own MMAs are complete, so it may overwrite its own buffers: stage what the others will finish
-        int oi = 0;
+        finish = rank < F;
+        if (finish) { tok0 = 8 * (rank * G8 / F); tok1 = 8 * ((rank + 1) * G8 / F); }
+        // 1. this CTA's MMAs are complete, so its pipeline is drained: tell every CTA of the cluster, wait for all
+        cluster_wait_all();                     // every CTA of the cluster has initialised its barriers
+        if (et < S) mbar_arrive_cluster(mapa_shared(smem_u32(&cfree_bar), et));
+        ok = wait_bounded_cluster(&cfree_bar, 0, abort, p.status);
+        if (!ok) break;
+        // 2. the sums of the tokens a peer finishes go straight from tensor memory into this rank's slot of the peer's
+        // shared memory, up to 32 columns' loads in flight (copied to a staging buffer and sent on with a bulk copy per peer
+        // the exchange took about twice as long: 61 tokens on 4096 weight rows, last MMA to end 6.0 us)
         for (int f = 0; f < F; ++f) {
           if (f == rank) continue;
           const int ft0 = 8 * (f * G8 / F), ft1 = 8 * ((f + 1) * G8 / F), fT = ft1 - ft0;
-          uint8_t* so = stage_out + static_cast<size_t>(oi) * slot_words * 4;
+          const uint32_t slot = mapa_shared(smem_u32(smem) + static_cast<uint32_t>((rank < f ? rank : rank - 1) * slot_words + r * 4) * 4u, f);
           for (int ps = 0; ps < passes; ++ps) {
-            uint8_t* srow = so + static_cast<size_t>(ps * fT * kTileN + r * 4) * 4;
+            const uint32_t dst = slot + static_cast<uint32_t>(ps * fT * kTileN) * 4u;
             for (int c = ft0; c < ft1; c += 32) {
-              const int nc = ft1 - c < 32 ? ft1 - c : 32;     // up to 32 columns per round, their TMEM loads in flight together
+              const int nc = ft1 - c < 32 ? ft1 - c : 32;
               uint32_t v[4][8];
 #pragma unroll
               for (int g = 0; g < 4; ++g)
@@ -584,51 +581,22 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
 #pragma unroll
               for (int g = 0; g < 4; ++g) {
                 if (g * 8 < nc) {
-                  uint8_t* d = srow + static_cast<size_t>(((c - ft0 + g * 8) >> 2) * (kTileN * 4)) * 4;
-                  *reinterpret_cast<uint4*>(d) = make_uint4(v[g][0], v[g][1], v[g][2], v[g][3]);
-                  *reinterpret_cast<uint4*>(d + kTileN * 16) = make_uint4(v[g][4], v[g][5], v[g][6], v[g][7]);
+                  const uint32_t d = dst + static_cast<uint32_t>(((c - ft0 + g * 8) >> 2) * (kTileN * 4)) * 4u;
+                  st_cluster_v4(d, v[g][0], v[g][1], v[g][2], v[g][3]);
+                  st_cluster_v4(d + kTileN * 16, v[g][4], v[g][5], v[g][6], v[g][7]);
                 }
               }
             }
           }
-          ++oi;
-        }
-        fence_proxy_async_smem();               // the copy engine reads what these threads wrote
-        finish = rank < F;
-        if (finish) {
-          tok0 = 8 * (rank * G8 / F);
-          tok1 = 8 * ((rank + 1) * G8 / F);
-          // bytes this CTA is going to receive (posted before any peer can start sending)
-          if (et == 0) mbar_arrive_expect_tx(&crecv_bar, static_cast<uint32_t>((S - 1) * passes * (tok1 - tok0) * kTileN * 4));
-        }
-        named_bar_sync(1, 128);
-        // 2. the pipelines of all CTAs of the cluster are drained: tell every CTA (itself included), wait for all
-        cluster_wait_all();                     // every CTA of the cluster has initialised its barriers
-        if (et < S) mbar_arrive_cluster(mapa_shared(smem_u32(&cfree_bar), et));
-        ok = wait_bounded_cluster(&cfree_bar, 0, abort, p.status);
-        if (!ok) break;
-        // 3. one bulk copy per finishing peer, straight into its slot for this rank
-        if (et == 0) {
-          oi = 0;
-          for (int f = 0; f < F; ++f) {
-            if (f == rank) continue;
-            const int fT = 8 * ((f + 1) * G8 / F) - 8 * (f * G8 / F);
-            const int slot = rank < f ? rank : rank - 1;
-            bulk_copy_to_peer(mapa_shared(smem_u32(smem) + static_cast<uint32_t>(slot * slot_words) * 4u, f),
-                              stage_out + static_cast<size_t>(oi) * slot_words * 4,
-                              static_cast<uint32_t>(passes * fT * kTileN * 4), mapa_shared(smem_u32(&crecv_bar), f));
-            ++oi;
-          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&crecv_bar), f));     // (release: the warp's stores come before it)
         }
         if (finish) {
           ok = wait_bounded_cluster(&crecv_bar, 0, abort, p.status);
           if (!ok) break;
-          // the senders may let go of their staging buffers (and exit)
-          if (et < S && et != rank) mbar_arrive_cluster(mapa_shared(smem_u32(&cdone_bar), et));
           rv.base = reinterpret_cast<const int32_t*>(smem);
           rv.S = S; rv.self = rank; rv.slot_words = slot_words; rv.T = tok1 - tok0; rv.t0 = tok0;
         }
-        sent_to = F - (rank < F ? 1 : 0);
       } else if (!complete) {
         // add this CTA's partial sums into the tile's meeting place, then find out whether it was the last contributor
         acc_tile = p.accum + static_cast<long long>(tile) * p.NB * kTileN;
@@ -672,8 +640,6 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
       ++seg;
       blk = seg_end;
     }
-    // mode 2: the staging buffers must outlive the copies that read them
-    if (sent_to > 0 && ok) wait_bounded_cluster(&cdone_bar, 0, abort, p.status);
     if (et == 0) { trace_mark(p, 10); if (p.trace) p.trace[blockIdx.x * 16 + 11] = seg; }
   }
 
@@ -777,9 +743,9 @@ static GemmW8Plan plan_w8(int64_t M, int64_t N, int64_t K, bool base = false) {
     if (S > 8) S = 8;
     if (S > pl.kblocks) S = pl.kblocks;
     for (; S >= 2; --S) {
-      // S-1 incoming and S-1 outgoing slots of [passes][longest token range][128] sums live in the drained pipeline
+      // S-1 incoming slots of [passes][longest token range][128] sums live in the drained pipeline
       const int G8 = pl.Mp / 8, F = S < G8 ? S : G8;
-      const size_t xfer = 2 * static_cast<size_t>(S - 1) * (base ? 1 : 2) * 8 * ((G8 + F - 1) / F) * kTileN * sizeof(int32_t);
+      const size_t xfer = static_cast<size_t>(S - 1) * (base ? 1 : 2) * 8 * ((G8 + F - 1) / F) * kTileN * sizeof(int32_t);
       if (xfer <= static_cast<size_t>(pl.epi_off)) break;
     }
     if (S >= 2) {

@@ -103,13 +103,6 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t caddr, uint32_t v) {
 __device__ __forceinline__ void st_cluster_v4(uint32_t caddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(caddr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-// Asynchronous copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from this CTA's shared memory into a
-// peer's; completion is counted in bytes on a barrier of the destination CTA.
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_caddr, const void* src_local, uint32_t bytes, uint32_t mbar_caddr) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst_caddr), "r"(smem_u32(src_local)), "r"(bytes), "r"(mbar_caddr)
-               : "memory");
-}
 // generic <-> async proxy ordering for every state space (global memory written with plain stores, read by TMA)
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void fence_acq_rel_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
