@@ -45,7 +45,9 @@ struct GemmW8Params {
   int csplit;              // mode 2: CTAs per cluster = K slices per weight tile
   int pre_stages;          // stages whose weight boxes are requested before waiting for the preceding kernel
   int epi_off;             // byte offset of the epilogue's transpose buffer in dynamic shared memory
-  int kb_rot_step;         // mode 1: CTA c starts its K loop at block (c * kb_rot_step) % kblocks
+  int kb_rot;              // mode 1: every CTA starts its K loop at a block of its own
+  int share_q, share_r;    // mode 1: groups8 = share_q * CTAs + share_r, mode 2: kblocks = share_q * csplit + share_r; the first
+                           // share_r get one more (the split without a division at the start of the kernel)
   int kblocks;             // K blocks per weight tile
   int num_tiles;
   long long total_blocks;  // num_tiles * kblocks
@@ -290,36 +292,47 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
   uint8_t* epi_buf = smem + p.epi_off;             // 16 KB transpose buffer of the epilogue, after the pipeline stages
   const int x_chunk_bytes = p.NB * kBlockK;
 
+  const int mode = kGrouped ? 0 : p.mode;          // a grouped launch is always stream-K: nothing of the other splits is compiled in
   const long long grid = gridDim.x;
-  // mode 0: this CTA's slice of the tile-major (tile, K block) sequence; mode 1: its row band and every K block
+  // mode 0: this CTA's slice of the tile-major (tile, K block) sequence; mode 1: its row band and every K block.
+  // Everything up to the first weight request is on the critical path of every call: with 64-bit divisions here that
+  // request left 2300 cycles after the kernel's start.
   long long blk_begin, blk_end;
   int band_row0 = 0, band_h = kTileN;
-  if (p.mode == 0) {
-    blk_begin = range_begin(blockIdx.x, p.total_blocks, grid);
-    blk_end = range_begin(blockIdx.x + 1, p.total_blocks, grid);
-  } else if (p.mode == 2) {
-    // a cluster of csplit CTAs per weight tile, CTA `rank` of it takes the rank-th slice of the tile's K blocks
-    const int tile2 = blockIdx.x / p.csplit, rank = blockIdx.x - tile2 * p.csplit;
-    blk_begin = static_cast<long long>(tile2) * p.kblocks + rank * p.kblocks / p.csplit;
-    blk_end = static_cast<long long>(tile2) * p.kblocks + (rank + 1) * p.kblocks / p.csplit;
-  } else {
-    const int g0 = static_cast<int>(range_begin(blockIdx.x, p.groups8, grid));
-    const int g1 = static_cast<int>(range_begin(blockIdx.x + 1, p.groups8, grid));
-    band_row0 = p.gran * g0;
-    band_h = p.gran * (g1 - g0);
+  int tile0, kbi0;                                   // tile and K block of blk_begin
+  if (mode == 1) {
+    const int c = blockIdx.x;
+    band_row0 = p.gran * (c * p.share_q + min(c, p.share_r));
+    band_h = p.gran * (p.share_q + (c < p.share_r ? 1 : 0));
+    tile0 = 0;
+    kbi0 = 0;
     blk_begin = 0;
     blk_end = p.kblocks;
+  } else if (mode == 2) {
+    // a cluster of csplit CTAs per weight tile, CTA `rank` of it takes the rank-th slice of the tile's K blocks
+    const int rank = static_cast<int>(cluster_ctarank());
+    tile0 = static_cast<int>(cluster_id());
+    kbi0 = rank * p.share_q + min(rank, p.share_r);
+    blk_begin = static_cast<long long>(tile0) * p.kblocks + kbi0;
+    blk_end = blk_begin + p.share_q + (rank < p.share_r ? 1 : 0);
+  } else {
+    blk_begin = range_begin(blockIdx.x, p.total_blocks, grid);
+    blk_end = range_begin(blockIdx.x + 1, p.total_blocks, grid);
+    tile0 = blk_begin < (1LL << 32) ? static_cast<int>(static_cast<unsigned>(blk_begin) / static_cast<unsigned>(p.kblocks))
+                                    : static_cast<int>(blk_begin / p.kblocks);
+    kbi0 = static_cast<int>(blk_begin - static_cast<long long>(tile0) * p.kblocks);
   }
   // One weight box in shared memory: a 3-D box packs its kw chunks back to back at this CTA's own band height (a
   // multiple of 8 rows, so every chunk still starts on a 1 KB swizzle atom); 2-D boxes sit at the plan's stride.
-  const int w_chunk = (p.tma3d && p.mode == 1) ? band_h * kBlockK : p.w_chunk_bytes;
+  const int w_chunk = (p.tma3d && mode == 1) ? band_h * kBlockK : p.w_chunk_bytes;
   const int w_stage_bytes = p.kw * w_chunk;
   const int stage_bytes = w_stage_bytes + p.kw * x_chunk_bytes;
   // Mode 1: every CTA walks K from its own starting block so that concurrent requests of the CTAs spread over the
   // whole row instead of hitting the same 128-byte column of every row (integer sums do not depend on the order).
-  const int kb_rot = (p.mode == 1) ? static_cast<int>((static_cast<long long>(blockIdx.x) * p.kb_rot_step) % p.kblocks) : 0;
-  const CUtensorMap* wmap = (p.mode == 1 && band_h != p.hmax) ? &tmap_w2 : &tmap_w;
-  const int tx_bytes = p.kw * ((p.mode == 0 ? kWStageBytes : band_h * kBlockK) + x_chunk_bytes);
+  // (the golden ratio's multiples, scaled to the number of blocks)
+  const int kb_rot = (mode == 1 && p.kb_rot) ? static_cast<int>(__umulhi(blockIdx.x * 0x9E3779B9u, static_cast<unsigned>(p.kblocks))) : 0;
+  const CUtensorMap* wmap = (mode == 1 && band_h != p.hmax) ? &tmap_w2 : &tmap_w;
+  const int tx_bytes = p.kw * ((mode == 0 ? kWStageBytes : band_h * kBlockK) + x_chunk_bytes);
 
   // the barriers of the pipeline stages one stage per lane of the producer warp, the others by its first lane
   if (warp == 0 && lane < p.num_stages) {
@@ -331,7 +344,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
       mbar_init(&tfull_bar[a], 1);
       mbar_init(&tempty_bar[a], 4);      // one arrival per epilogue warp
     }
-    if (p.mode == 2) {
+    if (mode == 2) {
       mbar_init(&cfree_bar, p.csplit);               // one arrival per CTA of the cluster
       mbar_init(&crecv_bar, 4 * (p.csplit - 1));     // one arrival per epilogue warp of every peer
     }
@@ -387,9 +400,6 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     c = w_lane ? lane : (lane - p.kw) % p.kw;
     x_half = w_lane ? 0 : (lane - p.kw) / p.kw;
     // (tile, K block) of the next block to load, advanced by one per stage; kbr = rotated K block
-    const int tile0 = blk_begin < (1LL << 32) ? static_cast<int>(static_cast<unsigned>(blk_begin) / static_cast<unsigned>(p.kblocks))
-                                              : static_cast<int>(blk_begin / p.kblocks);
-    const int kbi0 = static_cast<int>(blk_begin - static_cast<long long>(tile0) * p.kblocks);
     tile = tile0; kbi = kbi0;
     tile_first = tile0; kbi_first = kbi0;
     kbr = kbi + kb_rot;
@@ -410,7 +420,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
   }
   if (warp == 1) tmem_alloc(&tmem_base_slot, p.tmem_cols);
   tc_fence_before();
-  if (p.mode == 2) cluster_arrive_all();    // "my barriers are initialised": the epilogue warps wait for the peers' before their first remote arrive
+  if (mode == 2) cluster_arrive_relaxed_all();    // "my barriers are initialised": the epilogue warps wait for the peers' before their first remote arrive
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
@@ -547,7 +557,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
       int32_t* acc_tile = nullptr;
       int tok0 = 0, tok1 = p.Mp;
       RecvInfo rv = {nullptr, 0, 0, 0, 0, 0};
-      if (p.mode == 2 && p.csplit > 1) {
+      if (mode == 2 && p.csplit > 1) {
         // ---- split-K inside a cluster: partial sums travel through the peers' shared memory ----
         // Finishing is shared out as well: owner f < F completes the tokens of its groups of 8 for the whole tile.
         const int S = p.csplit, rank = static_cast<int>(blockIdx.x) - tile * S;
@@ -927,10 +937,11 @@ msd_status_t msd_gemm_w8a16_ex(const void* x_bf16, const int8_t* w, const float*
   GemmW8Params p;
   p.tma3d = t3 ? 1 : 0;
   p.M = static_cast<int>(M); p.Mp = pl.Mp; p.NB = pl.NB; p.N = static_cast<int>(N); p.K = static_cast<int>(K);
-  p.kb_rot_step = 5;
+  p.kb_rot = 1;
   p.pre_stages = 64;
   p.mode = pl.mode; p.groups8 = pl.groups8; p.gran = pl.gran; p.hmax = pl.hmax; p.w_chunk_bytes = pl.w_chunk_bytes; p.kw = pl.kw; p.epi_off = pl.epi_off; p.csplit = pl.csplit;
   p.kblocks = pl.kblocks; p.num_tiles = pl.num_tiles; p.total_blocks = pl.total_blocks;
+  { const int whole = pl.mode == 1 ? pl.groups8 : pl.kblocks, parts = pl.mode == 1 ? pl.grid : pl.csplit; p.share_q = whole / parts; p.share_r = whole % parts; }
   p.num_stages = pl.stages; p.tmem_cols = pl.tmem_cols; p.ytype = ytype;
   p.w_scale = w_scale; p.alpha = alpha; p.beta = beta; p.y = y; p.acc_dbg = acc_dbg;
   p.accum = reinterpret_cast<int32_t*>(ws + pl.off_slots);
@@ -983,10 +994,11 @@ msd_status_t msd_gemm_dequant_bf16(const void* x_bf16, const int8_t* w, const fl
   GemmW8Params p;
   p.tma3d = t3 ? 1 : 0;
   p.M = static_cast<int>(M); p.Mp = pl.Mp; p.NB = pl.NB; p.N = static_cast<int>(N); p.K = static_cast<int>(K);
-  p.kb_rot_step = 0;
+  p.kb_rot = 0;
   p.pre_stages = 64;
   p.mode = pl.mode; p.groups8 = pl.groups8; p.gran = pl.gran; p.hmax = pl.hmax; p.w_chunk_bytes = pl.w_chunk_bytes; p.kw = pl.kw; p.epi_off = pl.epi_off; p.csplit = pl.csplit;
   p.kblocks = pl.kblocks; p.num_tiles = pl.num_tiles; p.total_blocks = pl.total_blocks;
+  { const int whole = pl.mode == 1 ? pl.groups8 : pl.kblocks, parts = pl.mode == 1 ? pl.grid : pl.csplit; p.share_q = whole / parts; p.share_r = whole % parts; }
   p.num_stages = pl.stages; p.tmem_cols = pl.tmem_cols; p.ytype = ytype;
   p.w_scale = w_scale; p.alpha = nullptr; p.beta = nullptr; p.y = y; p.acc_dbg = nullptr;
   p.accum = reinterpret_cast<int32_t*>(ws + pl.off_slots);
@@ -1080,7 +1092,7 @@ msd_status_t msd_grouped_gemm_w8a16(const void* x_bf16, const int8_t* w, const f
 
   GemmW8Params p;
   p.M = pl.Mp; p.Mp = pl.Mp; p.NB = pl.NB; p.N = static_cast<int>(N); p.K = static_cast<int>(K);
-  p.kb_rot_step = 0; p.pre_stages = 64;
+  p.kb_rot = 0; p.pre_stages = 64; p.share_q = p.share_r = 0;
   p.mode = 0; p.groups8 = 1; p.gran = 8; p.hmax = kTileN; p.w_chunk_bytes = kWStageBytes; p.kw = kw; p.csplit = 1;
   p.tma3d = t3 ? 1 : 0;
   p.kblocks = kblocks; p.num_stages = pl.stages; p.tmem_cols = pl.tmem_cols; p.ytype = ytype;

@@ -91,6 +91,11 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+__device__ __forceinline__ uint32_t cluster_id() {      // along x
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
+  return r;
+}
 // shared::cluster address of the location that has CTA-local shared address `saddr` in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   uint32_t r;
@@ -144,6 +149,8 @@ __device__ __forceinline__ bool wait_bounded_cluster(uint64_t* bar, uint32_t par
 // the CTA's barriers are initialised (all CTAs of a cluster are certain to get there), and the threads that are
 // about to touch a peer's shared memory wait, much later, for all those arrivals.
 __device__ __forceinline__ void cluster_arrive_all() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// (without a release: for barriers whose initialisation was published with fence.mbarrier_init)
+__device__ __forceinline__ void cluster_arrive_relaxed_all() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait_all() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // ---- TMA ----------------------------------------------------------------------------------------
