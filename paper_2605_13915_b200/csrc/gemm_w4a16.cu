@@ -128,7 +128,90 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
 
-  if (threadIdx.x == 0) {
+  // Work items: (token tile, weight tile, K split).  With ksplit > 1 (few tiles, long K: decode shapes) every item
+  // covers kper K stages and its FP32 partial tile goes to rows [split * part_rows, ...) of a partial-sum buffer that a
+  // second kernel adds up in a fixed order.
+  const int total_tiles = p.m_tiles * p.n_tiles * p.ksplit;
+  // What a stage needs of the weights (the tile; with prepared scales its scale blocks) and of the activations.
+  struct Pos { int tile, ks, ks1, mt, nt; };
+  auto enter = [&](Pos& q) {                   // the first K stage of the work item q.tile
+    int split = 0;
+    if constexpr (kCluster) {                    // one token tile, a cluster per weight tile: nothing to divide
+      split = static_cast<int>(cluster_ctarank());
+      q.mt = 0;
+      q.nt = static_cast<int>(cluster_id());
+    } else {
+      const int tile_mn = kGrouped ? q.tile : q.tile / p.ksplit;      // (a grouped launch does not split K)
+      split = kGrouped ? 0 : q.tile - tile_mn * p.ksplit;
+      q.mt = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % p.m_tiles;
+      q.nt = p.n_fastest ? tile_mn % p.n_tiles : tile_mn / p.m_tiles;
+    }
+    q.ks = split * p.kper;
+    q.ks1 = q.ks + p.kper < p.kstages ? q.ks + p.kper : p.kstages;
+  };
+  auto advance = [&](Pos& q) {
+    if (++q.ks < q.ks1) return;
+    q.tile += gridDim.x;
+    if (q.tile < total_tiles) enter(q);
+  };
+  auto load_weights = [&](const Pos& q, int stage) {
+    uint8_t* dst = smem + stage * kStageBytes;
+    if (warp == 0) {
+      mbar_arrive_expect_tx(&full_bar[stage], kStageBytes);
+      int b_row = q.nt * kTN;
+      if constexpr (kGrouped) b_row += grp.expert[q.mt] * p.N;          // the weights of the group's expert
+      tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, b_row, &full_bar[stage]);
+    } else {
+      uint8_t* sf = dst + 2 * a_bytes + kBBytes;
+      size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
+      if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[q.mt]) * 2 * p.n_tiles;
+      bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
+      if constexpr (kSfbBlocks == 2) bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
+    }
+  };
+  auto load_activations = [&](const Pos& q, int stage) {
+    uint8_t* dst = smem + stage * kStageBytes;
+    if (warp == 0) {
+      tma_load_2d(dst, &tmap_a1, q.ks * 128, q.mt * kW4TileM, &full_bar[stage]);
+      tma_load_2d(dst + a_bytes, &tmap_a2, q.ks * 128, q.mt * kW4TileM, &full_bar[stage]);
+    } else {
+      uint8_t* sf = dst + 2 * a_bytes + kBBytes;
+      const size_t a_off = (static_cast<size_t>(q.mt) * p.sf_kgroups + 2 * q.ks) * 512;
+      bulk_load(sf, p.sfa1 + a_off, 1024, &full_bar[stage]);
+      bulk_load(sf + 1024, p.sfa2 + a_off, 1024, &full_bar[stage]);
+    }
+  };
+  constexpr int kGroupedEarly = 2;
+  Pos q = {}, first = {};
+  int pre = 0;                   // stages whose weights were asked for before the wait on the kernel launched just before
+
+  // Decode shapes (kCluster): warp 0 sets the barriers up, a stage per lane, and asks for the first stages' weight tiles right
+  // away, before the rest of the CTA's set-up (tensor memory, the CTA-wide barrier): 1 token, 4096 x 14336 and back 32.1 -> 31.6
+  // us.  Launches of many items are behind a decomposition of many rows, and asking that early takes bandwidth from it
+  // (32 experts 57.6 -> 58.9 us, 1000 rows 35.5 -> 37.9).
+  if constexpr (kCluster) {
+    if (warp == 0) {
+      if (lane < nstages) { mbar_init(&full_bar[lane], 1); mbar_init(&empty_bar[lane], 1); }
+      if (lane >= 8 && lane < 10) {
+        const int a = lane - 8;
+        mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 4);
+        mbar_init(&sf_ready[a], 4); mbar_init(&sf_free[a], 1);
+      }
+      if (lane == 10) abort_flag = 0;
+      mbar_init_fence();
+      __syncwarp();
+      if (lane == 0) {
+        q.tile = blockIdx.x;
+        enter(q);                                // (the grid has no more CTAs than work items)
+        first = q;
+        for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
+      }
+      __syncwarp();
+    } else if (threadIdx.x == 64) {
+      tma_prefetch_desc(&tmap_a1);
+      tma_prefetch_desc(&tmap_a2);
+    }
+  } else if (threadIdx.x == 0) {
     for (int s = 0; s < nstages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 4); }
     for (int a = 0; a < 2; ++a) { mbar_init(&sf_ready[a], 4); mbar_init(&sf_free[a], 1); }
@@ -144,10 +227,6 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
   volatile int* abort = &abort_flag;
-  // Work items: (token tile, weight tile, K split).  With ksplit > 1 (few tiles, long K: decode shapes) every item
-  // covers kper K stages and its FP32 partial tile goes to rows [split * part_rows, ...) of a partial-sum buffer that a
-  // second kernel adds up in a fixed order.
-  const int total_tiles = p.m_tiles * p.n_tiles * p.ksplit;
   bool ok_tile = true;           // kCluster: this warp's accumulator is complete
 
   if (warp == 0 || warp == 10) {
@@ -156,61 +235,21 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     // scale blocks (their bytes may be counted before warp 0's arrival announces them: the phase cannot end without it).
     if (lane == 0) {
       bool ok = true;
-      // What a stage needs of the weights (the tile; with prepared scales its scale blocks) and of the activations.
-      struct Pos { int tile, ks, ks1, mt, nt; };
-      auto enter = [&](Pos& q) {                   // the first K stage of the work item q.tile
-        const int split = q.tile % p.ksplit, tile_mn = q.tile / p.ksplit;
-        q.mt = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % p.m_tiles;
-        q.nt = p.n_fastest ? tile_mn % p.n_tiles : tile_mn / p.m_tiles;
-        q.ks = split * p.kper;
-        q.ks1 = q.ks + p.kper < p.kstages ? q.ks + p.kper : p.kstages;
-      };
-      auto advance = [&](Pos& q) {
-        if (++q.ks < q.ks1) return;
-        q.tile += gridDim.x;
-        if (q.tile < total_tiles) enter(q);
-      };
-      auto load_weights = [&](const Pos& q, int stage) {
-        uint8_t* dst = smem + stage * kStageBytes;
-        if (warp == 0) {
-          mbar_arrive_expect_tx(&full_bar[stage], kStageBytes);
-          int b_row = q.nt * kTN;
-          if constexpr (kGrouped) b_row += grp.expert[q.mt] * p.N;          // the weights of the group's expert
-          tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, b_row, &full_bar[stage]);
-        } else {
-          uint8_t* sf = dst + 2 * a_bytes + kBBytes;
-          size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
-          if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[q.mt]) * 2 * p.n_tiles;
-          bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
-          if constexpr (kSfbBlocks == 2) bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
-        }
-      };
-      auto load_activations = [&](const Pos& q, int stage) {
-        uint8_t* dst = smem + stage * kStageBytes;
-        if (warp == 0) {
-          tma_load_2d(dst, &tmap_a1, q.ks * 128, q.mt * kW4TileM, &full_bar[stage]);
-          tma_load_2d(dst + a_bytes, &tmap_a2, q.ks * 128, q.mt * kW4TileM, &full_bar[stage]);
-        } else {
-          uint8_t* sf = dst + 2 * a_bytes + kBBytes;
-          const size_t a_off = (static_cast<size_t>(q.mt) * p.sf_kgroups + 2 * q.ks) * 512;
-          bulk_load(sf, p.sfa1 + a_off, 1024, &full_bar[stage]);
-          bulk_load(sf + 1024, p.sfa2 + a_off, 1024, &full_bar[stage]);
-        }
-      };
       // (This kernel lets no dependent in early: the waiting decomposition of a next call beside it cost 2 us on 32 experts.)
-      // The first stages' weights are asked for before the kernel launched just before (the decomposition) has ended; the
-      // components and scales it writes - unprepared weight scales among them - after it.
-      Pos q;
-      q.tile = blockIdx.x;
-      enter(q);                                    // (the grid has no more CTAs than work items)
-      const Pos first = q;
-      const bool early = warp == 0 || p.sfb_ready;
-      if (!early) pdl_wait_primary();
-      int pre = 0;
-      for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
-      if (early) pdl_wait_primary();
+      if (warp == 10 || !kCluster) {
+        // neither weights nor prepared weight scales depend on the kernel launched just before; a grouped launch asks for two
+        // stages that early and leaves the bandwidth to the decomposition of its many rows (64 experts 40.2 -> 38.8 us, 32: 57.7 -> 57.1)
+        q.tile = blockIdx.x;
+        enter(q);
+        first = q;
+        if (warp == 10 && !p.sfb_ready) pdl_wait_primary();
+        for (; pre < (kGrouped ? kGroupedEarly : nstages) && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
+      }
+      // what the decomposition, launched just before, writes: the components and their scales
+      if (warp == 0 || p.sfb_ready) pdl_wait_primary();
       q = first;
       for (int i = 0; i < pre; ++i) { load_activations(q, i); advance(q); }
+      if (kGrouped) for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); load_activations(q, pre); advance(q); }
       int stage = pre == nstages ? 0 : pre;
       uint32_t phase = pre == nstages ? 1 : 0;
       while (q.tile < total_tiles) {
