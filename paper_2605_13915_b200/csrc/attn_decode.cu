@@ -307,11 +307,19 @@ attn_qstack_kernel(const AttnParams p, uint8_t* __restrict__ q_img, float* __res
   const int img_bytes = p.DC * p.Rp * kChunk;
   uint8_t* img = q_img + static_cast<size_t>(blockIdx.x) * img_bytes;
   float* sc = q_scales + static_cast<size_t>(blockIdx.x) * 2 * p.HG;
-  // unused head slots and the padding of the last D chunk must be zero
-  for (int i = threadIdx.x; i < img_bytes / 16; i += blockDim.x) reinterpret_cast<uint4*>(img)[i] = make_uint4(0, 0, 0, 0);
-  for (int i = threadIdx.x; i < 2 * p.HG; i += blockDim.x) sc[i] = 0.0f;
-  __syncthreads();
-  for (int h = warp; h < nh; h += static_cast<int>(blockDim.x >> 5)) attn_decompose_q_row(p, b, hk, grp, h, lane, img, sc + h, sc + p.HG + h);
+  // Every warp writes all of its head slots' rows itself - the components of a row that exists, zeros in the padding of the
+  // last D chunk and in unused slots - so nothing waits for a clean image (zero-filling it first and synchronising put
+  // the rows' loads behind 40 KB of stores).
+  for (int h = warp; h < p.HG; h += static_cast<int>(blockDim.x >> 5)) {
+    const int from = h < nh ? p.D : 0;
+    if (h < nh) attn_decompose_q_row(p, b, hk, grp, h, lane, img, sc + h, sc + p.HG + h);
+    else if (lane == 0) { sc[h] = 0.0f; sc[p.HG + h] = 0.0f; }
+    for (int d = from + 16 * lane; d < p.DC * kChunk; d += 16 * 32) {
+      uint8_t* chunk = img + (d >> 7) * p.Rp * kChunk;
+      *reinterpret_cast<uint4*>(chunk + swz_off(h, d & 127)) = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4*>(chunk + swz_off(p.HG + h, d & 127)) = make_uint4(0, 0, 0, 0);
+    }
+  }
 }
 
 // Head groups of up to 8 query rows per KV head (GQA).  kMaxHG: head slots one softmax thread looks after (8; the code
@@ -1167,10 +1175,10 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         if constexpr (kChunked) { /* the producer takes s_full as "the rotary chunk has been read" */ }
         else if (!p.v_alias) tc_commit(&kv_empty[st]);       // separate V: the K buffer is free once QK^T has read it
       };
-      // PV is issued by softmax threads (below), one dv tile each; this thread issues QK^T only.
+      // PV is issued by softmax threads or a warp of its own (below); this thread issues QK^T only.
       int q = 0;
       if constexpr (kChunked) {
-        // PV is issued by four softmax threads (below); this thread issues QK^T only.  QK^T(q) needs KV tile q in shared
+        // PV is issued by two softmax threads (below); this thread issues QK^T only.  QK^T(q) needs KV tile q in shared
         // memory and the score buffer q&1 read, i.e. P of tile q-2 written by every softmax warp (the slow path works
         // from registers).  The P buffer q&1 is free by then as well: KV tile q arrives in the stage that PV(q-2) gave
         // back chunk by chunk, so its arrival implies that PV(q-2) is complete.
@@ -1533,27 +1541,29 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         slow = true;
       }
       if constexpr (kChunked) {
-        // PV(t), one dv tile per thread: lane 0 of the first four softmax warps, which sit on the four different warp
-        // schedulers.  The softmax warps are idle here (the next score tile is not there yet), the product starts the
-        // moment P is final instead of when the QK^T-issuing thread gets round to it, and its 16 MMAs are issued four
-        // abreast.  An accumulator is only ever written by its own thread, so its MMAs stay in program order.
-        if (hh == 0 && lane == 0) {
+        // PV(t), two dv tiles per thread: lane 0 of the first two softmax warps, which sit on different warp schedulers.  The
+        // softmax warps are idle here (the next score tile is not there yet) and the product starts the moment P is final
+        // instead of when the QK^T-issuing thread gets round to it.  The value chunks are let go of in the order in which they are
+        // asked for again, 0 and 1 before 2 and 3: with four threads abreast all four came back at the end of the product (64 x
+        // 16384 tokens 276 us, now 270); one thread for all four takes too long to issue (281).  An accumulator is only ever
+        // written by its own thread, so its MMAs stay in program order.
+        if (hh == 0 && lane == 0 && wq < 2) {
           const int st = t & 1;
           if (slow) ok = wait_bounded(&p_redo, (n_slow - 1) & 1, abort, p.status);      // every warp has drained and rewritten P
-          if (ok) ok = wait_bounded(&ck_full[st][wq], (t >> 1) & 1, abort, p.status);      // its value chunk (long landed: QK^T(t) has read the tile)
-          if (ok) {
+          const uint32_t pa_lo = pv_pa_lo + (t & 1) * pv_p_step;
+#pragma unroll
+          for (int dv = wq; dv < 4; dv += 2) {
+            if (ok) ok = wait_bounded(&ck_full[st][dv], (t >> 1) & 1, abort, p.status);      // its value chunk (long landed: QK^T(t) has read the tile)
+            if (!ok) break;
             tc_fence_after();
-            if (wq == 0 && t >= 2 && t < 5) attn_mark(p, 8 + 6 * (t - 2));
-            const uint32_t va_lo = pv_va_lo + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + wq * (kChunkBytes >> 4);
-            const uint32_t pa_lo = pv_pa_lo + (t & 1) * pv_p_step;
-            const uint32_t acc = tmem_o + wq * (2 * kSlots);
+            const uint32_t va_lo = pv_va_lo + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + dv * (kChunkBytes >> 4);
+            const uint32_t acc = tmem_o + dv * (2 * kSlots);
             if (slow) mma_i8_lohi<false>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
             else mma_i8_lohi<true>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
 #pragma unroll
             for (int k = 1; k < 4; ++k)      // 32 tokens per MMA: four 8-token groups of 1024 bytes
               mma_i8_lohi<true>(acc, va_lo + k * (4096 >> 4), pv_v_hi, pa_lo + k * (32 * kPRow >> 4), pv_p_hi, pv_idesc);
-            tc_commit(&ck_empty[st][wq]);      // value chunk wq may be requested again; also "this dv tile of PV(t) is complete"
-            if (wq == 0 && t >= 2 && t < 5) attn_mark(p, 20 + t);
+            tc_commit(&ck_empty[st][dv]);      // value chunk dv may be requested again; also "this dv tile of PV(t) is complete"
           }
         }
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
