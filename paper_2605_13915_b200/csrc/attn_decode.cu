@@ -32,6 +32,36 @@ constexpr int kChunk = 128;         // bytes of D / Dv per TMA box and per share
 constexpr int kChunkBytes = kTok * kChunk;
 constexpr int kPartHdr = 4;         // words in front of a split's partial output row: reference maximum, sum of P, two unused
 
+// The split size of a call whose CTAs can all but be resident at once (wide head groups), taken on the device from the
+// lengths themselves: the host knows only the longest.  All splits of a call have the size, c tiles.  With A the tiles that
+// each of the machine's CTA slots has to do, c is A plus the start-up of the units' short last splits, over a share (0.06
+// for equal lengths, more the more they differ) that keeps those last splits, which run in the gaps, from ending later than
+// the full ones:  c = (A + units / slots + 1) / (1 - 0.06 - 0.25 (1 - mean / longest)).  Coefficients fitted to sweeps of the size over
+// 321 shapes (latent cache, 16 and 32 rows per KV head; 1024 to 32768 tokens; all lengths equal, from a half, from a tenth or a
+// quarter of the longest): time over that of the best size 1.012, 1.010 and 1.012 on average, against 1.082, 1.037 and
+// 1.057 with the size chosen from the longest length alone.  64 latent caches, 64 heads: 16384 tokens 270 us -> 238, 2048 to 8192 tokens
+// 130 -> 104; 16 GQA sequences of 1024 to 8192, 4 query tokens: 53.7 -> 47.9.
+struct AttnAdapt {
+  float per_token, base, inv_full;      // A = per_token * tokens + ..., 1 / (B * longest)
+  int c_min, c_max;                     // tiles; c_max = 0: the split size is the plan's
+};
+
+// (the host computes the same size for those who ask where the splits lie: every operation rounds by itself)
+__host__ __device__ __forceinline__ int attn_adapt_tiles(const AttnAdapt& a, int tokens) {
+#ifdef __CUDA_ARCH__
+  const float t = __int2float_rn(tokens), rho = fminf(__fmul_rn(t, a.inv_full), 1.0f);
+  const float c = __fdiv_rn(__fadd_rn(__fmul_rn(t, a.per_token), a.base), __fadd_rn(0.69f, __fmul_rn(0.25f, rho)));
+#else
+  volatile float m = static_cast<float>(tokens) * a.inv_full, x = static_cast<float>(tokens) * a.per_token;
+  const float rho = m < 1.0f ? m : 1.0f;
+  volatile float y = 0.25f * rho;
+  volatile float num = x + a.base, den = 0.69f + y;
+  const float c = num / den;
+#endif
+  const int n = static_cast<int>(ceilf(fminf(c, 1.0e9f)));
+  return n < a.c_min ? a.c_min : (n > a.c_max ? a.c_max : n);
+}
+
 struct AttnParams {
   const uint16_t* q;      // [B,Hq,D] BF16 (read by attn_qstack_kernel only)
   // written by attn_qstack_kernel, one entry per (sequence, KV head, head group): the stacked INT8 operand exactly as
@@ -74,6 +104,7 @@ struct AttnParams {
   float* qs_dbg;
   int32_t* s_dbg;
   long long dbg_T;
+  AttnAdapt adapt;          // wide head groups: the call's own split size, at least `chunk`
 };
 
 __device__ __forceinline__ void attn_mark(const AttnParams& p, int slot) {
@@ -950,6 +981,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   __shared__ int abort_flag;
   __shared__ int flush_stamp[2];                    // tile number + 1 of the last tile whose references had to move, per P buffer
   __shared__ float s_aq[kSlots];
+  __shared__ int span[2];                           // the split's first and past-the-last token (kept here: the softmax warps have no registers left for them)
   __shared__ float red[kSlots / kWideHS][4][kWideHS + 1];    // per-warp tile maxima (slow path only)
   constexpr int kWideWG = kSlots / kWideHS;
   constexpr int kNSW = 4 * kWideWG;
@@ -981,8 +1013,19 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   const int32_t* bt = kPaged ? p.block_table + static_cast<long long>(b) * p.max_blocks : nullptr;
   const int seq0 = kPaged ? 0 : p.cu[b];
   const int L = kPaged ? p.seqlens[b] : p.cu[b + 1] - seq0;
-  const int t_begin = split * p.chunk;
-  const int t_end = min(L, t_begin + p.chunk);
+  int chunk = p.chunk;
+  if (p.adapt.c_max > 0) {
+    int tokens = 0;
+    if constexpr (kPaged) {
+      for (int i = lane; i < p.B; i += 32) tokens += max(p.seqlens[i], 0);
+      tokens = __reduce_add_sync(0xffffffffu, tokens);
+    } else {
+      tokens = p.cu[p.B] - p.cu[0];
+    }
+    chunk = attn_adapt_tiles(p.adapt, tokens) * kTok;
+  }
+  const int t_begin = split * chunk;
+  const int t_end = min(L, t_begin + chunk);
   const int h0 = hk * p.G + grp * p.HG;
   const int nh = min(p.HG, p.G - grp * p.HG);
   const int ntiles = (t_end > t_begin) ? (t_end - t_begin + kTok - 1) / kTok : 0;
@@ -994,13 +1037,11 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     if (cta < 1024) { p.trace[cta * 32 + 1] = static_cast<long long>(g); p.trace[cta * 32 + 2] = ntiles; }
   }
 
-  if (ntiles == 0) {      // nothing in this split: neutral partials, before any barrier or TMEM use
+  if (ntiles == 0) {      // nothing in this split: a neutral header (the merge reads no further), before any barrier or TMEM use
     pdl_wait_primary();       // (this grid must not end before the kernel it depends on)
-    for (int i = threadIdx.x; i < nh * (p.Dv + kPartHdr); i += blockDim.x) {
-      const int h = i / (p.Dv + kPartHdr), e = i % (p.Dv + kPartHdr);
-      float* dst = p.partial + ((static_cast<long long>(b) * p.Hq + h0 + h) * p.n_splits + split) * (p.Dv + kPartHdr);
-      dst[e] = (e == 0) ? -INFINITY : 0.0f;
-    }
+    for (int i = threadIdx.x; i < nh * kPartHdr; i += blockDim.x)
+      p.partial[((static_cast<long long>(b) * p.Hq + h0 + i / kPartHdr) * p.n_splits + split) * (p.Dv + kPartHdr) + i % kPartHdr] =
+          (i % kPartHdr == 0) ? -INFINITY : 0.0f;
     return;
   }
 
@@ -1010,6 +1051,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   uint8_t* sm_p = sm_q + p.DC * p.Rp * kChunk;               // two buffers of [Rp x 128]
 
   if (threadIdx.x == 0) {
+    span[0] = t_begin; span[1] = t_end;
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(&kv_full[s], 1); mbar_init(&kv_empty[s], 1);
       mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1);
@@ -1322,8 +1364,8 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     const float kMagic = 12582912.0f;
 
     auto load_scales = [&](int t, float& ks_out, float& vs_out) {
-      const int tok_rel = t_begin + t * kTok + tl;
-      const bool valid = t < ntiles && tok_rel < t_end;
+      const int tok_rel = span[0] + t * kTok + tl;
+      const bool valid = t < ntiles && tok_rel < span[1];
       long long sidx;
       if constexpr (kPaged) {
         const long long prow = valid ? static_cast<long long>(__ldg(bt + (tok_rel >> p.page_shift))) * p.page + (tok_rel & (p.page - 1)) : 0;
@@ -1337,8 +1379,8 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     // c3: scores of this thread's token against its 8 head slots in the log2 domain (-inf where the token is past the
     // end of the split or not visible to the row)
     auto load_scores = [&](int t, float ks, float (&s)[kWideHS]) {
-      const int tok_rel = t_begin + t * kTok + tl;
-      const bool valid = tok_rel < t_end;
+      const int tok_rel = span[0] + t * kTok + tl;
+      const bool valid = tok_rel < span[1];
       const uint32_t srow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + (t & 1) * p.Rp;
       uint32_t v1[kWideHS], v2[kWideHS];
       tmem_ldw<kWideHS>(srow + hs0, v1);
@@ -1359,7 +1401,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       }
       // causal among the new tokens: only the tiles that reach them are masked row by row (a division per row and tile
       // took 0.8 of 2.5 us a tile when every tile was; as a condition on every score it cost all other calls 3 to 6 %)
-      if (p.Sq > 1 && t_begin + (t + 1) * kTok > L - p.Sq + 1) {
+      if (p.Sq > 1 && span[0] + (t + 1) * kTok > L - p.Sq + 1) {
 #pragma unroll
         for (int h = 0; h < kWideHS; ++h)
           if (tok_rel >= L - p.Sq + 1 + (grp * p.HG + hs0 + h) / p.Gr) s[h] = -INFINITY;
@@ -1643,11 +1685,17 @@ static int32_t* g_attn_s_dbg = nullptr;
 // (a separate small kernel: letting the last-arriving split do it inside the attention kernel measured slower).
 // One CTA per row; the weights e^{m_s - m} are computed once per split and the O_s rows are read as 16-byte vectors,
 // eight splits' loads in flight per thread.  O is summed over the splits in ascending order.
-__global__ void __launch_bounds__(128)
+// kTrim (wide head groups): the splits after the last that saw a token have no more than a header and are not read.
+// kMany (eight splits and more): registers for those eight loads.  Left to itself the compiler keeps to 32, for 16 CTAs an SM, and the
+// loads follow one another; with few splits the CTAs in flight are what counts (1 x 8192 tokens, 16 splits: the call 15.1 us, now
+// 12.6; 4 x 1000 to 4000, 11 splits: 16.0, now 14.7; 64 x 100 to 1000, one split: 28.3, 29.4 with 48 registers).
+template <bool kTrim, bool kMany>
+__global__ void __launch_bounds__(128, kMany ? 10 : 16)
 attn_combine_kernel(const float* __restrict__ partial, int n_splits_alloc, const int32_t* __restrict__ n_slots, int G, int HG,
                     int groups, int Dv, __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int Sq, int Gr, int Hkv) {
   __shared__ float s_w[128];
   __shared__ float s_red[2][4];
+  __shared__ int s_last[kTrim ? 4 : 1];
   pdl_wait_primary();              // the partial results come from the attention kernel launched just before
   const int PS = Dv + kPartHdr;
   const float* base = partial + static_cast<long long>(blockIdx.x) * n_splits_alloc * PS;
@@ -1669,12 +1717,22 @@ attn_combine_kernel(const float* __restrict__ partial, int n_splits_alloc, const
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float m = -INFINITY;
-  for (int s = tid; s < n_splits; s += 128) m = fmaxf(m, __ldg(base + static_cast<long long>(s) * PS));
+  int last = 0;
+  for (int s = tid; s < n_splits; s += 128) {
+    const float ms = __ldg(base + static_cast<long long>(s) * PS);
+    if constexpr (kTrim) last = (ms != -INFINITY) ? s + 1 : last;
+    m = fmaxf(m, ms);
+  }
+  if constexpr (kTrim) last = __reduce_max_sync(0xffffffffu, last);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) s_red[0][warp] = m;
+  if (lane == 0) {
+    s_red[0][warp] = m;
+    if constexpr (kTrim) s_last[warp] = last;
+  }
   __syncthreads();
   m = fmaxf(fmaxf(s_red[0][0], s_red[0][1]), fmaxf(s_red[0][2], s_red[0][3]));
+  if constexpr (kTrim) n_splits = max(max(s_last[0], s_last[1]), max(s_last[2], s_last[3]));
   const bool act = tid < (Dv >> 2);
   const float4* o4 = reinterpret_cast<const float4*>(base + kPartHdr) + tid;
   const int ps4 = PS >> 2;
@@ -1719,6 +1777,7 @@ attn_combine_kernel(const float* __restrict__ partial, int n_splits_alloc, const
 
 struct AttnPlan {
   int HG, Rp, groups, DC, DVT, n_splits, stages, tmem_cols, v_alias, chunk, kv_chunks;
+  AttnAdapt adapt;
   int balanced, q_min;      // balanced schedule: n_splits is the largest number of partial results a unit can have
   size_t smem_bytes, ws_bytes, ws_partial_bytes, ws_qimg_bytes, ws_qscale_bytes;
 };
@@ -1789,6 +1848,22 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
                                  : pl->HG == 16 ? AttnSplitCost{2, {1.3f, 1.75f, 1.75f}, 7.0f}
                                                 : AttnSplitCost{1, {small ? 1.3f : 2.0f, 2.0f, 2.0f}, small ? 7.0f : 11.0f};
   int chunk_tiles = option(OPT_ATTN_CHUNK_TILES);       // testing aid: a given split size
+  pl->adapt = AttnAdapt{0.0f, 0.0f, 0.0f, 0, 0};
+  const long long slots = static_cast<long long>(sm_count()) * split_cost.per_sm;
+  if (pl->HG > 8 && units <= slots && static_cast<long long>(B) * max_seqlen < 0x7FFFFFFFLL && chunk_tiles < 1 && option(OPT_ATTN_SPLITS) < 1) {
+    // wide head groups, at most one unit per CTA slot: the size comes from the lengths (AttnAdapt).  At most that with which
+    // full-length sequences fill one round of CTAs, at least (which sizes the workspace) the one for lengths of 40 % on average.
+    const float inv_slots = 1.0f / static_cast<float>(slots), per_seq = static_cast<float>(Hkv * pl->groups);
+    AttnAdapt& a = pl->adapt;
+    a.per_token = per_seq * inv_slots / static_cast<float>(kTok);
+    a.base = (0.5f * static_cast<float>(units) + static_cast<float>(units)) * inv_slots + 1.0f;      // (half a tile more per sequence: its last)
+    a.inv_full = 1.0f / (static_cast<float>(B) * static_cast<float>(std::max(max_seqlen, 1)));
+    const int rounds = static_cast<int>(slots / units);
+    a.c_max = std::min((tiles + rounds - 1) / rounds, kMaxHeldTiles);
+    a.c_max = std::max(a.c_max, std::min(2, std::max(tiles, 1)));
+    a.c_min = std::min(2, a.c_max);
+    chunk_tiles = a.c_min = attn_adapt_tiles(a, static_cast<int>(0.4 * static_cast<double>(B) * max_seqlen));
+  }
   if (chunk_tiles < 1) chunk_tiles = attn_split_tiles(units, tiles, split_cost);
   if (pl->HG > 8 && chunk_tiles > kMaxHeldTiles) chunk_tiles = kMaxHeldTiles;
   while ((tiles + chunk_tiles - 1) / chunk_tiles > 65535) chunk_tiles <<= 1;      // splits run along the grid's y axis
@@ -1837,7 +1912,7 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
 
 // The split merge for another attention kernel of this library (rows in output order, every row n_splits partial results).
 msd_status_t launch_attn_combine(const float* partial, int n_splits, int Dv, void* out_bf16, float* lse, int rows, cudaStream_t s) {
-  if (launch_pdl(attn_combine_kernel, dim3(rows), dim3(128), 0, s, option(OPT_NO_PDL) <= 0, partial, n_splits,
+  if (launch_pdl(n_splits >= 8 ? attn_combine_kernel<false, true> : attn_combine_kernel<false, false>, dim3(rows), dim3(128), 0, s, option(OPT_NO_PDL) <= 0, partial, n_splits,
                  static_cast<const int32_t*>(nullptr), 1, 1, 1, Dv, static_cast<__nv_bfloat16*>(out_bf16), lse, 1, 1, 1) != cudaSuccess)
     return MSD_ERR_CUDA;
   return launch_status();
@@ -1990,6 +2065,12 @@ static msd_status_t attn_split_starts(int32_t B, int32_t q_len, int32_t Hq, int3
     R = std::min<long long>(W / pl.q_min, ctas / U);
     R = R < 1 ? 1 : R;
   }
+  int chunk = pl.chunk;
+  if (pl.adapt.c_max > 0) {
+    int tokens = 0;
+    for (int b = 0; b < B; ++b) tokens += std::max(seqlens[b], 0);
+    chunk = attn_adapt_tiles(pl.adapt, tokens) * kTok;
+  }
   long long P = 0;                                   // tiles of the sequences in front
   for (int b = 0; b < B; ++b) {
     const int L = seqlens[b] > 0 ? seqlens[b] : 0;
@@ -2003,7 +2084,7 @@ static msd_status_t attn_split_starts(int32_t B, int32_t q_len, int32_t Hq, int3
         for (long long i = ((P + 1) * R - 1) / W + 1; i < R && i * W / R < P + nb && n < ns; ++i)
           first_row[n++] = static_cast<int32_t>((i * W / R - P) * kTok);
     } else {
-      for (int sidx = 1; sidx < ns; ++sidx) first_row[n++] = static_cast<int32_t>(std::min<long long>(L, static_cast<long long>(sidx) * pl.chunk));
+      for (int sidx = 1; sidx < ns; ++sidx) first_row[n++] = static_cast<int32_t>(std::min<long long>(L, static_cast<long long>(sidx) * chunk));
     }
     while (n <= ns) first_row[n++] = L;
     for (int r = 1; r < Hkv * G; ++r) std::copy(first_row, first_row + ns + 1, first_row + static_cast<long long>(r) * (ns + 1));
@@ -2086,6 +2167,7 @@ static msd_status_t attn_launch(const void* q_bf16, const int8_t* k_cache, const
   p.Sq = q_len; p.Gr = Hq_real / Hkv;
   p.HG = pl.HG; p.Rp = pl.Rp; p.groups = pl.groups; p.DC = pl.DC; p.DVT = pl.DVT;
   p.chunk = pl.chunk;
+  p.adapt = pl.adapt;
   p.n_splits = pl.n_splits; p.stages = pl.stages; p.v_alias = pl.v_alias; p.kv_chunks = pl.kv_chunks; p.tmem_cols = pl.tmem_cols;
   p.q_dbg = g_attn_q_dbg; p.qs_dbg = g_attn_qs_dbg; p.s_dbg = g_attn_s_dbg; p.dbg_T = total_tokens;
   p.scale = softmax_scale;
@@ -2108,7 +2190,10 @@ static msd_status_t attn_launch(const void* q_bf16, const int8_t* k_cache, const
     if (launch_pdl(attn_qstack_kernel, dim3(B * Hkv * pl.groups), dim3(32 * pl.HG), 0, s, pdl, p, q_img, q_scales) != cudaSuccess) return MSD_ERR_CUDA;
   }
   if (launch_pdl(kernel, grid, dim3(block_threads), pl.smem_bytes, s, pdl, tmap_k, tmap_v, p) != cudaSuccess) return MSD_ERR_CUDA;
-  if (launch_pdl(attn_combine_kernel, dim3(B * Hq), dim3(128), 0, s, pdl, static_cast<const float*>(p.partial),
+  const bool many = pl.n_splits >= 8 && !pl.balanced;
+  auto combine = pl.HG > 8 ? (many ? attn_combine_kernel<true, true> : attn_combine_kernel<true, false>)
+                           : (many ? attn_combine_kernel<false, true> : attn_combine_kernel<false, false>);
+  if (launch_pdl(combine, dim3(B * Hq), dim3(128), 0, s, pdl, static_cast<const float*>(p.partial),
                  pl.n_splits, static_cast<const int32_t*>(pl.balanced ? p.n_slots : nullptr), Hq / Hkv, pl.HG, pl.groups, Dv,
                  static_cast<__nv_bfloat16*>(out_bf16), lse, q_len, Hq / (Hkv * q_len), Hkv) != cudaSuccess)
     return MSD_ERR_CUDA;

@@ -98,6 +98,23 @@ def test_wide_groups_at_the_edges_of_the_slot_counts(rows, D):
     _check(inputs.gqa_case(6, 2 * rows, 2, D, [1, 127, 0, 128, 129, 2500], seed=rows + D))
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("rows,seqlens", [(16, [2500, 0, 130, 1]), (16, [2500] * 4), (32, [1, 127, 4000]), (64, [3000, 2990])])
+def test_split_size_from_the_lengths(rows, seqlens, paged):
+    """The split size that the device takes from the lengths (one long sequence among short ones, all alike, an empty one) is the
+    one the host reports, and the splits that a call leaves empty do not count."""
+    c = inputs.gqa_case(len(seqlens), rows, 1, 128, seqlens, seed=rows + len(seqlens))
+    if not paged:
+        _check(c)
+        return
+    k, v, ks, vs, table, sl = inputs.paginate(c, 16, seed=rows)
+    o = binding.attn_decode_int8kv_paged(bf16_dev(c.q), dev(k), dev(v), dev(ks), dev(vs), dev(table), dev(sl), 16, c.max_seqlen,
+                                         c.softmax_scale)
+    binding.last_device_status()
+    ref, _ = _run_gpu(c)
+    assert torch.equal(o, ref)
+
+
 @pytest.mark.parametrize("rows,D", [(4, 512), (8, 512), (4, 640), (16, 128)])
 def test_scores_at_the_largest_codes(rows, D):
     """Every code of the keys and of the queries' first components at its limit: the integer sums of both components, and
