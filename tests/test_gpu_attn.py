@@ -409,6 +409,19 @@ def test_speculative_decode_rows_are_causal_single_query_problems(Sq, Hq, Hkv):
         assert np.allclose(lse.cpu().numpy()[:, s], lse_ref, rtol=0, atol=2e-3)
 
 
+@pytest.mark.parametrize("Sq,Hq,Hkv,D", [(1, 8, 2, 128), (1, 8, 1, 64), (3, 8, 8, 128), (2, 16, 4, 64)])
+def test_one_split_is_written_as_the_merge_would(Sq, Hq, Hkv, D):
+    """One split a sequence: the attention kernel writes the result; bit for bit what the merge makes of the same partial
+    results when the call could have had a second split.  No token, one, the edges of a tile, a full split."""
+    binding.debug_set_option("MSD_ATTN_CHUNK_TILES", 3)
+    base = inputs.gqa_case(B=6, Hq=Hq * Sq, Hkv=Hkv, D=D, seqlens=[Sq, 0, 127, 128, 129, 384], seed=D + Sq)
+    q = bf16_dev(base.q.reshape(6, Sq, Hq, D))
+    args = [dev(x) for x in (base.k, base.v, base.k_scale, base.v_scale, base.cu_seqlens)]
+    (o1, l1), (o2, l2) = (binding.attn_decode_int8kv_spec(q, *args, m, base.softmax_scale, want_lse=True) for m in (384, 385))
+    binding.last_device_status()
+    assert torch.equal(o1, o2) and torch.equal(l1, l2)
+
+
 # ---- Alg. 3 lines 1-4 bit for bit: query components, their scales and both INT32 score planes -------------------------
 def _dump_buffers(rows, rows_per_seq, D, T):
     q_dbg = torch.full((2, rows, D), 99, dtype=torch.int8, device="cuda")
