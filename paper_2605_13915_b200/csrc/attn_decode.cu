@@ -38,7 +38,7 @@ constexpr int kPartHdr = 4;         // words in front of a split's partial outpu
 // for equal lengths, more the more they differ) that keeps those last splits, which run in the gaps, from ending later than
 // the full ones:  c = (A + units / slots + 1) / (1 - 0.06 - 0.25 (1 - mean / longest)).  Coefficients fitted to sweeps of the size over
 // 321 shapes (latent cache, 16 and 32 rows per KV head; 1024 to 32768 tokens; all lengths equal, from a half, from a tenth or a
-// quarter of the longest): time over that of the best size 1.012, 1.010 and 1.012 on average, against 1.082, 1.037 and
+// quarter of the longest): time over that of the best size (linear between swept sizes) 1.012, 1.010 and 1.012 on average, against 1.082, 1.037 and
 // 1.057 with the size chosen from the longest length alone.  64 latent caches, 64 heads: 16384 tokens 270 us -> 238, 2048 to 8192 tokens
 // 130 -> 104; 16 GQA sequences of 1024 to 8192, 4 query tokens: 53.7 -> 47.9.
 struct AttnAdapt {
