@@ -38,6 +38,7 @@ constexpr int kP8PairStageBytes = 2 * kP8ABytes + kP8BBytes / 2;    // 48 KB per
 constexpr int kP8PairStages = 4;
 constexpr int kP8StoreBytes = 2048;                             // one epilogue chunk: 32 rows x 64 bytes
 constexpr int kP8TmemCols = 512;
+constexpr int kP8PartPlanes = 2;                                // partial tiles of a piece of a cut tile: one per component
 
 struct GemmP8Params {
   int M, N, K;
@@ -46,7 +47,8 @@ struct GemmP8Params {
   int part_rows;                // ksplit > 1: rows per split of the FP32 partial-result buffer the tiles are written to
   int n_fastest;                // tile index -> (token tile, weight tile): weight tile fastest (1) or token tile fastest (0)
   // The tiles of a last round that would leave most units idle are cut along K instead (plan_p8): tiles [0, tail0) are
-  // whole items, tile tail0 + r (r < tail_n) is tail_s items of tail_k stages that write FP32 partial tiles.
+  // whole items, tile tail0 + r (r < tail_n) is tail_s items of tail_k stages that write their partial sums as they are:
+  // the two INT32 accumulators (kBase: the one FP32 accumulator) as tiles of their own, added by p8_tail_reduce_kernel.
   int tail0, tail_n, tail_s, tail_k;
   const float* alpha;           // [M]
   const float* beta;            // [M]
@@ -219,6 +221,22 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
       }
     };
     const uint32_t swz = static_cast<uint32_t>((lane >> 1) & 3);
+    // a chunk of 64 bytes of each of the warp's rows (a row a lane) to columns x.., rows y.. of a tensor map
+    auto stage_and_store = [&](const uint32_t (&v)[16], const CUtensorMap* map, int x, int y) {
+      if (lane == 0) bulk_wait_group_read<0>();    // the store of the previous chunk is done with the staging buffer
+      __syncwarp();
+      uint8_t* srow = sb + lane * 64;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<uint4*>(srow + ((static_cast<uint32_t>(j) ^ swz) << 4)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        tma_store_2d(map, x, y, sb);
+        bulk_commit_group();
+      }
+    };
+    constexpr int kPlanes = kBase ? 1 : kP8PartPlanes, unit_rows = (kPair ? 2 : 1) * kP8TileM;
     int it = 0;
     bool ok = true;
     pdl_wait_primary();             // alpha and beta come from the decomposition kernel launched just before
@@ -231,6 +249,7 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
       const bool bf = p.ytype == MSD_OUT_BF16 && part_tile < 0;
       const int ccols = bf ? 32 : 16;
       const int row0 = mt * kP8TileM + quad * 32, row = row0 + lane;
+      const int part_row = part_tile * kPlanes * unit_rows + static_cast<int>(rank) * kP8TileM + quad * 32;
       float a_i = 0.0f, b_i = 0.0f;
       if constexpr (!kBase) {
         if (row < p.M) { a_i = __ldg(p.alpha + row); b_i = __ldg(p.beta + row); }
@@ -278,6 +297,12 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
               p.acc_dbg[(static_cast<long long>(p.M) + row) * p.N + col + 16 * hsub + j] = static_cast<int32_t>(v2[j]);
             }
           }
+          if (part_tile >= 0) {      // a piece of a cut tile: both sums as they are, the first component's here
+            stage_and_store(v1, &tmap_part, part * 64 + c0, part_row);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) o[j] = v2[j];
+            continue;
+          }
           if (bf) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -305,19 +330,8 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
           }
         }
         if (c0 + ccols >= cend) release_acc();
-        if (lane == 0) bulk_wait_group_read<0>();    // the store of the previous chunk is done with the staging buffer
-        __syncwarp();
-        uint8_t* srow = sb + lane * 64;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          *reinterpret_cast<uint4*>(srow + ((static_cast<uint32_t>(j) ^ swz) << 4)) = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          if (part_tile < 0) tma_store_2d(&tmap_y, col, row0 + split * p.part_rows, sb);
-          else tma_store_2d(&tmap_part, part * 64 + c0, part_tile * ((kPair ? 2 : 1) * kP8TileM) + (kPair ? static_cast<int>(rank) * kP8TileM : 0) + quad * 32, sb);
-          bulk_commit_group();
-        }
+        if (part_tile < 0) stage_and_store(o, &tmap_y, col, row0 + split * p.part_rows);
+        else stage_and_store(o, &tmap_part, part * 64 + c0, part_row + (kPlanes - 1) * unit_rows);
       }
     }
     if (lane == 0) bulk_wait_group<0>();            // every store has been written before the CTA goes away
@@ -335,24 +349,43 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
   }
 }
 
-// Sums of the tail's partial tiles part[split][tile r][rows][256], split 0 first (fixed order), rounded once to y.
+// Results of the cut tiles from their pieces' partial sums part[piece][tile r][component][rows][256], 32-bit words.  The INT32
+// sums are added as integers and combined exactly as the epilogue combines those of a whole tile, so that a result does not
+// depend on whether its tile was cut; the FP32 sums of kBase are added in ascending order of the pieces.
+template <bool kBase>
 __global__ void __launch_bounds__(256)
-p8_tail_reduce_kernel(const float* __restrict__ part, const GemmP8Params p, int unit_rows, void* __restrict__ y, int ytype) {
+p8_tail_reduce_kernel(const uint32_t* __restrict__ part, const GemmP8Params p, int unit_rows, void* __restrict__ y, int ytype) {
   pdl_wait_primary();
   const int m_units = (p.m_tiles * kP8TileM + unit_rows - 1) / unit_rows;
-  const int quads = p.tail_n * unit_rows * (kP8TileN / 4);
-  const long long stride = static_cast<long long>(quads) * 4;              // floats per split
+  const int tile_quads = unit_rows * (kP8TileN / 4), quads = p.tail_n * tile_quads;
+  constexpr int kPlanes = kBase ? 1 : kP8PartPlanes;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += gridDim.x * blockDim.x) {
-    const int c = (i & (kP8TileN / 4 - 1)) * 4, rr = i / (kP8TileN / 4), r = rr / unit_rows;
+    const int r = i / tile_quads, q = i - r * tile_quads, c = (q & (kP8TileN / 4 - 1)) * 4, rr = q / (kP8TileN / 4);
     const int tile = p.tail0 + r;
     const int mu = p.n_fastest ? tile / p.n_tiles : tile % m_units, nt = p.n_fastest ? tile % p.n_tiles : tile / m_units;
-    const int row = mu * unit_rows + (rr - r * unit_rows), col = nt * kP8TileN + c;
+    const int row = mu * unit_rows + rr, col = nt * kP8TileN + c;
     if (row >= p.M || col >= p.N) continue;                                // (N is a multiple of 4)
-    const float* src = part + static_cast<long long>(i) * 4;
-    float4 acc = __ldg(reinterpret_cast<const float4*>(src));
-    for (int sp = 1; sp < p.tail_s; ++sp) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(src + sp * stride));
-      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    const uint4* src = reinterpret_cast<const uint4*>(part) + static_cast<long long>(r) * kPlanes * tile_quads + q;
+    const long long stride = static_cast<long long>(p.tail_n) * kPlanes * tile_quads;      // 16-byte pieces per split
+    float4 acc;
+    if constexpr (kBase) {
+      acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int sp = 0; sp < p.tail_s; ++sp) {
+        const uint4 v = __ldg(src + sp * stride);
+        acc.x += __uint_as_float(v.x); acc.y += __uint_as_float(v.y); acc.z += __uint_as_float(v.z); acc.w += __uint_as_float(v.w);
+      }
+    } else {
+      uint4 s1 = make_uint4(0, 0, 0, 0), s2 = s1;
+      for (int sp = 0; sp < p.tail_s; ++sp) {
+        const uint4 v1 = __ldg(src + sp * stride), v2 = __ldg(src + sp * stride + tile_quads);
+        s1.x += v1.x; s1.y += v1.y; s1.z += v1.z; s1.w += v1.w;
+        s2.x += v2.x; s2.y += v2.y; s2.z += v2.z; s2.w += v2.w;
+      }
+      const float a = __ldg(p.alpha + row), b = __ldg(p.beta + row);
+      auto combine = [&](int j, uint32_t t1, uint32_t t2) {
+        return __ldg(p.w_scale + col + j) * __fmaf_rn(a, static_cast<float>(static_cast<int32_t>(t1)), b * static_cast<float>(static_cast<int32_t>(t2)));
+      };
+      acc = make_float4(combine(0, s1.x, s2.x), combine(1, s1.y, s2.y), combine(2, s1.z, s2.z), combine(3, s1.w, s2.w));
     }
     const long long o = static_cast<long long>(row) * p.N + col;
     if (ytype == MSD_OUT_BF16) {
@@ -432,7 +465,7 @@ static GemmP8Plan plan_p8(int64_t M, int64_t N, int64_t K, bool base = false) {
   pl.off_beta = off;  off = round_up(off + static_cast<size_t>(M) * sizeof(float), 1024);
   pl.off_part = off;
   if (pl.ksplit > 1) off = round_up(off + static_cast<size_t>(pl.ksplit) * pl.m_tiles * kP8TileM * N * sizeof(float), 1024);
-  if (pl.tail_n > 0) off = round_up(off + static_cast<size_t>(pl.tail_s) * pl.tail_n * (pl.pair ? 2 : 1) * kP8TileM * kP8TileN * sizeof(float), 1024);
+  if (pl.tail_n > 0) off = round_up(off + static_cast<size_t>(pl.tail_s) * pl.tail_n * (base ? 1 : kP8PartPlanes) * (pl.pair ? 2 : 1) * kP8TileM * kP8TileN * sizeof(float), 1024);
   pl.bytes = off;
   return pl;
 }
@@ -462,7 +495,10 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
                               cudaStream_t s) {
   if (static_cast<long long>((M + kP8TileM - 1) / kP8TileM) * ((N + kP8TileN - 1) / kP8TileN) > 0x7FFFFFFFLL) return MSD_ERR_BAD_SHAPE;
   const GemmP8Plan pl = plan_p8(M, N, K, base);
-  if (workspace_bytes < pl.bytes) return MSD_ERR_WORKSPACE_TOO_SMALL;
+  // Cut tiles give the same results as whole ones, so a workspace without room for their partial sums still serves; the
+  // accumulators that acc_dbg asks for exist only in whole tiles.
+  const int tail_n = acc_dbg == nullptr && workspace_bytes >= pl.bytes ? pl.tail_n : 0;
+  if (workspace_bytes < (pl.tail_n > 0 ? pl.off_part : pl.bytes)) return MSD_ERR_WORKSPACE_TOO_SMALL;
   unsigned* status = device_status_ptr();
   if (!status) return MSD_ERR_CUDA;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -488,8 +524,6 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
   CUtensorMap tmap_a1, tmap_a2, tmap_b, tmap_y;
   const bool ybf = !split && ytype == MSD_OUT_BF16;
   const bool use_pair = pl.pair;
-  // (the INT32 accumulators exist only for whole tiles)
-  const int tail_n = acc_dbg == nullptr ? pl.tail_n : 0;
   const uint64_t unit_rows = (use_pair ? 2 : 1) * kP8TileM;
   if (!encode_tmap_2d(&tmap_a1, CU_TENSOR_MAP_DATA_TYPE_UINT8, a1_ptr, kb, M, kb, kP8BlockK, kP8TileM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_tmap_2d(&tmap_a2, CU_TENSOR_MAP_DATA_TYPE_UINT8, base ? a1_ptr : static_cast<const void*>(q2), kb, M, kb, kP8BlockK, kP8TileM, CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -499,7 +533,7 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
                       static_cast<uint64_t>(N) * (ybf ? 2 : 4), ybf ? 32 : 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
     return MSD_ERR_CUDA;
   CUtensorMap tmap_part = tmap_y;
-  if (tail_n > 0 && !encode_tmap_2d(&tmap_part, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, part, kP8TileN, unit_rows * tail_n * pl.tail_s,
+  if (tail_n > 0 && !encode_tmap_2d(&tmap_part, CU_TENSOR_MAP_DATA_TYPE_UINT32, part, kP8TileN, unit_rows * tail_n * pl.tail_s * (base ? 1 : kP8PartPlanes),
                                     kP8TileN * sizeof(float), 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
     return MSD_ERR_CUDA;
 
@@ -544,7 +578,8 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
   if (tail_n > 0) {
     const long long quads = static_cast<long long>(tail_n) * unit_rows * (kP8TileN / 4);
     const unsigned blocks = static_cast<unsigned>(std::min<long long>((quads + 255) / 256, 4LL * sm_count()));
-    if (launch_pdl(p8_tail_reduce_kernel, dim3(blocks), dim3(256), 0, s, pdl, static_cast<const float*>(part), p, static_cast<int>(unit_rows), y, ytype) != cudaSuccess)
+    if (launch_pdl(base ? p8_tail_reduce_kernel<true> : p8_tail_reduce_kernel<false>, dim3(blocks), dim3(256), 0, s, pdl,
+                   reinterpret_cast<const uint32_t*>(part), p, static_cast<int>(unit_rows), y, ytype) != cudaSuccess)
       return MSD_ERR_CUDA;
   }
   return MSD_OK;

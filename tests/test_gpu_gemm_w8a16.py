@@ -234,22 +234,25 @@ def test_prefill_regime_with_k_split(M, N, K):
 @pytest.mark.parametrize("M,N,K,pair", [(200, 19200, 2048, 1), (300, 19000, 2064, 1), (300, 12792, 2048, 0), (385, 9736, 4096, 0),
                                         (1000, 9480, 2176, 1)])
 def test_prefill_last_round_cut_along_k(M, N, K, pair):
-    """A few tiles more than fill the machine once: those are cut along K and their FP32 partial tiles added.  Against the same
-    call with the accumulators asked for, which keeps every tile whole (and is checked against the oracle above): at most
-    32 partial sums rounded to FP32, each within 2^-24 of itself, so 32 * 2^-24 < 2e-6 of the row's norm; BF16 outputs
-    may land one unit in the last place apart."""
+    """A few tiles more than fill the machine once: those are cut along K and their pieces' INT32 sums added, so every bit is
+    that of the same call with the accumulators asked for, which keeps every tile whole (and is checked against the oracle
+    above).  That tiles were cut shows in the workspace, which holds the pieces' sums; one without room for them still
+    serves, uncut, and one that is smaller still is refused."""
     binding.debug_set_option("MSD_P8_PAIR", pair)
     c = inputs.gemm_w8_case(M, N, K, seed=M)
     x, w, s = bf16_dev(c.x), dev(c.w), dev(c.w_scale)
+    up = lambda v: (v + 1023) // 1024 * 1024
+    whole_bytes = 2 * up(M * K) + 2 * up(4 * M)
+    assert binding.gemm_w8a16_workspace_bytes(M, N, K) > whole_bytes
     for dt in (torch.float32, torch.bfloat16):
         whole, _acc = binding.gemm_w8a16(x, w, s, out_dtype=dt, want_acc=True)
         cut = binding.gemm_w8a16(x, w, s, out_dtype=dt)
+        short = binding.gemm_w8a16(x, w, s, out_dtype=dt, ws=binding.workspace(whole_bytes))
         torch.cuda.synchronize()
         binding.last_device_status()
-        a, b = whole.float().cpu().numpy(), cut.float().cpu().numpy()
-        slack = 2e-6 * np.linalg.norm(a, axis=1, keepdims=True) + (np.abs(a) * 2.0 ** -7 if dt == torch.bfloat16 else 0)
-        assert np.all(np.abs(a - b) <= slack)
-        assert dt == torch.bfloat16 or not np.array_equal(a, b)          # the cut tiles are really summed in another order
+        assert torch.equal(cut, whole) and torch.equal(short, whole)
+    with pytest.raises(binding.MsdError):
+        binding.gemm_w8a16(x, w, s, ws=binding.workspace(whole_bytes)[:whole_bytes - 1])
 
 
 @pytest.mark.parametrize("pair", ["0", "1"])
