@@ -337,8 +337,8 @@ msd_status_t msd_attn_decode_int8kv_paged(const void* q_bf16, const int8_t* k_ca
 /* The split schedule msd_attn_decode_int8kv uses (so a checker can mirror it): writes the tile size, the largest
  * number of context splits a (sequence, query row) can have and the tokens per split.  With *split_tokens > 0 split s
  * of a sequence of length L covers tokens [s*split_tokens, min(L, (s+1)*split_tokens)) and is walked in tiles of
- * `tile` tokens (splits past L are empty); with more than 8 rows per KV head a call may use a larger size, one for all its
- * sequences, that it takes from their lengths (msd_attn_decode_split_starts knows it).  *split_tokens = 0: the splits depend on the lengths of all sequences of
+ * `tile` tokens (splits past L are empty); a call may use a larger size, one for all its sequences, that it takes from their
+ * lengths (msd_attn_decode_split_starts knows it).  *split_tokens = 0: the splits depend on the lengths of all sequences of
  * the call (Sec. 4.3 leaves the partition of the context open; head groups of up to 8 rows per KV head may cut the list
  * of all sequences' tiles into equal runs, as many as fit the machine at once, so that no SM is left with more work
  * than another) - msd_attn_decode_split_starts lists them. */

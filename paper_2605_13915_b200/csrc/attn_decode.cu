@@ -32,31 +32,42 @@ constexpr int kChunk = 128;         // bytes of D / Dv per TMA box and per share
 constexpr int kChunkBytes = kTok * kChunk;
 constexpr int kPartHdr = 4;         // words in front of a split's partial output row: reference maximum, sum of P, two unused
 
-// The split size of a call whose CTAs can all but be resident at once (wide head groups), taken on the device from the
-// lengths themselves: the host knows only the longest.  All splits of a call have the size, c tiles.  With A the tiles that
-// each of the machine's CTA slots has to do, c is A plus the start-up of the units' short last splits, over a share (0.06
-// for equal lengths, more the more they differ) that keeps those last splits, which run in the gaps, from ending later than
-// the full ones:  c = (A + units / slots + 1) / (1 - 0.06 - 0.25 (1 - mean / longest)).  Coefficients fitted to sweeps of the size over
-// 321 shapes (latent cache, 16 and 32 rows per KV head; 1024 to 32768 tokens; all lengths equal, from a half, from a tenth or a
-// quarter of the longest): time over that of the best size (linear between swept sizes) 1.012, 1.010 and 1.012 on average, against 1.082, 1.037 and
-// 1.057 with the size chosen from the longest length alone.  64 latent caches, 64 heads: 16384 tokens 270 us -> 238, 2048 to 8192 tokens
-// 130 -> 104; 16 GQA sequences of 1024 to 8192, 4 query tokens: 53.7 -> 47.9.
+// The split size of a call, taken on the device from the lengths themselves: the host knows only a bound of the longest.
+// All splits of a call have the size, c tiles, between c_min (which the workspace and the grid are laid out for) and c_max.
+// With A the tiles that each of the machine's CTA slots has to do and U the slots' share of units, x = A + 1.5 U:
+//   narrow kernel                              c = (x + 1) / 0.9
+//   wide kernel, lengths 40 % of the bound or more on average (rho = mean / bound)     c = (x + 1) / (0.69 + 0.25 rho)
+//   wide kernel, less: skewed lengths or a generous bound                              c = x / 0.85
+// c is a slot's work plus the start-up of the units' short last splits, over a share that keeps those, which run in the gaps,
+// from ending after the full ones.  Fitted to sweeps of the size over 152 calls with up to 8 rows per KV head and 104 with more
+// (equal and mixed lengths, one long sequence in ten or thirty, bounds two to eight times the longest; 1 to 64 sequences of up to
+// 32768 tokens): time over that of the best size swept 1.012 and 1.023 on average.
+constexpr int kAdaptMaxPaged = 256;     // sequences of a paged call up to which every CTA sums their lengths
 struct AttnAdapt {
-  float per_token, base, inv_full;      // A = per_token * tokens + ..., 1 / (B * longest)
+  float per_token, base, inv_bound;     // x (narrow: c) = per_token * tokens + base; rho = inv_bound * tokens
   int c_min, c_max;                     // tiles; c_max = 0: the split size is the plan's
 };
 
 // (the host computes the same size for those who ask where the splits lie: every operation rounds by itself)
+template <bool kWide>
 __host__ __device__ __forceinline__ int attn_adapt_tiles(const AttnAdapt& a, int tokens) {
+  float c;
 #ifdef __CUDA_ARCH__
-  const float t = __int2float_rn(tokens), rho = fminf(__fmul_rn(t, a.inv_full), 1.0f);
-  const float c = __fdiv_rn(__fadd_rn(__fmul_rn(t, a.per_token), a.base), __fadd_rn(0.69f, __fmul_rn(0.25f, rho)));
+  const float t = __int2float_rn(tokens), x = __fadd_rn(__fmul_rn(t, a.per_token), a.base);
+  c = x;
+  if constexpr (kWide) {
+    const float rho = fminf(__fmul_rn(t, a.inv_bound), 1.0f);
+    c = rho >= 0.4f ? __fdiv_rn(__fadd_rn(x, 1.0f), __fadd_rn(0.69f, __fmul_rn(0.25f, rho))) : __fdiv_rn(x, 0.85f);
+  }
 #else
-  volatile float m = static_cast<float>(tokens) * a.inv_full, x = static_cast<float>(tokens) * a.per_token;
-  const float rho = m < 1.0f ? m : 1.0f;
-  volatile float y = 0.25f * rho;
-  volatile float num = x + a.base, den = 0.69f + y;
-  const float c = num / den;
+  volatile float p = static_cast<float>(tokens) * a.per_token, x = p + a.base;
+  c = x;
+  if constexpr (kWide) {
+    volatile float m = static_cast<float>(tokens) * a.inv_bound;
+    const float rho = m < 1.0f ? m : 1.0f;
+    volatile float r = 0.25f * rho, num = x + 1.0f, den = 0.69f + r;
+    c = rho >= 0.4f ? num / den : x / 0.85f;
+  }
 #endif
   const int n = static_cast<int>(ceilf(fminf(c, 1.0e9f)));
   return n < a.c_min ? a.c_min : (n > a.c_max ? a.c_max : n);
@@ -113,6 +124,44 @@ struct AttnParams {
 __device__ __forceinline__ long long attn_out_row(const AttnParams& p, int b, int hk, int r) {
   const int sq = r / p.Gr;
   return (static_cast<long long>(b) * p.Sq + sq) * (p.Hkv * p.Gr) + hk * p.Gr + (r - sq * p.Gr);
+}
+
+// Tokens [t_begin, t_end) of split `split` of a sequence of L tokens.
+__device__ __forceinline__ void attn_split_span(int L, int split, int chunk, int* t_begin, int* t_end) {
+  const long long t0 = static_cast<long long>(split) * chunk;      // (splits past the end: beyond 2^31 for a careless max_seqlen)
+  *t_begin = t0 < L ? static_cast<int>(t0) : max(L, 0);
+  *t_end = L - *t_begin > chunk ? *t_begin + chunk : L;
+}
+
+// A split without tokens: the first of a unit marks the end of the unit's splits for the merge (reference maximum -inf), the
+// others leave no trace, so that they are gone as soon as they are launched.
+__device__ __forceinline__ void attn_end_of_splits(const AttnParams& p, int b, int hk, int grp, int nh, int split, int chunk, int L) {
+  if (split > 0 && static_cast<long long>(split - 1) * chunk >= L) return;
+  for (int i = threadIdx.x; i < nh; i += blockDim.x)
+    p.partial[((static_cast<long long>(b) * p.Hq + hk * p.G + grp * p.HG + i) * p.n_splits + split) * (p.Dv + kPartHdr)] = -INFINITY;
+}
+
+// Sequence b of a call (first row in a contiguous cache, tokens) and the call's tokens per split.  Every warp for itself, all
+// lanes; the loads are independent of one another, this is the start of a CTA and nothing goes on before they return.
+template <bool kWide, bool kPaged, bool kAdapt>
+__device__ __forceinline__ void attn_call_lengths(const AttnParams& p, int b, int lane, int* seq0, int* L, int* chunk) {
+  const bool adapt = kAdapt && p.adapt.c_max > 0;
+  int tokens = 0;
+  if constexpr (kPaged) {
+    *seq0 = 0;
+    *L = __ldg(p.seqlens + b);
+    if (adapt && p.B <= kAdaptMaxPaged) {
+      for (int i = lane; i < p.B; i += 32) tokens += max(__ldg(p.seqlens + i), 0);
+      tokens = __reduce_add_sync(0xffffffffu, tokens);
+    }
+  } else {
+    const int last = __ldg(p.cu + (adapt ? p.B : b)), first = __ldg(p.cu);
+    *seq0 = __ldg(p.cu + b);
+    *L = __ldg(p.cu + b + 1) - *seq0;
+    tokens = last - first;
+  }
+  *chunk = p.chunk;
+  if (adapt && (!kPaged || p.B <= kAdaptMaxPaged)) *chunk = attn_adapt_tiles<kWide>(p.adapt, tokens) * kTok;
 }
 
 __device__ __forceinline__ void attn_mark(const AttnParams& p, int slot) {
@@ -410,28 +459,24 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     if (!attn_walk_init(p, s_scan, &w0, &slot0)) return;
   } else {
     const int split = blockIdx.y, b = blockIdx.x / U;
-    const int L = attn_seq_tokens(p, b);
-    const int t_begin = split * p.chunk;                       // every split covers the same number of tokens
-    const int t_end = min(L, t_begin + p.chunk);
+    int L, chunk;                              // every split covers the same number of tokens
+    attn_call_lengths<false, kPaged, !kDirect>(p, b, lane, &w0.seq0, &L, &chunk);
+    int t_begin, t_end;
+    attn_split_span(L, split, chunk, &t_begin, &t_end);
     const int ntiles = (t_end > t_begin) ? (t_end - t_begin + kTok - 1) / kTok : 0;
-    if (ntiles == 0) {      // nothing in this split: neutral partials, before any barrier or TMEM use
-      const int grp = blockIdx.x % p.groups, hk = (blockIdx.x / p.groups) % p.Hkv;
-      const int h0 = hk * p.G + grp * p.HG, nh = min(p.HG, p.G - grp * p.HG);
+    if (ntiles == 0) {      // nothing in this split, and nothing set up yet
+      const int grp = blockIdx.x % p.groups, hk = (blockIdx.x / p.groups) % p.Hkv, nh = min(p.HG, p.G - grp * p.HG);
       if constexpr (kDirect) {          // no token at all
         for (int i = threadIdx.x; i < nh * p.Dv; i += blockDim.x)
           p.out[attn_out_row(p, b, hk, grp * p.HG + i / p.Dv) * p.Dv + i % p.Dv] = __float2bfloat16_rn(0.0f);
         if (p.lse && threadIdx.x < nh) p.lse[attn_out_row(p, b, hk, grp * p.HG + threadIdx.x)] = -INFINITY;
-        return;
-      }
-      for (int i = threadIdx.x; i < nh * (p.Dv + kPartHdr); i += blockDim.x) {
-        const int h = i / (p.Dv + kPartHdr), e = i % (p.Dv + kPartHdr);
-        float* dst = p.partial + ((static_cast<long long>(b) * p.Hq + h0 + h) * p.n_splits + split) * (p.Dv + kPartHdr);
-        dst[e] = (e == 0) ? -INFINITY : 0.0f;
+      } else {
+        attn_end_of_splits(p, b, hk, grp, nh, split, chunk, L);
       }
       return;
     }
     w0.b = b; w0.u = blockIdx.x % U; w0.t = t_begin / kTok; w0.left = ntiles;
-    attn_walk_load(p, w0);
+    w0.L = L; w0.nb = (L + kTok - 1) / kTok;
     slot0 = split;
   }
   const int total_tiles = w0.left;
@@ -1039,21 +1084,10 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   const int b = (blockIdx.x - grp * pairs) / p.Hkv, hk = blockIdx.x - grp * pairs - b * p.Hkv;
   const int unit_q = (b * p.Hkv + hk) * p.groups + grp;      // index of the stacked query operand (attn_qstack_kernel)
   const int32_t* bt = kPaged ? p.block_table + static_cast<long long>(b) * p.max_blocks : nullptr;
-  const int seq0 = kPaged ? 0 : p.cu[b];
-  const int L = kPaged ? p.seqlens[b] : p.cu[b + 1] - seq0;
-  int chunk = p.chunk;
-  if (p.adapt.c_max > 0) {
-    int tokens = 0;
-    if constexpr (kPaged) {
-      for (int i = lane; i < p.B; i += 32) tokens += max(p.seqlens[i], 0);
-      tokens = __reduce_add_sync(0xffffffffu, tokens);
-    } else {
-      tokens = p.cu[p.B] - p.cu[0];
-    }
-    chunk = attn_adapt_tiles(p.adapt, tokens) * kTok;
-  }
-  const int t_begin = split * chunk;
-  const int t_end = min(L, t_begin + chunk);
+  int seq0, L, chunk;
+  attn_call_lengths<true, kPaged, true>(p, b, lane, &seq0, &L, &chunk);
+  int t_begin, t_end;
+  attn_split_span(L, split, chunk, &t_begin, &t_end);
   const int h0 = hk * p.G + grp * p.HG;
   const int nh = min(p.HG, p.G - grp * p.HG);
   const int ntiles = (t_end > t_begin) ? (t_end - t_begin + kTok - 1) / kTok : 0;
@@ -1065,11 +1099,9 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     if (cta < 1024) { p.trace[cta * 32 + 1] = static_cast<long long>(g); p.trace[cta * 32 + 2] = ntiles; }
   }
 
-  if (ntiles == 0) {      // nothing in this split: a neutral header (the merge reads no further), before any barrier or TMEM use
-    pdl_wait_primary();       // (this grid must not end before the kernel it depends on)
-    for (int i = threadIdx.x; i < nh * kPartHdr; i += blockDim.x)
-      p.partial[((static_cast<long long>(b) * p.Hq + h0 + i / kPartHdr) * p.n_splits + split) * (p.Dv + kPartHdr) + i % kPartHdr] =
-          (i % kPartHdr == 0) ? -INFINITY : 0.0f;
+  if (ntiles == 0) {      // nothing in this split, and nothing set up yet
+    if (split == 0) pdl_wait_primary();       // (the grid must not end before the kernel it depends on, even if every sequence is empty)
+    attn_end_of_splits(p, b, hk, grp, nh, split, chunk, L);
     return;
   }
 
@@ -1711,19 +1743,18 @@ static int32_t* g_attn_s_dbg = nullptr;
 
 // c8: merge the splits of one (sequence, query head) and normalise:  O = sum_s e^{m_s - m} O_s / sum_s e^{m_s - m} l_s
 // (a separate small kernel: letting the last-arriving split do it inside the attention kernel measured slower).
-// One CTA per row; the weights e^{m_s - m} are computed once per split and the O_s rows are read as 16-byte vectors,
-// eight splits' loads in flight per thread.  O is summed over the splits in ascending order.
-// kTrim (wide head groups): the splits after the last that saw a token have no more than a header and are not read.
-// kMany (eight splits and more): registers for those eight loads.  Left to itself the compiler keeps to 32, for 16 CTAs an SM, and the
-// loads follow one another; with few splits the CTAs in flight are what counts (1 x 8192 tokens, 16 splits: the call 15.1 us, now
-// 12.6; 4 x 1000 to 4000, 11 splits: 16.0, now 14.7; 64 x 100 to 1000, one split: 28.3, 29.4 with 48 registers).
+// One CTA per row; the weights e^{m_s - m} are computed once per split and the O_s rows are read as 16-byte vectors, a batch of
+// splits' loads in flight per thread.  O is summed over the splits in ascending order.
+// kTrim (fixed splits): a row's splits end at the first whose reference maximum is -inf; what lies behind it is not read.
+// kMany (more than four splits): batches of eight and the registers for them.  Left to itself the compiler keeps to 32, for 16
+// CTAs an SM, which is what counts with few splits (64 x 100 to 1000 tokens, one split: 28.3 us, 29.4 with 48 registers); with more
+// the loads do (2 x 1158 to 2316 tokens, 7 splits: 10.4 us the call, 11.7 where those past the last whole batch followed one another).
 template <bool kTrim, bool kMany>
 __global__ void __launch_bounds__(128, kMany ? 10 : 16)
 attn_combine_kernel(const float* __restrict__ partial, int n_splits_alloc, const int32_t* __restrict__ n_slots, int G, int HG,
                     int groups, int Dv, __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int Sq, int Gr, int Hkv) {
   __shared__ float s_w[128];
-  __shared__ float s_red[2][4];
-  __shared__ int s_last[kTrim ? 4 : 1];
+  __shared__ float s_red[4];
   pdl_wait_primary();              // the partial results come from the attention kernel launched just before
   const int PS = Dv + kPartHdr;
   const float* base = partial + static_cast<long long>(blockIdx.x) * n_splits_alloc * PS;
@@ -1744,23 +1775,26 @@ attn_combine_kernel(const float* __restrict__ partial, int n_splits_alloc, const
     row = (bq * Sq + sq) * (Hkv * Gr) + hk * Gr + (r - sq * Gr);
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // every warp for itself: the largest reference maximum, and with kTrim the end of the row's splits
   float m = -INFINITY;
-  int last = 0;
-  for (int s = tid; s < n_splits; s += 128) {
-    const float ms = __ldg(base + static_cast<long long>(s) * PS);
-    if constexpr (kTrim) last = (ms != -INFINITY) ? s + 1 : last;
-    m = fmaxf(m, ms);
+  for (int s0 = 0, end = n_splits; s0 < end; s0 += 128) {
+    float ms[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ms[j] = s0 + 32 * j + lane < end ? __ldg(base + static_cast<long long>(s0 + 32 * j + lane) * PS) : -INFINITY;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if constexpr (kTrim) {
+        const unsigned stop = __ballot_sync(0xffffffffu, ms[j] == -INFINITY);      // (past the last split too)
+        if (stop != 0 && n_splits == end) n_splits = min(end, s0 + 32 * j + __ffs(stop) - 1);
+        if (s0 + 32 * j + lane >= n_splits) ms[j] = -INFINITY;
+      }
+      m = fmaxf(m, ms[j]);
+    }
+    if (kTrim && n_splits < end) break;
   }
-  if constexpr (kTrim) last = __reduce_max_sync(0xffffffffu, last);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) {
-    s_red[0][warp] = m;
-    if constexpr (kTrim) s_last[warp] = last;
-  }
-  __syncthreads();
-  m = fmaxf(fmaxf(s_red[0][0], s_red[0][1]), fmaxf(s_red[0][2], s_red[0][3]));
-  if constexpr (kTrim) n_splits = max(max(s_last[0], s_last[1]), max(s_last[2], s_last[3]));
+  constexpr int kBatch = kMany ? 8 : 4;
   const bool act = tid < (Dv >> 2);
   const float4* o4 = reinterpret_cast<const float4*>(base + kPartHdr) + tid;
   const int ps4 = PS >> 2;
@@ -1778,19 +1812,24 @@ attn_combine_kernel(const float* __restrict__ partial, int n_splits_alloc, const
     const int n = min(128, n_splits - s0);
     if (act) {
       const float4* q = o4 + static_cast<long long>(s0) * ps4;
-#pragma unroll 8
-      for (int i = 0; i < n; ++i) {
-        const float4 v = __ldg(q + static_cast<long long>(i) * ps4);
-        const float wi = s_w[i];
-        acc.x += wi * v.x; acc.y += wi * v.y; acc.z += wi * v.z; acc.w += wi * v.w;
+      // (a batch at a time, the last one with the loads it needs: a remainder loop would wait for them one by one)
+      for (int i = 0; i < n; i += kBatch) {
+        float4 v[kBatch];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) v[j] = i + j < n ? __ldg(q + static_cast<long long>(i + j) * ps4) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          const float wi = s_w[i + j];          // (0 past the last split)
+          acc.x += wi * v[j].x; acc.y += wi * v[j].y; acc.z += wi * v[j].z; acc.w += wi * v[j].w;
+        }
       }
     }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if (lane == 0) s_red[1][warp] = l;
+  if (lane == 0) s_red[warp] = l;
   __syncthreads();
-  l = (s_red[1][0] + s_red[1][1]) + (s_red[1][2] + s_red[1][3]);
+  l = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
   if (act) {
     const float o0 = l > 0.0f ? acc.x / l : 0.0f, o1 = l > 0.0f ? acc.y / l : 0.0f;
     const float o2 = l > 0.0f ? acc.z / l : 0.0f, o3 = l > 0.0f ? acc.w / l : 0.0f;
@@ -1812,15 +1851,14 @@ struct AttnPlan {
 
 // What a context split costs, in microseconds (fitted to sweeps over split sizes): `per_sm` CTAs of the kernel fit an SM, a
 // tile takes tile_us[k - 1] with k of them on it, a CTA's set-up, first tiles, partial results and their merge `fixed_us`.
-struct AttnSplitCost { int per_sm; float tile_us[3], fixed_us; };
+// CTA that finds nothing to do adds empty_us to a call that has many of them.
+struct AttnSplitCost { int per_sm; float tile_us[3], fixed_us, empty_us; };
 
-// Tiles per context split.  The CTAs of a call run in rounds of as many as fit the machine, so the split size decides how
-// many rounds there are and how full the last is; powers of two missed both (one latent cache of 64 heads, 8 sequences of 4096 to
-// 8192 tokens: 2 tiles a split 57.8 us, 8 tiles 38.2; 12 GQA sequences of 6000: 4 tiles 42.9, 12 tiles 32.8; 128 query / 8 KV
-// heads, 32 x 4096: 8 tiles 85, 32 tiles 68).  The host knows the longest sequence, not the others: the size taken has the
-// smallest sum of the costs with every sequence at full length (whole rounds) and with lengths of 60 % on average (mixed
-// lengths fill the rounds up; half a split is left over at the end).  Against the best size found by sweeping it lost 4 % on
-// average over 18 shapes, 18 % at most.
+// Tiles per context split that suit a call whose sequences are near their bound, or mixed with a mean of 60 % of it: what the
+// lengths may make of it, and whether one split will do, is attn_adapt_plan's.  The CTAs of a call run in rounds of as many as
+// fit the machine, so the split size decides how many rounds there are and how full the last is; powers of two miss both.  The
+// size taken has the smallest sum of the costs with every sequence at full length (whole rounds) and with lengths of 60 % on
+// average (mixed lengths fill the rounds up; half a split is left over at the end).
 static int attn_split_tiles(long long units, int tiles, const AttnSplitCost& k) {
   const float sms = static_cast<float>(sm_count()), slots = sms * static_cast<float>(k.per_sm), u = static_cast<float>(units);
   const float frac = 0.6f;
@@ -1845,8 +1883,51 @@ static int attn_split_tiles(long long units, int tiles, const AttnSplitCost& k) 
   return best;
 }
 
+// Shapes for which the narrow kernel that writes the result of a single split itself is built.
+static bool attn_direct_built(const AttnPlan& pl) { return pl.HG == 8 && pl.DVT == 1 && pl.DC <= 4; }
+
 // The held references' integer accumulators take at most this many tiles: 127 * 127 * 128 * 512 < 2^31.
 constexpr int kMaxHeldTiles = 512;
+
+static int attn_call_tiles(const AttnPlan& pl, int tokens) {
+  return pl.HG > 8 ? attn_adapt_tiles<true>(pl.adapt, tokens) : attn_adapt_tiles<false>(pl.adapt, tokens);
+}
+
+// The range of the split size that a call takes from its lengths (AttnAdapt); returns the smallest, or `tiles` for one split.
+//
+// Smallest: the host cannot tell one sequence of `tiles` tiles among short ones from a batch of such sequences, nor either from
+// short sequences under a generous bound.  The first is over no sooner than the c tiles of one of its splits, every unit that
+// is short leaves tiles / c - 1 CTAs with nothing to do, and the sum of the two is smallest at the root below (one sequence of
+// 32768 and 15, 31, 127, 255 of 512 or 1024 tokens, 32 / 8 heads: best sizes swept 16, 24, 43, 96; the root is 15, 21, 43, 60).
+// Largest: that with which full-length sequences fill one round of CTAs; more units than CTA slots, two
+// splits a sequence or the size that suits full lengths.
+static int attn_adapt_plan(AttnPlan* pl, int B, int Hkv, long long units, int tiles, int max_seqlen, int c_model, const AttnSplitCost& k) {
+  const float slots = static_cast<float>(sm_count()) * static_cast<float>(k.per_sm), u = static_cast<float>(units), t1 = k.tile_us[0];
+  const int held = pl->HG > 8 ? kMaxHeldTiles : 1 << 20;
+  int c_min = static_cast<int>(std::min(std::ceil(std::sqrt(k.empty_us / t1 * static_cast<float>(tiles) * u)), 1.0e6f));
+  c_min = std::min(std::max(c_min, 2), std::min(tiles, held));
+  int c_max = std::max(tiles - tiles / 3, c_model);
+  if (u <= slots) {
+    const int rounds = static_cast<int>(slots / u);
+    c_max = (tiles + rounds - 1) / rounds;
+  }
+  c_max = std::min(c_max, held);
+  if (u > slots) c_min = std::min(c_min, c_max);
+  int ns = (tiles + c_min - 1) / c_min;
+  // One split, which the narrow kernel finishes without a merge, where that is the better size for full lengths and no worse
+  // for a single long sequence.
+  const float split_us = t1 * static_cast<float>(c_min) + k.empty_us * static_cast<float>(ns) * u + 3.0f;
+  if (ns <= 1 || (attn_direct_built(*pl) && c_model >= tiles && t1 * static_cast<float>(tiles) <= split_us)) return tiles;
+  c_min = (tiles + ns - 1) / ns;
+  const float share = pl->HG > 8 ? 1.0f / slots : 1.0f / (0.9f * slots);
+  pl->adapt.per_token = static_cast<float>(Hkv * pl->groups) * share / static_cast<float>(kTok);
+  pl->adapt.base = (1.5f * u + (pl->HG > 8 ? 0.0f : slots)) * share;
+  pl->adapt.inv_bound = 1.0f / (static_cast<float>(B) * static_cast<float>(std::max(max_seqlen, 1)));
+  pl->adapt.c_min = c_min;
+  pl->adapt.c_max = c_max;
+  if (c_max <= c_min || attn_call_tiles(*pl, B * max_seqlen) <= c_min) pl->adapt.c_max = 0;      // no lengths ask for more
+  return c_min;
+}
 
 static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, bool v_alias, AttnPlan* pl) {
   if (B < 1 || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || D < 16 || D % 16 != 0 || Dv < 16 || Dv % 16 != 0) return false;
@@ -1872,27 +1953,16 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   const int tiles = (max_seqlen + kTok - 1) / kTok;
   const long long units = static_cast<long long>(B) * Hkv * pl->groups;
   const bool small = pl->DC == 1 && pl->DVT == 1;
-  const AttnSplitCost split_cost = pl->HG == 8 ? (small ? AttnSplitCost{3, {1.0f, 1.5f, 2.2f}, 6.0f} : AttnSplitCost{1, {2.0f, 2.0f, 2.0f}, 8.0f})
-                                 : pl->HG == 16 ? AttnSplitCost{2, {1.3f, 1.75f, 1.75f}, 7.0f}
-                                                : AttnSplitCost{1, {small ? 1.3f : 2.0f, 2.0f, 2.0f}, small ? 7.0f : 11.0f};
+  const AttnSplitCost split_cost = pl->HG == 8 ? (small ? AttnSplitCost{3, {1.0f, 1.5f, 2.2f}, 6.0f, 0.009f} : AttnSplitCost{1, {2.0f, 2.0f, 2.0f}, 8.0f, 0.0085f})
+                                 : pl->HG == 16 ? AttnSplitCost{2, {1.3f, 1.75f, 1.75f}, 7.0f, 0.0075f}
+                                                : AttnSplitCost{1, {small ? 1.3f : 2.0f, 2.0f, 2.0f}, small ? 7.0f : 11.0f, 0.0085f};
   int chunk_tiles = option(OPT_ATTN_CHUNK_TILES);       // testing aid: a given split size
   pl->adapt = AttnAdapt{0.0f, 0.0f, 0.0f, 0, 0};
-  const long long slots = static_cast<long long>(sm_count()) * split_cost.per_sm;
-  if (pl->HG > 8 && units <= slots && static_cast<long long>(B) * max_seqlen < 0x7FFFFFFFLL && chunk_tiles < 1 && option(OPT_ATTN_SPLITS) < 1) {
-    // wide head groups, at most one unit per CTA slot: the size comes from the lengths (AttnAdapt).  At most that with which
-    // full-length sequences fill one round of CTAs, at least (which sizes the workspace) the one for lengths of 40 % on average.
-    const float inv_slots = 1.0f / static_cast<float>(slots), per_seq = static_cast<float>(Hkv * pl->groups);
-    AttnAdapt& a = pl->adapt;
-    a.per_token = per_seq * inv_slots / static_cast<float>(kTok);
-    a.base = (0.5f * static_cast<float>(units) + static_cast<float>(units)) * inv_slots + 1.0f;      // (half a tile more per sequence: its last)
-    a.inv_full = 1.0f / (static_cast<float>(B) * static_cast<float>(std::max(max_seqlen, 1)));
-    const int rounds = static_cast<int>(slots / units);
-    a.c_max = std::min((tiles + rounds - 1) / rounds, kMaxHeldTiles);
-    a.c_max = std::max(a.c_max, std::min(2, std::max(tiles, 1)));
-    a.c_min = std::min(2, a.c_max);
-    chunk_tiles = a.c_min = attn_adapt_tiles(a, static_cast<int>(0.4 * static_cast<double>(B) * max_seqlen));
+  if (chunk_tiles < 1) {
+    chunk_tiles = attn_split_tiles(units, tiles, split_cost);      // what the lengths may at most make it
+    if (option(OPT_ATTN_SPLITS) < 1 && static_cast<long long>(B) * max_seqlen < 0x7FFFFFFFLL)
+      chunk_tiles = attn_adapt_plan(pl, B, Hkv, units, tiles, max_seqlen, chunk_tiles, split_cost);
   }
-  if (chunk_tiles < 1) chunk_tiles = attn_split_tiles(units, tiles, split_cost);
   if (pl->HG > 8 && chunk_tiles > kMaxHeldTiles) chunk_tiles = kMaxHeldTiles;
   while ((tiles + chunk_tiles - 1) / chunk_tiles > 65535) chunk_tiles <<= 1;      // splits run along the grid's y axis
   int ns = (tiles + chunk_tiles - 1) / chunk_tiles;
@@ -1940,7 +2010,7 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
 
 // The split merge for another attention kernel of this library (rows in output order, every row n_splits partial results).
 msd_status_t launch_attn_combine(const float* partial, int n_splits, int Dv, void* out_bf16, float* lse, int rows, cudaStream_t s) {
-  if (launch_pdl(n_splits >= 8 ? attn_combine_kernel<false, true> : attn_combine_kernel<false, false>, dim3(rows), dim3(128), 0, s, option(OPT_NO_PDL) <= 0, partial, n_splits,
+  if (launch_pdl(n_splits > 4 ? attn_combine_kernel<false, true> : attn_combine_kernel<false, false>, dim3(rows), dim3(128), 0, s, option(OPT_NO_PDL) <= 0, partial, n_splits,
                  static_cast<const int32_t*>(nullptr), 1, 1, 1, Dv, static_cast<__nv_bfloat16*>(out_bf16), lse, 1, 1, 1) != cudaSuccess)
     return MSD_ERR_CUDA;
   return launch_status();
@@ -1951,7 +2021,7 @@ using AttnKernel = void (*)(CUtensorMap, CUtensorMap, AttnParams);
 // A single split of each sequence has nothing to merge: the narrow kernel writes the result, one launch and one round trip through
 // memory fewer (32 / 8 heads, 64 x 100 to 1000 tokens: 28.3 us, now 26.3; 48 x 750 to 1500: 30.2 and 27.5; 8 / 8, 32 x 512 to
 // 2048: 27.4 and 24.5).  Instantiations of their own: the branch at the end of the others cost 4 x 1000 to 4000 tokens 2.6 %.
-static bool attn_direct(const AttnPlan& pl) { return pl.HG == 8 && !pl.balanced && pl.n_splits == 1 && pl.DVT == 1 && pl.DC <= 4; }
+static bool attn_direct(const AttnPlan& pl) { return attn_direct_built(pl) && !pl.balanced && pl.n_splits == 1; }
 
 // The kernel instantiation for a plan (G: query rows per KV head) and its block size.
 static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* block_threads) {
@@ -1984,7 +2054,7 @@ static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* b
     }
   }
 #undef MSD_ATTN_PICK
-#undef MSD_ATTN_PICK_B
+#undef MSD_ATTN_PICK_P
   return kernel;
 }
 
@@ -2102,10 +2172,10 @@ static msd_status_t attn_split_starts(int32_t B, int32_t q_len, int32_t Hq, int3
     R = R < 1 ? 1 : R;
   }
   int chunk = pl.chunk;
-  if (pl.adapt.c_max > 0) {
+  if (pl.adapt.c_max > 0 && !(paged && B > kAdaptMaxPaged)) {
     int tokens = 0;
     for (int b = 0; b < B; ++b) tokens += std::max(seqlens[b], 0);
-    chunk = attn_adapt_tiles(pl.adapt, tokens) * kTok;
+    chunk = attn_call_tiles(pl, tokens) * kTok;
   }
   long long P = 0;                                   // tiles of the sequences in front
   for (int b = 0; b < B; ++b) {
@@ -2230,9 +2300,8 @@ static msd_status_t attn_launch(const void* q_bf16, const int8_t* k_cache, const
   }
   if (launch_pdl(kernel, grid, dim3(block_threads), pl.smem_bytes, s, pdl, tmap_k, tmap_v, p) != cudaSuccess) return MSD_ERR_CUDA;
   if (direct) return launch_status();
-  const bool many = pl.n_splits >= 8 && !pl.balanced;
-  auto combine = pl.HG > 8 ? (many ? attn_combine_kernel<true, true> : attn_combine_kernel<true, false>)
-                           : (many ? attn_combine_kernel<false, true> : attn_combine_kernel<false, false>);
+  const bool many = pl.n_splits > 4 && !pl.balanced;
+  auto combine = pl.balanced ? attn_combine_kernel<false, false> : (many ? attn_combine_kernel<true, true> : attn_combine_kernel<true, false>);
   if (launch_pdl(combine, dim3(B * Hq), dim3(128), 0, s, pdl, static_cast<const float*>(p.partial),
                  pl.n_splits, static_cast<const int32_t*>(pl.balanced ? p.n_slots : nullptr), Hq / Hkv, pl.HG, pl.groups, Dv,
                  static_cast<__nv_bfloat16*>(out_bf16), lse, q_len, Hq / (Hkv * q_len), Hkv) != cudaSuccess)

@@ -85,3 +85,32 @@ def test_schedule_choice_by_shape():
     assert sched(32, 128, 8, 128, 128, 8192)[2] > 0
     assert sched(64, 64, 1, 576, 512, 16384)[2] > 0
     assert sched(32, 32, 8, 256, 256, 8192)[2] > 0
+
+
+# smallest, largest: the sizes in tiles that took about a tenth longer than the best at most when the size was swept on a B200;
+# the one that a call takes from its lengths has to be among them (bound: max_seqlen over the longest sequence)
+@pytest.mark.parametrize("seqlens,Hq,Hkv,D,Dv,bound,smallest,largest", [
+    ([32768] + [1024] * 15, 64, 1, 576, 512, 1, 6, 13),           # one long latent cache among short ones
+    ([16384] + [512] * 63, 64, 1, 576, 512, 1, 5, 12),
+    ([16384] + [512] * 127, 64, 1, 576, 512, 1, 8, 20),           # more units than SMs
+    ([2048] * 8, 64, 1, 576, 512, 8, 2, 4),                       # a bound eight times the longest
+    ([4096] * 32, 64, 1, 576, 512, 8, 14, 19),
+    ([32768] + [1024] * 15, 32, 8, 128, 128, 1, 10, 24),          # grouped queries, one long sequence among short ones
+    ([32768] + [512] * 31, 32, 8, 128, 128, 1, 16, 32),
+    ([16384] + [512] * 63, 32, 8, 128, 128, 1, 16, 32),
+    ([32768] + [512] * 127, 32, 8, 128, 128, 1, 36, 72),
+    ([6000] + [500] * 11, 32, 8, 128, 128, 1, 4, 9),
+    ([8192] + [512] * 23, 32, 8, 128, 128, 1, 6, 15),
+    ([2048] * 8, 32, 8, 128, 128, 8, 5, 10),
+    ([4096] * 32, 32, 8, 128, 128, 8, 22, 32),
+    ([16384] + [512] * 15, 128, 8, 128, 128, 1, 6, 18),           # 16 rows per KV head
+    ([2048] * 16, 128, 8, 128, 128, 8, 8, 12),
+])
+def test_split_size_follows_the_lengths(seqlens, Hq, Hkv, D, Dv, bound, smallest, largest):
+    L = np.array(seqlens, np.int32)
+    starts, _ = binding.attn_decode_split_starts(L, Hq, Hkv, D, Dv, bound * int(L.max()), v_aliased=D != Dv, resident_ctas=444)
+    longest = int(np.argmax(L))
+    size = int(starts[longest, 0, 0, 1]) // TILE
+    assert smallest <= size <= largest
+    s = starts[:, 0, 0].astype(np.int64)
+    assert np.array_equal(s, np.minimum(L[:, None], np.arange(s.shape[1])[None, :] * size * TILE))

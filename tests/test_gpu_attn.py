@@ -115,6 +115,49 @@ def test_split_size_from_the_lengths(rows, seqlens, paged):
     assert torch.equal(o, ref)
 
 
+@pytest.mark.parametrize("page", [0, 16, 64])
+@pytest.mark.parametrize("Hq,seqlens,bound", [(16, [2000] * 7, 1), (64, [2000, 0, 2000, 1999, 1, 2000, 2000, 2000, 2000], 1),
+                                              (128, [1000] * 8, 2), (16, [3000] * 12, 4)])
+def test_split_size_from_the_lengths_few_rows(Hq, seqlens, bound, page):
+    """Up to 8 rows per KV head: a split size that the device takes from the lengths, larger than the smallest, is the one the host
+    reports, under an exact and a generous max_seqlen, contiguous and paged."""
+    c = inputs.gqa_case(len(seqlens), Hq, 16, 128, seqlens, seed=Hq)
+    mx = bound * c.max_seqlen
+    starts, _ = _split_starts(c, max_seqlen=mx)
+    assert starts[0, 0, 0, 1] > binding.attn_decode_schedule(len(seqlens), Hq, 16, 128, 128, mx)[2] > 0
+    if page:
+        k, v, ks, vs, table, sl = inputs.paginate(c, page, seed=Hq)
+        table = np.pad(table, ((0, 0), (0, (bound - 1) * table.shape[1] + bound)))
+        o, lse = binding.attn_decode_int8kv_paged(bf16_dev(c.q), dev(k), dev(v), dev(ks), dev(vs), dev(table), dev(sl), page, mx,
+                                                  c.softmax_scale, want_lse=True)
+    else:
+        o, lse = binding.attn_decode_int8kv(bf16_dev(c.q), dev(c.k), dev(c.v), dev(c.k_scale), dev(c.v_scale), dev(c.cu_seqlens), mx,
+                                            c.softmax_scale, want_lse=True)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    ref, lse_ref = _oracle_tiled(c, max_seqlen=mx, paged=page > 0)
+    _assert_close(oracle.bf16_bits_to_f64(bf16_bits(o)), ref)
+    live = np.isfinite(lse_ref)
+    assert np.allclose(lse.cpu().numpy()[live], lse_ref[live], rtol=0, atol=2e-3) and np.all(np.isneginf(lse.cpu().numpy()[~live]))
+
+
+@pytest.mark.parametrize("rows", [4, 16, 64])
+def test_merge_ends_where_the_splits_end(rows):
+    """More splits than a pass of the merge looks at (157), and a second call of short sequences in the same workspace: what the
+    first left behind the end of the second's splits does not count."""
+    binding.debug_set_option("MSD_ATTN_CHUNK_TILES", 1)
+    lens = [20000, 0, 130]
+    c = inputs.gqa_case(3, rows, 1, 128, lens, seed=rows)
+    ws = binding.workspace(binding.attn_decode_int8kv_workspace_bytes(3, rows, 1, 128, 128, 20000))
+    for case in (c, inputs.gqa_case(3, rows, 1, 128, [100, 0, 700], seed=rows + 1)):
+        o = binding.attn_decode_int8kv(bf16_dev(case.q), dev(case.k), dev(case.v), dev(case.k_scale), dev(case.v_scale),
+                                       dev(case.cu_seqlens), 20000, case.softmax_scale, ws=ws)
+        torch.cuda.synchronize()
+        binding.last_device_status()
+        ref, _ = _oracle_tiled(case, max_seqlen=20000)
+        _assert_close(oracle.bf16_bits_to_f64(bf16_bits(o)), ref)
+
+
 @pytest.mark.parametrize("rows,D", [(4, 512), (8, 512), (4, 640), (16, 128)])
 def test_scores_at_the_largest_codes(rows, D):
     """Every code of the keys and of the queries' first components at its limit: the integer sums of both components, and
