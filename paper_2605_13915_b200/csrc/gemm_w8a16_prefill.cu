@@ -375,15 +375,19 @@ p8_tail_reduce_kernel(const uint32_t* __restrict__ part, const GemmP8Params p, i
         acc.x += __uint_as_float(v.x); acc.y += __uint_as_float(v.y); acc.z += __uint_as_float(v.z); acc.w += __uint_as_float(v.w);
       }
     } else {
+      const float a = __ldg(p.alpha + row), b = __ldg(p.beta + row);      // (on their way while the sums arrive)
+      float sw[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sw[j] = __ldg(p.w_scale + col + j);
       uint4 s1 = make_uint4(0, 0, 0, 0), s2 = s1;
+#pragma unroll 4
       for (int sp = 0; sp < p.tail_s; ++sp) {
         const uint4 v1 = __ldg(src + sp * stride), v2 = __ldg(src + sp * stride + tile_quads);
         s1.x += v1.x; s1.y += v1.y; s1.z += v1.z; s1.w += v1.w;
         s2.x += v2.x; s2.y += v2.y; s2.z += v2.z; s2.w += v2.w;
       }
-      const float a = __ldg(p.alpha + row), b = __ldg(p.beta + row);
       auto combine = [&](int j, uint32_t t1, uint32_t t2) {
-        return __ldg(p.w_scale + col + j) * __fmaf_rn(a, static_cast<float>(static_cast<int32_t>(t1)), b * static_cast<float>(static_cast<int32_t>(t2)));
+        return sw[j] * __fmaf_rn(a, static_cast<float>(static_cast<int32_t>(t1)), b * static_cast<float>(static_cast<int32_t>(t2)));
       };
       acc = make_float4(combine(0, s1.x, s2.x), combine(1, s1.y, s2.y), combine(2, s1.z, s2.z), combine(3, s1.w, s2.w));
     }
@@ -404,24 +408,26 @@ struct GemmP8Plan {
   size_t off_q1, off_q2, off_alpha, off_beta, off_part, bytes;
 };
 
-// The round structure of `tiles` output tiles on `units` pairs or CTAs; returns its length in rounds.
+// The round structure of `tiles` output tiles of `tile_rows` tokens on `units` pairs or CTAs; returns its length in rounds.
 // A last round of at most half the units is cut along K (stages of 128) so that all of them share it: 1000 tokens on 14336
-// weight rows are 224 pair tiles on 74 pairs, 3.03 rounds that took four (an MLP of 4096 x 14336, both layers: 188 -> 179 us;
-// 1100 tokens, 5120 x 10240: 206 -> 186).  Pieces keep at least four
-// stages (a shorter one is all pipeline fill), and the partial tiles and their sum cost about 8 us, eleven stages.
-static double p8_rounds(long long tiles, long long units, int kstages, int* tail0, int* tail_n, int* tail_s, int* tail_k) {
+// weight rows are 224 pair tiles on 74 pairs, 3.03 rounds that took four (98.6 us, 90.2 cut; 1100 tokens, 5120 x 10240: 120.6 and
+// 97.6).  Pieces keep at least four stages (a shorter one is all pipeline fill).  The pieces' sums and their addition cost
+// about as much as eleven stages and one more for every twenty pieces of 256 tokens; where the round gets no shorter than that,
+// the cut loses (1168 tokens, 12800 x 3264, 56 pieces, 13 stages shorter: 83.7 us whole, 85.5 cut).
+static double p8_rounds(long long tiles, long long units, int tile_rows, int kstages, int* tail0, int* tail_n, int* tail_s, int* tail_k) {
   const long long full = tiles / units * units, rest = tiles - full;
   *tail0 = static_cast<int>(full); *tail_n = 0; *tail_s = 1; *tail_k = kstages;
   if (rest == 0) return static_cast<double>(full / units);
   long long sp = units / rest;
   if (sp > kstages / 4) sp = kstages / 4;
   if (full > 0 && sp >= 2) {
-    const int per = static_cast<int>((kstages + sp - 1) / sp);
-    if (kstages - per > 11) {
+    const int per = static_cast<int>((kstages + sp - 1) / sp), pieces = (kstages + per - 1) / per;
+    const double cost = 11.0 + static_cast<double>(rest * pieces) * tile_rows / (20 * 256);
+    if (kstages - per > cost) {
       *tail_n = static_cast<int>(rest);
       *tail_k = per;
-      *tail_s = (kstages + per - 1) / per;
-      return static_cast<double>(full / units) + static_cast<double>(per + 11) / kstages;
+      *tail_s = pieces;
+      return static_cast<double>(full / units) + (per + cost) / kstages;
     }
   }
   return static_cast<double>(full / units + 1);
@@ -451,8 +457,8 @@ static GemmP8Plan plan_p8(int64_t M, int64_t N, int64_t K, bool base = false) {
   // idle); the option MSD_P8_PAIR forces the choice.
   const long long pair_tiles = static_cast<long long>((pl.m_tiles + 1) / 2) * pl.n_tiles;
   int t1[4], t2[4];
-  const double r1 = p8_rounds(tiles, sm_count(), pl.kstages, &t1[0], &t1[1], &t1[2], &t1[3]);
-  const double r2 = p8_rounds(pair_tiles, sm_count() / 2, pl.kstages, &t2[0], &t2[1], &t2[2], &t2[3]);
+  const double r1 = p8_rounds(tiles, sm_count(), kP8TileM, pl.kstages, &t1[0], &t1[1], &t1[2], &t1[3]);
+  const double r2 = p8_rounds(pair_tiles, sm_count() / 2, 2 * kP8TileM, pl.kstages, &t2[0], &t2[1], &t2[2], &t2[3]);
   const int forced_pair = option(OPT_P8_PAIR);       // testing aid
   pl.pair = pl.ksplit == 1 && pl.m_tiles >= 2 && (forced_pair >= 0 ? forced_pair != 0 : r2 <= 1.01 * r1);
   const int* t = pl.pair ? t2 : t1;
