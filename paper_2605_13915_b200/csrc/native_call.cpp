@@ -9,7 +9,9 @@
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include <vector>
 
@@ -102,7 +104,7 @@ bool dims(Args& a, std::initializer_list<std::pair<const at::Tensor*, int>> want
 }
 
 // (x, w, w_scale, ws, y, acc or None, scaling)
-PyObject* gemm_w8a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+PyObject* gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
   const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(), *ws = a.tensor(false, false), *y = a.tensor(false, false),
                    *acc = a.tensor(true, false);
@@ -114,7 +116,7 @@ PyObject* gemm_w8a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
 }
 
 // (x, w_fp4, scales, prepared, ws, y)
-PyObject* gemm_w4a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+PyObject* gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
   const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor();
   const bool prepared = a.integer() != 0;
@@ -128,21 +130,17 @@ PyObject* gemm_w4a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
 
 // Rows per expert from a Python sequence; their sum must be the number of rows of x.
 bool group_sizes(Args& a, PyObject* seq, int64_t E, int64_t rows, std::vector<int32_t>& out) {
-  PyObject* fast = PySequence_Fast(seq, "group_sizes: expected a sequence");
+  const THPObjectPtr fast(PySequence_Fast(seq, "group_sizes: expected a sequence"));
   if (!fast) return false;
   int64_t sum = 0;
-  const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast);
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast.get());
   out.reserve(static_cast<size_t>(E));
   for (Py_ssize_t i = 0; i < n; ++i) {
-    const long v = PyLong_AsLong(PySequence_Fast_GET_ITEM(fast, i));
-    if (v == -1 && PyErr_Occurred()) {
-      Py_DECREF(fast);
-      return false;
-    }
+    const long v = PyLong_AsLong(PySequence_Fast_GET_ITEM(fast.get(), i));
+    if (v == -1 && PyErr_Occurred()) return false;
     out.push_back(static_cast<int32_t>(v));
     sum += v;
   }
-  Py_DECREF(fast);
   if (n != E || sum != rows) {
     a.fail(PyExc_AssertionError, "group_sizes: one per expert, adding up to the rows of x");
     return false;
@@ -151,7 +149,7 @@ bool group_sizes(Args& a, PyObject* seq, int64_t E, int64_t rows, std::vector<in
 }
 
 // (x, w, w_scale, group_sizes, ws, y)
-PyObject* grouped_gemm_w8a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+PyObject* grouped_gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   if (n != 6) return PyErr_Format(PyExc_TypeError, "expected 6 arguments");
   Args t(args, 3), u(args + 4, 2);
   const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
@@ -166,7 +164,7 @@ PyObject* grouped_gemm_w8a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
 }
 
 // (x, w_fp4, scales, group_sizes, prepared, ws, y)
-PyObject* grouped_gemm_w4a16(PyObject*, PyObject* const* args, Py_ssize_t n) {
+PyObject* grouped_gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   if (n != 7) return PyErr_Format(PyExc_TypeError, "expected 7 arguments");
   Args t(args, 3), u(args + 4, 3);
   const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
@@ -206,11 +204,8 @@ PyObject* attn_decode(PyObject* const* args, Py_ssize_t n) {
                                             Dv, scale, addr(out), addr_as<float>(lse), w.p, w.bytes, stream()));
 }
 
-PyObject* attn_decode_int8kv(PyObject*, PyObject* const* args, Py_ssize_t n) { return attn_decode<false>(args, n); }
-PyObject* attn_decode_int8kv_spec(PyObject*, PyObject* const* args, Py_ssize_t n) { return attn_decode<true>(args, n); }
-
 // (q, k, v or None, k_scale, v_scale or None, block_table, seqlens, page_size, max_seqlen, softmax_scale, Dv, ws, out, lse or None)
-PyObject* attn_decode_int8kv_paged(PyObject*, PyObject* const* args, Py_ssize_t n) {
+PyObject* attn_decode_int8kv_paged(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
   const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(), *vs = a.tensor(true), *table = a.tensor(),
                    *len = a.tensor();
@@ -228,11 +223,23 @@ PyObject* attn_decode_int8kv_paged(PyObject*, PyObject* const* args, Py_ssize_t 
       addr_as<float>(lse), w.p, w.bytes, stream()));
 }
 
+// What the interpreter calls: C++ exceptions (a tensor without storage or with another layout, no memory) become Python's.
+template <PyObject* (*fn)(PyObject* const*, Py_ssize_t)>
+PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  return fn(args, n);
+  END_HANDLE_TH_ERRORS
+}
+
+template <PyObject* (*fn)(PyObject* const*, Py_ssize_t)>
+PyMethodDef method(const char* name) {
+  return {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(entry<fn>)), METH_FASTCALL, nullptr};
+}
+
 PyMethodDef methods[] = {
-#define MSD_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(name)), METH_FASTCALL, nullptr}
-    MSD_METHOD(gemm_w8a16), MSD_METHOD(gemm_w4a16), MSD_METHOD(grouped_gemm_w8a16), MSD_METHOD(grouped_gemm_w4a16),
-    MSD_METHOD(attn_decode_int8kv), MSD_METHOD(attn_decode_int8kv_spec), MSD_METHOD(attn_decode_int8kv_paged),
-#undef MSD_METHOD
+    method<gemm_w8a16>("gemm_w8a16"), method<gemm_w4a16>("gemm_w4a16"), method<grouped_gemm_w8a16>("grouped_gemm_w8a16"),
+    method<grouped_gemm_w4a16>("grouped_gemm_w4a16"), method<attn_decode<false>>("attn_decode_int8kv"),
+    method<attn_decode<true>>("attn_decode_int8kv_spec"), method<attn_decode_int8kv_paged>("attn_decode_int8kv_paged"),
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
