@@ -153,7 +153,7 @@ def workspace(nbytes, device="cuda"):
 def _ws_ptr(ws):
     base = ws.data_ptr()
     al = (base + 1023) // 1024 * 1024
-    return C.c_void_p(al), ws.numel() - (al - base)
+    return C.c_void_p(al), max(0, ws.numel() * ws.element_size() - (al - base))
 
 
 SCALING_DEFAULT, SCALING_FRACTIONAL = 0, 1

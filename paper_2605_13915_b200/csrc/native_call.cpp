@@ -26,21 +26,9 @@ class Args {
   Args(PyObject* const* a, Py_ssize_t n) : a_(a), n_(n) {}
   bool ok() const { return ok_; }
 
-  const at::Tensor* tensor(bool nullable = false, bool device = true) {
-    PyObject* o = next();
-    if (!o) return nullptr;
-    if (o == Py_None && nullable) return nullptr;
-    if (!THPVariable_Check(o)) {
-      fail(PyExc_TypeError, "expected a tensor");
-      return nullptr;
-    }
-    const at::Tensor& t = THPVariable_Unpack(o);
-    if (device && (!t.is_cuda() || !t.is_contiguous())) {
-      fail(PyExc_ValueError, "expected contiguous CUDA tensors");
-      return nullptr;
-    }
-    return &t;
-  }
+  const at::Tensor* tensor(bool nullable = false) { return take(nullable, false); }
+  // written by the kernels: a contiguous CUDA tensor, or page-locked host memory that they can reach
+  const at::Tensor* buffer(bool nullable = false) { return take(nullable, true); }
   int64_t integer() {
     PyObject* o = next();
     if (!o) return 0;
@@ -61,6 +49,21 @@ class Args {
   }
 
  private:
+  const at::Tensor* take(bool nullable, bool pinned) {
+    PyObject* o = next();
+    if (!o) return nullptr;
+    if (o == Py_None && nullable) return nullptr;
+    if (!THPVariable_Check(o)) {
+      fail(PyExc_TypeError, "expected a tensor");
+      return nullptr;
+    }
+    const at::Tensor& t = THPVariable_Unpack(o);
+    if (!(t.is_cuda() || (pinned && t.is_pinned())) || !t.is_contiguous()) {
+      fail(PyExc_ValueError, "expected contiguous CUDA tensors");
+      return nullptr;
+    }
+    return &t;
+  }
   PyObject* next() {
     if (!ok_) return nullptr;
     if (i_ >= n_) {
@@ -80,14 +83,14 @@ T* addr_as(const at::Tensor* t) { return static_cast<T*>(addr(t)); }
 msd_out_t out_type(const at::Tensor* y) { return y->scalar_type() == at::kBFloat16 ? MSD_OUT_BF16 : MSD_OUT_FP32; }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// The workspace a tensor of bytes offers: from its first 1024-byte boundary on.
+// The workspace a tensor offers: its bytes from the first 1024-byte boundary on, none where it ends before that.
 struct Workspace {
   void* p;
   size_t bytes;
   explicit Workspace(const at::Tensor* t) {
     const uintptr_t base = reinterpret_cast<uintptr_t>(t->data_ptr()), al = (base + 1023) / 1024 * 1024;
     p = reinterpret_cast<void*>(al);
-    bytes = static_cast<size_t>(t->numel()) - (al - base);
+    bytes = t->nbytes() > al - base ? t->nbytes() - (al - base) : 0;
   }
 };
 
@@ -106,8 +109,8 @@ bool dims(Args& a, std::initializer_list<std::pair<const at::Tensor*, int>> want
 // (x, w, w_scale, ws, y, acc or None, scaling)
 PyObject* gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
-  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(), *ws = a.tensor(false, false), *y = a.tensor(false, false),
-                   *acc = a.tensor(true, false);
+  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(), *ws = a.buffer(), *y = a.buffer(),
+                   *acc = a.buffer(true);
   const int64_t scaling = a.integer();
   if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
   const Workspace k(ws);
@@ -120,7 +123,7 @@ PyObject* gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
   const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor();
   const bool prepared = a.integer() != 0;
-  const at::Tensor *ws = a.tensor(false, false), *y = a.tensor(false, false);
+  const at::Tensor *ws = a.buffer(), *y = a.buffer();
   if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
   const Workspace k(ws);
   const auto fn = prepared ? msd_gemm_w4a16_prepared : msd_gemm_w4a16;
@@ -154,7 +157,7 @@ PyObject* grouped_gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   Args t(args, 3), u(args + 4, 2);
   const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
   if (!dims(t, {{x, 2}, {w, 3}})) return nullptr;
-  const at::Tensor *ws = u.tensor(false, false), *y = u.tensor(false, false);
+  const at::Tensor *ws = u.buffer(), *y = u.buffer();
   std::vector<int32_t> sizes;
   if (!u.ok() || !group_sizes(u, args[3], w->size(0), x->size(0), sizes)) return nullptr;
   if (x->size(1) != w->size(2)) return PyErr_Format(PyExc_AssertionError, "x and w differ in K");
@@ -170,7 +173,7 @@ PyObject* grouped_gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
   if (!dims(t, {{x, 2}, {w, 3}})) return nullptr;
   const bool prepared = u.integer() != 0;
-  const at::Tensor *ws = u.tensor(false, false), *y = u.tensor(false, false);
+  const at::Tensor *ws = u.buffer(), *y = u.buffer();
   std::vector<int32_t> sizes;
   if (!u.ok() || !group_sizes(u, args[3], w->size(0), x->size(0), sizes)) return nullptr;
   if (x->size(1) != 2 * w->size(2)) return PyErr_Format(PyExc_AssertionError, "x and w_fp4 differ in K");
@@ -189,7 +192,7 @@ PyObject* attn_decode(PyObject* const* args, Py_ssize_t n) {
   const int32_t max_seqlen = static_cast<int32_t>(a.integer());
   const float scale = static_cast<float>(a.number());
   const int32_t Dv = static_cast<int32_t>(a.integer());
-  const at::Tensor *ws = a.tensor(false, false), *out = a.tensor(false, false), *lse = a.tensor(true, false);
+  const at::Tensor *ws = a.buffer(), *out = a.buffer(), *lse = a.buffer(true);
   constexpr int rank = spec ? 4 : 3;
   if (!dims(a, {{q, rank}, {k, 3}})) return nullptr;
   const Workspace w(ws);
@@ -212,7 +215,7 @@ PyObject* attn_decode_int8kv_paged(PyObject* const* args, Py_ssize_t n) {
   const int32_t page = static_cast<int32_t>(a.integer()), max_seqlen = static_cast<int32_t>(a.integer());
   const float scale = static_cast<float>(a.number());
   const int32_t Dv = static_cast<int32_t>(a.integer());
-  const at::Tensor *ws = a.tensor(false, false), *out = a.tensor(false, false), *lse = a.tensor(true, false);
+  const at::Tensor *ws = a.buffer(), *out = a.buffer(), *lse = a.buffer(true);
   if (!dims(a, {{q, 3}, {k, 3}, {table, 2}})) return nullptr;
   if (page < 1) return PyErr_Format(PyExc_ValueError, "page_size must be positive");
   const Workspace w(ws);

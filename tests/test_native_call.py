@@ -1,9 +1,13 @@
-"""The call module's behaviour at its edges, on a host without a GPU: each case runs in a child process, since what is tested
-would otherwise take the test process down."""
+"""The call module's behaviour at its edges.  What could take the test process down runs in a child process."""
 import os
 import subprocess
 import sys
 import textwrap
+
+import pytest
+import torch
+
+from paper_2605_13915_b200 import binding
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -15,7 +19,8 @@ def _child(code):
 
 
 def test_exceptions_of_the_tensor_library_become_python_exceptions():
-    """Tensors whose storage or layout cannot be asked for raise; an exception that left the C++ code would end the process."""
+    """An exception of the tensor library (here from asking for a stream without a driver, or for the address of a tensor without
+    storage) is raised in Python; one that left the C++ code would end the process."""
     out = _child("""
         import torch
         from torch._subclasses.fake_tensor import FakeTensorMode
@@ -35,8 +40,47 @@ def test_exceptions_of_the_tensor_library_become_python_exceptions():
                                ("attn_decode_int8kv_spec", (q[None], k, k, ks, ks, cu, 8, 0.1, 64, ws, q[None], None)),
                                ("attn_decode_int8kv_paged", (q, k, k, ks, ks, cu[None], cu, 8, 8, 0.1, 64, ws, q, None))):
                 try:
-                    getattr(calls, name)(*args)
+                    print("refused" if getattr(calls, name)(*args) != binding.MSD_OK else "launched", name)
                 except RuntimeError as e:
                     print("raised", name)
         """)
-    assert out.count("raised") == 7
+    # (with a driver a fake tensor's address is null, which the library refuses; without one, asking for the stream throws)
+    assert out.count("raised") + out.count("refused") == 7 and "launched" not in out
+
+
+def test_workspace_that_ends_before_its_first_boundary_is_empty():
+    """The wrappers that go through ctypes: what lies before the first 1024-byte boundary is no workspace, and none is left of a
+    tensor that ends there (the difference, as an unsigned size, would pass for any amount)."""
+    buf = torch.zeros(4096, dtype=torch.uint8)
+    off = -buf.data_ptr() % 1024
+    assert binding._ws_ptr(buf[off + 1:off + 2])[1] == 0
+    assert binding._ws_ptr(buf[off:off + 2048])[1] == 2048
+    assert binding._ws_ptr(buf[off:off + 2048].view(torch.int32))[1] == 2048      # bytes, whatever the elements
+    assert binding._ws_ptr(buf[off + 1000:off + 2048])[1] == 1024
+
+
+@pytest.mark.gpu
+def test_workspace_and_outputs_are_checked():
+    """Workspaces that are too small are refused however they lie; outputs and workspaces that the kernels cannot write are refused
+    before a launch."""
+    dev = "cuda"
+    x, w, s = torch.ones(16, 64, dtype=torch.bfloat16, device=dev), torch.ones(64, 64, dtype=torch.int8, device=dev), torch.ones(64, device=dev)
+    y = torch.empty(16, 64, dtype=torch.bfloat16, device=dev)
+    need = binding.gemm_w8a16_workspace_bytes(16, 64, 64)
+    buf = torch.zeros(need + 4096, dtype=torch.uint8, device=dev)
+    off = -buf.data_ptr() % 1024
+    for ws in (buf[off + 1:off + 2], buf[off + 1:off + 2 + need], buf[off:off + need - 1]):
+        with pytest.raises(binding.MsdError) as e:
+            binding.gemm_w8a16(x, w, s, ws=ws, out=y)
+        assert e.value.code == 5                                     # MSD_ERR_WORKSPACE_TOO_SMALL
+    good = buf[off:off + need]
+    assert torch.equal(binding.gemm_w8a16(x, w, s, ws=good, out=y), torch.full_like(y, 64.0))
+    wide = torch.empty(16, 128, dtype=torch.bfloat16, device=dev)
+    for bad in (dict(ws=good, out=y.cpu()), dict(ws=good.cpu(), out=y), dict(ws=good, out=wide[:, :64]), dict(ws=good, out=y.T)):
+        with pytest.raises(ValueError):
+            binding.gemm_w8a16(x, w, s, **bad)
+    for bad in (y.to_sparse(), torch.empty(16, 64, dtype=torch.bfloat16, device="meta")):
+        with pytest.raises((RuntimeError, ValueError)):
+            binding.gemm_w8a16(x, w, s, ws=good, out=bad)
+    torch.cuda.synchronize()
+    binding.last_device_status()
