@@ -2058,20 +2058,24 @@ static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* b
   return kernel;
 }
 
-// Raises the dynamic shared-memory limit once per kernel instantiation.
+// Raises the dynamic shared-memory limit once per kernel instantiation and device.
 static bool prepare_attn_kernel(AttnKernel kernel) {
+  struct Entry { void* kernel; DeviceOnce once; };
   static std::mutex mu;
-  static void* done[32] = {};
-  std::lock_guard<std::mutex> lock(mu);
-  int free_slot = -1;
-  for (int i = 0; i < 32; ++i) {
-    if (done[i] == reinterpret_cast<void*>(kernel)) return true;
-    if (!done[i] && free_slot < 0) free_slot = i;
+  static Entry entries[32];
+  Entry* e = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (Entry& i : entries) {
+      if (!i.kernel) i.kernel = reinterpret_cast<void*>(kernel);
+      if (i.kernel == reinterpret_cast<void*>(kernel)) { e = &i; break; }
+    }
   }
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess) return false;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) return false;
-  if (free_slot >= 0) done[free_slot] = reinterpret_cast<void*>(kernel);
-  return true;
+  const auto set_up = [&] {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+           cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+  };
+  return e ? e->once(set_up) : set_up();
 }
 
 // Grid of the balanced schedule: as many CTAs as are resident at once, rounded down to whole sets of U (one CTA per

@@ -221,11 +221,8 @@ msd_status_t launch_decompose_mxfp4(const void* x_bf16, int64_t M, int64_t K, in
   const int64_t want = (nblocks + kMxThreads - 1) / kMxThreads;
   const int64_t cap = static_cast<int64_t>(sm_count()) * per_sm;
   const unsigned grid = static_cast<unsigned>(want < cap ? want : cap) + static_cast<unsigned>(rl.blocks);
-  static bool carve_done = false;
-  if (!carve_done) {
-    cudaFuncSetAttribute(decompose_mxfp4_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    carve_done = true;
-  }
+  static DeviceOnce once;
+  once([] { return cudaFuncSetAttribute(decompose_mxfp4_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess; });
   const cudaError_t err = launch_pdl(decompose_mxfp4_kernel, dim3(grid), dim3(kMxThreads), 0, stream, option(OPT_NO_PDL) <= 0,
                                      static_cast<const uint16_t*>(x_bf16), ldx, M, static_cast<int>(K), q1, q2, e1, e2, sf_kgroups, rl, rg);
   return err == cudaSuccess ? MSD_OK : MSD_ERR_CUDA;

@@ -846,15 +846,18 @@ static int w4_resident_clusters(int tile_n, int S) {
   static std::mutex mu;
   static Entry cache[32];
   static int used = 0;
+  static DeviceOnce once;
+  if (!once([] {
+        for (const int w : {128, 224, 256})
+          if (cudaFuncSetAttribute(w4_cluster_kernel(w), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess) return false;
+        return true;
+      }))
+    return 0;
   std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < used; ++i)
     if (cache[i].tile_n == tile_n && cache[i].S == S) return cache[i].n;
   const W4Kernel kernel = w4_cluster_kernel(tile_n);
   int n = 0;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(S) * 64);
   cfg.blockDim = dim3(kW4ThreadsSf);
@@ -866,7 +869,7 @@ static int w4_resident_clusters(int tile_n, int S) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
   if (used < 32) cache[used++] = Entry{tile_n, S, n};
   return n;
 }
@@ -1146,13 +1149,12 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
                         CU_TENSOR_MAP_SWIZZLE_128B))
       return MSD_ERR_CUDA;
     const size_t smem_pair = static_cast<size_t>(kW4PairStages) * (2 * kW4ABytes + (pl.tile_n / 2) * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
-    static bool attr_pair_done = false;
-    if (!attr_pair_done) {
-      if (cudaFuncSetAttribute(gemm_w4a16_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess ||
-          cudaFuncSetAttribute(gemm_w4a16_pair_kernel<224>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess)
-        return MSD_ERR_CUDA;
-      attr_pair_done = true;
-    }
+    static DeviceOnce once;
+    if (!once([] {
+          return cudaFuncSetAttribute(gemm_w4a16_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+                 cudaFuncSetAttribute(gemm_w4a16_pair_kernel<224>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
+        }))
+      return MSD_ERR_CUDA;
     const int pair_tiles = ((pl.m_tiles + 1) / 2) * pl.n_tiles;
     int clusters = sm_count() / 2;
     if (clusters > pair_tiles) clusters = pair_tiles;
@@ -1175,13 +1177,12 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
     return MSD_OK;
   }
   const size_t smem_bytes = static_cast<size_t>(pl.nstages) * (2 * pl.a_rows * 128 + pl.tile_n * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(gemm_w4a16_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w4a16_kernel<224, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess)
-      return MSD_ERR_CUDA;
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  if (!once([] {
+        return cudaFuncSetAttribute(gemm_w4a16_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w4a16_kernel<224, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
+      }))
+    return MSD_ERR_CUDA;
   const cudaError_t le = pl.tile_n == 256
       ? launch_pdl(gemm_w4a16_kernel<256, false>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, GemmW4NoGroups())
       : launch_pdl(gemm_w4a16_kernel<224, false>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, GemmW4NoGroups());
@@ -1263,13 +1264,12 @@ static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w
   int nstages = static_cast<int>((227 * 1024 - 2048 - 8 * kW4StoreBytes - 1024) / stage_bytes);
   if (nstages > 8) nstages = 8;
   const size_t smem_bytes = nstages * stage_bytes + 8 * kW4StoreBytes + 1024;
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(gemm_w4a16_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w4a16_kernel<224, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess)
-      return MSD_ERR_CUDA;
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  if (!once([] {
+        return cudaFuncSetAttribute(gemm_w4a16_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w4a16_kernel<224, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
+      }))
+    return MSD_ERR_CUDA;
   const bool pdl = option(OPT_NO_PDL) <= 0;
 
   // up to 64 non-empty groups per pair of launches (decomposition + GEMM); the weight scales of all experts are brought

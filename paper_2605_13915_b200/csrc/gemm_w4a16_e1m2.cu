@@ -442,12 +442,9 @@ msd_status_t msd_gemm_w4a16_e1m2(const void* x_bf16, const uint8_t* w_fp4, const
                       static_cast<uint64_t>(M), static_cast<uint64_t>(N) * (ybf ? 2 : 4), ybf ? 32 : 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
     return MSD_ERR_CUDA;
   const size_t smem_bytes = static_cast<size_t>(kE1Stages) * kE1StageBytes + 8 * kE1StoreBytes + 1024;
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(gemm_w4a16_e1m2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes)) != cudaSuccess)
-      return MSD_ERR_CUDA;
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  if (!once([=] { return cudaFuncSetAttribute(gemm_w4a16_e1m2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes)) == cudaSuccess; }))
+    return MSD_ERR_CUDA;
   const bool pdl = option(OPT_NO_PDL) <= 0;
   if (launch_pdl(gemm_w4a16_e1m2_kernel, dim3(pl.grid), dim3(kE1Threads), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p) != cudaSuccess)
     return MSD_ERR_CUDA;

@@ -781,27 +781,23 @@ static GemmW8Plan plan_w8(int64_t M, int64_t N, int64_t K, bool base = false) {
 }
 
 static bool ensure_smem_attr() {
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(gemm_w8a16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a16_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess)
-    {
-      cudaGetLastError();
-      return false;
-    }
-    attr_done = true;
-  }
-  return true;
+  static DeviceOnce once;
+  return once([] {
+    return cudaFuncSetAttribute(gemm_w8a16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_w8a16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_w8a16_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
+  });
 }
 
 static int max_resident_clusters(bool base, int S, size_t smem_bytes) {
   struct Entry { bool base; int S; size_t smem; int n; };
+  static std::mutex mu;
   static Entry cache[32];
   static int used = 0;
+  if (!ensure_smem_attr()) return 0;
+  std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < used; ++i)
     if (cache[i].base == base && cache[i].S == S && cache[i].smem == smem_bytes) return cache[i].n;
-  if (!ensure_smem_attr()) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(S) * 64);
   cfg.blockDim = dim3(kGemmThreads);
@@ -816,7 +812,7 @@ static int max_resident_clusters(bool base, int S, size_t smem_bytes) {
   int n = 0;
   const cudaError_t e = base ? cudaOccupancyMaxActiveClusters(&n, gemm_w8a16_kernel<true>, &cfg)
                              : cudaOccupancyMaxActiveClusters(&n, gemm_w8a16_kernel<false>, &cfg);
-  if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
+  if (e != cudaSuccess) { cudaGetLastError(); return 0; }
   if (used < 32) cache[used++] = Entry{base, S, smem_bytes, n};
   return n;
 }

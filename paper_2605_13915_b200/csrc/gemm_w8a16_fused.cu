@@ -290,12 +290,9 @@ msd_status_t msd_gemm_w8a16_fused_dequant(const void* x_bf16, const int8_t* w, c
   p.band_h = pl.band_h; p.bands = pl.bands; p.ksplit = pl.ksplit; p.kper = pl.kper; p.kstages = pl.kstages; p.kw = pl.kw;
   p.stages = pl.stages; p.ytype = ytype; p.w_scale = w_scale; p.y = y;
   p.part = static_cast<float*>(workspace); p.status = status;
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(gemm_w8a16_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) != cudaSuccess)
-      return MSD_ERR_CUDA;
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  if (!once([] { return cudaFuncSetAttribute(gemm_w8a16_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess; }))
+    return MSD_ERR_CUDA;
   gemm_w8a16_fused_kernel<<<static_cast<unsigned>(pl.bands * pl.ksplit), kFzThreads, pl.smem_bytes, s>>>(tmap_w, tmap_x, p);
   if (cudaGetLastError() != cudaSuccess) return MSD_ERR_CUDA;
   if (pl.ksplit > 1)

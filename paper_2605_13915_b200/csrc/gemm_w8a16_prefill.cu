@@ -558,15 +558,14 @@ static msd_status_t p8_launch(bool base, const void* x_bf16, const int8_t* w, co
   }
   const size_t smem_bytes = static_cast<size_t>(kP8Stages) * kP8StageBytes + 16 * kP8StoreBytes + 1024;
   const size_t smem_pair = static_cast<size_t>(kP8PairStages) * kP8PairStageBytes + 16 * kP8StoreBytes + 1024;
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes)) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_pair)) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes)) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_pair)) != cudaSuccess)
-      return MSD_ERR_CUDA;
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  if (!once([=] {
+        return cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes)) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_pair)) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes)) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w8a16_prefill_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_pair)) == cudaSuccess;
+      }))
+    return MSD_ERR_CUDA;
   const bool pdl = option(OPT_NO_PDL) <= 0;
   const long long units = use_pair ? sm_count() / 2 : sm_count();
   const long long tiles = static_cast<long long>(use_pair ? (pl.m_tiles + 1) / 2 : pl.m_tiles) * pl.n_tiles;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "msd.h"
 
 namespace msd {
@@ -39,6 +41,29 @@ bool encode_tmap_2d(CUtensorMap* out, CUtensorMapDataType dtype, const void* bas
 bool encode_tmap_3d(CUtensorMap* out, CUtensorMapDataType dtype, const void* base, uint64_t d0, uint64_t d1, uint64_t d2,
                     uint64_t stride1_bytes, uint64_t stride2_bytes, uint32_t b0, uint32_t b1, uint32_t b2,
                     CUtensorMapSwizzle swizzle);
+
+// Set-up that a kernel needs once on every device (attributes of functions belong to a device's context).  Calls may come from
+// several threads at once: then it may run more than once, which does no harm.  Returns false when it failed; it is then tried
+// again by the next call.
+class DeviceOnce {
+ public:
+  template <typename F>
+  bool operator()(F&& set_up) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    const uint64_t bit = uint64_t{1} << dev;
+    if (done_.load(std::memory_order_acquire) & bit) return true;
+    if (!set_up()) {
+      cudaGetLastError();
+      return false;
+    }
+    done_.fetch_or(bit, std::memory_order_release);
+    return true;
+  }
+
+ private:
+  std::atomic<uint64_t> done_{0};
+};
 
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }

@@ -94,7 +94,16 @@ struct Workspace {
   }
 };
 
-PyObject* status(msd_status_t s) { return PyLong_FromLong(static_cast<long>(s)); }
+// Calls into the library without the interpreter's lock: a launch waits where the stream's queue is full, and what is ahead in
+// the queue may need a Python thread to go on.  Everything the call needs has been read off the arguments by then (the
+// caller's frame keeps the tensors).
+template <typename Call>
+PyObject* status_of(const Call& call) {
+  PyThreadState* lock = PyEval_SaveThread();
+  const msd_status_t s = call();
+  PyEval_RestoreThread(lock);
+  return PyLong_FromLong(static_cast<long>(s));
+}
 
 bool dims(Args& a, std::initializer_list<std::pair<const at::Tensor*, int>> want) {
   if (!a.ok()) return false;
@@ -114,8 +123,13 @@ PyObject* gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   const int64_t scaling = a.integer();
   if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
   const Workspace k(ws);
-  return status(msd_gemm_w8a16_ex(addr(x), addr_as<int8_t>(w), addr_as<float>(s), x->size(0), w->size(0), x->size(1), addr(y), out_type(y),
-                                  addr_as<int32_t>(acc), static_cast<msd_scaling_t>(scaling), k.p, k.bytes, stream()));
+  const int64_t M = x->size(0), N = w->size(0), K = x->size(1);
+  void *xp = addr(x), *yp = addr(y), *st = stream();
+  const auto *wp = addr_as<int8_t>(w);
+  const auto *sp = addr_as<float>(s);
+  auto *ap = addr_as<int32_t>(acc);
+  const msd_out_t yt = out_type(y);
+  return status_of([&] { return msd_gemm_w8a16_ex(xp, wp, sp, M, N, K, yp, yt, ap, static_cast<msd_scaling_t>(scaling), k.p, k.bytes, st); });
 }
 
 // (x, w_fp4, scales, prepared, ws, y)
@@ -127,8 +141,11 @@ PyObject* gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
   const Workspace k(ws);
   const auto fn = prepared ? msd_gemm_w4a16_prepared : msd_gemm_w4a16;
-  return status(fn(addr(x), addr_as<uint8_t>(w), addr_as<uint8_t>(s), x->size(0), w->size(0), x->size(1), addr(y), out_type(y), k.p, k.bytes,
-                   stream()));
+  const int64_t M = x->size(0), N = w->size(0), K = x->size(1);
+  void *xp = addr(x), *yp = addr(y), *st = stream();
+  const auto *wp = addr_as<uint8_t>(w), *sp = addr_as<uint8_t>(s);
+  const msd_out_t yt = out_type(y);
+  return status_of([&] { return fn(xp, wp, sp, M, N, K, yp, yt, k.p, k.bytes, st); });
 }
 
 // Rows per expert from a Python sequence; their sum must be the number of rows of x.
@@ -162,8 +179,13 @@ PyObject* grouped_gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   if (!u.ok() || !group_sizes(u, args[3], w->size(0), x->size(0), sizes)) return nullptr;
   if (x->size(1) != w->size(2)) return PyErr_Format(PyExc_AssertionError, "x and w differ in K");
   const Workspace k(ws);
-  return status(msd_grouped_gemm_w8a16(addr(x), addr_as<int8_t>(w), addr_as<float>(s), sizes.data(), static_cast<int32_t>(w->size(0)),
-                                       w->size(1), w->size(2), addr(y), out_type(y), k.p, k.bytes, stream()));
+  const int32_t E = static_cast<int32_t>(w->size(0));
+  const int64_t N = w->size(1), K = w->size(2);
+  void *xp = addr(x), *yp = addr(y), *st = stream();
+  const auto *wp = addr_as<int8_t>(w);
+  const auto *sp = addr_as<float>(s);
+  const msd_out_t yt = out_type(y);
+  return status_of([&] { return msd_grouped_gemm_w8a16(xp, wp, sp, sizes.data(), E, N, K, yp, yt, k.p, k.bytes, st); });
 }
 
 // (x, w_fp4, scales, group_sizes, prepared, ws, y)
@@ -179,8 +201,12 @@ PyObject* grouped_gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   if (x->size(1) != 2 * w->size(2)) return PyErr_Format(PyExc_AssertionError, "x and w_fp4 differ in K");
   const Workspace k(ws);
   const auto fn = prepared ? msd_grouped_gemm_w4a16_prepared : msd_grouped_gemm_w4a16;
-  return status(fn(addr(x), addr_as<uint8_t>(w), addr_as<uint8_t>(s), sizes.data(), static_cast<int32_t>(w->size(0)), w->size(1),
-                   2 * w->size(2), addr(y), out_type(y), k.p, k.bytes, stream()));
+  const int32_t E = static_cast<int32_t>(w->size(0));
+  const int64_t N = w->size(1), K = 2 * w->size(2);
+  void *xp = addr(x), *yp = addr(y), *st = stream();
+  const auto *wp = addr_as<uint8_t>(w), *sp = addr_as<uint8_t>(s);
+  const msd_out_t yt = out_type(y);
+  return status_of([&] { return fn(xp, wp, sp, sizes.data(), E, N, K, yp, yt, k.p, k.bytes, st); });
 }
 
 // (q, k, v or None, k_scale, v_scale or None, cu_seqlens, max_seqlen, softmax_scale, Dv, ws, out, lse or None);
@@ -197,14 +223,19 @@ PyObject* attn_decode(PyObject* const* args, Py_ssize_t n) {
   if (!dims(a, {{q, rank}, {k, 3}})) return nullptr;
   const Workspace w(ws);
   const int32_t B = static_cast<int32_t>(q->size(0)), Hq = static_cast<int32_t>(q->size(rank - 2)), D = static_cast<int32_t>(q->size(rank - 1));
-  const int32_t Hkv = static_cast<int32_t>(k->size(1));
-  if constexpr (!spec)
-    return status(msd_attn_decode_int8kv(addr(q), addr_as<int8_t>(k), addr_as<int8_t>(v), addr_as<float>(ks), addr_as<float>(vs),
-                                         addr_as<int32_t>(cu), k->size(0), max_seqlen, B, Hq, Hkv, D, Dv, scale, addr(out),
-                                         addr_as<float>(lse), w.p, w.bytes, stream()));
-  return status(msd_attn_decode_int8kv_spec(addr(q), addr_as<int8_t>(k), addr_as<int8_t>(v), addr_as<float>(ks), addr_as<float>(vs),
-                                            addr_as<int32_t>(cu), k->size(0), max_seqlen, B, static_cast<int32_t>(q->size(1)), Hq, Hkv, D,
-                                            Dv, scale, addr(out), addr_as<float>(lse), w.p, w.bytes, stream()));
+  const int32_t Hkv = static_cast<int32_t>(k->size(1)), q_len = spec ? static_cast<int32_t>(q->size(1)) : 1;
+  const int64_t T = k->size(0);
+  void *qp = addr(q), *op = addr(out), *st = stream();
+  const auto *kp = addr_as<int8_t>(k), *vp = addr_as<int8_t>(v);
+  const auto *ksp = addr_as<float>(ks), *vsp = addr_as<float>(vs);
+  const auto *cup = addr_as<int32_t>(cu);
+  auto *lp = addr_as<float>(lse);
+  return status_of([&] {
+    if constexpr (spec)
+      return msd_attn_decode_int8kv_spec(qp, kp, vp, ksp, vsp, cup, T, max_seqlen, B, q_len, Hq, Hkv, D, Dv, scale, op, lp, w.p, w.bytes, st);
+    else
+      return msd_attn_decode_int8kv(qp, kp, vp, ksp, vsp, cup, T, max_seqlen, B, Hq, Hkv, D, Dv, scale, op, lp, w.p, w.bytes, st);
+  });
 }
 
 // (q, k, v or None, k_scale, v_scale or None, block_table, seqlens, page_size, max_seqlen, softmax_scale, Dv, ws, out, lse or None)
@@ -219,11 +250,18 @@ PyObject* attn_decode_int8kv_paged(PyObject* const* args, Py_ssize_t n) {
   if (!dims(a, {{q, 3}, {k, 3}, {table, 2}})) return nullptr;
   if (page < 1) return PyErr_Format(PyExc_ValueError, "page_size must be positive");
   const Workspace w(ws);
-  return status(msd_attn_decode_int8kv_paged(
-      addr(q), addr_as<int8_t>(k), addr_as<int8_t>(v), addr_as<float>(ks), addr_as<float>(vs), addr_as<int32_t>(table), addr_as<int32_t>(len),
-      k->size(0) / page, page, static_cast<int32_t>(table->size(1)), max_seqlen, static_cast<int32_t>(q->size(0)),
-      static_cast<int32_t>(q->size(1)), static_cast<int32_t>(k->size(1)), static_cast<int32_t>(q->size(2)), Dv, scale, addr(out),
-      addr_as<float>(lse), w.p, w.bytes, stream()));
+  const int32_t B = static_cast<int32_t>(q->size(0)), Hq = static_cast<int32_t>(q->size(1)), D = static_cast<int32_t>(q->size(2));
+  const int32_t Hkv = static_cast<int32_t>(k->size(1)), max_blocks = static_cast<int32_t>(table->size(1));
+  const int64_t blocks = k->size(0) / page;
+  void *qp = addr(q), *op = addr(out), *st = stream();
+  const auto *kp = addr_as<int8_t>(k), *vp = addr_as<int8_t>(v);
+  const auto *ksp = addr_as<float>(ks), *vsp = addr_as<float>(vs);
+  const auto *tp = addr_as<int32_t>(table), *np = addr_as<int32_t>(len);
+  auto *lp = addr_as<float>(lse);
+  return status_of([&] {
+    return msd_attn_decode_int8kv_paged(qp, kp, vp, ksp, vsp, tp, np, blocks, page, max_blocks, max_seqlen, B, Hq, Hkv, D, Dv, scale, op, lp,
+                                        w.p, w.bytes, st);
+  });
 }
 
 // What the interpreter calls: C++ exceptions (a tensor without storage or with another layout, no memory) become Python's.

@@ -84,3 +84,35 @@ def test_workspace_and_outputs_are_checked():
             binding.gemm_w8a16(x, w, s, ws=good, out=bad)
     torch.cuda.synchronize()
     binding.last_device_status()
+
+
+@pytest.mark.gpu
+def test_other_python_threads_run_during_a_call(tmp_path):
+    """A launch waits where the stream's queue is full; the interpreter's other threads must not wait with it.  A stand-in for the
+    library's function that sleeps takes its place in the child, so that nothing is launched."""
+    (tmp_path / "slow.c").write_text("#include <unistd.h>\nint msd_gemm_w8a16_ex() { usleep(1500000); return 0; }\n")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(tmp_path / "slow.so"), str(tmp_path / "slow.c")], check=True)
+    out = _child(f"""
+        import ctypes, threading, time
+        ctypes.CDLL({str(tmp_path / "slow.so")!r}, mode=ctypes.RTLD_GLOBAL)
+        import torch
+        from paper_2605_13915_b200 import binding
+        calls = binding._calls()
+        t = lambda *s, dtype=torch.int8: torch.zeros(*s, dtype=dtype, device="cuda")
+        args = (t(16, 64, dtype=torch.bfloat16), t(32, 64), t(32, dtype=torch.float32), t(4096), t(16, 32, dtype=torch.bfloat16), None, 0)
+        torch.cuda.synchronize()
+        spent = []
+        def call():
+            t0 = time.monotonic()
+            calls.gemm_w8a16(*args)
+            spent.append(time.monotonic() - t0)
+        thread = threading.Thread(target=call)
+        t0 = time.monotonic()
+        thread.start()
+        time.sleep(0.2)
+        print("others", time.monotonic() - t0)
+        thread.join()
+        print("call", spent[0])
+        """)
+    took = dict(line.split() for line in out.splitlines())
+    assert float(took["call"]) >= 1.4 and float(took["others"]) < 1.0
