@@ -105,23 +105,24 @@ PyObject* status_of(const Call& call) {
   return PyLong_FromLong(static_cast<long>(s));
 }
 
+// (-n: at least n; the sizes past them are not asked for)
 bool dims(Args& a, std::initializer_list<std::pair<const at::Tensor*, int>> want) {
   if (!a.ok()) return false;
   for (const auto& w : want)
-    if (w.first->dim() != w.second) {
+    if (w.second < 0 ? w.first->dim() < -w.second : w.first->dim() != w.second) {
       a.fail(PyExc_ValueError, "a tensor has the wrong number of dimensions");
       return false;
     }
   return true;
 }
 
-// (x, w, w_scale, ws, y, acc or None, scaling)
+// (x, w, w_scale, ws, y, acc or None, scaling); None for a pointer that the library requires is passed on, and refused there
 PyObject* gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
-  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(), *ws = a.buffer(), *y = a.buffer(),
+  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(true), *ws = a.buffer(), *y = a.buffer(),
                    *acc = a.buffer(true);
   const int64_t scaling = a.integer();
-  if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
+  if (!dims(a, {{x, 2}, {w, -1}})) return nullptr;
   const Workspace k(ws);
   const int64_t M = x->size(0), N = w->size(0), K = x->size(1);
   void *xp = addr(x), *yp = addr(y), *st = stream();
@@ -135,10 +136,10 @@ PyObject* gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
 // (x, w_fp4, scales, prepared, ws, y)
 PyObject* gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
-  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor();
+  const at::Tensor *x = a.tensor(), *w = a.tensor(), *s = a.tensor(true);
   const bool prepared = a.integer() != 0;
   const at::Tensor *ws = a.buffer(), *y = a.buffer();
-  if (!dims(a, {{x, 2}, {w, 2}})) return nullptr;
+  if (!dims(a, {{x, 2}, {w, -1}})) return nullptr;
   const Workspace k(ws);
   const auto fn = prepared ? msd_gemm_w4a16_prepared : msd_gemm_w4a16;
   const int64_t M = x->size(0), N = w->size(0), K = x->size(1);
@@ -156,7 +157,14 @@ bool group_sizes(Args& a, PyObject* seq, int64_t E, int64_t rows, std::vector<in
   const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast.get());
   out.reserve(static_cast<size_t>(E));
   for (Py_ssize_t i = 0; i < n; ++i) {
-    const long v = PyLong_AsLong(PySequence_Fast_GET_ITEM(fast.get(), i));
+    PyObject* item = PySequence_Fast_GET_ITEM(fast.get(), i);
+    THPObjectPtr as_int;
+    if (!PyLong_Check(item)) {                   // whatever int() takes
+      as_int = PyNumber_Long(item);
+      if (!as_int) return false;
+      item = as_int.get();
+    }
+    const long v = PyLong_AsLong(item);
     if (v == -1 && PyErr_Occurred()) return false;
     out.push_back(static_cast<int32_t>(v));
     sum += v;
@@ -172,7 +180,7 @@ bool group_sizes(Args& a, PyObject* seq, int64_t E, int64_t rows, std::vector<in
 PyObject* grouped_gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
   if (n != 6) return PyErr_Format(PyExc_TypeError, "expected 6 arguments");
   Args t(args, 3), u(args + 4, 2);
-  const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
+  const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor(true);
   if (!dims(t, {{x, 2}, {w, 3}})) return nullptr;
   const at::Tensor *ws = u.buffer(), *y = u.buffer();
   std::vector<int32_t> sizes;
@@ -192,7 +200,7 @@ PyObject* grouped_gemm_w8a16(PyObject* const* args, Py_ssize_t n) {
 PyObject* grouped_gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
   if (n != 7) return PyErr_Format(PyExc_TypeError, "expected 7 arguments");
   Args t(args, 3), u(args + 4, 3);
-  const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor();
+  const at::Tensor *x = t.tensor(), *w = t.tensor(), *s = t.tensor(true);
   if (!dims(t, {{x, 2}, {w, 3}})) return nullptr;
   const bool prepared = u.integer() != 0;
   const at::Tensor *ws = u.buffer(), *y = u.buffer();
@@ -214,13 +222,13 @@ PyObject* grouped_gemm_w4a16(PyObject* const* args, Py_ssize_t n) {
 template <bool spec>
 PyObject* attn_decode(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
-  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(), *vs = a.tensor(true), *cu = a.tensor();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(true), *vs = a.tensor(true), *cu = a.tensor(true);
   const int32_t max_seqlen = static_cast<int32_t>(a.integer());
   const float scale = static_cast<float>(a.number());
   const int32_t Dv = static_cast<int32_t>(a.integer());
   const at::Tensor *ws = a.buffer(), *out = a.buffer(), *lse = a.buffer(true);
   constexpr int rank = spec ? 4 : 3;
-  if (!dims(a, {{q, rank}, {k, 3}})) return nullptr;
+  if (!dims(a, {{q, rank}, {k, -2}})) return nullptr;
   const Workspace w(ws);
   const int32_t B = static_cast<int32_t>(q->size(0)), Hq = static_cast<int32_t>(q->size(rank - 2)), D = static_cast<int32_t>(q->size(rank - 1));
   const int32_t Hkv = static_cast<int32_t>(k->size(1)), q_len = spec ? static_cast<int32_t>(q->size(1)) : 1;
@@ -241,18 +249,17 @@ PyObject* attn_decode(PyObject* const* args, Py_ssize_t n) {
 // (q, k, v or None, k_scale, v_scale or None, block_table, seqlens, page_size, max_seqlen, softmax_scale, Dv, ws, out, lse or None)
 PyObject* attn_decode_int8kv_paged(PyObject* const* args, Py_ssize_t n) {
   Args a(args, n);
-  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(), *vs = a.tensor(true), *table = a.tensor(),
-                   *len = a.tensor();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(true), *ks = a.tensor(true), *vs = a.tensor(true), *table = a.tensor(),
+                   *len = a.tensor(true);
   const int32_t page = static_cast<int32_t>(a.integer()), max_seqlen = static_cast<int32_t>(a.integer());
   const float scale = static_cast<float>(a.number());
   const int32_t Dv = static_cast<int32_t>(a.integer());
   const at::Tensor *ws = a.buffer(), *out = a.buffer(), *lse = a.buffer(true);
-  if (!dims(a, {{q, 3}, {k, 3}, {table, 2}})) return nullptr;
-  if (page < 1) return PyErr_Format(PyExc_ValueError, "page_size must be positive");
+  if (!dims(a, {{q, 3}, {k, -2}, {table, -2}})) return nullptr;
   const Workspace w(ws);
   const int32_t B = static_cast<int32_t>(q->size(0)), Hq = static_cast<int32_t>(q->size(1)), D = static_cast<int32_t>(q->size(2));
   const int32_t Hkv = static_cast<int32_t>(k->size(1)), max_blocks = static_cast<int32_t>(table->size(1));
-  const int64_t blocks = k->size(0) / page;
+  const int64_t blocks = page > 0 ? k->size(0) / page : 0;      // (the library refuses other pages)
   void *qp = addr(q), *op = addr(out), *st = stream();
   const auto *kp = addr_as<int8_t>(k), *vp = addr_as<int8_t>(v);
   const auto *ksp = addr_as<float>(ks), *vsp = addr_as<float>(vs);

@@ -4,6 +4,7 @@ import subprocess
 import sys
 import textwrap
 
+import numpy as np
 import pytest
 import torch
 
@@ -116,3 +117,36 @@ def test_other_python_threads_run_during_a_call(tmp_path):
         """)
     took = dict(line.split() for line in out.splitlines())
     assert float(took["call"]) >= 1.4 and float(took["others"]) < 1.0
+
+
+@pytest.mark.gpu
+def test_argument_forms():
+    """Rows per expert as anything that int() takes; a missing scale or length array is the library's null pointer, a page size it
+    does not know its MSD_ERR_UNSUPPORTED."""
+    dev = "cuda"
+    x, w, s = torch.ones(5, 64, dtype=torch.bfloat16, device=dev), torch.ones(2, 64, 64, dtype=torch.int8, device=dev), torch.ones(2, 64, device=dev)
+    want = torch.full((5, 64), 64.0, dtype=torch.bfloat16, device=dev)
+    for sizes in ([2, 3], (2.0, 3.0), np.array([2, 3]), np.array([2.0, 3.0], np.float32), torch.tensor([2, 3]), torch.tensor([2.0, 3.0]),
+                  ["2", "3"]):
+        assert torch.equal(binding.grouped_gemm_w8a16(x, w, s, sizes), want)
+    with pytest.raises(ValueError):
+        binding.grouped_gemm_w8a16(x, w, s, ["two", 3])
+    with pytest.raises(AssertionError):
+        binding.grouped_gemm_w8a16(x, w, s, [2, 2])
+
+    def code(fn, *args, **kw):
+        with pytest.raises(binding.MsdError) as e:
+            fn(*args, **kw)
+        return e.value.code
+    assert code(binding.gemm_w8a16, x, w[0], None) == 1
+    q, k, ks = torch.ones(1, 4, 64, dtype=torch.bfloat16, device=dev), torch.ones(16, 1, 64, dtype=torch.int8, device=dev), torch.ones(16, 1, device=dev)
+    cu, table, lens = (torch.tensor(v, dtype=torch.int32, device=dev) for v in ([0, 16], [[0, 1]], [16]))
+    assert code(binding.attn_decode_int8kv, q, k, k, None, ks, cu, 16, 0.125) == 1
+    assert code(binding.attn_decode_int8kv, q, k, k, ks, ks, None, 16, 0.125) == 1
+    assert code(binding.attn_decode_int8kv_paged, q, k, k, ks, ks, table, None, 8, 16, 0.125) == 1
+    for page in (-8, 0, 24):
+        assert code(binding.attn_decode_int8kv_paged, q, k, k, ks, ks, table, lens, page, 16, 0.125) == 4
+    split = binding.attn_decode_int8kv(q, k.view(16, 1, 4, 16), k, ks, ks, cu, 16, 0.125)       # rows in pieces: the same bytes
+    assert torch.equal(split, binding.attn_decode_int8kv(q, k, k, ks, ks, cu, 16, 0.125))
+    torch.cuda.synchronize()
+    binding.last_device_status()
