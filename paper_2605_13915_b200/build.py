@@ -35,17 +35,30 @@ def _headers():
 
 
 def needs_build() -> bool:
+    return _lib_stale() or _native_stale()
+
+
+def _lib_stale() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(d) > t for d in sources() + _headers()) or _native_stale()
+    return any(os.path.getmtime(d) > t for d in sources() + _headers())
+
+
+def _native_tag() -> str:
+    """What the call module is built for, and carries as a string: torch's binary interface changes with its version."""
+    import torch
+    return "msd call module for torch %s, python %d.%d" % (torch.__version__, sys.version_info[0], sys.version_info[1])
 
 
 def _native_stale() -> bool:
     if not os.path.exists(NATIVE_PATH):
         return True
     t = os.path.getmtime(NATIVE_PATH)
-    return any(os.path.getmtime(d) > t for d in (NATIVE_SRC, os.path.join(_ROOT, "include", "msd.h")))
+    if any(os.path.getmtime(d) > t for d in (NATIVE_SRC, os.path.join(_ROOT, "include", "msd.h"))):
+        return True
+    with open(NATIVE_PATH, "rb") as f:
+        return _native_tag().encode() + b"\0" not in f.read()
 
 
 def _build_native():
@@ -54,7 +67,7 @@ def _build_native():
     import torch
     troot = os.path.dirname(torch.__file__)
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++20", "-fPIC", "-shared", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), NATIVE_SRC, "-o", NATIVE_PATH,
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), '-DMSD_BUILT_FOR="%s"' % _native_tag(), NATIVE_SRC, "-o", NATIVE_PATH,
            "-I", os.path.join(_ROOT, "include"), "-I", sysconfig.get_paths()["include"],
            "-isystem", os.path.join(troot, "include"), "-isystem", os.path.join(troot, "include", "torch", "csrc", "api", "include"),
            "-isystem", os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include"),
@@ -72,7 +85,9 @@ def _obj(src):
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu under csrc/ and link them into one shared library (nvcc cross-compiles without a GPU)."""
-    if not force and not needs_build():
+    if not force and not _lib_stale():
+        if _native_stale():
+            _build_native()
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ_DIR, exist_ok=True)

@@ -294,4 +294,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 }  // namespace
 
+// (build.py looks for it: a module built for another torch is built again)
+extern "C" __attribute__((used, visibility("default"))) const char msd_call_module_built_for[] = MSD_BUILT_FOR;
+
 PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }

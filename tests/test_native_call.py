@@ -60,6 +60,15 @@ def test_workspace_that_ends_before_its_first_boundary_is_empty():
     assert binding._ws_ptr(buf[off + 1000:off + 2048])[1] == 1024
 
 
+
+def test_module_built_for_another_torch_is_stale(monkeypatch):
+    from paper_2605_13915_b200 import build
+    binding.lib()
+    assert not build.needs_build()
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".post1")
+    assert build.needs_build()
+
+
 @pytest.mark.gpu
 def test_workspace_and_outputs_are_checked():
     """Workspaces that are too small are refused however they lie; outputs and workspaces that the kernels cannot write are refused
