@@ -410,11 +410,13 @@ attn_qstack_kernel(const AttnParams p, uint8_t* __restrict__ q_img, float* __res
   }
 }
 
-// Head groups of up to 8 query rows per KV head (GQA).  kMaxHG: head slots one softmax thread looks after (8; the code
-// also compiles for 16, which the planner no longer picks);
-// kNH: heads its code is unrolled for (<= kMaxHG); kMaxDVT: 128-wide tiles of Dv.
+// Head slots that one softmax thread looks after.
+constexpr int kThreadSlots = 8;
+
+// Head groups of up to 8 query rows per KV head (GQA).  kNH: heads the softmax code is unrolled for (<= 8); kMaxDVT: 128-wide
+// tiles of Dv.
 // kPaged: the cache is paged (block table); a template parameter so that the contiguous kernels carry none of it.
-template <int kMaxHG, int kNH, int kMaxDVT, bool kPaged, int kMode>
+template <int kNH, int kMaxDVT, bool kPaged, int kMode>
 __global__ void __launch_bounds__(kAttnThreads, (kNH <= 8 && kMaxDVT == 1) ? 3 : 1)
 attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v, const AttnParams p) {
   constexpr bool kBalanced = kMode == 1, kDirect = kMode == 2;      // kDirect: one split a sequence, the result written here (p.out)
@@ -424,7 +426,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
   __shared__ int abort_flag;
   // The CTA decomposes its few query rows itself (beside the other CTAs of the SM); wide head groups, where that
   // would be repeated by every context split, take them from attn_qstack_kernel instead (attn_decode_wide_kernel).
-  constexpr int kSlots = kMaxHG;                   // head slots of the stacked operands: rows [0,kSlots) first
+  constexpr int kSlots = kThreadSlots;             // head slots of the stacked operands: rows [0,kSlots) first
   constexpr int kNSW = 4;                          // component, rows [kSlots, 2*kSlots) second component
   __shared__ float s_aq[kSlots], s_bq[kSlots];
   __shared__ float red[2][4][kNH + 1];             // per-warp tile maxima, double buffered by tile parity
@@ -745,7 +747,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
       const int t_end = min(L, t_begin + ntiles * kTok);
       // c1: decompose the query rows of this segment's heads (one warp per head, round robin) into the stacked operand
       // (the head slots and padding columns that were zeroed at the start are never written)
-      if (kNH > 4 && kMaxHG == 8 && p.D <= 128) {
+      if (kNH > 4 && p.D <= 128) {
         // more than four rows of at most 128 values: a warp takes its two rows side by side, 16 lanes each (one after
         // the other the stacked operand was ready 5.4 us after the CTA's start instead of 3.0 us with one row per warp)
         if (wi < nh) attn_decompose_q_pair(p, b, hk, grp, wi, wi + kNSW < nh ? wi + kNSW : -1, lane, sm_q, s_aq, s_bq);
@@ -809,14 +811,14 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         float s[kNH];
         const uint32_t srow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + (gt & 1) * p.Rp;
         {
-          uint32_t v1[kMaxHG], v2[kMaxHG];          // first / second component columns
-          tmem_ldw<kMaxHG>(srow + hs0, v1);
-          tmem_ldw<kMaxHG>(srow + kSlots + hs0, v2);
+          uint32_t v1[kThreadSlots], v2[kThreadSlots];          // first / second component columns
+          tmem_ld8(srow + hs0, v1);
+          tmem_ld8(srow + kSlots + hs0, v2);
           tmem_ld_wait();
           if (p.s_dbg && valid) {
             long long tok_row = seq0 + tok_rel;
             if constexpr (kPaged) tok_row = static_cast<long long>(__ldg(bt + (tok_rel >> p.page_shift))) * p.page + (tok_rel & (p.page - 1));
-            attn_dump_scores<kMaxHG>(p, tok_row, hk, grp, hs0, nh, v1, v2);
+            attn_dump_scores<kThreadSlots>(p, tok_row, hk, grp, hs0, nh, v1, v2);
           }
 #pragma unroll
           for (int h = 0; h < kNH; ++h)
@@ -916,9 +918,9 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         for (int j = 0; j < kMaxDVT; ++j) {
           if (j < p.DVT) {
             const uint32_t orow = tmem_o + (static_cast<uint32_t>(quad * 32) << 16) + j * p.Rp;
-            uint32_t v1[kMaxHG], v2[kMaxHG];
-            tmem_ldw<kMaxHG>(orow + hs0, v1);
-            tmem_ldw<kMaxHG>(orow + kSlots + hs0, v2);
+            uint32_t v1[kThreadSlots], v2[kThreadSlots];
+            tmem_ld8(orow + hs0, v1);
+            tmem_ld8(orow + kSlots + hs0, v2);
             tmem_ld_wait();
 #pragma unroll
             for (int h = 0; h < kNH; ++h)
@@ -1029,23 +1031,16 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 // that fit shared memory for a 576-byte row bound the pipeline, not the latency of L2 misses.)
 constexpr float kHoldMarginLog2 = 3.0f;
 constexpr float kHoldScaleGrowth = 1.25f;
-template <int W> __device__ __forceinline__ void tmem_stw(uint32_t taddr, const uint32_t (&v)[W]) {
-  static_assert(W == 8 || W == 16, "8 or 16 columns per store");
-  if constexpr (W == 8) tmem_st8(taddr, v);
-  else tmem_st16(taddr, v);
-}
-
 
 // kSlots: head slots per CTA (2 kSlots stacked rows).  32 for latent caches and for more than 16 rows per KV head: one CTA
 // per SM, all 512 tensor-memory columns.  16 for 9 to 16 rows at D, Dv <= 128: 128 columns, 78 KB of shared memory and 80
 // registers (the block is bounded as 12 warps: the register file is four banks, one per scheduler, and two CTAs of 11 warps put
 // six on one of them), so two CTAs share an SM and one's softmax runs while the other waits for its products.
-// kWideHS: head slots per softmax thread (8 or 16); the slots are shared out over kSlots / kWideHS groups of
-// four softmax warps.  kFixDC / kFixDVT: the chunk counts of D and Dv when known at compile time (0: taken from the
+// The slots are shared out over kSlots / 8 groups of four softmax warps.  kFixDC / kFixDVT: the chunk counts of D and Dv when known at compile time (0: taken from the
 // plan) - the MMA thread shares its scheduler with four busy softmax warps, so every instruction it spends per MMA on
 // loop control and address arithmetic delays the tensor pipe; with fixed counts its loops unroll to an add per operand.
-template <int kSlots, int kWideHS, bool kPaged, int kFixDC, int kFixDVT>
-__global__ void __launch_bounds__(kSlots == 16 ? 384 : ((kFixDC == 5 && kFixDVT == 4 && !kPaged) ? 64 : 96) + 128 * (kSlots / kWideHS),
+template <int kSlots, bool kPaged, int kFixDC, int kFixDVT>
+__global__ void __launch_bounds__(kSlots == 16 ? 384 : ((kFixDC == 5 && kFixDVT == 4 && !kPaged) ? 64 : 96) + 128 * (kSlots / kThreadSlots),
                                   kSlots == 16 ? 2 : 1)
 attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v, const AttnParams p) {
   extern __shared__ uint8_t smem_dyn[];
@@ -1055,8 +1050,8 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   __shared__ int flush_stamp[2];                    // tile number + 1 of the last tile whose references had to move, per P buffer
   __shared__ float s_aq[kSlots];
   __shared__ int span[2];                           // the split's first and past-the-last token (kept here: the softmax warps have no registers left for them)
-  __shared__ float red[kSlots / kWideHS][4][kWideHS + 1];    // per-warp tile maxima (slow path only)
-  constexpr int kWideWG = kSlots / kWideHS;
+  __shared__ float red[kSlots / kThreadSlots][4][kThreadSlots + 1];    // per-warp tile maxima (slow path only)
+  constexpr int kWideWG = kSlots / kThreadSlots;
   constexpr int kNSW = 4 * kWideWG;
   // Latent cache of 576 bytes per token with V aliased to its first 512 (the launcher picks this instantiation only
   // then): the two KV stages are given back chunk by chunk (five 128-byte-wide chunks of 16 KB): every chunk is
@@ -1382,7 +1377,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     const int wi = warp - 2;                        // 0 .. 15
     const int hh = wi >> 2;                         // which group of head slots this warp looks after
     const int wq = wi & 3;
-    const int hs0 = hh * kWideHS;                   // its first head slot
+    const int hs0 = hh * kThreadSlots;                   // its first head slot
     {
       // alpha_Q of this CTA's heads, computed by attn_qstack_kernel (launched just before this kernel);
       // beta_Q = alpha_Q / 254 is applied as a constant factor
@@ -1400,21 +1395,21 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     // this thread's tokens.  The FP32 running output of this thread's dv lane (4 x 8 values) lives in the tensor-memory
     // columns behind the accumulators: it is touched only by the rare drains, and 32 registers fewer per thread let
     // the compiler keep the eight heads' dependent chains of the per-tile code in flight side by side.
-    float aq[kWideHS], nm[kWideHS], l_part[kWideHS];
+    float aq[kThreadSlots], nm[kThreadSlots], l_part[kThreadSlots];
     const uint32_t orun_row = tmem_o + kDVT * p.Rp + (static_cast<uint32_t>(quad * 32) << 16) + hs0;
 #pragma unroll
-    for (int h = 0; h < kWideHS; ++h) {
+    for (int h = 0; h < kThreadSlots; ++h) {
       const bool present = hs0 + h < nh;
       aq[h] = present ? (kIntCombine ? s_aq[hs0 + h] * (1.0f / 254.0f) : s_aq[hs0 + h]) : 0.0f;
       nm[h] = present ? 1e30f : -1e30f;
       l_part[h] = 0.0f;
     }
     {
-      uint32_t z[kWideHS];
+      uint32_t z[kThreadSlots];
 #pragma unroll
-      for (int h = 0; h < kWideHS; ++h) z[h] = 0u;
+      for (int h = 0; h < kThreadSlots; ++h) z[h] = 0u;
 #pragma unroll
-      for (int j = 0; j < kDVT; ++j) tmem_stw<kWideHS>(orun_row + j * kSlots, z);
+      for (int j = 0; j < kDVT; ++j) tmem_st8(orun_row + j * kSlots, z);
       tmem_st_wait();
     }
     float a_ref = 0.0f, alpha_p = 0.0f, inv_a = 0.0f, inv_b = 0.0f;
@@ -1438,21 +1433,21 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     };
     // c3: scores of this thread's token against its 8 head slots in the log2 domain (-inf where the token is past the
     // end of the split or not visible to the row)
-    auto load_scores = [&](int t, float ks, float (&s)[kWideHS]) {
+    auto load_scores = [&](int t, float ks, float (&s)[kThreadSlots]) {
       const int tok_rel = span[0] + t * kTok + tl;
       const bool valid = tok_rel < span[1];
       const uint32_t srow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + (t & 1) * p.Rp;
-      uint32_t v1[kWideHS], v2[kWideHS];
-      tmem_ldw<kWideHS>(srow + hs0, v1);
-      tmem_ldw<kWideHS>(srow + kSlots + hs0, v2);
+      uint32_t v1[kThreadSlots], v2[kThreadSlots];
+      tmem_ld8(srow + hs0, v1);
+      tmem_ld8(srow + kSlots + hs0, v2);
       tmem_ld_wait();
       if (p.s_dbg && valid) {
         long long tok_row = seq0 + tok_rel;
         if constexpr (kPaged) tok_row = static_cast<long long>(__ldg(bt + (tok_rel >> p.page_shift))) * p.page + (tok_rel & (p.page - 1));
-        attn_dump_scores<kWideHS>(p, tok_row, hk, grp, hs0, nh, v1, v2);
+        attn_dump_scores<kThreadSlots>(p, tok_row, hk, grp, hs0, nh, v1, v2);
       }
 #pragma unroll
-      for (int h = 0; h < kWideHS; ++h) {
+      for (int h = 0; h < kThreadSlots; ++h) {
         // S1 + S2 / 254; with D <= 512 as (254 S1 + S2) / 254 (|254 S1 + S2| <= 255 * 127 * 128 * D < 2^31): one conversion
         // instead of two on a pipe that takes a warp every eighth cycle (the factor is in aq)
         const float tsum = kIntCombine ? static_cast<float>(254 * static_cast<int32_t>(v1[h]) + static_cast<int32_t>(v2[h]))
@@ -1463,21 +1458,21 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       // took 0.8 of 2.5 us a tile when every tile was; as a condition on every score it cost all other calls 3 to 6 %)
       if (p.Sq > 1 && span[0] + (t + 1) * kTok > L - p.Sq + 1) {
 #pragma unroll
-        for (int h = 0; h < kWideHS; ++h)
+        for (int h = 0; h < kThreadSlots; ++h)
           if (tok_rel >= L - p.Sq + 1 + (grp * p.HG + hs0 + h) / p.Gr) s[h] = -INFINITY;
       }
     };
     // c4-c5: P = 2^(s - reference), value scale folded in, two-pass INT8 with the scale in force, into P buffer t&1.
     // Returns the largest s - reference of this thread (> 0: the reference must move).
-    auto write_p = [&](int t, const float (&s)[kWideHS], float vs, float (&pl)[kWideHS]) -> float {
+    auto write_p = [&](int t, const float (&s)[kThreadSlots], float vs, float (&pl)[kThreadSlots]) -> float {
       // this token's row of the P buffer: 64 (32) bytes, the 16-byte pieces XORed with address bits 7 and 8 (bit 7)
       uint8_t* prow = sm_p + (t & 1) * p.Rp * kChunk + tl * kPRow;
       constexpr int kPieces = kPRow / 16;
       const int sw = (tl * kPRow >> 7) & (kPieces - 1);
-      uint32_t c1[kWideHS], c2[kWideHS];
+      uint32_t c1[kThreadSlots], c2[kThreadSlots];
       float xm = -INFINITY;
 #pragma unroll
-      for (int h = 0; h < kWideHS; ++h) {
+      for (int h = 0; h < kThreadSlots; ++h) {
         const float x = s[h] + nm[h];
         xm = fmaxf(xm, x);
         const float pr = ex2_approx(x);
@@ -1490,42 +1485,37 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         c1[h] = __float_as_uint(u1);
         c2[h] = __float_as_uint(u2);
       }
-      // the codes are the low bytes; kWideHS of them make one 8- or 16-byte store per component
-      uint32_t w1[kWideHS / 4], w2[kWideHS / 4];
+      // the codes are the low bytes; eight of them make one store per component
+      uint32_t w1[kThreadSlots / 4], w2[kThreadSlots / 4];
 #pragma unroll
-      for (int g = 0; g < kWideHS / 4; ++g) {
+      for (int g = 0; g < kThreadSlots / 4; ++g) {
         w1[g] = __byte_perm(__byte_perm(c1[4 * g], c1[4 * g + 1], 0x0040), __byte_perm(c1[4 * g + 2], c1[4 * g + 3], 0x0040), 0x5410);
         w2[g] = __byte_perm(__byte_perm(c2[4 * g], c2[4 * g + 1], 0x0040), __byte_perm(c2[4 * g + 2], c2[4 * g + 3], 0x0040), 0x5410);
       }
       uint8_t* d1 = prow + ((((hs0 >> 4) ^ sw) & (kPieces - 1)) << 4) + (hs0 & 15);
       uint8_t* d2 = prow + (((((kSlots + hs0) >> 4) ^ sw) & (kPieces - 1)) << 4) + (hs0 & 15);
-      if constexpr (kWideHS == 8) {
-        *reinterpret_cast<uint2*>(d1) = make_uint2(w1[0], w1[1]);
-        *reinterpret_cast<uint2*>(d2) = make_uint2(w2[0], w2[1]);
-      } else {
-        *reinterpret_cast<uint4*>(d1) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-        *reinterpret_cast<uint4*>(d2) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
-      }
+      *reinterpret_cast<uint2*>(d1) = make_uint2(w1[0], w1[1]);
+      *reinterpret_cast<uint2*>(d2) = make_uint2(w2[0], w2[1]);
       return xm;
     };
     // Alg. 3 line 12 for everything accumulated since the last drain: O <- (O + alpha_P (O1 + O2 / 254)) * resc
-    auto drain = [&](const float (&resc)[kWideHS], float alpha_old) {
+    auto drain = [&](const float (&resc)[kThreadSlots], float alpha_old) {
 #pragma unroll
       for (int j = 0; j < kDVT; ++j) {
         if (j < p.DVT) {
           const uint32_t orow = tmem_o + (static_cast<uint32_t>(quad * 32) << 16) + j * p.Rp;
-          uint32_t v1[kWideHS], v2[kWideHS], o[kWideHS];
-          tmem_ldw<kWideHS>(orow + hs0, v1);
-          tmem_ldw<kWideHS>(orow + kSlots + hs0, v2);
-          tmem_ldw<kWideHS>(orun_row + j * kSlots, o);
+          uint32_t v1[kThreadSlots], v2[kThreadSlots], o[kThreadSlots];
+          tmem_ld8(orow + hs0, v1);
+          tmem_ld8(orow + kSlots + hs0, v2);
+          tmem_ld8(orun_row + j * kSlots, o);
           tmem_ld_wait();
 #pragma unroll
-          for (int h = 0; h < kWideHS; ++h) {
+          for (int h = 0; h < kThreadSlots; ++h) {
             const float acc = __fmaf_rn(static_cast<float>(static_cast<int32_t>(v2[h])), kInv254, static_cast<float>(static_cast<int32_t>(v1[h])));
             // the drained sums belong to the OLD reference: add them, then rescale
             o[h] = __float_as_uint(__fmaf_rn(alpha_old, acc, __uint_as_float(o[h])) * resc[h]);
           }
-          tmem_stw<kWideHS>(orun_row + j * kSlots, o);
+          tmem_st8(orun_row + j * kSlots, o);
         }
       }
       tmem_st_wait();
@@ -1554,7 +1544,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       if (!ok) break;
       if (threadIdx.x == 64 && t >= 2 && t < 5) attn_mark(p, 4 + 6 * (t - 2));
       tc_fence_after();
-      float s[kWideHS], pl[kWideHS];
+      float s[kThreadSlots], pl[kThreadSlots];
       if (active) {
         load_scores(t, ks, s);
         if constexpr (!kChunked) {
@@ -1569,7 +1559,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         // a group of head slots without a head (9 to 24 rows per KV head): nothing to compute, but the barriers count
         // every softmax warp; its P columns keep whatever codes they hold and its accumulator columns are never read
 #pragma unroll
-        for (int h = 0; h < kWideHS; ++h) pl[h] = 0.0f;
+        for (int h = 0; h < kThreadSlots; ++h) pl[h] = 0.0f;
       }
       fence_proxy_async_smem();
       tc_fence_before();
@@ -1591,18 +1581,18 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       } else if (stamp[t & 1] == t + 1) {
         // ---- the references move: tile maxima per head over the group's 128 tokens, largest value scale ----
 #pragma unroll
-        for (int h = 0; h < kWideHS; ++h) {
+        for (int h = 0; h < kThreadSlots; ++h) {
           const float wm = warp_max(s[h]);
           if (lane == 0) red[hh][wq][h] = wm;
         }
         {
           const float wv = warp_max(vs);
-          if (lane == 0) red[hh][wq][kWideHS] = wv;
+          if (lane == 0) red[hh][wq][kThreadSlots] = wv;
         }
         named_bar_sync(bar_id, 128);
-        float resc[kWideHS];
+        float resc[kThreadSlots];
 #pragma unroll
-        for (int h = 0; h < kWideHS; ++h) {
+        for (int h = 0; h < kThreadSlots; ++h) {
           const float tmax = fmaxf(fmaxf(red[hh][0][h], red[hh][1][h]), fmaxf(red[hh][2][h], red[hh][3][h]));
           resc[h] = 1.0f;
           if (hs0 + h < nh && tmax + nm[h] > 0.0f) {
@@ -1611,7 +1601,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
             nm[h] = -m_new;
           }
         }
-        const float vmax = fmaxf(fmaxf(red[hh][0][kWideHS], red[hh][1][kWideHS]), fmaxf(red[hh][2][kWideHS], red[hh][3][kWideHS]));
+        const float vmax = fmaxf(fmaxf(red[hh][0][kThreadSlots], red[hh][1][kThreadSlots]), fmaxf(red[hh][2][kThreadSlots], red[hh][3][kThreadSlots]));
         const float alpha_old = alpha_p;
         if (vmax > a_ref) {
           a_ref = vmax * kHoldScaleGrowth;
@@ -1631,7 +1621,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
           tc_fence_after();
           drain(resc, alpha_old);
 #pragma unroll
-          for (int h = 0; h < kWideHS; ++h) l_part[h] *= resc[h];
+          for (int h = 0; h < kThreadSlots; ++h) l_part[h] *= resc[h];
         }
         write_p(t, s, vs, pl);
         fence_proxy_async_smem();
@@ -1671,7 +1661,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       }
 #pragma unroll
-      for (int h = 0; h < kWideHS; ++h) l_part[h] += pl[h];
+      for (int h = 0; h < kThreadSlots; ++h) l_part[h] += pl[h];
     }
     if (ok) {
       // what the accumulators still hold
@@ -1683,9 +1673,9 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       }
       if (ok && active) {
         tc_fence_after();
-        float one[kWideHS];
+        float one[kThreadSlots];
 #pragma unroll
-        for (int h = 0; h < kWideHS; ++h) one[h] = 1.0f;
+        for (int h = 0; h < kThreadSlots; ++h) one[h] = 1.0f;
         drain(one, alpha_p);
       }
     }
@@ -1693,7 +1683,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     // partial results of this split: reference maximum, sum of P and unnormalised output per head
     if (ok) {
 #pragma unroll
-      for (int h = 0; h < kWideHS; ++h) {
+      for (int h = 0; h < kThreadSlots; ++h) {
         float l = l_part[h];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
@@ -1701,7 +1691,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       }
       named_bar_sync(bar_id, 128);
 #pragma unroll
-      for (int h = 0; h < kWideHS; ++h) {
+      for (int h = 0; h < kThreadSlots; ++h) {
         if (hs0 + h < nh) {
           float* dst = p.partial + ((static_cast<long long>(b) * p.Hq + h0 + hs0 + h) * p.n_splits + split) * (p.Dv + kPartHdr);
           if (tl == 0) {
@@ -1714,11 +1704,11 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
 #pragma unroll
       for (int j = 0; j < kDVT; ++j) {
         if (j < p.DVT) {            // (warp-uniform: the tensor-memory load is a whole-warp instruction)
-          uint32_t o[kWideHS];
-          tmem_ldw<kWideHS>(orun_row + j * kSlots, o);
+          uint32_t o[kThreadSlots];
+          tmem_ld8(orun_row + j * kSlots, o);
           tmem_ld_wait();
 #pragma unroll
-          for (int h = 0; h < kWideHS; ++h)
+          for (int h = 0; h < kThreadSlots; ++h)
             if (hs0 + h < nh && j * kChunk + tl < p.Dv)
               p.partial[((static_cast<long long>(b) * p.Hq + h0 + hs0 + h) * p.n_splits + split) * (p.Dv + kPartHdr) + kPartHdr + j * kChunk + tl] =
                   __uint_as_float(o[h]);
@@ -2026,31 +2016,31 @@ static bool attn_direct(const AttnPlan& pl) { return attn_direct_built(pl) && !p
 // The kernel instantiation for a plan (G: query rows per KV head) and its block size.
 static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* block_threads) {
   AttnKernel kernel = nullptr;
-#define MSD_ATTN_PICK_P(HG_, NH_, P_) \
-  kernel = (pl.DVT == 1 && pl.DC <= 4) ? attn_decode_kernel<HG_, NH_, 1, P_, 0> : (pl.DVT == 2) ? attn_decode_kernel<HG_, NH_, 2, P_, 0> \
-                                                                                   : attn_decode_kernel<HG_, NH_, 4, P_, 0>
-#define MSD_ATTN_PICK(HG_, NH_) \
-  do { if (paged) { MSD_ATTN_PICK_P(HG_, NH_, true); } else { MSD_ATTN_PICK_P(HG_, NH_, false); } } while (0)
+#define MSD_ATTN_PICK_P(NH_, P_) \
+  kernel = (pl.DVT == 1 && pl.DC <= 4) ? attn_decode_kernel<NH_, 1, P_, 0> : (pl.DVT == 2) ? attn_decode_kernel<NH_, 2, P_, 0> \
+                                                                                           : attn_decode_kernel<NH_, 4, P_, 0>
+#define MSD_ATTN_PICK(NH_) \
+  do { if (paged) { MSD_ATTN_PICK_P(NH_, true); } else { MSD_ATTN_PICK_P(NH_, false); } } while (0)
   *block_threads = kAttnThreads;
   if (pl.balanced) {        // (plan_attn: HG == 8, one chunk of D and of Dv)
-    if (G <= 4) kernel = paged ? attn_decode_kernel<8, 4, 1, true, 1> : attn_decode_kernel<8, 4, 1, false, 1>;
-    else kernel = paged ? attn_decode_kernel<8, 8, 1, true, 1> : attn_decode_kernel<8, 8, 1, false, 1>;
+    if (G <= 4) kernel = paged ? attn_decode_kernel<4, 1, true, 1> : attn_decode_kernel<4, 1, false, 1>;
+    else kernel = paged ? attn_decode_kernel<8, 1, true, 1> : attn_decode_kernel<8, 1, false, 1>;
   } else if (attn_direct(pl)) {
-    if (G <= 4) kernel = paged ? attn_decode_kernel<8, 4, 1, true, 2> : attn_decode_kernel<8, 4, 1, false, 2>;
-    else kernel = paged ? attn_decode_kernel<8, 8, 1, true, 2> : attn_decode_kernel<8, 8, 1, false, 2>;
+    if (G <= 4) kernel = paged ? attn_decode_kernel<4, 1, true, 2> : attn_decode_kernel<4, 1, false, 2>;
+    else kernel = paged ? attn_decode_kernel<8, 1, true, 2> : attn_decode_kernel<8, 1, false, 2>;
   } else if (pl.HG == 8) {
-    if (G <= 4) { MSD_ATTN_PICK(8, 4); } else { MSD_ATTN_PICK(8, 8); }
+    if (G <= 4) { MSD_ATTN_PICK(4); } else { MSD_ATTN_PICK(8); }
   } else {
     // wide head groups: 32 or 16 head slots per CTA, held references (attn_decode_wide_kernel)
     const bool mla = pl.DC == 5 && pl.DVT == 4 && pl.v_alias && pl.stages == 2;     // a 513..640-byte latent row whose first 512 bytes are V
     *block_threads = ((mla && !paged) ? 64 : 96) + 128 * 4;      // producer, QK^T issuer, 16 softmax warps and, except for the chunk-wise kernel, a PV issuer
     if (pl.HG == 16) {
-      kernel = paged ? attn_decode_wide_kernel<16, 8, true, 1, 1> : attn_decode_wide_kernel<16, 8, false, 1, 1>;
+      kernel = paged ? attn_decode_wide_kernel<16, true, 1, 1> : attn_decode_wide_kernel<16, false, 1, 1>;
       *block_threads = 96 + 128 * 2;
     } else if (paged) {
-      kernel = mla ? attn_decode_wide_kernel<32, 8, true, 5, 4> : attn_decode_wide_kernel<32, 8, true, 0, 0>;
+      kernel = mla ? attn_decode_wide_kernel<32, true, 5, 4> : attn_decode_wide_kernel<32, true, 0, 0>;
     } else {
-      kernel = mla ? attn_decode_wide_kernel<32, 8, false, 5, 4> : attn_decode_wide_kernel<32, 8, false, 0, 0>;
+      kernel = mla ? attn_decode_wide_kernel<32, false, 5, 4> : attn_decode_wide_kernel<32, false, 0, 0>;
     }
   }
 #undef MSD_ATTN_PICK

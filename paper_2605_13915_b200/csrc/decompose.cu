@@ -1,6 +1,6 @@
 // Online activation decomposition kernels.
-//   INT8  (Sec. 3.2, Eqs. alpha..x2; Alg. 1 lines 1-5): one CTA per row, 128-bit BF16 loads, warp-shuffle
-//          row maximum, IEEE FP32 division + round-half-to-even, packed 128-bit INT8 stores.
+//   INT8  (Sec. 3.2, Eqs. alpha..x2; Alg. 1 lines 1-5): one CTA per row, 128-bit BF16 loads, row maximum by warp
+//          shuffles, the rounded IEEE quotients without a division per value (quant.cuh), 8 codes per store.
 //   MXFP4 (Sec. 3.2.1, Alg. 2, on the E2M1 grid): one thread per 32-element block - the block maximum needs
 //          no cross-thread reduction and beta follows from alpha by a shift.
 #include <cuda_bf16.h>

@@ -772,8 +772,8 @@ static GemmW8Plan plan_w8(int64_t M, int64_t N, int64_t K, bool base = false) {
   pl.off_q = off;         off = round_up(off + (base ? static_cast<size_t>(N) * K * 2 : static_cast<size_t>(pl.NB) * K), 1024);
   pl.off_alpha = off;     off = round_up(off + 128 * sizeof(float), 256);
   pl.off_beta = off;      off = round_up(off + 128 * sizeof(float), 256);
-  // one arrival counter per weight tile, then the two counters of the in-kernel decomposition
-  pl.off_counters = off;  off = round_up(off + static_cast<size_t>(pl.num_tiles + 2) * sizeof(unsigned), 1024);
+  // one arrival counter per weight tile
+  pl.off_counters = off;  off = round_up(off + static_cast<size_t>(pl.num_tiles) * sizeof(unsigned), 1024);
   // split-K meeting place: one [NB x 128] tile of sums per weight tile (used by the stream-K split only)
   pl.off_slots = off;     off = round_up(off + static_cast<size_t>(pl.num_tiles) * pl.NB * kTileN * sizeof(int32_t), 1024);
   pl.bytes = off;
@@ -1031,7 +1031,7 @@ static GroupedPlan plan_grouped(int64_t M_total, int max_group, int E, int64_t N
   g.off_q = off;        off = round_up(off + 2 * static_cast<size_t>(g.mt_pad) * K, 1024);
   g.off_alpha = off;    off = round_up(off + static_cast<size_t>(M_total + 1) * sizeof(float), 256);
   g.off_beta = off;     off = round_up(off + static_cast<size_t>(M_total + 1) * sizeof(float), 256);
-  g.off_counters = off; off = round_up(off + (tiles + 2) * sizeof(unsigned), 1024);
+  g.off_counters = off; off = round_up(off + tiles * sizeof(unsigned), 1024);
   g.off_slots = off;    off = round_up(off + tiles * g.base.NB * kTileN * sizeof(int32_t), 1024);
   g.bytes = off;
   return g;

@@ -1,5 +1,4 @@
-// Element-wise INT8 quantisation shared by the decomposition kernel, the GEMM's in-kernel row decomposition and the
-// attention kernel's query set-up.
+// Element-wise INT8 quantisation shared by the decomposition kernel and the attention kernels' query set-up.
 #pragma once
 #include <cuda_runtime.h>
 
