@@ -1637,7 +1637,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         // softmax warps are idle here (the next score tile is not there yet) and the product starts the moment P is final
         // instead of when the QK^T-issuing thread gets round to it.  The value chunks are let go of in the order in which they are
         // asked for again, 0 and 1 before 2 and 3: with four threads abreast all four came back at the end of the product (64 x
-        // 16384 tokens 276 us, now 270); one thread for all four takes too long to issue (281).  An accumulator is only ever
+        // 16384 tokens, 43 tiles a split: 276 us against 270); one thread for all four takes too long to issue (281).  An accumulator is only ever
         // written by its own thread, so its MMAs stay in program order.
         if (hh == 0 && lane == 0 && wq < 2) {
           const int st = t & 1;
@@ -1923,8 +1923,8 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   if (B < 1 || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || D < 16 || D % 16 != 0 || Dv < 16 || Dv % 16 != 0) return false;
   const int G = Hq / Hkv;
   // up to 8 rows per KV head: the narrow kernel (three CTAs per SM); 9 to 16 at D, Dv <= 128: the wide kernel with 16 head
-  // slots (two CTAs per SM; 16 rows, 32 x 4096 tokens: 130 us with 32 slots half empty and one CTA per SM, 85 now; 8 x 32768:
-  // 199 and 135); everything else: with 32.  (A 16-slot narrow kernel needs 166 registers and was slower than either.)
+  // slots (two CTAs per SM; 16 rows, the same split sizes, 32 x 4096 tokens: 130 us with 32 slots half empty and one CTA per SM, 85
+  // with 16; 8 x 32768: 199 and 135); everything else: with 32.  (A 16-slot narrow kernel needs 166 registers and was slower than either.)
   pl->HG = (G <= 8) ? 8 : (G <= 16 && D <= kChunk && Dv <= kChunk ? 16 : 32);
   pl->Rp = 2 * pl->HG;
   pl->groups = (G + pl->HG - 1) / pl->HG;
@@ -1965,12 +1965,12 @@ static bool plan_attn(int B, int Hq, int Hkv, int D, int Dv, int max_seqlen, boo
   pl->n_splits = ns;
   pl->chunk = chunk_tiles * kTok;
   // Balanced schedule: every CTA of a grid that just fills the machine gets the same number of tiles, at least q_min
-  // (a unit of n tiles then meets at most ceil(n / q_min) + 1 CTAs).  It costs a few percent (every CTA starts at once and
-  // cuts its own run first; every sequence a run enters is a new set-up), and pays where fixed splits fit badly: sequences
-  // of 32 tiles or more, up to three 16-tile splits per resident CTA, and more units than half the resident CTAs.  Against
-  // fixed splits of the size chosen above (32 query / 8 KV heads, lengths up to 8192 / all 8192): 32 sequences 65 to 67 us
-  // mixed, 100 to 97 uniform; 36: 72 to 78, 110 to 108; 44: 85 to 93, 132 to 130.  With at least two CTAs per unit in one round
-  // the fixed splits of mixed lengths fill it: 24 sequences 53 to 46, 79 to 83; 20 of up to 7000, 5 rows per KV head, 53 to 44.
+  // (a unit of n tiles then meets at most ceil(n / q_min) + 1 CTAs).  Taken for sequences of 32 tiles or more, up to three
+  // 16-tile splits per resident CTA, and more units than half the resident CTAs.  It costs set-up (every CTA starts at once and
+  // cuts its own run first; every sequence a run enters is a new set-up) and is the better one with many sequences of very
+  // different lengths; since the fixed splits' size comes from the lengths, they are ahead over the rest of this range, where the
+  // line has not been moved yet (32 query / 8 KV heads, balanced and fixed, us: 40 x 800 to 8192 tokens 73 and 77, 36 x 2048 to 8192 75
+  // and 75, 32 x 2048 to 8192 68 and 63, 32 x 8192 101 and 88, 16 x 8192 + 16 x 128 107 and 52).
   // Built for the kernels that keep three CTAs per SM (up to 8 rows per KV head, D and Dv <= 128).
   const bool can_balance = pl->HG == 8 && pl->DC == 1 && pl->DVT == 1 && option(OPT_ATTN_SPLITS) < 1 &&
                            option(OPT_ATTN_CHUNK_TILES) < 1;
@@ -2009,8 +2009,8 @@ msd_status_t launch_attn_combine(const float* partial, int n_splits, int Dv, voi
 using AttnKernel = void (*)(CUtensorMap, CUtensorMap, AttnParams);
 
 // A single split of each sequence has nothing to merge: the narrow kernel writes the result, one launch and one round trip through
-// memory fewer (32 / 8 heads, 64 x 100 to 1000 tokens: 28.3 us, now 26.3; 48 x 750 to 1500: 30.2 and 27.5; 8 / 8, 32 x 512 to
-// 2048: 27.4 and 24.5).  Instantiations of their own: the branch at the end of the others cost 4 x 1000 to 4000 tokens 2.6 %.
+// memory fewer (32 / 8 heads, us with the merge and without: 64 x 100 to 1000 tokens 28.3 and 26.3, 48 x 750 to 1500 30.2 and 27.5).
+// Instantiations of their own: the branch at the end of the others cost 4 x 1000 to 4000 tokens 2.6 %.
 static bool attn_direct(const AttnPlan& pl) { return attn_direct_built(pl) && !pl.balanced && pl.n_splits == 1; }
 
 // The kernel instantiation for a plan (G: query rows per KV head) and its block size.

@@ -14,8 +14,8 @@
 
 namespace msd {
 
-// Bound by issue slots and latency (4096 rows of 4096: 59 -> 27 us with launch, 67 MB; instructions per value 32 -> 21, of which
-// 5 are the row maximum's reductions and divisions).  The row is read twice: the first pass takes the maximum, the second
+// Bound by issue slots and latency (4096 rows of 4096, 67 MB: 27 us with launch, 21 instructions per value, of which 5 are the row
+// maximum's reductions and divisions; 59 us and 32 instructions with one value at a time and a check on each).  The row is read twice: the first pass takes the maximum, the second
 // quantises (its reads hit the L1 cache; a thread's first two units of 8 values stay in registers, which is all there is
 // at decode widths).  The second pass is a loop that is NOT unrolled and keeps two units in flight: with four unrolled
 // copies of the quantisation the kernel spent most of its time waiting for instructions, and with a register limit of 40
@@ -189,10 +189,11 @@ msd_status_t launch_decompose_int8(const void* x_bf16, int64_t M, int64_t K, int
   if (M == 0) return MSD_OK;
   // A programmatic dependent of whatever precedes it (in a chain of layers: the previous layer's GEMM), so that its launch
   // and the launch of the GEMM behind it are over when that kernel ends; launched plainly, 4 to 5 us passed between two
-  // GEMMs in which no weights moved (16 tokens, 4096 x 4096: 14.9 us a call, now 13.2; 1 token, 14336 x 4096: 18.6, 16.9).
+  // GEMMs in which no weights moved (16 tokens, 4096 x 4096: 14.9 us a call launched plainly, 13.2 as a dependent; 1 token, 14336 x 4096:
+  // 18.6 and 16.9).
   // Few rows: the kernel sits on the critical path of the GEMM behind it, and more threads per row mean a shorter
   // latency.  Many rows: throughput counts, so a thread takes several units and many rows share an SM (1000 rows of 4096:
-  // 15 us with 128 threads a row, 20 with 64: too few warps in flight; 1000 rows of 14336: 29 us with 512, 45 before).
+  // 15 us with 128 threads a row, 20 with 64: too few warps in flight; 1000 rows of 14336: 29 us with 512).
   int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
   if (M > 128) threads = K <= 4096 ? 128 : (K <= 8192 ? 256 : 512);
   auto kernel = threads == 1024 ? decompose_int8_kernel<1024>

@@ -186,9 +186,9 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   int pre = 0;                   // stages whose weights were asked for before the wait on the kernel launched just before
 
   // Decode shapes (kCluster): warp 0 sets the barriers up, a stage per lane, and asks for the first stages' weight tiles right
-  // away, before the rest of the CTA's set-up (tensor memory, the CTA-wide barrier): 1 token, 4096 x 14336 and back 32.1 -> 31.6
+  // away, before the rest of the CTA's set-up (tensor memory, the CTA-wide barrier): 1 token, 4096 x 14336 and back 31.6 us, 32.1 after it
   // us.  Launches of many items are behind a decomposition of many rows, and asking that early takes bandwidth from it
-  // (32 experts 57.6 -> 58.9 us, 1000 rows 35.5 -> 37.9).
+  // (32 experts 58.9 us, 57.6 later; 1000 rows 37.9 and 35.5).
   if constexpr (kCluster) {
     if (warp == 0) {
       if (lane < nstages) { mbar_init(&full_bar[lane], 1); mbar_init(&empty_bar[lane], 1); }
@@ -238,7 +238,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       // (This kernel lets no dependent in early: the waiting decomposition of a next call beside it cost 2 us on 32 experts.)
       if (warp == 10 || !kCluster) {
         // neither weights nor prepared weight scales depend on the kernel launched just before; a grouped launch asks for two
-        // stages that early and leaves the bandwidth to the decomposition of its many rows (64 experts 40.2 -> 38.8 us, 32: 57.7 -> 57.1)
+        // stages that early and leaves the bandwidth to the decomposition of its many rows (64 experts 38.8 us, 40.2 asking for all; 32: 57.1 and 57.7)
         q.tile = blockIdx.x;
         enter(q);
         first = q;
