@@ -116,23 +116,29 @@ def test_split_size_from_the_lengths(rows, seqlens, paged):
 
 
 @pytest.mark.parametrize("page", [0, 16, 64])
-@pytest.mark.parametrize("Hq,seqlens,bound", [(16, [2000] * 7, 1), (64, [2000, 0, 2000, 1999, 1, 2000, 2000, 2000, 2000], 1),
-                                              (128, [1000] * 8, 2), (16, [3000] * 12, 4)])
-def test_split_size_from_the_lengths_few_rows(Hq, seqlens, bound, page):
-    """Up to 8 rows per KV head: a split size that the device takes from the lengths, larger than the smallest, is the one the host
-    reports, under an exact and a generous max_seqlen, contiguous and paged."""
-    c = inputs.gqa_case(len(seqlens), Hq, 16, 128, seqlens, seed=Hq)
-    mx = bound * c.max_seqlen
+@pytest.mark.parametrize("Hq,Hkv,seqlens,bound", [
+    # up to 8 rows per KV head
+    (16, 16, [2000] * 7, 1), (64, 16, [2000, 0, 2000, 1999, 1, 2000, 2000, 2000, 2000], 1), (128, 16, [1000] * 8, 2), (16, 16, [3000] * 12, 4),
+    # 16 and 32 rows, and a latent cache (Hkv = 0); lengths of 40 % of the bound or more on average, and less
+    (128, 8, [2000, 0, 2000, 1999, 1, 2000, 2000], 1), (128, 8, [1500] * 16, 4), (256, 8, [700] * 7, 1), (256, 8, [1500] * 6, 4),
+    (64, 0, [1000] * 10, 2), (64, 0, [500] * 24, 4)])
+def test_larger_split_sizes_from_the_lengths(Hq, Hkv, seqlens, bound, page):
+    """A split size that the device takes from the lengths, larger than the smallest, is the one the host reports, under an exact
+    and a generous max_seqlen, contiguous and paged, in every kernel that takes one."""
+    B, mx = len(seqlens), bound * max(seqlens)
+    c = inputs.gqa_case(B, Hq, Hkv, 128, seqlens, seed=Hq) if Hkv else inputs.mla_case(B, Hq, 576, 512, seqlens, seed=Hq)
+    D, n_kv = c.q.shape[2], max(Hkv, 1)
     starts, _ = _split_starts(c, max_seqlen=mx)
-    assert starts[0, 0, 0, 1] > binding.attn_decode_schedule(len(seqlens), Hq, 16, 128, 128, mx)[2] > 0
+    assert starts[0, 0, 0, 1] > binding.attn_decode_schedule(B, Hq, n_kv, D, c.dv, mx)[2] > 0
+    cache = [c.k, c.v, c.k_scale, c.v_scale]
     if page:
-        k, v, ks, vs, table, sl = inputs.paginate(c, page, seed=Hq)
+        *cache, table, sl = inputs.paginate(c, page, seed=Hq)
         table = np.pad(table, ((0, 0), (0, (bound - 1) * table.shape[1] + bound)))
-        o, lse = binding.attn_decode_int8kv_paged(bf16_dev(c.q), dev(k), dev(v), dev(ks), dev(vs), dev(table), dev(sl), page, mx,
-                                                  c.softmax_scale, want_lse=True)
+    k, v, ks, vs = (None if t is None else dev(t) for t in cache)
+    if page:
+        o, lse = binding.attn_decode_int8kv_paged(bf16_dev(c.q), k, v, ks, vs, dev(table), dev(sl), page, mx, c.softmax_scale, dv=c.dv, want_lse=True)
     else:
-        o, lse = binding.attn_decode_int8kv(bf16_dev(c.q), dev(c.k), dev(c.v), dev(c.k_scale), dev(c.v_scale), dev(c.cu_seqlens), mx,
-                                            c.softmax_scale, want_lse=True)
+        o, lse = binding.attn_decode_int8kv(bf16_dev(c.q), k, v, ks, vs, dev(c.cu_seqlens), mx, c.softmax_scale, dv=c.dv, want_lse=True)
     torch.cuda.synchronize()
     binding.last_device_status()
     ref, lse_ref = _oracle_tiled(c, max_seqlen=mx, paged=page > 0)
