@@ -881,30 +881,38 @@ static void w4_stages(int a_rows, int tile_n, size_t extra_bytes, int* nstages, 
   *nstages = ns > 8 ? 8 : ns;
 }
 
-// Decode shapes (one token tile): tile width and K splits as a cluster.  Every CTA has one item, so the call takes as long as
-// the longest item, width x stages: the smallest wins, of equal ones the smaller cluster.  At most 8 CTAs a cluster, items
-// of at least two stages, all clusters resident at once.  cluster = 1: no split gains anything, or none fits.
+// Decode shapes (one token tile): tile width and K splits as a cluster.  Every CTA has one item, so a call takes about as long
+// as its longest: in us, fitted to 105 shapes swept over all widths and splits,
+//   stages x (0.22 + 0.00172 x width) + 0.000135 x tokens x width x (S - 1) / S (the sums a CTA sends to its peers) + 0.2 x S.
+// The choice with the smallest is 1.008 of the best swept on average and 1.08 at most; width x stages alone, without what a stage and
+// the exchange cost whatever the width, 1.038 and 1.37 (125 tokens, 2848 x 4096: 8 CTAs of 224 columns 15.3 us, 4 of 128 11.2).
+// At most 8 CTAs a cluster, items of at least two stages, all clusters resident at once.  cluster = 1, K unsplit or split
+// through memory: no split gains anything or none fits; few stages (then exchange and cluster cost more than the stages saved: 125
+// tokens, 15904 x 1280 11.5 us split, 10.1 whole); or a single weight tile with so many stages that eight CTAs are too few
+// (1 token, 8 x 14592: 12.1 us in eight, 10.0 in fourteen through memory).
 static void w4_decode_shape(int64_t M, int64_t N, int kstages, int* tile_n, int* cluster) {
   const int a_rows = static_cast<int>((M + 7) / 8 * 8);
   *cluster = 1;
-  long long best = 0;
+  if (N <= 224 && kstages > 28) return;
+  auto cost = [&](int w, int S) {
+    const int per = (kstages + S - 1) / S;
+    return static_cast<float>(per) * (0.22f + 1.72e-3f * static_cast<float>(w)) +
+           (S > 1 ? 1.35e-4f * static_cast<float>(M) * static_cast<float>(w) * static_cast<float>(S - 1) / static_cast<float>(S) + 0.2f * static_cast<float>(S) : 0.0f);
+  };
+  float best = kstages < 8 ? cost(224, 1) : 1e30f;       // (with eight stages and more the kernel without clusters splits too)
   for (const int w : {128, 224, 256}) {
     const long long tiles = (N + w - 1) / w;
-    long long S = sm_count() / tiles;
-    if (S > 8) S = 8;
-    if (S > kstages / 2) S = kstages / 2;
-    for (; S >= 2; --S) {
-      const int per = static_cast<int>((kstages + S - 1) / S);
+    int nstages;
+    size_t stage_bytes;
+    w4_stages(a_rows, w, 0, &nstages, &stage_bytes);
+    for (int S = 2; S <= 8 && S <= kstages / 2 && S * tiles <= sm_count(); ++S) {
+      const int per = (kstages + S - 1) / S;
       if ((kstages + per - 1) / per != S) continue;                     // a split without stages
-      const long long cost = static_cast<long long>(w) * per * 16 + S;
-      if (best != 0 && cost >= best) break;
-      int nstages;
-      size_t stage_bytes;
-      w4_stages(a_rows, w, 0, &nstages, &stage_bytes);
+      const float c = cost(w, S);
+      if (c >= best) continue;
       const size_t slots = static_cast<size_t>(S) * ((w / 16 + S - 1) / S) * 64 * a_rows;        // what the peers send, in the drained pipeline
-      if (slots > nstages * stage_bytes || w4_resident_clusters(w, static_cast<int>(S)) < tiles) continue;
-      best = cost; *tile_n = w; *cluster = static_cast<int>(S);
-      break;
+      if (slots > nstages * stage_bytes || w4_resident_clusters(w, S) < tiles) continue;
+      best = c; *tile_n = w; *cluster = S;
     }
   }
 }

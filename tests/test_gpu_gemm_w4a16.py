@@ -131,11 +131,15 @@ def test_prepared_weight_scales(M, N, K, pair, tile):
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 4096, 2048), (16, 4088, 14336), (33, 1000, 1280), (61, 14336, 1024), (128, 2056, 4096),
-                                   (8, 8, 4096), (100, 136, 8192), (17, 16776, 1152)])
+                                   (8, 8, 4096), (100, 136, 8192), (17, 16776, 1152), (4, 8248, 4096), (125, 15904, 1280), (5, 16, 7424)])
 def test_decode_k_split_as_a_cluster(M, N, K):
     """One token tile with the K splits of a weight tile as the CTAs of a cluster: every tile width, ragged last tiles (one 8-column
-    piece among them), uneven last splits, one row to a full tile; row-major and prepared scales give the same bits, FP32
-    against the oracle, BF16 the FP32 result rounded once."""
+    piece among them), uneven last splits, one row to a full tile, and the shapes left whole or split through memory beside
+    them; row-major and prepared scales give the same bits, FP32 against the oracle, BF16 the FP32 result rounded once.  Partial
+    tiles in memory show in the workspace: a single weight tile with a long K has them, a shape with clusters does not."""
+    up, groups = lambda v: (v + 1023) // 1024 * 1024, 2 * ((K + 255) // 256)
+    no_partial = 2 * up(M * K // 2) + 2 * up(512 * groups) + up(2 * ((N + 223) // 224) * groups * 512)
+    assert (binding.gemm_w4a16_workspace_bytes(M, N, K) > no_partial) == (N <= 224 and K > 28 * 256)
     c = inputs.gemm_w4_case(M, N, K, seed=M + N)
     x, w, e = bf16_dev(c.x), dev(c.w_fp4), dev(c.w_e8m0)
     y = binding.gemm_w4a16(x, w, e, out_dtype=torch.float32)
