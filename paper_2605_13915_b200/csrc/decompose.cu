@@ -192,10 +192,13 @@ msd_status_t launch_decompose_int8(const void* x_bf16, int64_t M, int64_t K, int
   // GEMMs in which no weights moved (16 tokens, 4096 x 4096: 14.9 us a call launched plainly, 13.2 as a dependent; 1 token, 14336 x 4096:
   // 18.6 and 16.9).
   // Few rows: the kernel sits on the critical path of the GEMM behind it, and more threads per row mean a shorter
-  // latency.  Many rows: throughput counts, so a thread takes several units and many rows share an SM (1000 rows of 4096:
-  // 15 us with 128 threads a row, 20 with 64: too few warps in flight; 1000 rows of 14336: 29 us with 512).
+  // latency.  Many rows: throughput counts, so a thread takes several units and many rows share an SM.  Whole calls, us with 128 / 256 /
+  // 512 / 1024 threads a row: 160 rows, 4096 x 4096 21.0 / 18.5 / 17.7 / 18.9; 400, 24.9 with 256 and 24.7 with 512; 1000, 35.1 / 32.7 /
+  // 34.2 / 39.5; 129 rows, 4096 x 14336 48.1 / 39.6 / 36.2 / 34.3; 600, 102.9 / 88.7 / 84.8 / 87.2; 2500, 231 / 221 / 242 / 258; 1000 rows,
+  // 2048 x 1024 14.4 / 14.7 / 17.0 / 22.0.
   int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
-  if (M > 128) threads = K <= 4096 ? 128 : (K <= 8192 ? 256 : 512);
+  if (M > 448) threads /= 2;
+  if (M > 800 && threads == 512) threads = 256;
   auto kernel = threads == 1024 ? decompose_int8_kernel<1024>
               : threads == 512 ? decompose_int8_kernel<512>
               : threads == 256 ? decompose_int8_kernel<256> : decompose_int8_kernel<128>;

@@ -102,7 +102,7 @@ def test_decompose_int8_fractional_scaling_bit_exact(M, K):
     binding.last_device_status()
 
 
-@pytest.mark.parametrize("M,K", [(128, 2832), (129, 2832), (256, 4112), (130, 8208), (3, 16400)])
+@pytest.mark.parametrize("M,K", [(128, 2832), (129, 2832), (256, 4112), (130, 8208), (3, 16400), (449, 1040), (449, 2832), (801, 8208)])
 @pytest.mark.parametrize("fractional", [False, True])
 def test_decompose_int8_ties_bit_exact(M, K, fractional):
     """Quotients on and next to half-integers: every BF16 mantissa at 11 exponents below row maxima that run over all
