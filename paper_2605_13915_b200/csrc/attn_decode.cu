@@ -1070,7 +1070,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
   constexpr bool kIntCombine = kFixDC >= 1 && kFixDC <= 4;      // D <= 512
   constexpr auto kPSwizzle = kSlots == 32 ? kSwizzle64B : kSwizzle32B;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // Splits along y: the early splits of every sequence, which are always full, start first and the short last ones fill
   // the tail.  Units along x, head group slowest: the head groups of a sequence split read the same tiles, and launched side
   // by side they miss L2 together.
@@ -1217,20 +1217,20 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0) {
+    {
       const uint32_t idesc_qk = idesc_dense(2, 1, 1, 0, 0, kTok, p.Rp);     // S8 x S8 -> S32, both K-major
       const uint32_t idesc_pv = idesc_dense(2, 1, 1, 1, 1, kTok, p.Rp);     // A (V^T) and B (P) MN-major
       bool ok = true;
       // the stacked Q operand of this (sequence, KV head, head group) comes ready-made from attn_qstack_kernel, the
       // kernel launched just before this one (the producer's KV loads, which do not depend on it, are already under way)
       pdl_wait_primary();
-      {
+      if (lane == 0) {
         const int chunk_bytes = p.Rp * kChunk;
         mbar_arrive_expect_tx(&q_ready, p.DC * chunk_bytes);
         for (int c = 0; c < p.DC; ++c)
           bulk_load(sm_q + c * chunk_bytes, p.q_img + (static_cast<size_t>(unit_q) * p.DC + c) * chunk_bytes, chunk_bytes, &q_ready);
       }
-      ok = wait_bounded(&q_ready, 0, abort, p.status);
+      ok = wait_bounded_warp(&q_ready, 0, abort, p.status);
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);         // K-major tiles: K, stacked Q
       const uint64_t dvt = smem_desc(0, 16384, 1024, kSwizzle128B);     // V^T read MN-major from the token-major tile
       const uint64_t q_enc = dk + (smem_u32(sm_q) >> 4);
@@ -1254,28 +1254,28 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
             for (int k = 0; k < 4; ++k)
               if (c + 1 < kFixDC || k < last_steps) {
                 if (c > 0 || k > 0)
-                  mma_i8_lohi<true>(d, ka_lo + (c * (kChunkBytes >> 4) + 2 * k), k_hi, qa_lo + (c * ((kSlots * 2 * kChunk) >> 4) + 2 * k), q_hi, idesc_qk);
+                  mma_i8_lohi_warp<true>(d, ka_lo + (c * (kChunkBytes >> 4) + 2 * k), k_hi, qa_lo + (c * ((kSlots * 2 * kChunk) >> 4) + 2 * k), q_hi, idesc_qk);
                 else
-                  mma_i8_lohi<false>(d, ka_lo, k_hi, qa_lo, q_hi, idesc_qk);
+                  mma_i8_lohi_warp<false>(d, ka_lo, k_hi, qa_lo, q_hi, idesc_qk);
               }
         } else {
           uint64_t kc = ka, qa = q_enc;
           for (int c = 0; c < nDC; ++c) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-              if (c + 1 < nDC || k < last_steps) mma_i8(d, kc + 2 * k, qa + 2 * k, idesc_qk, (c > 0 || k > 0) ? 1u : 0u);
+              if (c + 1 < nDC || k < last_steps) mma_i8_warp(d, kc + 2 * k, qa + 2 * k, idesc_qk, (c > 0 || k > 0) ? 1u : 0u);
             kc += kChunkBytes >> 4;
             qa += q_step;
           }
         }
-        tc_commit(&s_full[t & 1]);
+        tc_commit_warp(&s_full[t & 1]);
         if constexpr (kChunked) { /* the producer takes s_full as "the rotary chunk has been read" */ }
-        else if (!p.v_alias) tc_commit(&kv_empty[st]);       // separate V: the K buffer is free once QK^T has read it
+        else if (!p.v_alias) tc_commit_warp(&kv_empty[st]);       // separate V: the K buffer is free once QK^T has read it
       };
       // PV is issued by softmax threads or a warp of its own (below); this thread issues QK^T only.
       int q = 0;
       if constexpr (kChunked) {
-        // PV is issued by two softmax threads (below); this thread issues QK^T only.  QK^T(q) needs KV tile q in shared
+        // PV is issued by two softmax warps (below); this warp issues QK^T only.  QK^T(q) needs KV tile q in shared
         // memory and the score buffer q&1 read, i.e. P of tile q-2 written by every softmax warp (the slow path works
         // from registers).  The P buffer q&1 is free by then as well: KV tile q arrives in the stage that PV(q-2) gave
         // back chunk by chunk, so its arrival implies that PV(q-2) is complete.
@@ -1287,40 +1287,40 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         for (; q < ntiles && ok; ++q) {
           const int st = q & 1;
           const uint32_t ph = (q >> 1) & 1;
-          if (q >= 2) ok = wait_bounded(&p_full[q & 1], ((q - 2) >> 1) & 1, abort, p.status);
+          if (q >= 2) ok = wait_bounded_warp(&p_full[q & 1], ((q - 2) >> 1) & 1, abort, p.status);
           if (!ok) break;
           const uint32_t d = tmem_base + (q & 1) * p.Rp;
           const uint32_t k_lo = k_lo0 + static_cast<uint32_t>(st * (kv_stage_bytes >> 4));
 #pragma unroll
           for (int i = 0; i < 5; ++i) {
             const int c = (i == 0) ? 4 : i - 1;
-            ok = wait_bounded(&ck_full[st][c], ph, abort, p.status);
+            ok = wait_bounded_warp(&ck_full[st][c], ph, abort, p.status);
             if (!ok) break;
-            if (i == 0 && q >= 2 && q < 5) attn_mark(p, 7 + 6 * (q - 2));
+            if (i == 0 && q >= 2 && q < 5 && lane == 0) attn_mark(p, 7 + 6 * (q - 2));
             tc_fence_after();
 #pragma unroll
             for (int k = 0; k < 4; ++k)
               if (c < 4 || k < last_steps) {
                 const uint32_t ka = k_lo + (c * (kChunkBytes >> 4) + 2 * k), qa = q_lo0 + (c * ((kSlots * 2 * kChunk) >> 4) + 2 * k);
-                if (i == 0 && k == 0) mma_i8_lohi<false>(d, ka, k_hi, qa, q_hi, idesc_qk);
-                else mma_i8_lohi<true>(d, ka, k_hi, qa, q_hi, idesc_qk);
+                if (i == 0 && k == 0) mma_i8_lohi_warp<false>(d, ka, k_hi, qa, q_hi, idesc_qk);
+                else mma_i8_lohi_warp<true>(d, ka, k_hi, qa, q_hi, idesc_qk);
               }
           }
           if (!ok) break;
-          tc_commit(&s_full[q & 1]);
-          if (q >= 2 && q < 5) attn_mark(p, q == 4 ? 30 : 23 + q);
+          tc_commit_warp(&s_full[q & 1]);
+          if (q >= 2 && q < 5 && lane == 0) attn_mark(p, q == 4 ? 30 : 23 + q);
         }
       } else {
         // QK^T(q) needs KV tile q in shared memory and the score buffer q&1 read (P of tile q-2 written by every softmax
         // warp; the slow path works from registers).  PV is issued by a warp of its own (below); that PV(q-2) has read
         // the P buffer before P of tile q is written there is the softmax warps' wait on pv_done.
         for (; q < ntiles && ok; ++q) {
-          if (q >= 2) ok = wait_bounded(&p_full[q & 1], ((q - 2) >> 1) & 1, abort, p.status);
-          if (ok) ok = wait_bounded(&kv_full[q % p.stages], (q / p.stages) & 1, abort, p.status);
+          if (q >= 2) ok = wait_bounded_warp(&p_full[q & 1], ((q - 2) >> 1) & 1, abort, p.status);
+          if (ok) ok = wait_bounded_warp(&kv_full[q % p.stages], (q / p.stages) & 1, abort, p.status);
           if (!ok) break;
-          if (q >= 2 && q < 5) attn_mark(p, 7 + 6 * (q - 2));
+          if (q >= 2 && q < 5 && lane == 0) attn_mark(p, 7 + 6 * (q - 2));
           issue_qk(q);
-          if (q >= 2 && q < 5) attn_mark(p, q == 4 ? 30 : 23 + q);
+          if (q >= 2 && q < 5 && lane == 0) attn_mark(p, q == 4 ? 30 : 23 + q);
         }
       }
     }
@@ -1330,7 +1330,7 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
     // 4 commits and its polling, everything else waiting for it), and a softmax thread issuing PV puts it on the
     // softmax warps' critical path.
     if constexpr (!kChunked) {
-      if (lane == 0) {
+      {
         const uint64_t vdesc = smem_desc(0, 16384, 1024, kSwizzle128B) + (smem_u32(smem) >> 4);       // V^T, MN-major from the token-major tile
         const uint64_t pdesc = smem_desc(0, 8 * kPRow, 8 * kPRow, kPSwizzle) + (smem_u32(sm_p) >> 4);           // P, token-major
         const uint32_t va0 = static_cast<uint32_t>(vdesc), v_hi = static_cast<uint32_t>(vdesc >> 32);
@@ -1343,30 +1343,30 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         for (int t = 0; t < ntiles && ok; ++t) {
           const int st = t % p.stages;
           // P of tile t final: written by every softmax warp and, when the references had to move, written again
-          ok = wait_bounded(&p_full[t & 1], (t >> 1) & 1, abort, p.status);
+          ok = wait_bounded_warp(&p_full[t & 1], (t >> 1) & 1, abort, p.status);
           bool fresh = false;
-          if (ok && stamp[t & 1] == t + 1) {
-            ok = wait_bounded(&p_redo, n_slow & 1, abort, p.status);
+          if (ok && __any_sync(0xffffffffu, stamp[t & 1] == t + 1)) {
+            ok = wait_bounded_warp(&p_redo, n_slow & 1, abort, p.status);
             ++n_slow;
             fresh = true;                          // the accumulators were drained: start them again
           }
-          if (ok) ok = wait_bounded(p.v_alias ? &kv_full[st] : &v_full[st], (t / p.stages) & 1, abort, p.status);     // the value tile
+          if (ok) ok = wait_bounded_warp(p.v_alias ? &kv_full[st] : &v_full[st], (t / p.stages) & 1, abort, p.status);     // the value tile
           if (!ok) break;
           tc_fence_after();
-          if (t >= 2 && t < 5) attn_mark(p, 8 + 6 * (t - 2));
+          if (t >= 2 && t < 5 && lane == 0) attn_mark(p, 8 + 6 * (t - 2));
           const uint32_t va = va0 + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + (p.v_alias ? 0u : static_cast<uint32_t>(p.DC * (kChunkBytes >> 4)));
           const uint32_t pa = pa0 + (t & 1) * p_step;
           for (int j = 0; j < n_dvt; ++j) {
             const uint32_t acc = tmem_o + j * (2 * kSlots);
-            if (fresh) mma_i8_lohi<false>(acc, va + j * (kChunkBytes >> 4), v_hi, pa, p_hi, idesc);
-            else mma_i8_lohi<true>(acc, va + j * (kChunkBytes >> 4), v_hi, pa, p_hi, idesc);
+            if (fresh) mma_i8_lohi_warp<false>(acc, va + j * (kChunkBytes >> 4), v_hi, pa, p_hi, idesc);
+            else mma_i8_lohi_warp<true>(acc, va + j * (kChunkBytes >> 4), v_hi, pa, p_hi, idesc);
 #pragma unroll
             for (int k = 1; k < 4; ++k)      // 32 tokens per MMA: four 8-token groups of 1024 bytes
-              mma_i8_lohi<true>(acc, va + j * (kChunkBytes >> 4) + k * (4096 >> 4), v_hi, pa + k * (32 * kPRow >> 4), p_hi, idesc);
+              mma_i8_lohi_warp<true>(acc, va + j * (kChunkBytes >> 4) + k * (4096 >> 4), v_hi, pa + k * (32 * kPRow >> 4), p_hi, idesc);
           }
-          tc_commit(&pv_done[t & 1]);
-          tc_commit(p.v_alias ? &kv_empty[st] : &v_empty[st]);
-          if (t >= 2 && t < 5) attn_mark(p, 20 + t);
+          tc_commit_warp(&pv_done[t & 1]);
+          tc_commit_warp(p.v_alias ? &kv_empty[st] : &v_empty[st]);
+          if (t >= 2 && t < 5 && lane == 0) attn_mark(p, 20 + t);
         }
       }
     }
@@ -1633,29 +1633,29 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         slow = true;
       }
       if constexpr (kChunked) {
-        // PV(t), two dv tiles per thread: lane 0 of the first two softmax warps, which sit on different warp schedulers.  The
+        // PV(t), two dv tiles each by the first two softmax warps, which sit on different warp schedulers.  The
         // softmax warps are idle here (the next score tile is not there yet) and the product starts the moment P is final
         // instead of when the QK^T-issuing thread gets round to it.  The value chunks are let go of in the order in which they are
         // asked for again, 0 and 1 before 2 and 3: with four threads abreast all four came back at the end of the product (64 x
         // 16384 tokens, 43 tiles a split: 276 us against 270); one thread for all four takes too long to issue (281).  An accumulator is only ever
         // written by its own thread, so its MMAs stay in program order.
-        if (hh == 0 && lane == 0 && wq < 2) {
+        if (wi < 2) {
           const int st = t & 1;
-          if (slow) ok = wait_bounded(&p_redo, (n_slow - 1) & 1, abort, p.status);      // every warp has drained and rewritten P
+          if (slow) ok = wait_bounded_warp(&p_redo, (n_slow - 1) & 1, abort, p.status);      // every warp has drained and rewritten P
           const uint32_t pa_lo = pv_pa_lo + (t & 1) * pv_p_step;
 #pragma unroll
           for (int dv = wq; dv < 4; dv += 2) {
-            if (ok) ok = wait_bounded(&ck_full[st][dv], (t >> 1) & 1, abort, p.status);      // its value chunk (long landed: QK^T(t) has read the tile)
+            if (ok) ok = wait_bounded_warp(&ck_full[st][dv], (t >> 1) & 1, abort, p.status);      // its value chunk (long landed: QK^T(t) has read the tile)
             if (!ok) break;
             tc_fence_after();
             const uint32_t va_lo = pv_va_lo + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + dv * (kChunkBytes >> 4);
             const uint32_t acc = tmem_o + dv * (2 * kSlots);
-            if (slow) mma_i8_lohi<false>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
-            else mma_i8_lohi<true>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
+            if (slow) mma_i8_lohi_warp<false>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
+            else mma_i8_lohi_warp<true>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
 #pragma unroll
             for (int k = 1; k < 4; ++k)      // 32 tokens per MMA: four 8-token groups of 1024 bytes
-              mma_i8_lohi<true>(acc, va_lo + k * (4096 >> 4), pv_v_hi, pa_lo + k * (32 * kPRow >> 4), pv_p_hi, pv_idesc);
-            tc_commit(&ck_empty[st][dv]);      // value chunk dv may be requested again; also "this dv tile of PV(t) is complete"
+              mma_i8_lohi_warp<true>(acc, va_lo + k * (4096 >> 4), pv_v_hi, pa_lo + k * (32 * kPRow >> 4), pv_p_hi, pv_idesc);
+            tc_commit_warp(&ck_empty[st][dv]);      // value chunk dv may be requested again; also "this dv tile of PV(t) is complete"
           }
         }
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;

@@ -125,7 +125,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
 
   // Work items: (token tile, weight tile, K split).  With ksplit > 1 (few tiles, long K: decode shapes) every item
@@ -262,7 +262,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       int stage = 0; uint32_t phase = 0;
       int it = 0;
       bool ok = true;
@@ -275,12 +275,12 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
         const int acc = (kAcc == 2) ? (it & 1) : 0;
         const uint32_t tphase = (kAcc == 2) ? ((it >> 1) & 1) : (it & 1);
         const uint32_t d_tmem = tmem_base + acc * kTN;
-        ok = wait_bounded(&tempty_bar[acc], tphase ^ 1, abort, p.status);      // epilogue has drained this accumulator
+        ok = wait_bounded_warp(&tempty_bar[acc], tphase ^ 1, abort, p.status);      // epilogue has drained this accumulator
         if (!ok) break;
         tc_fence_after();
         const int ks0 = (tile % p.ksplit) * p.kper, ks1 = ks0 + p.kper < p.kstages ? ks0 + p.kper : p.kstages;
         for (int ks = ks0; ks < ks1; ++ks) {
-          ok = wait_bounded(&full_bar[stage], phase, abort, p.status);
+          ok = wait_bounded_warp(&full_bar[stage], phase, abort, p.status);
           if (!ok) break;
           tc_fence_after();
           // Descriptors differ from the templates only in the 16-byte-granular address field (bits 0-13; shared
@@ -293,24 +293,24 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           const uint32_t sfb_t = sfa1_t + 16;                            // 2 k-groups x 8 columns (256 weight rows)
           // the scale columns of this stage were written by warps 6..9 (tcgen05.cp copies issued by this thread run in
           // order with the MMAs in the tensor pipe and cost a sixth of its time)
-          ok = wait_bounded(&sf_ready[sfpar], (nstage >> 1) & 1, abort, p.status);
+          ok = wait_bounded_warp(&sf_ready[sfpar], (nstage >> 1) & 1, abort, p.status);
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {                    // 64 elements (32 bytes) per MMA
             const int g = kk >> 1;
             const uint32_t idesc = (kk & 1) ? idesc_hi : idesc_lo;   // which pair of scale bytes of the 4-scale column
-            mma_mxf4(d_tmem, a1d + 2 * kk, bd + 2 * kk, idesc, sfa1_t + 4 * g, sfb_t + 8 * g, (ks > ks0 || kk > 0) ? 1u : 0u);
-            mma_mxf4(d_tmem, a2d + 2 * kk, bd + 2 * kk, idesc, sfa2_t + 4 * g, sfb_t + 8 * g, 1u);
+            mma_mxf4_warp(d_tmem, a1d + 2 * kk, bd + 2 * kk, idesc, sfa1_t + 4 * g, sfb_t + 8 * g, (ks > ks0 || kk > 0) ? 1u : 0u);
+            mma_mxf4_warp(d_tmem, a2d + 2 * kk, bd + 2 * kk, idesc, sfa2_t + 4 * g, sfb_t + 8 * g, 1u);
           }
-          tc_commit(&sf_free[sfpar]);                // this set of scale columns may be rewritten once these MMAs are done
+          tc_commit_warp(&sf_free[sfpar]);                // this set of scale columns may be rewritten once these MMAs are done
           sfpar ^= 1;
           ++nstage;
-          tc_commit(&empty_bar[stage]);
+          tc_commit_warp(&empty_bar[stage]);
           if (++stage == nstages) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        tc_commit(&tfull_bar[acc]);
+        tc_commit_warp(&tfull_bar[acc]);
       }
     }
   } else if (warp >= 6) {      // (warp 10 went the producers' way above)
@@ -569,8 +569,8 @@ gemm_w4a16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);          // 0 = leader of the pair
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
 
   if (threadIdx.x == 0) {
@@ -632,7 +632,7 @@ gemm_w4a16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       int stage = 0; uint32_t phase = 0;
       int it = 0, nstage = 0;
       bool ok = true;
@@ -643,14 +643,14 @@ gemm_w4a16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid
         const int acc = (kAcc == 2) ? (it & 1) : 0;
         const uint32_t tphase = (kAcc == 2) ? ((it >> 1) & 1) : (it & 1);
         const uint32_t d_tmem = tmem_base + acc * kTN;
-        ok = wait_bounded(&tempty_bar[acc], tphase ^ 1, abort, p.status);   // both epilogues have drained this accumulator
+        ok = wait_bounded_warp(&tempty_bar[acc], tphase ^ 1, abort, p.status);   // both epilogues have drained this accumulator
         if (!ok) break;
         tc_fence_after();
         for (int ks = 0; ks < p.kstages; ++ks, ++nstage) {
           const int set = nstage & 1;
-          ok = wait_bounded(&full_bar[stage], phase, abort, p.status);
+          ok = wait_bounded_warp(&full_bar[stage], phase, abort, p.status);
           if (!ok) break;
-          ok = wait_bounded(&sf_ready[set], (nstage >> 1) & 1, abort, p.status);
+          ok = wait_bounded_warp(&sf_ready[set], (nstage >> 1) & 1, abort, p.status);
           if (!ok) break;
           tc_fence_after();
           const uint64_t enc = static_cast<uint64_t>(smem_u32(smem + stage * kStageBytes) >> 4);
@@ -662,15 +662,15 @@ gemm_w4a16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid
           for (int kk = 0; kk < 4; ++kk) {                    // 64 elements (32 bytes) per MMA
             const int g = kk >> 1;
             const uint32_t idesc = (kk & 1) ? idesc_hi : idesc_lo;   // which pair of scale bytes of the 4-scale column
-            mma_mxf4_pair(d_tmem, a1d + 2 * kk, bd + 2 * kk, idesc, sfa1_t + 4 * g, sfb_t + 8 * g, (ks > 0 || kk > 0) ? 1u : 0u);
-            mma_mxf4_pair(d_tmem, a2d + 2 * kk, bd + 2 * kk, idesc, sfa2_t + 4 * g, sfb_t + 8 * g, 1u);
+            mma_mxf4_pair_warp(d_tmem, a1d + 2 * kk, bd + 2 * kk, idesc, sfa1_t + 4 * g, sfb_t + 8 * g, (ks > 0 || kk > 0) ? 1u : 0u);
+            mma_mxf4_pair_warp(d_tmem, a2d + 2 * kk, bd + 2 * kk, idesc, sfa2_t + 4 * g, sfb_t + 8 * g, 1u);
           }
-          tc_commit_pair(&sf_free[set], 3);         // this set of scale columns may be rewritten in both CTAs
-          tc_commit_pair(&empty_bar[stage], 3);     // frees the stage in both CTAs
+          tc_commit_pair_warp(&sf_free[set], 3);         // this set of scale columns may be rewritten in both CTAs
+          tc_commit_pair_warp(&empty_bar[stage], 3);     // frees the stage in both CTAs
           if (++stage == kW4PairStages) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        tc_commit_pair(&tfull_bar[acc], 3);
+        tc_commit_pair_warp(&tfull_bar[acc], 3);
       }
     }
   } else if (warp >= 6) {      // (warp 10 went the producers' way above)

@@ -272,7 +272,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
   __shared__ int is_last_flag;
   __shared__ __align__(16) float s_alpha[128], s_beta[128];
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);      // (the same in all lanes, known to be so)
   const int lane = threadIdx.x & 31;
   if (p.num_stages < 1 || p.kw < 1 || p.kblocks < 1) return;     // malformed plan: touch nothing
   // lets a decomposition kernel queued behind this GEMM become resident early (it still waits for this grid to finish)
@@ -467,9 +467,10 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0) {
+    {
       const uint32_t idesc = kBase ? idesc_dense(/*D=F32*/ 1, /*A=BF16*/ 1, /*B=BF16*/ 1, 0, 0, kTileN, p.NB)
                                    : idesc_dense(/*D=S32*/ 2, /*A=S8*/ 1, /*B=S8*/ 1, 0, 0, kTileN, p.NB);
+      const uint64_t op_desc = smem_desc(0, 16, 1024, kSwizzle128B);
       int stage = 0;
       uint32_t phase = 0;
       int seg = 0;
@@ -480,36 +481,36 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
         const long long tile_end = static_cast<long long>(tile + 1) * p.kblocks;
         const long long seg_end = tile_end < blk_end ? tile_end : blk_end;
         const int acc = seg & 1;
-        ok = wait_bounded(&tempty_bar[acc], ((seg >> 1) & 1) ^ 1, abort, p.status);
+        ok = wait_bounded_warp(&tempty_bar[acc], ((seg >> 1) & 1) ^ 1, abort, p.status);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * p.NB;
         for (long long b = blk; b < seg_end; ++b) {
-          ok = wait_bounded(&full_bar[stage], phase, abort, p.status);
+          ok = wait_bounded_warp(&full_bar[stage], phase, abort, p.status);
           if (!ok) break;
-          if (b == blk_begin) trace_mark(p, 6);
+          if (b == blk_begin && lane == 0) trace_mark(p, 6);
           tc_fence_after();
-          const uint32_t wa = smem_u32(smem + stage * stage_bytes);
-          const uint32_t xa = wa + w_stage_bytes;     // the MMA reads 128 A rows; rows past the band are never used
-          for (int c = 0; c < p.kw; ++c) {
+          // (descriptors of one kernel differ in their address field only)
+          uint64_t wd = op_desc + static_cast<uint64_t>(smem_u32(smem + stage * stage_bytes) >> 4);
+          uint64_t xd = wd + static_cast<uint64_t>(w_stage_bytes >> 4);     // the MMA reads 128 A rows; rows past the band are never used
+          for (int c = 0; c < p.kw; ++c, wd += w_chunk >> 4, xd += x_chunk_bytes >> 4) {
 #pragma unroll
             for (int k = 0; k < kBlockK / 32; ++k) {
-              const uint64_t adesc = smem_desc(wa + c * w_chunk + k * 32, 16, 1024, kSwizzle128B);
-              const uint64_t bdesc = smem_desc(xa + c * x_chunk_bytes + k * 32, 16, 1024, kSwizzle128B);
+              const uint64_t adesc = wd + 2 * k, bdesc = xd + 2 * k;
               const uint32_t accum = (b > blk || c > 0 || k > 0) ? 1u : 0u;
-              if constexpr (kBase) mma_f16(d_tmem, adesc, bdesc, idesc, accum);
-              else mma_i8(d_tmem, adesc, bdesc, idesc, accum);
+              if constexpr (kBase) mma_f16_warp(d_tmem, adesc, bdesc, idesc, accum);
+              else mma_i8_warp(d_tmem, adesc, bdesc, idesc, accum);
             }
           }
-          tc_commit(&empty_bar[stage]);          // frees the stage once these MMAs have read it
+          tc_commit_warp(&empty_bar[stage]);          // frees the stage once these MMAs have read it
           if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        tc_commit(&tfull_bar[acc]);              // accumulator of this segment complete
+        tc_commit_warp(&tfull_bar[acc]);              // accumulator of this segment complete
         ++seg;
         blk = seg_end;
       }
-      trace_mark(p, 7);
+      if (lane == 0) trace_mark(p, 7);
     }
   } else {
     // ------------------------------ epilogue (warps 2..5) ------------------------------

@@ -73,8 +73,8 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = kPair ? cluster_ctarank() : 0u;     // 0 = leader of the pair
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const uint32_t rank = kPair ? __shfl_sync(0xffffffffu, cluster_ctarank(), 0) : 0u;     // 0 = leader of the pair
   pdl_launch_dependents();       // the decomposition of a next layer sets up beside this kernel (1000 tokens: 188 us a layer pair, 200 without)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
 
@@ -164,7 +164,7 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       int stage = 0; uint32_t phase = 0;
       int it = 0;
       bool ok = true;
@@ -172,13 +172,13 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
       const uint32_t idesc = kBase ? idesc_dense(/*D=F32*/ 1, /*A=BF16*/ 1, /*B=BF16*/ 1, 0, 0, kPair ? 2 * kP8TileM : kP8TileM, kP8TileN)
                                    : idesc_dense(/*D=S32*/ 2, /*A=S8*/ 1, /*B=S8*/ 1, 0, 0, kPair ? 2 * kP8TileM : kP8TileM, kP8TileN);
       for (int tile = first; tile < total_tiles && ok; tile += step, ++it) {
-        ok = wait_bounded(&tempty_bar, (it & 1) ^ 1, abort, p.status);        // the epilogue has drained both accumulators
+        ok = wait_bounded_warp(&tempty_bar, (it & 1) ^ 1, abort, p.status);        // the epilogue has drained both accumulators
         if (!ok) break;
         tc_fence_after();
         int tile_mn, ks0, ks1, split, part_tile;
         item_of(tile, tile_mn, ks0, ks1, split, part_tile);
         for (int ks = ks0; ks < ks1; ++ks) {
-          ok = wait_bounded(&full_bar[stage], phase, abort, p.status);
+          ok = wait_bounded_warp(&full_bar[stage], phase, abort, p.status);
           if (!ok) break;
           tc_fence_after();
           const uint64_t enc = static_cast<uint64_t>(smem_u32(smem + stage * kStageBytes) >> 4);
@@ -187,21 +187,21 @@ gemm_w8a16_prefill_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __g
           for (int kk = 0; kk < 4; ++kk) {                    // 32 elements (32 bytes) per MMA
             const uint32_t acc = (ks > ks0 || kk > 0) ? 1u : 0u;
             if constexpr (kBase) {              // 16 BF16 elements (32 bytes) per MMA
-              if (kPair) mma_f16_pair(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
-              else mma_f16(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
+              if (kPair) mma_f16_pair_warp(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
+              else mma_f16_warp(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
             } else if (kPair) {
-              mma_i8_pair(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
-              mma_i8_pair(tmem_base + kP8TileN, a2d + 2 * kk, bd + 2 * kk, idesc, acc);
+              mma_i8_pair_warp(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
+              mma_i8_pair_warp(tmem_base + kP8TileN, a2d + 2 * kk, bd + 2 * kk, idesc, acc);
             } else {
-              mma_i8(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
-              mma_i8(tmem_base + kP8TileN, a2d + 2 * kk, bd + 2 * kk, idesc, acc);
+              mma_i8_warp(tmem_base, a1d + 2 * kk, bd + 2 * kk, idesc, acc);
+              mma_i8_warp(tmem_base + kP8TileN, a2d + 2 * kk, bd + 2 * kk, idesc, acc);
             }
           }
-          if (kPair) tc_commit_pair(&empty_bar[stage], 3); else tc_commit(&empty_bar[stage]);    // frees the stage (in both CTAs)
+          if (kPair) tc_commit_pair_warp(&empty_bar[stage], 3); else tc_commit_warp(&empty_bar[stage]);    // frees the stage (in both CTAs)
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        if (kPair) tc_commit_pair(&tfull_bar, 3); else tc_commit(&tfull_bar);
+        if (kPair) tc_commit_pair_warp(&tfull_bar, 3); else tc_commit_warp(&tfull_bar);
       }
     }
   } else {
