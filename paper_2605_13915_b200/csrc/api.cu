@@ -38,7 +38,7 @@ int sm_count() {
 }
 
 static const char* const kOptionNames[OPT_COUNT] = {
-    "MSD_NO_PDL", "MSD_GEMM_MODE", "MSD_GEMM_CTAS", "MSD_P8_PAIR", "MSD_P8_KSPLIT", "MSD_W4_PAIR", "MSD_W4_TILEN", "MSD_W4_KSPLIT",
+    "MSD_NO_PDL", "MSD_GEMM_MODE", "MSD_GEMM_CTAS", "MSD_P8_PAIR", "MSD_P8_KSPLIT", "MSD_W4_PAIR", "MSD_W4_TILEN", "MSD_W4_KSPLIT", "MSD_W4_DECODE",
     "MSD_ATTN_SPLITS", "MSD_ATTN_CHUNK_TILES", "MSD_ATTN_BALANCED"};
 static int g_options[OPT_COUNT];
 static std::mutex g_options_mu;

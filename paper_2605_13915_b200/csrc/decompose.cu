@@ -122,11 +122,13 @@ decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, i
     const int64_t row_in = b / kblocks;
     const int kb = static_cast<int>(b - row_in * kblocks);
     const uint4* src = reinterpret_cast<const uint4*>(x + row_in * ldx + kb * 32);
-    int64_t row = row_in;                   // where the row's components and scales go
+    int64_t row = row_in, srow = row_in;    // where the row's components and scales go
     if (rg.n > 0) {
       int g = 0;
-      while (g + 1 < rg.n && row_in >= rg.off[g + 1]) ++g;
-      row = static_cast<int64_t>(g) * 128 + (row_in - rg.off[g]);
+      for (int step = kMaxRowGroups / 2; step > 0; step >>= 1)
+        if (g + step < rg.n && row_in >= rg.off[g + step]) g += step;
+      row = static_cast<int64_t>(g) * rg.rows + (row_in - rg.off[g]);
+      srow = static_cast<int64_t>(g) * rg.srows + (row_in - rg.off[g]);
     }
     uint32_t w[16];
 #pragma unroll
@@ -164,21 +166,22 @@ decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, i
     *reinterpret_cast<uint4*>(q2 + row * (K >> 1) + kb * 16) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
     // sf_kgroups == 0: row-major [M, K/32]; otherwise the 512-byte blocks (128 rows x 4 scales) the block-scaled
     // MMA's shared-memory -> TMEM scale copy expects: block (row/128, kb/4), byte (row%32)*16 + ((row/32)%4)*4 + kb%4
-    const int64_t so = sf_kgroups == 0
-                           ? row * kblocks + kb
-                           : ((row >> 7) * sf_kgroups + (kb >> 2)) * 512 + (row & 31) * 16 + ((row >> 5) & 3) * 4 + (kb & 3);
+    auto scale_at = [&](int64_t r) {
+      return sf_kgroups == 0 ? r * kblocks + kb : ((r >> 7) * sf_kgroups + (kb >> 2)) * 512 + (r & 31) * 16 + ((r >> 5) & 3) * 4 + (kb & 3);
+    };
+    const int64_t so1 = scale_at(srow), so2 = scale_at(srow + rg.srow2);
     if (pack4) {
       // four neighbouring lanes hold the four scales of one aligned 32-bit word (kblocks is a multiple of 4)
       uint32_t w1 = static_cast<uint32_t>(a + 127) << (8 * (threadIdx.x & 3)), w2 = static_cast<uint32_t>(bexp + 127) << (8 * (threadIdx.x & 3));
       w1 |= __shfl_xor_sync(lanes, w1, 1); w2 |= __shfl_xor_sync(lanes, w2, 1);
       w1 |= __shfl_xor_sync(lanes, w1, 2); w2 |= __shfl_xor_sync(lanes, w2, 2);
       if ((threadIdx.x & 3) == 0) {
-        *reinterpret_cast<uint32_t*>(e1 + so) = w1;
-        *reinterpret_cast<uint32_t*>(e2 + so) = w2;
+        *reinterpret_cast<uint32_t*>(e1 + so1) = w1;
+        *reinterpret_cast<uint32_t*>(e2 + so2) = w2;
       }
     } else {
-      e1[so] = static_cast<uint8_t>(a + 127);
-      e2[so] = static_cast<uint8_t>(bexp + 127);
+      e1[so1] = static_cast<uint8_t>(a + 127);
+      e2[so2] = static_cast<uint8_t>(bexp + 127);
     }
     }
   }

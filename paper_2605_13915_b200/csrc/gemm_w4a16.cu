@@ -10,8 +10,8 @@
 // (token tile, weight tile, K split) in an order chosen by which operand stays in L2.
 //
 // Warps: 0 = operand producer, 1 = MMA issuer + TMEM owner, 2..5 = epilogue (TMEM -> BF16/FP32 -> swizzled staging
-// buffer -> TMA store), 6..9 = scale warps, 10 = scale producer.  The same kernel serves the grouped
-// (mixture-of-experts) entry point: group g is token tile g.  gemm_w4a16_pair_kernel is the opt-in cta_group::2 variant.
+// buffer -> TMA store), 6..9 = scale warps, 10 = scale producer.  gemm_w4a16_pair_kernel is the cta_group::2 variant for prefill
+// shapes; few tokens per weight matrix and mixture-of-experts calls run in gemm_w4a16_decode.cu.
 #include <cuda_bf16.h>
 
 #include <cstdlib>
@@ -46,21 +46,11 @@ struct GemmW4Params {
   int part_rows;                // ksplit > 1: rows per split of the partial-sum buffer the tiles are written to
   int nstages;                  // pipeline stages that fit with a_rows rows per component tile
   int a_rows;                   // rows of a token tile that are loaded (the box of the component tensor maps): 128, or
-                                // fewer when no group of a grouped launch is longer; the MMA reads stale rows beyond them,
+                                // fewer when there is one token tile; the MMA reads stale rows beyond them,
                                 // whose results are never stored
   int n_fastest;                // tile index -> (token tile, weight tile): weight tile fastest (1) or token tile fastest (0)
   unsigned* status;
 };
-
-// Mixture-of-experts launch: token tile g holds the rows of group g (at most 128), which multiply the weights of expert
-// expert[g]; the rows of the result go to y rows off[g] ...
-struct GemmW4Groups {
-  int n;
-  int expert[kMaxRowGroups], off[kMaxRowGroups + 1];
-};
-struct GemmW4NoGroups {};
-template <bool kGrouped> struct W4GroupArg { using type = GemmW4NoGroups; };
-template <> struct W4GroupArg<true> { using type = GemmW4Groups; };
 
 // Sum of the K-split partial tiles, split 0 first (fixed order: the same inputs give the same bits), rounded once.
 __global__ void __launch_bounds__(256)
@@ -100,12 +90,12 @@ msd_status_t launch_ksplit_reduce(const float* part, int ksplit, int64_t part_st
 // kCluster: one token tile of at most 128 rows, one work item per CTA, and the K splits of a weight tile are the CTAs of a
 // thread-block cluster: when all of them are done every CTA writes the columns that a peer finishes into that peer's
 // shared memory (the drained pipeline), and after a second cluster barrier sums its own columns, split 0 first.  Without it
-// the FP32 partial tiles went through memory and a reduce kernel of their own (see w4_decode_shape).
-template <int kTN, bool kGrouped = false, bool kCluster = false>
+// the FP32 partial tiles went through memory and a reduce kernel of their own (see w4_tile_decode_shape).
+template <int kTN, bool kCluster = false>
 __global__ void __launch_bounds__(kW4ThreadsSf, 1)
 gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_a2,
                   const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_y,
-                  const GemmW4Params p, const typename W4GroupArg<kGrouped>::type grp) {
+                  const GemmW4Params p) {
   constexpr int kBBytes = kTN * 128;
   // Shared-memory stage: the two component tiles, the weight tile, the scale blocks.  Launches with few rows (one
   // token tile of M < 128 rows, short groups) load only a_rows <= 128 rows per component (whole 1 KB swizzle atoms), pack the stage accordingly and use the room for more
@@ -141,8 +131,8 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       q.mt = 0;
       q.nt = static_cast<int>(cluster_id());
     } else {
-      const int tile_mn = kGrouped ? q.tile : q.tile / p.ksplit;      // (a grouped launch does not split K)
-      split = kGrouped ? 0 : q.tile - tile_mn * p.ksplit;
+      const int tile_mn = q.tile / p.ksplit;
+      split = q.tile - tile_mn * p.ksplit;
       q.mt = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % p.m_tiles;
       q.nt = p.n_fastest ? tile_mn % p.n_tiles : tile_mn / p.m_tiles;
     }
@@ -158,13 +148,10 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     uint8_t* dst = smem + stage * kStageBytes;
     if (warp == 0) {
       mbar_arrive_expect_tx(&full_bar[stage], kStageBytes);
-      int b_row = q.nt * kTN;
-      if constexpr (kGrouped) b_row += grp.expert[q.mt] * p.N;          // the weights of the group's expert
-      tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, b_row, &full_bar[stage]);
+      tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, q.nt * kTN, &full_bar[stage]);
     } else {
       uint8_t* sf = dst + 2 * a_bytes + kBBytes;
-      size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
-      if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[q.mt]) * 2 * p.n_tiles;
+      const size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
       bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
       if constexpr (kSfbBlocks == 2) bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
     }
@@ -181,14 +168,12 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       bulk_load(sf + 1024, p.sfa2 + a_off, 1024, &full_bar[stage]);
     }
   };
-  constexpr int kGroupedEarly = 2;
   Pos q = {}, first = {};
   int pre = 0;                   // stages whose weights were asked for before the wait on the kernel launched just before
 
-  // Decode shapes (kCluster): warp 0 sets the barriers up, a stage per lane, and asks for the first stages' weight tiles right
-  // away, before the rest of the CTA's set-up (tensor memory, the CTA-wide barrier): 1 token, 4096 x 14336 and back 31.6 us, 32.1 after it
-  // us.  Launches of many items are behind a decomposition of many rows, and asking that early takes bandwidth from it
-  // (32 experts 58.9 us, 57.6 later; 1000 rows 37.9 and 35.5).
+  // kCluster: warp 0 sets the barriers up, a stage per lane, and asks for the first stages' weight tiles right away, before the rest
+  // of the CTA's set-up (tensor memory, the CTA-wide barrier).  Launches of many items are behind a decomposition of many rows, and
+  // asking that early takes bandwidth from it (1000 rows 37.9 us, 35.5 later).
   if constexpr (kCluster) {
     if (warp == 0) {
       if (lane < nstages) { mbar_init(&full_bar[lane], 1); mbar_init(&empty_bar[lane], 1); }
@@ -235,21 +220,18 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     // scale blocks (their bytes may be counted before warp 0's arrival announces them: the phase cannot end without it).
     if (lane == 0) {
       bool ok = true;
-      // (This kernel lets no dependent in early: the waiting decomposition of a next call beside it cost 2 us on 32 experts.)
       if (warp == 10 || !kCluster) {
-        // neither weights nor prepared weight scales depend on the kernel launched just before; a grouped launch asks for two
-        // stages that early and leaves the bandwidth to the decomposition of its many rows (64 experts 38.8 us, 40.2 asking for all; 32: 57.1 and 57.7)
+        // neither weights nor prepared weight scales depend on the kernel launched just before
         q.tile = blockIdx.x;
         enter(q);
         first = q;
         if (warp == 10 && !p.sfb_ready) pdl_wait_primary();
-        for (; pre < (kGrouped ? kGroupedEarly : nstages) && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
+        for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
       }
       // what the decomposition, launched just before, writes: the components and their scales
       if (warp == 0 || p.sfb_ready) pdl_wait_primary();
       q = first;
       for (int i = 0; i < pre; ++i) { load_activations(q, i); advance(q); }
-      if (kGrouped) for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); load_activations(q, pre); advance(q); }
       int stage = pre == nstages ? 0 : pre;
       uint32_t phase = pre == nstages ? 1 : 0;
       while (q.tile < total_tiles) {
@@ -374,17 +356,12 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       ok = wait_bounded(&tfull_bar[acc], tphase, abort, p.status);
       if (!ok) break;
       tc_fence_after();
-      int row0 = mt * kW4TileM + quad * 32;              // first output row of this warp
-      int rows_end = p.M;                                // output rows at or past it belong to nobody (or somebody else)
-      if constexpr (kGrouped) {
-        row0 = grp.off[mt] + quad * 32;
-        rows_end = grp.off[mt + 1];
-      }
+      const int row0 = mt * kW4TileM + quad * 32;        // first output row of this warp
       const uint32_t trow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + acc * kTN;
       // columns of this tile inside the matrix (a warp whose rows are all past M has nothing to store); chunks
       // beyond them are skipped altogether, so every pass through the loop commits exactly one store group
       const int cols_here = p.N - nt * kTN < kTN ? p.N - nt * kTN : kTN;
-      const int cend = row0 < rows_end ? cols_here : 0;
+      const int cend = row0 < p.M ? cols_here : 0;
       if (cend == 0) {
         tc_fence_before();
         __syncwarp();
@@ -411,9 +388,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           if (lane == 0) mbar_arrive(&tempty_bar[acc]);
         }
         uint8_t* sb = stage_buf + buf * kW4StoreBytes;
-        // the store that read this buffer two chunks ago is done with it (grouped launches may skip a commit when a
-        // group ends inside the warp's rows, so there all earlier stores are waited for)
-        if (lane == 0) { if constexpr (kGrouped) bulk_wait_group_read<0>(); else bulk_wait_group_read<1>(); }
+        if (lane == 0) bulk_wait_group_read<1>();      // the store that read this buffer two chunks ago is done with it
         __syncwarp();
         uint8_t* srow = sb + lane * 64;
 #pragma unroll
@@ -421,27 +396,9 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           *reinterpret_cast<uint4*>(srow + ((static_cast<uint32_t>(j) ^ swz) << 4)) = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
         fence_proxy_async_smem();
         __syncwarp();
-        if (!kGrouped || row0 + 32 <= rows_end) {
-          if (lane == 0) {
-            tma_store_2d(&tmap_y, nt * kTN + c0, row0 + split * p.part_rows, sb);
-            bulk_commit_group();
-          }
-        } else {
-          // the group ends inside this warp's 32 rows: the rows below belong to the next group, so the box store
-          // is replaced by 16-byte stores of the group's own rows (lane -> row lane / 4 + 8 i, 16-byte piece lane % 4)
-          const int esize = (p.ytype == MSD_OUT_BF16) ? 2 : 4;
-          const int col = nt * kTN + c0, piece = lane & 3;
-          if ((col + (piece + 1) * (16 / esize)) <= p.N) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int r = (lane >> 2) + 8 * i;
-              if (row0 + r < rows_end) {
-                const uint4 v = *reinterpret_cast<const uint4*>(sb + r * 64 + ((static_cast<uint32_t>(piece) ^ static_cast<uint32_t>((r >> 1) & 3)) << 4));
-                *reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.y) + (static_cast<size_t>(row0 + r) * p.N + col) * esize + piece * 16) = v;
-              }
-            }
-          }
-          __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&tmap_y, nt * kTN + c0, row0 + split * p.part_rows, sb);
+          bulk_commit_group();
         }
       }
     }
@@ -806,6 +763,8 @@ gemm_w4a16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid
 struct GemmW4Plan {
   int m_tiles, n_tiles, kstages, sf_kgroups, grid, tile_n;
   int cluster;                  // > 1: K splits of a weight tile = CTAs of a cluster (kCluster)
+  bool few;                     // few tokens: the kernel of gemm_w4a16_decode.cu, cut up as `d` says
+  W4DecodeShape d;
   int sf_tile_rows;             // weight rows per tile of the blocked scale layout (224 or 256; 128-row tiles use 256)
   int ksplit, kper, a_rows, nstages;
   size_t off_q1, off_q2, off_sfa1, off_sfa2, off_sfb, off_part, bytes;
@@ -835,9 +794,9 @@ static int w4_tile_n(bool pair = false) {
   return pair ? 256 : 224;
 }
 
-using W4Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmW4Params, GemmW4NoGroups);
+using W4Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmW4Params);
 static W4Kernel w4_cluster_kernel(int tile_n) {
-  return tile_n == 128 ? gemm_w4a16_kernel<128, false, true> : tile_n == 224 ? gemm_w4a16_kernel<224, false, true> : gemm_w4a16_kernel<256, false, true>;
+  return tile_n == 128 ? gemm_w4a16_kernel<128, true> : tile_n == 224 ? gemm_w4a16_kernel<224, true> : gemm_w4a16_kernel<256, true>;
 }
 
 // How many clusters of S CTAs of that kernel the device holds at once (0 on error).
@@ -890,7 +849,7 @@ static void w4_stages(int a_rows, int tile_n, size_t extra_bytes, int* nstages, 
 // through memory: no split gains anything or none fits; few stages (then exchange and cluster cost more than the stages saved: 125
 // tokens, 15904 x 1280 11.5 us split, 10.1 whole); or a single weight tile with so many stages that eight CTAs are too few
 // (1 token, 8 x 14592: 12.1 us in eight, 10.0 in fourteen through memory).
-static void w4_decode_shape(int64_t M, int64_t N, int kstages, int* tile_n, int* cluster) {
+static void w4_tile_decode_shape(int64_t M, int64_t N, int kstages, int* tile_n, int* cluster) {
   const int a_rows = static_cast<int>((M + 7) / 8 * 8);
   *cluster = 1;
   if (N <= 224 && kstages > 28) return;
@@ -917,17 +876,31 @@ static void w4_decode_shape(int64_t M, int64_t N, int kstages, int* tile_n, int*
   }
 }
 
+// Calls of at most 128 tokens that the kernel of gemm_w4a16_decode.cu takes: all where it leaves K whole, and up to 32 tokens where it
+// splits it (then the sums exchanged and the components each CTA loads grow with the tokens, and tiles of 128 tokens x 128 to 256
+// weight rows with half as many CTAs per row cost less: 4096 x 14336, 16 tokens 12.7 us here and 15.1 there, 61 tokens 16.5
+// and 15.0; 2560 x 9984, 29 tokens 10.7 and 12.0; K whole, 14336 x 4096, 61 tokens 12.5 and 14.4, 128 tokens 15.4 and 16.0).
+// One weight tile with so long a K that eight CTAs are too few for it is split through memory.
+static bool w4_decode_takes(W4DecodeShape* d, int64_t M, int64_t N, int64_t K, int kstages) {
+  const int forced = option(OPT_W4_DECODE);          // testing aid: 0 never, a shape wherever it fits
+  if (M > kW4TileM || forced == 0 || (N <= 224 && kstages > 28)) return false;
+  return w4_decode_shape(d, static_cast<int>(M), 0, N, K) && (forced > 0 || d->S == 1 || M <= 32);
+}
+
 static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   GemmW4Plan pl;
   int tile_n = w4_tile_n(w4_use_pair(M, N, K));
   pl.cluster = 1;
-  if (M <= kW4TileM && option(OPT_W4_TILEN) < 0 && option(OPT_W4_KSPLIT) < 0 && option(OPT_W4_PAIR) < 0)
-    w4_decode_shape(M, N, static_cast<int>((K + kW4BlockK - 1) / kW4BlockK), &tile_n, &pl.cluster);
-  pl.sf_tile_rows = tile_n == 224 ? 224 : 256;
+  pl.few = false;
+  pl.kstages = static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
+  if (M <= kW4TileM && option(OPT_W4_TILEN) < 0 && option(OPT_W4_KSPLIT) < 0 && option(OPT_W4_PAIR) < 0) {
+    pl.few = w4_decode_takes(&pl.d, M, N, K, pl.kstages);
+    if (!pl.few) w4_tile_decode_shape(M, N, pl.kstages, &tile_n, &pl.cluster);
+  }
+  pl.sf_tile_rows = tile_n == 224 && !pl.few ? 224 : 256;
   pl.tile_n = tile_n;
   pl.m_tiles = static_cast<int>((M + kW4TileM - 1) / kW4TileM);
   pl.n_tiles = static_cast<int>((N + tile_n - 1) / tile_n);
-  pl.kstages = static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
   pl.sf_kgroups = 2 * pl.kstages;
   const int tiles = pl.m_tiles * pl.n_tiles;
   // Few output tiles and a long K (decode shapes): split K so that there is about one work item per SM, each at
@@ -956,6 +929,14 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   size_t stage_bytes;
   w4_stages(pl.a_rows, tile_n, pl.cluster > 1 ? 0 : 8 * kW4StoreBytes, &pl.nstages, &stage_bytes);
   size_t off = 0;
+  if (pl.few) {                 // components and their scales as one stack of rows
+    pl.off_q1 = off;   off = round_up(off + static_cast<size_t>(pl.d.Mp + M) * (K / 2), 1024);
+    pl.off_q2 = pl.off_q1 + static_cast<size_t>(pl.d.Mp) * (K / 2);
+    pl.off_sfa1 = pl.off_sfa2 = off; off = round_up(off + static_cast<size_t>(pl.d.nsfx) * pl.sf_kgroups * 512, 1024);
+    pl.off_sfb = off;  off = round_up(off + static_cast<size_t>(2 * ((N + 255) / 256)) * pl.sf_kgroups * 512, 1024);
+    pl.off_part = pl.bytes = off;
+    return pl;
+  }
   pl.off_q1 = off;   off = round_up(off + static_cast<size_t>(M) * (K / 2), 1024);
   pl.off_q2 = off;   off = round_up(off + static_cast<size_t>(M) * (K / 2), 1024);
   pl.off_sfa1 = off; off = round_up(off + static_cast<size_t>(pl.m_tiles) * pl.sf_kgroups * 512, 1024);
@@ -968,35 +949,19 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
 }
 
 // ---- grouped (mixture of experts) ----------------------------------------------------------------------------------
-// Workspace: components of up to 64 groups at a time as token tiles of 128 rows, their scale blocks, and the blocked
-// scales of all experts' weights.
+// Workspace: stacked components of up to 64 groups at a time, their scale blocks, and the blocked scales of all experts' weights.
 struct GroupedW4Plan {
-  int n_tiles, kstages, sf_kgroups, tile_n;
-  size_t off_q1, off_q2, off_sfa1, off_sfa2, off_sfb, bytes;
+  int sf_kgroups, row_blocks;
+  size_t off_q, off_sfx, off_sfw, bytes;
 };
-static GroupedW4Plan plan_grouped_w4(int32_t E, int64_t N, int64_t K, int groups) {
+static GroupedW4Plan plan_grouped_w4(int32_t E, int64_t N, int64_t K) {
   GroupedW4Plan pl;
-  // Tile width: the one whose tiles fill the SMs in fewer, or shorter, rounds (groups = non-empty groups of the first
-  // launch; the workspace is sized for the wider layout of the blocked weight scales either way)
-  if (const int forced = option(OPT_W4_TILEN); forced >= 0) {
-    pl.tile_n = forced == 256 ? 256 : 224;
-  } else {
-    const long long g = groups < 1 ? 1 : (groups > kMaxRowGroups ? kMaxRowGroups : groups);
-    const long long t224 = g * ((N + 223) / 224), t256 = g * ((N + 255) / 256);
-    const long long c224 = (t224 + sm_count() - 1) / sm_count() * 224, c256 = (t256 + sm_count() - 1) / sm_count() * 256;
-    pl.tile_n = c256 < c224 ? 256 : 224;
-  }
-  pl.n_tiles = static_cast<int>((N + pl.tile_n - 1) / pl.tile_n);
-  pl.kstages = static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
-  pl.sf_kgroups = 2 * pl.kstages;
-  const size_t rows = static_cast<size_t>(kMaxRowGroups) * kW4TileM;
+  pl.sf_kgroups = 2 * static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
+  pl.row_blocks = 2 * static_cast<int>((N + 255) / 256);
   size_t off = 0;
-  pl.off_q1 = off;   off = round_up(off + rows * (K / 2), 1024);
-  pl.off_q2 = off;   off = round_up(off + rows * (K / 2), 1024);
-  pl.off_sfa1 = off; off = round_up(off + static_cast<size_t>(kMaxRowGroups) * pl.sf_kgroups * 512, 1024);
-  pl.off_sfa2 = off; off = round_up(off + static_cast<size_t>(kMaxRowGroups) * pl.sf_kgroups * 512, 1024);
-  // (N + 223) / 224 tiles is the larger count of the two widths
-  pl.off_sfb = off;  off = round_up(off + static_cast<size_t>(E) * 2 * ((N + 223) / 224) * pl.sf_kgroups * 512, 1024);
+  pl.off_q = off;   off = round_up(off + static_cast<size_t>(kMaxRowGroups) * 2 * kW4TileM * (K / 2), 1024);
+  pl.off_sfx = off; off = round_up(off + static_cast<size_t>(kMaxRowGroups) * 2 * pl.sf_kgroups * 512, 1024);
+  pl.off_sfw = off; off = round_up(off + static_cast<size_t>(E) * pl.row_blocks * pl.sf_kgroups * 512, 1024);
   pl.bytes = off;
   return pl;
 }
@@ -1115,9 +1080,14 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
     const PreparedScales ps = prepared_scales_layout(1, N, K);
     sfb = prepared + (pl.sf_tile_rows == 224 ? ps.off224 : ps.off256);
   }
+  RowGroups rg = {};
+  if (pl.few) rg.srow2 = pl.d.Mp;
   msd_status_t st = launch_decompose_mxfp4(x_bf16, M, K, K, q1, q2, ws + pl.off_sfa1, ws + pl.off_sfa2, pl.sf_kgroups, s,
-                                           prepared ? nullptr : &rl);
+                                           prepared ? nullptr : &rl, &rg);
   if (st != MSD_OK) return st;
+  if (pl.few)
+    return w4_decode_launch(pl.d, w_fp4, q1, pl.d.Mp + M, N, static_cast<int>(M), N, K, sfb, prepared != nullptr, ws + pl.off_sfa1, y,
+                            static_cast<int>(ytype), 0, nullptr, nullptr, status, s);
 
   CUtensorMap tmap_a1, tmap_a2, tmap_b;
   const uint64_t kb = static_cast<uint64_t>(K / 2);
@@ -1180,20 +1150,20 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
     size_t stage_bytes;
     w4_stages(pl.a_rows, pl.tile_n, 0, &nstages, &stage_bytes);
     if (launch_pdl_cluster(w4_cluster_kernel(pl.tile_n), dim3(pl.grid), dim3(kW4ThreadsSf), nstages * stage_bytes + 1024, s, pdl,
-                           static_cast<unsigned>(pl.cluster), tmap_a1, tmap_a2, tmap_b, tmap_y, p, GemmW4NoGroups()) != cudaSuccess)
+                           static_cast<unsigned>(pl.cluster), tmap_a1, tmap_a2, tmap_b, tmap_y, p) != cudaSuccess)
       return MSD_ERR_CUDA;
     return MSD_OK;
   }
   const size_t smem_bytes = static_cast<size_t>(pl.nstages) * (2 * pl.a_rows * 128 + pl.tile_n * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
   static DeviceOnce once;
   if (!once([] {
-        return cudaFuncSetAttribute(gemm_w4a16_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
-               cudaFuncSetAttribute(gemm_w4a16_kernel<224, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
+        return cudaFuncSetAttribute(gemm_w4a16_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w4a16_kernel<224>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
       }))
     return MSD_ERR_CUDA;
   const cudaError_t le = pl.tile_n == 256
-      ? launch_pdl(gemm_w4a16_kernel<256, false>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, GemmW4NoGroups())
-      : launch_pdl(gemm_w4a16_kernel<224, false>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, GemmW4NoGroups());
+      ? launch_pdl(gemm_w4a16_kernel<256>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p)
+      : launch_pdl(gemm_w4a16_kernel<224>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p);
   if (le != cudaSuccess) return MSD_ERR_CUDA;
   if (split) {
     const msd_status_t rs = launch_ksplit_reduce(part, pl.ksplit, static_cast<int64_t>(part_rows) * N, M, N, y, static_cast<int>(ytype), s, pdl);
@@ -1208,7 +1178,7 @@ extern "C" {
 
 size_t msd_grouped_gemm_w4a16_workspace_bytes(int32_t E, int64_t N, int64_t K) {
   if (E < 1 || N < 1 || K < 128 || K % 128 != 0) return 0;
-  return msd::plan_grouped_w4(E, N, K, E).bytes;
+  return msd::plan_grouped_w4(E, N, K).bytes;
 }
 
 msd_status_t msd_grouped_gemm_w4a16(const void* x_bf16, const uint8_t* w_fp4, const uint8_t* w_e8m0,
@@ -1241,98 +1211,61 @@ static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w
       !aligned(workspace, 1024))
     return MSD_ERR_BAD_ALIGNMENT;
   int64_t M_total = 0;
-  int nonempty = 0, largest = 0;
+  int largest = 0;
   for (int e = 0; e < E; ++e) {
     if (group_sizes_host[e] < 0 || group_sizes_host[e] > kW4TileM) return MSD_ERR_BAD_SHAPE;     // decode regime per expert
     M_total += group_sizes_host[e];
-    nonempty += group_sizes_host[e] > 0 ? 1 : 0;
     if (group_sizes_host[e] > largest) largest = group_sizes_host[e];
   }
   if (M_total > 0x7FFFFFFFLL) return MSD_ERR_BAD_SHAPE;
-  const GroupedW4Plan pl = plan_grouped_w4(E, N, K, nonempty);
-  const int a_rows = (largest + 7) / 8 * 8;             // rows of a token tile worth loading (whole 8-row swizzle atoms)
+  const GroupedW4Plan pl = plan_grouped_w4(E, N, K);
   if (workspace_bytes < pl.bytes) return MSD_ERR_WORKSPACE_TOO_SMALL;
   if (M_total == 0) return MSD_OK;
   unsigned* status = device_status_ptr();
   if (!status) return MSD_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  uint8_t* q1 = ws + pl.off_q1;
-  uint8_t* q2 = ws + pl.off_q2;
-  const bool ybf = ytype == MSD_OUT_BF16;
-  const uint64_t kb = static_cast<uint64_t>(K / 2);
-  CUtensorMap tmap_a1, tmap_a2, tmap_b, tmap_y;
-  if (!encode_tmap_2d(&tmap_a1, CU_TENSOR_MAP_DATA_TYPE_UINT8, q1, kb, static_cast<uint64_t>(kMaxRowGroups) * kW4TileM, kb, 128, static_cast<uint32_t>(a_rows), CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_tmap_2d(&tmap_a2, CU_TENSOR_MAP_DATA_TYPE_UINT8, q2, kb, static_cast<uint64_t>(kMaxRowGroups) * kW4TileM, kb, 128, static_cast<uint32_t>(a_rows), CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_tmap_2d(&tmap_b, CU_TENSOR_MAP_DATA_TYPE_UINT8, w_fp4, kb, static_cast<uint64_t>(E) * N, kb, 128, static_cast<uint32_t>(pl.tile_n), CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_tmap_2d(&tmap_y, ybf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, y, static_cast<uint64_t>(N),
-                      static_cast<uint64_t>(M_total), static_cast<uint64_t>(N) * (ybf ? 2 : 4), ybf ? 32 : 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
-    return MSD_ERR_CUDA;
-  const size_t stage_bytes = static_cast<size_t>(2 * a_rows * 128 + pl.tile_n * 128 + kW4SfBytes);
-  int nstages = static_cast<int>((227 * 1024 - 2048 - 8 * kW4StoreBytes - 1024) / stage_bytes);
-  if (nstages > 8) nstages = 8;
-  const size_t smem_bytes = nstages * stage_bytes + 8 * kW4StoreBytes + 1024;
-  static DeviceOnce once;
-  if (!once([] {
-        return cudaFuncSetAttribute(gemm_w4a16_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
-               cudaFuncSetAttribute(gemm_w4a16_kernel<224, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
-      }))
-    return MSD_ERR_CUDA;
-  const bool pdl = option(OPT_NO_PDL) <= 0;
+  uint8_t* q = ws + pl.off_q;
+  uint8_t* sfx = ws + pl.off_sfx;
 
   // up to 64 non-empty groups per pair of launches (decomposition + GEMM); the weight scales of all experts are brought
   // into the blocked layout by the first decomposition launch
   bool scales_done = prepared != nullptr;
-  const uint8_t* sfb = ws + pl.off_sfb;
-  if (prepared) {
-    const PreparedScales ps = prepared_scales_layout(E, N, K);
-    sfb = prepared + (pl.tile_n == 224 ? ps.off224 : ps.off256);
-  }
+  const uint8_t* sfw = prepared ? prepared + prepared_scales_layout(E, N, K).off256 : ws + pl.off_sfw;
   int e = 0;
   int64_t row = 0;
   while (e < E) {
-    GemmW4Groups grp = {};
+    int expert[kMaxRowGroups], off[kMaxRowGroups + 1];
     RowGroups rg = {};
     const int64_t row_first = row;
-    while (e < E && grp.n < kMaxRowGroups) {
+    while (e < E && rg.n < kMaxRowGroups) {
       const int sz = group_sizes_host[e];
       if (sz > 0) {
-        grp.expert[grp.n] = e;
-        grp.off[grp.n] = static_cast<int>(row);
-        rg.off[grp.n] = static_cast<int>(row - row_first);
+        expert[rg.n] = e;
+        off[rg.n] = static_cast<int>(row);
+        rg.off[rg.n] = static_cast<int>(row - row_first);
         row += sz;
-        ++grp.n;
+        ++rg.n;
       }
       ++e;
     }
-    if (grp.n == 0) break;
-    grp.off[grp.n] = static_cast<int>(row);
-    rg.off[grp.n] = static_cast<int>(row - row_first);
-    rg.n = grp.n;
+    if (rg.n == 0) break;
+    off[rg.n] = static_cast<int>(row);
+    rg.off[rg.n] = static_cast<int>(row - row_first);
+    W4DecodeShape d;
+    if (!w4_decode_shape(&d, largest, rg.n, N, K)) return MSD_ERR_UNSUPPORTED;      // (one exists for every call accepted above)
+    rg.rows = d.NB; rg.srows = 128 * d.nsfx; rg.srow2 = d.Mp;
     SfRelayout rl = {};
-    rl.src = w_e8m0; rl.dst = ws + pl.off_sfb; rl.rows = N; rl.kblocks = static_cast<int>(K / 32);
-    rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = pl.tile_n; rl.row_blocks = 2 * pl.n_tiles; rl.matrices = E;
-    msd_status_t st = launch_decompose_mxfp4(static_cast<const uint16_t*>(x_bf16) + row_first * K, row - row_first, K, K, q1, q2,
-                                             ws + pl.off_sfa1, ws + pl.off_sfa2, pl.sf_kgroups, s, scales_done ? nullptr : &rl, &rg);
+    rl.src = w_e8m0; rl.dst = ws + pl.off_sfw; rl.rows = N; rl.kblocks = static_cast<int>(K / 32);
+    rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = 256; rl.row_blocks = pl.row_blocks; rl.matrices = E;
+    msd_status_t st = launch_decompose_mxfp4(static_cast<const uint16_t*>(x_bf16) + row_first * K, row - row_first, K, K, q,
+                                             q + static_cast<size_t>(d.Mp) * (K / 2), sfx, sfx, pl.sf_kgroups, s, scales_done ? nullptr : &rl, &rg);
+    if (st != MSD_OK) return st;
+    // (a later launch finds weight scales that the first one's decomposition laid out: complete before its own began)
+    st = w4_decode_launch(d, w_fp4, q, static_cast<int64_t>(rg.n) * d.NB, static_cast<int64_t>(E) * N, 0, N, K, sfw, scales_done, sfx, y,
+                          static_cast<int>(ytype), rg.n, expert, off, status, s);
     if (st != MSD_OK) return st;
     scales_done = true;
-
-    GemmW4Params p;
-    p.M = static_cast<int>(M_total); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
-    p.m_tiles = grp.n; p.n_tiles = pl.n_tiles; p.kstages = pl.kstages; p.sf_kgroups = pl.sf_kgroups;
-    p.sfa1 = ws + pl.off_sfa1; p.sfa2 = ws + pl.off_sfa2; p.sfb = sfb; p.sfb_ready = prepared != nullptr;
-    p.y = y; p.ytype = ytype; p.status = status;
-    p.a_rows = a_rows; p.nstages = nstages;
-    p.ksplit = 1; p.kper = pl.kstages; p.part_rows = 0;
-    p.n_fastest = 1;              // the CTAs of a wave share a group's components; every expert's weights are read once
-    {
-    }
-    const long long tiles = static_cast<long long>(grp.n) * pl.n_tiles;
-    const int grid = static_cast<int>(tiles < sm_count() ? tiles : sm_count());
-    const cudaError_t le = pl.tile_n == 256
-        ? launch_pdl(gemm_w4a16_kernel<256, true>, dim3(grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, grp)
-        : launch_pdl(gemm_w4a16_kernel<224, true>, dim3(grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, grp);
-    if (le != cudaSuccess) return MSD_ERR_CUDA;
   }
   return MSD_OK;
 }

@@ -27,6 +27,7 @@ enum Option {
   OPT_W4_PAIR,              // MSD_W4_PAIR: W4A16 kernel on CTA pairs (1) or single CTAs (0)
   OPT_W4_TILEN,             // MSD_W4_TILEN: tile width of the single-CTA W4A16 kernel (224 or 256)
   OPT_W4_KSPLIT,            // MSD_W4_KSPLIT: its K split
+  OPT_W4_DECODE,            // MSD_W4_DECODE: shape of the few-token W4A16 kernel: 100000 kw + 1000 CTAs per band + rows per band
   OPT_ATTN_SPLITS,          // MSD_ATTN_SPLITS: number of context splits of the attention kernels
   OPT_ATTN_CHUNK_TILES,     // MSD_ATTN_CHUNK_TILES: tiles per context split
   OPT_ATTN_BALANCED,        // MSD_ATTN_BALANCED: 1 balanced schedule wherever a kernel for it exists, 0 never
@@ -142,16 +143,32 @@ struct SfRelayout {
                        // weights), each cut into its own `row_blocks` blocks
   int blocks;          // filled in by the launcher
 };
-// Rows sorted by group (mixture of experts): group g owns rows [off[g], off[g+1]) and its decomposition is written as
-// token tile g (rows 128 g ...) of the component and scale buffers.
+// Rows sorted by group (mixture of experts): group g owns rows [off[g], off[g+1]) and its decomposition is written to rows
+// g * rows ... of the component buffers and rows g * srows ... of the scale buffers.
 constexpr int kMaxRowGroups = 64;
 struct RowGroups {
   int n;                       // 0: no regrouping, output row = input row
+  int rows, srows;             // rows per group in the component buffers / in the scale buffers (128-row blocks)
+  int srow2;                   // the second component's scales are this many rows further down (stacked components)
   int off[kMaxRowGroups + 1];
 };
 msd_status_t launch_decompose_mxfp4(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, uint8_t* q1, uint8_t* q2,
                                     uint8_t* e1, uint8_t* e2, int sf_kgroups, cudaStream_t stream,
                                     SfRelayout* relayout = nullptr, const RowGroups* groups = nullptr);
+
+// W4A16 layers with few tokens per weight matrix (gemm_w4a16_decode.cu): how the kernel cuts a call up, and its launch.
+// Components: one stack [Q1 (Mp rows); Q2] per group of NB rows; scales: nsfx blocks of 128 stacked rows per group.
+struct W4DecodeShape {
+  int h, kw, S;                        // weight rows per band, 256-element K blocks per stage, CTAs (K splits) per band
+  int Mp, NB, nsfx, kblocks, ksteps, kper, bands, items, grid;
+  int x_off, sf_off, stage_bytes, nstages, set_cols, nsets, sf_col, nacc, epi_off, smem;
+};
+// (groups: matrices of a grouped launch, 0 for an ungrouped call)
+bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K);
+// expert == nullptr: one matrix, M tokens; otherwise `nonempty` groups, group g = rows [off[g], off[g + 1]) of y and weights expert[g]
+msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, const uint8_t* q, int64_t q_rows, int64_t w_rows, int M, int64_t N,
+                              int64_t K, const uint8_t* sfw, bool sfw_ready, const uint8_t* sfx, void* y, int ytype, int nonempty,
+                              const int* expert, const int* off, unsigned* status, cudaStream_t s);
 
 #ifdef __CUDACC__
 // Relayout of row-major E8M0 scales [rows, kblocks] into the 512-byte blocks (128 rows x 4 scales) of the block-scaled

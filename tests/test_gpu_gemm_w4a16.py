@@ -150,3 +150,23 @@ def test_decode_k_split_as_a_cluster(M, N, K):
     binding.last_device_status()
     assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
     _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)
+
+
+@pytest.mark.parametrize("M,N,K,kw,S,h", [(1, 8, 128, 1, 1, 128), (16, 1000, 1152, 2, 1, 96), (33, 264, 3072, 4, 2, 40), (64, 2056, 1408, 1, 3, 112),
+                                          (65, 392, 4096, 2, 8, 128), (128, 520, 1024, 2, 2, 104), (7, 20488, 512, 2, 1, 128), (128, 20480, 384, 1, 1, 112)])
+def test_few_token_kernel_in_every_shape(M, N, K, kw, S, h):
+    """The few-token kernel with its shape given: every stage width, K whole and split over clusters of 2 to 8 CTAs (uneven last splits,
+    stages with fewer K blocks than they hold, a K that ends inside a block), bands that cross 128-row scale blocks, a ragged last
+    band, one and two scale blocks of components, several bands a CTA with one and two accumulators.  Row-major and prepared scales
+    give the same bits, FP32 against the oracle, BF16 the FP32 result rounded once."""
+    c = inputs.gemm_w4_case(M, N, K, seed=5 + M + N)
+    x, w, e = bf16_dev(c.x), dev(c.w_fp4), dev(c.w_e8m0)
+    binding.debug_set_option("MSD_W4_DECODE", 100000 * kw + 1000 * S + h)
+    y = binding.gemm_w4a16(x, w, e, out_dtype=torch.float32)
+    prep = binding.prepare_w4a16_scales(e)
+    y2 = binding.gemm_w4a16(x, w, None, out_dtype=torch.float32, prepared=prep)
+    yb = binding.gemm_w4a16(x, w, None, out_dtype=torch.bfloat16, prepared=prep)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
+    _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)
