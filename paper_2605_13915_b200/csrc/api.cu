@@ -108,10 +108,13 @@ static TmapSlot g_tmap_cache[kTmapCacheSlots];
 static std::mutex g_tmap_mu;
 
 static bool encode_cached(CUtensorMap* out, const TmapKey& k) {
+  // (everything is mixed in before the multiplication that brings it to the top: maps of one buffer that differ in their boxes only
+  // would otherwise share a slot and be encoded anew on every call)
   uint64_t h = reinterpret_cast<uintptr_t>(k.base) * 0x9E3779B97F4A7C15ull;
-  h ^= (k.dims[0] * 31 + k.dims[1]) * 0xC2B2AE3D27D4EB4Full + k.dims[2] * 131 + k.box[0] * 7 + k.box[1] * 3 + k.box[2] + k.strides[0] +
-       static_cast<uint64_t>(k.swizzle) * 17 + static_cast<uint64_t>(k.dtype);
-  TmapSlot& slot = g_tmap_cache[(h >> 20) % kTmapCacheSlots];
+  for (const uint64_t v : {k.dims[0], k.dims[1], k.dims[2], k.strides[0], static_cast<uint64_t>(k.box[0]), static_cast<uint64_t>(k.box[1]),
+                           static_cast<uint64_t>(k.box[2]), static_cast<uint64_t>(k.swizzle * 32 + k.dtype)})
+    h = (h ^ v) * 0x9E3779B97F4A7C15ull;
+  TmapSlot& slot = g_tmap_cache[(h >> 32) % kTmapCacheSlots];
   {
     std::lock_guard<std::mutex> lock(g_tmap_mu);
     if (slot.used && slot.key == k) { *out = slot.map; return true; }
