@@ -122,13 +122,15 @@ decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, i
     const int64_t row_in = b / kblocks;
     const int kb = static_cast<int>(b - row_in * kblocks);
     const uint4* src = reinterpret_cast<const uint4*>(x + row_in * ldx + kb * 32);
-    int64_t row = row_in, srow = row_in;    // where the row's components and scales go
+    int64_t row = row_in, srow = row_in;    // where the row's first component and its scales go
+    int second = rg.second;                 // rows from there to the second component's
     if (rg.n > 0) {
       int g = 0;
       for (int step = kMaxRowGroups / 2; step > 0; step >>= 1)
         if (g + step < rg.n && row_in >= rg.off[g + step]) g += step;
       row = static_cast<int64_t>(g) * rg.rows + (row_in - rg.off[g]);
       srow = static_cast<int64_t>(g) * rg.srows + (row_in - rg.off[g]);
+      second = (rg.off[g + 1] - rg.off[g] + 7) & ~7;
     }
     uint32_t w[16];
 #pragma unroll
@@ -163,13 +165,13 @@ decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, i
       o2[i >> 2] |= static_cast<uint32_t>(c2) << (8 * (i & 3));
     }
     *reinterpret_cast<uint4*>(q1 + row * (K >> 1) + kb * 16) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
-    *reinterpret_cast<uint4*>(q2 + row * (K >> 1) + kb * 16) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
+    *reinterpret_cast<uint4*>(q2 + (row + second) * (K >> 1) + kb * 16) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
     // sf_kgroups == 0: row-major [M, K/32]; otherwise the 512-byte blocks (128 rows x 4 scales) the block-scaled
     // MMA's shared-memory -> TMEM scale copy expects: block (row/128, kb/4), byte (row%32)*16 + ((row/32)%4)*4 + kb%4
     auto scale_at = [&](int64_t r) {
       return sf_kgroups == 0 ? r * kblocks + kb : ((r >> 7) * sf_kgroups + (kb >> 2)) * 512 + (r & 31) * 16 + ((r >> 5) & 3) * 4 + (kb & 3);
     };
-    const int64_t so1 = scale_at(srow), so2 = scale_at(srow + rg.srow2);
+    const int64_t so1 = scale_at(srow), so2 = scale_at(srow + second);
     if (pack4) {
       // four neighbouring lanes hold the four scales of one aligned 32-bit word (kblocks is a multiple of 4)
       uint32_t w1 = static_cast<uint32_t>(a + 127) << (8 * (threadIdx.x & 3)), w2 = static_cast<uint32_t>(bexp + 127) << (8 * (threadIdx.x & 3));

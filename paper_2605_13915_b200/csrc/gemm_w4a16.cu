@@ -931,7 +931,7 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   size_t off = 0;
   if (pl.few) {                 // components and their scales as one stack of rows
     pl.off_q1 = off;   off = round_up(off + static_cast<size_t>(pl.d.Mp + M) * (K / 2), 1024);
-    pl.off_q2 = pl.off_q1 + static_cast<size_t>(pl.d.Mp) * (K / 2);
+    pl.off_q2 = pl.off_q1;
     pl.off_sfa1 = pl.off_sfa2 = off; off = round_up(off + static_cast<size_t>(pl.d.nsfx) * pl.sf_kgroups * 512, 1024);
     pl.off_sfb = off;  off = round_up(off + static_cast<size_t>(2 * ((N + 255) / 256)) * pl.sf_kgroups * 512, 1024);
     pl.off_part = pl.bytes = off;
@@ -1081,7 +1081,7 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
     sfb = prepared + (pl.sf_tile_rows == 224 ? ps.off224 : ps.off256);
   }
   RowGroups rg = {};
-  if (pl.few) rg.srow2 = pl.d.Mp;
+  if (pl.few) rg.second = pl.d.Mp;
   msd_status_t st = launch_decompose_mxfp4(x_bf16, M, K, K, q1, q2, ws + pl.off_sfa1, ws + pl.off_sfa2, pl.sf_kgroups, s,
                                            prepared ? nullptr : &rl, &rg);
   if (st != MSD_OK) return st;
@@ -1254,12 +1254,12 @@ static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w
     rg.off[rg.n] = static_cast<int>(row - row_first);
     W4DecodeShape d;
     if (!w4_decode_shape(&d, largest, rg.n, N, K)) return MSD_ERR_UNSUPPORTED;      // (one exists for every call accepted above)
-    rg.rows = d.NB; rg.srows = 128 * d.nsfx; rg.srow2 = d.Mp;
+    rg.rows = d.NB; rg.srows = 128 * d.nsfx;
     SfRelayout rl = {};
     rl.src = w_e8m0; rl.dst = ws + pl.off_sfw; rl.rows = N; rl.kblocks = static_cast<int>(K / 32);
     rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = 256; rl.row_blocks = pl.row_blocks; rl.matrices = E;
-    msd_status_t st = launch_decompose_mxfp4(static_cast<const uint16_t*>(x_bf16) + row_first * K, row - row_first, K, K, q,
-                                             q + static_cast<size_t>(d.Mp) * (K / 2), sfx, sfx, pl.sf_kgroups, s, scales_done ? nullptr : &rl, &rg);
+    msd_status_t st = launch_decompose_mxfp4(static_cast<const uint16_t*>(x_bf16) + row_first * K, row - row_first, K, K, q, q,
+                                             sfx, sfx, pl.sf_kgroups, s, scales_done ? nullptr : &rl, &rg);
     if (st != MSD_OK) return st;
     // (a later launch finds weight scales that the first one's decomposition laid out: complete before its own began)
     st = w4_decode_launch(d, w_fp4, q, static_cast<int64_t>(rg.n) * d.NB, static_cast<int64_t>(E) * N, 0, N, K, sfw, scales_done, sfx, y,

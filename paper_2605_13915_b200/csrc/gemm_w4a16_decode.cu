@@ -14,6 +14,7 @@
 namespace msd {
 
 constexpr int kDecThreads = 384;                  // weight producer, MMA issuer, four epilogue warps, four scale warps, component and scale producers
+constexpr int kDecBoxes = 4;                      // heights of component boxes in a grouped launch
 constexpr int kDecBlockK = 256;                   // elements per K block (128 packed bytes, one swizzle row)
 constexpr int kDecMaxStages = 16;
 constexpr int kDecMaxSets = 4;
@@ -22,7 +23,7 @@ constexpr int kDecSmem = 227 * 1024 - 2048;
 constexpr int kDecTmemCols = 512;
 
 struct W4DecodeParams {
-  int M, Mp, NB, N;             // tokens (ungrouped), rows reserved per component, MMA N, weight rows of a matrix
+  int M, NB, N;                 // tokens (ungrouped), most stacked component rows of a group, weight rows of a matrix
   int h, bands, items;          // weight rows per band, bands per matrix, bands of all groups
   int kblocks, kw, ksteps;      // 256-element K blocks, of which a stage holds kw; stages that cover K
   int S, kper;                  // CTAs per band (a cluster) and stages each takes
@@ -46,6 +47,10 @@ struct W4DecodeGroups {
   int expert[kMaxRowGroups], off[kMaxRowGroups + 1];
 };
 struct W4DecodeNoGroups {};
+// Component boxes: in a grouped launch of a quarter, half, three quarters and all of NB rows, of which a group loads the smallest that
+// holds its own (32 experts of 2048 x 7168, 6 to 35 tokens each: 51.1 us with one, 49.5 with four).
+template <bool kGrouped> struct W4DecodeXMaps { CUtensorMap m[kGrouped ? kDecBoxes : 1]; };
+__host__ __device__ inline int w4d_box_rows(int NB, int i) { return (NB * (i + 1) / kDecBoxes + 15) / 16 * 16; }
 template <bool kGrouped> struct W4DecodeArg { using type = W4DecodeNoGroups; };
 template <> struct W4DecodeArg<true> { using type = W4DecodeGroups; };
 
@@ -66,7 +71,7 @@ __device__ __forceinline__ void w4d_stage_value(uint8_t* buf, int j, int r, floa
 
 template <bool kGrouped>
 __global__ void __launch_bounds__(kDecThreads, 1)
-gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const W4DecodeParams p,
+gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ W4DecodeXMaps<kGrouped> tmap_x, const W4DecodeParams p,
                          const __grid_constant__ typename W4DecodeArg<kGrouped>::type grp) {
   extern __shared__ uint8_t smem_dyn[];
   __shared__ __align__(8) uint64_t full_bar[kDecMaxStages], empty_bar[kDecMaxStages], tfull_bar[2], tempty_bar[2];
@@ -83,8 +88,21 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
   const int item_step = S > 1 ? p.items : static_cast<int>(gridDim.x);     // (a cluster has one item)
   const int ks0 = rank * p.kper, ks1 = min(ks0 + p.kper, p.ksteps);
 
+  // Stacked component rows of an item's group: two components of ceil8(tokens) rows, and the rows of the box that brings them.
+  struct Rows { int Mp, NB, box, box_rows; };
+  auto rows_of = [&](int item) {
+    Rows r = {p.NB >> 1, p.NB, 0, p.NB};
+    if constexpr (kGrouped) {
+      const int g = item / p.bands;
+      r.Mp = (grp.off[g + 1] - grp.off[g] + 7) & ~7;
+      r.NB = 2 * r.Mp;
+      r.box = 0;
+      while ((r.box_rows = w4d_box_rows(p.NB, r.box)) < r.NB) ++r.box;
+    }
+    return r;
+  };
   // Where an item's operands lie; ks counts stages.
-  struct Pos { int item, ks, w_row, x_row, rb, need2, sfx_off; };
+  struct Pos { int item, ks, w_row, x_row, rb, need2, sfx_off; Rows rows; };
   auto enter = [&](Pos& q) {
     int g = 0, band = q.item, e = 0;
     if constexpr (kGrouped) { g = q.item / p.bands; band = q.item - g * p.bands; e = grp.expert[g]; }
@@ -96,6 +114,7 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     q.need2 = (row0 & 127) + p.h > 128 && q.rb + 1 < p.row_blocks;
     q.rb += e * p.row_blocks;
     q.sfx_off = g * p.nsfx;
+    q.rows = rows_of(q.item);
   };
   auto advance = [&](Pos& q) {
     if (++q.ks < ks1) return;
@@ -110,7 +129,7 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
   auto load_w = [&](const Pos& q, int stage) {
     const int v = valid_blocks(q.ks);
     if (lane == 0)
-      mbar_arrive_expect_tx(&full_bar[stage], static_cast<uint32_t>((p.t3 ? p.kw : v) * (p.h + p.NB) * 128 + v * 1024 * (1 + q.need2 + p.nsfx)));
+      mbar_arrive_expect_tx(&full_bar[stage], static_cast<uint32_t>((p.t3 ? p.kw : v) * (p.h + q.rows.box_rows) * 128 + v * 1024 * (1 + q.need2 + p.nsfx)));
     __syncwarp();
     uint8_t* dst = smem + stage * p.stage_bytes;
     if (p.t3) {
@@ -123,9 +142,9 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
   auto load_x = [&](const Pos& q, int stage) {
     uint8_t* dst = smem + stage * p.stage_bytes + p.x_off;
     if (p.t3) {
-      if (lane == 0) tma_load_3d_hint(dst, &tmap_x, 0, q.x_row, q.ks * p.kw, &full_bar[stage], pol_x);
+      if (lane == 0) tma_load_3d_hint(dst, &tmap_x.m[q.rows.box], 0, q.x_row, q.ks * p.kw, &full_bar[stage], pol_x);
     } else if (lane < valid_blocks(q.ks)) {
-      tma_load_2d_hint(dst + lane * p.NB * 128, &tmap_x, (q.ks * p.kw + lane) * 128, q.x_row, &full_bar[stage], pol_x);
+      tma_load_2d_hint(dst + lane * q.rows.box_rows * 128, &tmap_x.m[q.rows.box], (q.ks * p.kw + lane) * 128, q.x_row, &full_bar[stage], pol_x);
     }
   };
   auto load_sf = [&](const Pos& q, int stage, bool w, bool x) {
@@ -140,7 +159,7 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
 
   Pos q = {}, first = {};
   int pre = 0;
-  const bool producer = warp == 0 || warp >= 10;
+  const bool producer = warp == 0 || warp == 10 || warp == 11;
   if (warp == 0) {
     if (lane < p.nstages) { mbar_init(&full_bar[lane], 1); mbar_init(&empty_bar[lane], 1); }
     if (lane >= 16 && lane < 18) { mbar_init(&tfull_bar[lane - 16], 1); mbar_init(&tempty_bar[lane - 16], 4); }
@@ -149,8 +168,8 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     mbar_init_fence();
     __syncwarp();
     pol_w = policy_evict_first();
-  } else if (threadIdx.x == 64) {
-    tma_prefetch_desc(&tmap_x);
+  } else if (warp == 2 && lane < (kGrouped ? kDecBoxes : 1)) {
+    tma_prefetch_desc(&tmap_x.m[lane]);
   }
   if (producer) {
     pol_x = policy_evict_last();
@@ -198,9 +217,11 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     uint32_t phase = 0, set_phase = 0;
     bool ok = true;
     const uint64_t op_desc = smem_desc(0, 16, 1024, kSwizzle128B);
-    const uint32_t idesc_lo = idesc_block_scaled(/*E2M1*/ 1, 1, 128, p.NB, 0, 0), idesc_hi = idesc_block_scaled(1, 1, 128, p.NB, 2, 2);
-    const int w_blk = p.h * 8, x_blk = p.NB * 8, x_off = p.x_off >> 4;       // in 16-byte units, as descriptors count
+    const int w_blk = p.h * 8, x_off = p.x_off >> 4;       // in 16-byte units, as descriptors count
     for (int item = item0; item < p.items && ok; item += item_step, ++it) {
+      const Rows rows = rows_of(item);
+      const uint32_t idesc_lo = idesc_block_scaled(/*E2M1*/ 1, 1, 128, rows.NB, 0, 0), idesc_hi = idesc_block_scaled(1, 1, 128, rows.NB, 2, 2);
+      const int x_blk = rows.box_rows * 8;
       const int acc = p.nacc == 2 ? (it & 1) : 0;
       const uint32_t tphase = p.nacc == 2 ? ((it >> 1) & 1) : (it & 1);
       const uint32_t d_tmem = tmem_base + acc * p.NB;
@@ -306,12 +327,12 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         ok = named_bar_and(1, 128, wait_bounded(&tfull_bar[acc], tphase, abort, p.status));
         if (!ok) break;
         tc_fence_after();
-        const int n0 = band * p.h, rows = min(p.h, p.N - n0);
+        const int n0 = band * p.h, rows = min(p.h, p.N - n0), Mp = (tokens + 7) & ~7;
         const uint32_t t_row = t_lane + acc * p.NB;
         for (int c0 = 0; c0 < tokens; c0 += 16, buf ^= 1) {
           uint32_t a[16], b[16];
           tmem_ld16(t_row + c0, a);
-          tmem_ld16(t_row + p.Mp + c0, b);      // (a last chunk of 8 tokens reads columns beyond its own, never used)
+          tmem_ld16(t_row + Mp + c0, b);      // (a last chunk of 8 tokens reads columns beyond its own, never used)
           tmem_ld_wait();
           if (c0 + 16 >= tokens) {
             tc_fence_before();
@@ -352,7 +373,7 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         uint32_t a[16], b[16];
         __syncwarp();
         tmem_ld16(t_lane + 4 * g0, a);
-        tmem_ld16(t_lane + p.Mp + 4 * g0, b);
+        tmem_ld16(t_lane + (p.NB >> 1) + 4 * g0, b);
         tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -480,11 +501,11 @@ static bool w4_decode_layout(W4DecodeShape* d, int tokens, int groups, int64_t N
 }
 
 // Band height, stage width and K split by what they cost, in us:
-//   a stage       the largest of 0.4 + 0.16 kw (waits, scales into tensor memory, MMA issue), its bytes at 80 GB/s (what an SM takes in)
-//                 and the weights of all active CTAs' stages at 6.3 TB/s; 1.4 times that with fewer than three stages in flight
+//   a stage       the largest of 0.35 + 0.2 kw (waits, scales into tensor memory, MMA issue), its bytes at 60 GB/s (what an SM takes in)
+//                 and the weights of all active CTAs' stages at 6.3 TB/s; 1.2 times that with fewer than three stages in flight
 //   a K split     1 + tokens (S - 1) / (32 S): two cluster barriers, and the sums sent to the peers
-// Against the best of every (kw, S, height) swept over 30 layers (1 to 128 tokens, 2048 to 16384 x 2048 to 16384) and 15 calls with
-// experts (8 to 60 of them, 8 to 69 tokens the longest group): 1.010 on average, 1.06 at most; bands of 128 rows only 1.013 and 1.19.
+// Against the best of every (kw, S, height) swept over 30 layers (1 to 128 tokens, 2048 to 16384 x 2048 to 16384) and 26 calls with
+// experts (9 to 64 of them, 6 to 77 tokens the longest group): 1.013 on average, 1.10 at most.
 bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K) {
   const int sms = sm_count();
   if (const int forced = option(OPT_W4_DECODE); forced > 0)
@@ -498,10 +519,10 @@ bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int
         if (S > 1 && (d.items * S > sms || w4_decode_clusters(S) < d.items)) continue;
         const int full = d.items * S / d.grid, rest = d.items * S - full * d.grid;
         auto stage_us = [&](int ctas) {
-          float us = 0.4f + 0.16f * static_cast<float>(kw);
-          us = fmaxf(us, static_cast<float>(d.stage_bytes) / 80.0e3f);
+          float us = 0.35f + 0.2f * static_cast<float>(kw);
+          us = fmaxf(us, static_cast<float>(d.stage_bytes) / 60.0e3f);
           us = fmaxf(us, 136.0f * static_cast<float>(h * kw) * static_cast<float>(ctas) / 6.3e6f);
-          return d.nstages < 3 && d.kper > d.nstages ? 1.4f * us : us;
+          return d.nstages < 3 && d.kper > d.nstages ? 1.2f * us : us;
         };
         float c = static_cast<float>(d.kper) * (static_cast<float>(full) * stage_us(d.grid) + (rest ? stage_us(rest) : 0.0f));
         if (S > 1) c += 1.0f + static_cast<float>(tokens * (S - 1)) / static_cast<float>(32 * S);
@@ -518,15 +539,20 @@ msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, cons
   const bool t3 = K % kDecBlockK == 0;
   const CUtensorMapDataType u8 = CU_TENSOR_MAP_DATA_TYPE_UINT8;
   const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B;
-  CUtensorMap tmap_w, tmap_x;
-  const bool ok =
-      t3 ? encode_tmap_3d(&tmap_w, u8, w_fp4, 128, static_cast<uint64_t>(w_rows), kb / 128, kb, 128, 128, static_cast<uint32_t>(d.h), static_cast<uint32_t>(d.kw), sw) &&
-               encode_tmap_3d(&tmap_x, u8, q, 128, static_cast<uint64_t>(q_rows), kb / 128, kb, 128, 128, static_cast<uint32_t>(d.NB), static_cast<uint32_t>(d.kw), sw)
-         : encode_tmap_2d(&tmap_w, u8, w_fp4, kb, static_cast<uint64_t>(w_rows), kb, 128, static_cast<uint32_t>(d.h), sw) &&
-               encode_tmap_2d(&tmap_x, u8, q, kb, static_cast<uint64_t>(q_rows), kb, 128, static_cast<uint32_t>(d.NB), sw);
+  CUtensorMap tmap_w;
+  W4DecodeXMaps<true> tmap_x;
+  const int boxes = expert ? kDecBoxes : 1;
+  bool ok =
+      t3 ? encode_tmap_3d(&tmap_w, u8, w_fp4, 128, static_cast<uint64_t>(w_rows), kb / 128, kb, 128, 128, static_cast<uint32_t>(d.h), static_cast<uint32_t>(d.kw), sw)
+         : encode_tmap_2d(&tmap_w, u8, w_fp4, kb, static_cast<uint64_t>(w_rows), kb, 128, static_cast<uint32_t>(d.h), sw);
+  for (int i = 0; i < boxes && ok; ++i) {
+    const uint32_t rows = static_cast<uint32_t>(expert ? w4d_box_rows(d.NB, i) : d.NB);
+    ok = t3 ? encode_tmap_3d(&tmap_x.m[i], u8, q, 128, static_cast<uint64_t>(q_rows), kb / 128, kb, 128, 128, rows, static_cast<uint32_t>(d.kw), sw)
+            : encode_tmap_2d(&tmap_x.m[i], u8, q, kb, static_cast<uint64_t>(q_rows), kb, 128, rows, sw);
+  }
   if (!ok) return MSD_ERR_CUDA;
   W4DecodeParams p;
-  p.M = M; p.Mp = d.Mp; p.NB = d.NB; p.N = static_cast<int>(N);
+  p.M = M; p.NB = d.NB; p.N = static_cast<int>(N);
   p.h = d.h; p.bands = d.bands; p.items = d.items;
   p.kblocks = d.kblocks; p.kw = d.kw; p.ksteps = d.ksteps; p.S = d.S; p.kper = d.kper;
   p.nstages = d.nstages; p.stage_bytes = d.stage_bytes; p.x_off = d.x_off; p.sf_off = d.sf_off; p.nsfx = d.nsfx;
@@ -546,7 +572,7 @@ msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, cons
     e = launch_pdl(gemm_w4a16_decode_kernel<true>, dim3(d.grid), dim3(kDecThreads), static_cast<size_t>(d.smem), s, pdl, tmap_w, tmap_x, p, g);
   } else {
     e = launch_pdl_cluster(gemm_w4a16_decode_kernel<false>, dim3(d.grid), dim3(kDecThreads), static_cast<size_t>(d.smem), s, pdl, static_cast<unsigned>(d.S),
-                           tmap_w, tmap_x, p, W4DecodeNoGroups());
+                           tmap_w, W4DecodeXMaps<false>{{tmap_x.m[0]}}, p, W4DecodeNoGroups());
   }
   return e == cudaSuccess ? MSD_OK : MSD_ERR_CUDA;
 }

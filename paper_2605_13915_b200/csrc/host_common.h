@@ -143,13 +143,14 @@ struct SfRelayout {
                        // weights), each cut into its own `row_blocks` blocks
   int blocks;          // filled in by the launcher
 };
-// Rows sorted by group (mixture of experts): group g owns rows [off[g], off[g+1]) and its decomposition is written to rows
-// g * rows ... of the component buffers and rows g * srows ... of the scale buffers.
+// Rows sorted by group (mixture of experts): group g owns rows [off[g], off[g+1]).  Its two components go, one below the other, to
+// rows g * rows ... of ONE buffer: the first from there, the second ceil8(rows of the group) further down; their scales likewise
+// to rows g * srows ... of one scale buffer (whole 128-row blocks per group).
 constexpr int kMaxRowGroups = 64;
 struct RowGroups {
-  int n;                       // 0: no regrouping, output row = input row
-  int rows, srows;             // rows per group in the component buffers / in the scale buffers (128-row blocks)
-  int srow2;                   // the second component's scales are this many rows further down (stacked components)
+  int n;                       // 0: no groups, output row = input row
+  int rows, srows;
+  int second;                  // no groups: rows from the first component's to the second's (0: buffers of their own)
   int off[kMaxRowGroups + 1];
 };
 msd_status_t launch_decompose_mxfp4(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, uint8_t* q1, uint8_t* q2,
@@ -157,7 +158,7 @@ msd_status_t launch_decompose_mxfp4(const void* x_bf16, int64_t M, int64_t K, in
                                     SfRelayout* relayout = nullptr, const RowGroups* groups = nullptr);
 
 // W4A16 layers with few tokens per weight matrix (gemm_w4a16_decode.cu): how the kernel cuts a call up, and its launch.
-// Components: one stack [Q1 (Mp rows); Q2] per group of NB rows; scales: nsfx blocks of 128 stacked rows per group.
+// Components: one stack (see RowGroups) per group in room for NB rows; scales: nsfx blocks of 128 stacked rows per group.
 struct W4DecodeShape {
   int h, kw, S;                        // weight rows per band, 256-element K blocks per stage, CTAs (K splits) per band
   int Mp, NB, nsfx, kblocks, ksteps, kper, bands, items, grid;
