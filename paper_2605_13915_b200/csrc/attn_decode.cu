@@ -1040,7 +1040,7 @@ constexpr float kHoldScaleGrowth = 1.25f;
 // plan) - the MMA thread shares its scheduler with four busy softmax warps, so every instruction it spends per MMA on
 // loop control and address arithmetic delays the tensor pipe; with fixed counts its loops unroll to an add per operand.
 template <int kSlots, bool kPaged, int kFixDC, int kFixDVT>
-__global__ void __launch_bounds__(kSlots == 16 ? 384 : ((kFixDC == 5 && kFixDVT == 4 && !kPaged) ? 64 : 96) + 128 * (kSlots / kThreadSlots),
+__global__ void __launch_bounds__(kSlots == 16 ? 384 : 96 + 128 * (kSlots / kThreadSlots),
                                   kSlots == 16 ? 2 : 1)
 attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v, const AttnParams p) {
   extern __shared__ uint8_t smem_dyn[];
@@ -1135,32 +1135,34 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
 
   if (warp == 0) {
     // ------------------------------ TMA producer: K (and V) tiles ------------------------------
-    if (lane == 0) {
-      const int k_bytes = p.DC * kChunkBytes, v_bytes = p.DVT * kChunkBytes;
-      int kq = 0, vq = p.v_alias ? ntiles : 0;
-      if constexpr (kChunked) {
-        bool okp = true;
-        for (; kq < ntiles && okp; ++kq) {
-          const int st = kq & 1;
-          const uint32_t ph = (kq >> 1) & 1;
-          uint8_t* dst = smem + st * kv_stage_bytes;
-          const int tok0 = seq0 + t_begin + kq * kTok;
-          if (kq >= 2 && kq < 5) attn_mark(p, 9 + 6 * (kq - 2));
-          // Chunk by chunk as the tile two back lets go of the stage: the rotary chunk (read by QK^T only) when its
-          // scores are complete (s_full of that tile: same index, same phase; a commit costs its thread about 80 ns,
-          // so the rotary chunk has no barrier of its own), value chunk j when the dv tile of PV that reads it is
-          // complete.  (Parity ph ^ 1 passes at once on a barrier that has not completed a phase yet.)
+    const int k_bytes = p.DC * kChunkBytes, v_bytes = p.DVT * kChunkBytes;
+    int kq = 0, vq = p.v_alias ? ntiles : 0;
+    if constexpr (kChunked) {
+      bool okp = true;
+      for (; kq < ntiles && okp; ++kq) {
+        const int st = kq & 1;
+        const uint32_t ph = (kq >> 1) & 1;
+        uint8_t* dst = smem + st * kv_stage_bytes;
+        const int tok0 = seq0 + t_begin + kq * kTok;
+        if (kq >= 2 && kq < 5 && lane == 0) attn_mark(p, 9 + 6 * (kq - 2));
+        // Chunk by chunk as the tile two back lets go of the stage: the rotary chunk (read by QK^T only) when its
+        // scores are complete (s_full of that tile: same index, same phase; a commit costs its thread about 80 ns,
+        // so the rotary chunk has no barrier of its own), value chunk j when the dv tile of PV that reads it is
+        // complete.  (Parity ph ^ 1 passes at once on a barrier that has not completed a phase yet.)
 #pragma unroll
-          for (int i = 0; i < 5; ++i) {
-            const int c = (i == 0) ? 4 : i - 1;
-            if (i == 0) okp = wait_bounded(&s_full[st], ph ^ 1, abort, p.status);
-            else okp = wait_bounded(&ck_empty[st][c], ph ^ 1, abort, p.status);
-            if (!okp) break;
+        for (int i = 0; i < 5; ++i) {
+          const int c = (i == 0) ? 4 : i - 1;
+          if (i == 0) okp = wait_bounded_warp(&s_full[st], ph ^ 1, abort, p.status);
+          else okp = wait_bounded_warp(&ck_empty[st][c], ph ^ 1, abort, p.status);
+          if (!okp) break;
+          if (elect_one()) {
             mbar_arrive_expect_tx(&ck_full[st][c], kChunkBytes);      // every chunk lands on a barrier of its own
             tma_load_3d(dst + c * kChunkBytes, &tmap_k, c * kChunk, hk, tok0, &ck_full[st][c]);
           }
         }
       }
+    }
+    if (!kChunked && lane == 0) {
       long long t_idle = clock64();
       while (kq < ntiles || vq < ntiles) {
         bool progressed = false;
@@ -1272,10 +1274,10 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         if constexpr (kChunked) { /* the producer takes s_full as "the rotary chunk has been read" */ }
         else if (!p.v_alias) tc_commit_warp(&kv_empty[st]);       // separate V: the K buffer is free once QK^T has read it
       };
-      // PV is issued by softmax threads or a warp of its own (below); this thread issues QK^T only.
+      // PV is issued by a warp of its own (below); this one issues QK^T only.
       int q = 0;
       if constexpr (kChunked) {
-        // PV is issued by two softmax warps (below); this warp issues QK^T only.  QK^T(q) needs KV tile q in shared
+        // QK^T(q) needs KV tile q in shared
         // memory and the score buffer q&1 read, i.e. P of tile q-2 written by every softmax warp (the slow path works
         // from registers).  The P buffer q&1 is free by then as well: KV tile q arrives in the stage that PV(q-2) gave
         // back chunk by chunk, so its arrival implies that PV(q-2) is complete.
@@ -1325,10 +1327,42 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       }
     }
   } else if (warp == 2 + kNSW) {
-    // ------------------------------ PV issuer (rows whose tiles are not handled chunk by chunk) ------------------------------
+    // ------------------------------ PV issuer ------------------------------
     // A warp of its own: one thread issuing QK^T and PV alike was never idle (1.7 us per tile at D = Dv = 128 for 8 MMAs,
-    // 4 commits and its polling, everything else waiting for it), and a softmax thread issuing PV puts it on the
-    // softmax warps' critical path.
+    // 4 commits and its polling, everything else waiting for it), and softmax warps issuing PV put it on their critical path
+    // (latent cache, 64 x 16384 tokens: 250 us with the first two softmax warps issuing two dv tiles each, 241 here).
+    if constexpr (kChunked) {
+      // dv tile by dv tile, in the order in which the value chunks are asked for again
+      const uint64_t vdesc = smem_desc(0, 16384, 1024, kSwizzle128B) + (smem_u32(smem) >> 4);       // V^T, MN-major from the token-major tile
+      const uint64_t pdesc = smem_desc(0, 8 * kPRow, 8 * kPRow, kPSwizzle) + (smem_u32(sm_p) >> 4);           // P, token-major
+      const uint32_t idesc = idesc_dense(2, 1, 1, 1, 1, kTok, p.Rp);     // S8 x S8 -> S32, A (V^T) and B (P) MN-major
+      bool ok = true;
+      int n_slow = 0;
+      for (int t = 0; t < ntiles && ok; ++t) {
+        const int st = t & 1;
+        const uint32_t ph = (t >> 1) & 1;
+        ok = wait_bounded_warp(&p_full[st], ph, abort, p.status);
+        bool fresh = false;
+        if (ok && __any_sync(0xffffffffu, stamp[st] == t + 1)) {
+          ok = wait_bounded_warp(&p_redo, n_slow & 1, abort, p.status);
+          ++n_slow;
+          fresh = true;                            // the accumulators were drained: start them again
+        }
+        if (!ok) break;
+        const uint64_t pa = pdesc + static_cast<uint32_t>(st) * (static_cast<uint32_t>(p.Rp * kChunk) >> 4);
+#pragma unroll
+        for (int dv = 0; dv < 4; ++dv) {
+          ok = wait_bounded_warp(&ck_full[st][dv], ph, abort, p.status);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t va = vdesc + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + dv * (kChunkBytes >> 4);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)              // 32 tokens per MMA: four 8-token groups of 1024 bytes
+            mma_i8_warp(tmem_o + dv * (2 * kSlots), va + k * (4096 >> 4), pa + k * (32 * kPRow >> 4), idesc, (k > 0 || !fresh) ? 1u : 0u);
+          tc_commit_warp(&ck_empty[st][dv]);
+        }
+      }
+    }
     if constexpr (!kChunked) {
       {
         const uint64_t vdesc = smem_desc(0, 16384, 1024, kSwizzle128B) + (smem_u32(smem) >> 4);       // V^T, MN-major from the token-major tile
@@ -1521,15 +1555,6 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       tmem_st_wait();
     };
 
-    // operand descriptors of PV as lower / upper words (see mma_i8_lohi): V^T read MN-major from the token-major KV tile,
-    // P an MN-major operand too
-    const uint64_t pv_vdesc = smem_desc(0, 16384, 1024, kSwizzle128B) + (smem_u32(smem) >> 4);
-    const uint64_t pv_pdesc = smem_desc(0, 8 * kPRow, 8 * kPRow, kPSwizzle) + (smem_u32(sm_p) >> 4);
-    const uint32_t pv_va_lo = static_cast<uint32_t>(pv_vdesc), pv_v_hi = static_cast<uint32_t>(pv_vdesc >> 32);
-    const uint32_t pv_pa_lo = static_cast<uint32_t>(pv_pdesc), pv_p_hi = static_cast<uint32_t>(pv_pdesc >> 32);
-    const uint32_t pv_p_step = static_cast<uint32_t>(p.Rp * kChunk) >> 4;
-    const uint32_t pv_idesc = idesc_dense(2, 1, 1, 1, 1, kTok, p.Rp);     // S8 x S8 -> S32, A (V^T) and B (P) MN-major
-
     bool ok = true;
     int n_slow = 0;
     // this warp's group of head slots holds at least one head (the kernel for 576-byte rows, where every instruction
@@ -1570,13 +1595,11 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
       ok = wait_bounded(&p_full[t & 1], (t >> 1) & 1, abort, p.status);
       if (!ok) break;
       if (threadIdx.x == 64 && t >= 2 && t < 5) attn_mark(p, 6 + 6 * (t - 2));
-      bool slow = false;
       if (!active) {
         if (stamp[t & 1] == t + 1) {      // the other groups drain and write P again: be counted among the warps that are done
           __syncwarp();
           if (lane == 0) mbar_arrive(&p_redo);
           ++n_slow;
-          slow = true;
         }
       } else if (stamp[t & 1] == t + 1) {
         // ---- the references move: tile maxima per head over the group's 128 tokens, largest value scale ----
@@ -1630,35 +1653,6 @@ attn_decode_wide_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid
         if (lane == 0) mbar_arrive(&p_redo);
         ++n_slow;
         named_bar_sync(bar_id, 128);          // `red` may be rewritten
-        slow = true;
-      }
-      if constexpr (kChunked) {
-        // PV(t), two dv tiles each by the first two softmax warps, which sit on different warp schedulers.  The
-        // softmax warps are idle here (the next score tile is not there yet) and the product starts the moment P is final
-        // instead of when the QK^T-issuing thread gets round to it.  The value chunks are let go of in the order in which they are
-        // asked for again, 0 and 1 before 2 and 3: with four threads abreast all four came back at the end of the product (64 x
-        // 16384 tokens, 43 tiles a split: 276 us against 270); one thread for all four takes too long to issue (281).  An accumulator is only ever
-        // written by its own thread, so its MMAs stay in program order.
-        if (wi < 2) {
-          const int st = t & 1;
-          if (slow) ok = wait_bounded_warp(&p_redo, (n_slow - 1) & 1, abort, p.status);      // every warp has drained and rewritten P
-          const uint32_t pa_lo = pv_pa_lo + (t & 1) * pv_p_step;
-#pragma unroll
-          for (int dv = wq; dv < 4; dv += 2) {
-            if (ok) ok = wait_bounded_warp(&ck_full[st][dv], (t >> 1) & 1, abort, p.status);      // its value chunk (long landed: QK^T(t) has read the tile)
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t va_lo = pv_va_lo + static_cast<uint32_t>(st * (kv_stage_bytes >> 4)) + dv * (kChunkBytes >> 4);
-            const uint32_t acc = tmem_o + dv * (2 * kSlots);
-            if (slow) mma_i8_lohi_warp<false>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
-            else mma_i8_lohi_warp<true>(acc, va_lo, pv_v_hi, pa_lo, pv_p_hi, pv_idesc);
-#pragma unroll
-            for (int k = 1; k < 4; ++k)      // 32 tokens per MMA: four 8-token groups of 1024 bytes
-              mma_i8_lohi_warp<true>(acc, va_lo + k * (4096 >> 4), pv_v_hi, pa_lo + k * (32 * kPRow >> 4), pv_p_hi, pv_idesc);
-            tc_commit_warp(&ck_empty[st][dv]);      // value chunk dv may be requested again; also "this dv tile of PV(t) is complete"
-          }
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       }
 #pragma unroll
       for (int h = 0; h < kThreadSlots; ++h) l_part[h] += pl[h];
@@ -2033,7 +2027,7 @@ static AttnKernel pick_attn_kernel(const AttnPlan& pl, int G, bool paged, int* b
   } else {
     // wide head groups: 32 or 16 head slots per CTA, held references (attn_decode_wide_kernel)
     const bool mla = pl.DC == 5 && pl.DVT == 4 && pl.v_alias && pl.stages == 2;     // a 513..640-byte latent row whose first 512 bytes are V
-    *block_threads = ((mla && !paged) ? 64 : 96) + 128 * 4;      // producer, QK^T issuer, 16 softmax warps and, except for the chunk-wise kernel, a PV issuer
+    *block_threads = 96 + 128 * 4;      // producer, QK^T issuer, 16 softmax warps, PV issuer
     if (pl.HG == 16) {
       kernel = paged ? attn_decode_wide_kernel<16, true, 1, 1> : attn_decode_wide_kernel<16, false, 1, 1>;
       *block_threads = 96 + 128 * 2;
