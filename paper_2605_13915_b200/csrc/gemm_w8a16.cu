@@ -358,7 +358,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
   // Runs before the CTA-wide barrier below: the thread that initialised the mbarriers is in this warp, and the sooner
   // the first weight boxes are requested the sooner the stream from HBM starts.
   uint64_t pol_w = 0, pol_x = 0;
-  bool w_lane = false, x_lane = false;
+  bool x_lane = false;
   int c = 0, x_half = 0, tile = 0, kbi = 0, kbr = 0, kbr0 = 0, pre = 0, pre0 = 0, tile_first = 0, kbi_first = 0;
   // first weight row of a tile in the weight tensor, and first row of its stacked components in the component buffer
   auto w_row = [&](int t) -> int {
@@ -378,27 +378,30 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     if (++kbi == p.kblocks) { kbi = 0; ++tile; }
     if (++kbr == p.kblocks) kbr = 0;
   };
-  // the weight box(es) / component box(es) of K block `kblk` (in units of stages) into stage memory at `dst`
-  auto load_w = [&](uint8_t* dst, int kblk, int row, uint64_t* bar) {
-    if (p.tma3d) tma_load_3d_hint(dst, wmap, 0, row, kblk * p.kw, bar, pol_w);
-    else tma_load_2d_hint(dst + c * w_chunk, wmap, (kblk * p.kw + c) * kBlockK, row, bar, pol_w);
+  // The weight box(es) of K block `kblk` (in units of stages), with the announcement of a stage's bytes, and its component box(es) into
+  // stage memory at `dst`.  One 3-D box per operand where there is one, issued by the converged warp; else lanes [0, kw) issue a
+  // weight box each and lanes [kw, 2 kw) one of the stacked components (grouped: [kw, 3 kw), one box per component).
+  auto request_w = [&](uint8_t* dst, int kblk, int row, uint64_t* bar) {
+    if (p.tma3d) {
+      mbar_arrive_expect_tx_warp(bar, tx_bytes);
+      tma_load_3d_hint_warp(dst, wmap, 0, row, kblk * p.kw, bar, pol_w);
+    } else {
+      if (lane == 0) mbar_arrive_expect_tx(bar, tx_bytes);
+      __syncwarp();
+      if (lane < p.kw) tma_load_2d_hint(dst + lane * w_chunk, wmap, (kblk * p.kw + lane) * kBlockK, row, bar, pol_w);
+    }
   };
-  auto load_x = [&](uint8_t* dst, int kblk, int row, uint64_t* bar) {
-    if (p.tma3d && !kGrouped) tma_load_3d_hint(dst + w_stage_bytes, &tmap_x, 0, row, kblk * p.kw, bar, pol_x);
-    else tma_load_2d_hint(dst + w_stage_bytes + c * x_chunk_bytes + x_half * x_half_bytes, &tmap_x, (kblk * p.kw + c) * kBlockK, row, bar, pol_x);
+  auto request_x = [&](uint8_t* dst, int kblk, int row, uint64_t* bar) {
+    if (p.tma3d && !kGrouped) tma_load_3d_hint_warp(dst + w_stage_bytes, &tmap_x, 0, row, kblk * p.kw, bar, pol_x);
+    else if (x_lane) tma_load_2d_hint(dst + w_stage_bytes + c * x_chunk_bytes + x_half * x_half_bytes, &tmap_x, (kblk * p.kw + c) * kBlockK, row, bar, pol_x);
   };
   if (warp == 0) {
     __syncwarp();
-    // The whole warp takes part: lane 0 owns the barriers, lanes [0, kw) each issue one weight box of a stage and
-    // lanes [kw, 2 kw) one box of the stacked components, so the copies of a stage are issued side by side instead
-    // of one after another by a single thread.
     pol_w = policy_evict_first();    // weights are streamed once
     pol_x = policy_evict_last();      // the stacked components are re-read by every CTA
-    w_lane = lane < (p.tma3d ? 1 : p.kw);
     x_lane = lane >= p.kw && lane < (kGrouped ? 3 : 2) * p.kw;     // grouped: one box per component
-    if (p.tma3d && !kGrouped) x_lane = lane == p.kw;              // one 3-D box of the stacked components per stage
-    c = w_lane ? lane : (lane - p.kw) % p.kw;
-    x_half = w_lane ? 0 : (lane - p.kw) / p.kw;
+    c = x_lane ? (lane - p.kw) % p.kw : 0;
+    x_half = x_lane ? (lane - p.kw) / p.kw : 0;
     // (tile, K block) of the next block to load, advanced by one per stage; kbr = rotated K block
     tile = tile0; kbi = kbi0;
     tile_first = tile0; kbi_first = kbi0;
@@ -411,9 +414,7 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     pre0 = pre < p.pre_stages ? pre : p.pre_stages;
     if constexpr (kBase) pdl_wait_primary();     // here the weights themselves come from the preceding kernel
     for (int i = 0; i < pre0; ++i) {
-      if (lane == 0) mbar_arrive_expect_tx(&full_bar[i], tx_bytes);
-      __syncwarp();
-      if (w_lane) load_w(smem + i * stage_bytes, kbr, w_row(tile), &full_bar[i]);
+      request_w(smem + i * stage_bytes, kbr, w_row(tile), &full_bar[i]);
       advance();
     }
     if (lane == 0) trace_mark(p, 3);
@@ -434,12 +435,10 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
       int kx = kbr0;
       for (int i = 0; i < pre; ++i) {
         if (i >= pre0) {     // weight boxes held back so that the wait above was not queued behind them
-          if (lane == 0) mbar_arrive_expect_tx(&full_bar[i], tx_bytes);
-          __syncwarp();
-          if (w_lane) load_w(smem + i * stage_bytes, kbr, w_row(tile), &full_bar[i]);
+          request_w(smem + i * stage_bytes, kbr, w_row(tile), &full_bar[i]);
           advance();
         }
-        if (x_lane) load_x(smem + i * stage_bytes, kx, x_row(tile_first + (kbi_first + i) / p.kblocks), &full_bar[i]);
+        request_x(smem + i * stage_bytes, kx, x_row(tile_first + (kbi_first + i) / p.kblocks), &full_bar[i]);
         if (++kx == p.kblocks) kx = 0;
       }
     }
@@ -447,15 +446,11 @@ gemm_w8a16_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     uint32_t phase = (pre == p.num_stages) ? 1 : 0;
     bool ok = true;
     for (long long blk = blk_begin + pre; blk < blk_end; ++blk) {
-      if (lane == 0) {
-        ok = wait_bounded(&empty_bar[stage], phase ^ 1, abort, p.status);
-        if (ok) mbar_arrive_expect_tx(&full_bar[stage], tx_bytes);
-      }
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      ok = wait_bounded_warp(&empty_bar[stage], phase ^ 1, abort, p.status);
       if (!ok) break;
       uint8_t* dst = smem + stage * stage_bytes;
-      if (w_lane) load_w(dst, kbr, w_row(tile), &full_bar[stage]);
-      else if (x_lane) load_x(dst, kbr, x_row(tile), &full_bar[stage]);
+      request_w(dst, kbr, w_row(tile), &full_bar[stage]);
+      request_x(dst, kbr, x_row(tile), &full_bar[stage]);
       advance();
       if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
     }
