@@ -67,8 +67,9 @@ msd_status_t msd_debug_timeout_selftest(int64_t budget_cycles, void* stream);
  * what the environment says.  Unknown names: MSD_ERR_UNSUPPORTED.  None of them changes results.
  *   MSD_NO_PDL (1: no programmatic dependent launches), MSD_GEMM_MODE / MSD_GEMM_CTAS (work split and CTA count of the
  *   W8A16 decode kernel: 0 stream-K, 1 row bands, 2 clusters), MSD_P8_PAIR / MSD_P8_KSPLIT (W8A16 many-row kernel: CTA
- *   pairs, K split), MSD_W4_PAIR / MSD_W4_TILEN / MSD_W4_KSPLIT (W4A16 kernels), MSD_ATTN_SPLITS / MSD_ATTN_CHUNK_TILES
- *   (context splits of the attention kernels; msd_attn_decode_schedule reports the schedule in force),
+ *   pairs, K split), MSD_W4_PAIR / MSD_W4_TILEN / MSD_W4_KSPLIT (W4A16 kernels), MSD_W4_DECODE (W4A16 with few tokens: 0 keeps
+ *   calls for one matrix on the tile kernel, else 100000 x K blocks per stage + 1000 x CTAs per band + weight rows per band),
+ *   MSD_ATTN_SPLITS / MSD_ATTN_CHUNK_TILES (context splits of the attention kernels; msd_attn_decode_schedule reports the schedule in force),
  *   MSD_ATTN_BALANCED (1: the balanced split schedule for every shape that has a kernel for it, 0: never; a forced
  *   split count or size switches it off as well). */
 msd_status_t msd_debug_set_option(const char* name, int32_t value);

@@ -3,6 +3,10 @@
 // Operands are swapped against the many-row kernels of gemm_w4a16.cu: a band of up to 128 weight rows is the MMA A operand, the
 // stacked components [Q1; Q2] (NB = 2 ceil8(tokens) rows) are B, and the two passes land in different columns of one accumulator,
 // so a weight tile passes the tensor core once and an MMA costs what its tokens are worth.
+//
+// Bound: HBM for experts (32 of 2048 x 7168, 512 tokens: 53 us, 4.8 TB/s), the chain of two kernels for single layers (16 tokens, 4096 x 14336
+// and back: 11.2 and 12.6 us for 31 MB each).  With tiles of 128 token rows, padded and once per component, a 256 x 256 weight stage
+// took 0.65 us of tensor time where HBM needs 0.8 for all SMs: 68 and 32 us for the two.
 #include <cuda_bf16.h>
 
 #include <cmath>
