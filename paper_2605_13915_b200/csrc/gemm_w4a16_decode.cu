@@ -510,17 +510,15 @@ static bool w4_decode_layout(W4DecodeShape* d, int tokens, int groups, int64_t N
 //   a K split     1 + tokens (S - 1) / (32 S): two cluster barriers, and the sums sent to the peers
 // Against the best of every (kw, S, height) swept over 30 layers (1 to 128 tokens, 2048 to 16384 x 2048 to 16384) and 26 calls with
 // experts (9 to 64 of them, 6 to 77 tokens the longest group): 1.013 on average, 1.10 at most.
-bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K) {
-  const int sms = sm_count();
-  if (const int forced = option(OPT_W4_DECODE); forced > 0)
-    return w4_decode_layout(best, tokens, groups, N, K, forced % 1000, forced / 100000, forced / 1000 % 100);
+static bool w4_decode_search(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K, int sms) {
   float cost = 1e30f;
   for (int kw = 4; kw >= 1; kw >>= 1)
     for (int S = 1; S <= (groups > 0 ? 1 : 8); ++S)
       for (int h = 128; h >= 96; h -= 16) {
         W4DecodeShape d;
+        if (S > 1 && (N + h - 1) / h * S > sms) continue;
         if (!w4_decode_layout(&d, tokens, groups, N, K, h, kw, S)) continue;
-        if (S > 1 && (d.items * S > sms || w4_decode_clusters(S) < d.items)) continue;
+        if (S > 1 && w4_decode_clusters(S) < d.items) continue;
         const int full = d.items * S / d.grid, rest = d.items * S - full * d.grid;
         auto stage_us = [&](int ctas) {
           float us = 0.35f + 0.2f * static_cast<float>(kw);
@@ -533,6 +531,30 @@ bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int
         if (c < cost) { cost = c; *best = d; }
       }
   return cost < 1e30f;
+}
+
+// The search looks at up to 72 shapes, several microseconds of host time: a layer's is remembered (64 direct-mapped slots by everything
+// it depends on; calls with experts, whose groups change from call to call, have nine to look at).
+bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K) {
+  if (const int forced = option(OPT_W4_DECODE); forced > 0)
+    return w4_decode_layout(best, tokens, groups, N, K, forced % 1000, forced / 100000, forced / 1000 % 100);
+  const int sms = sm_count();
+  if (groups > 0) return w4_decode_search(best, tokens, groups, N, K, sms);
+  struct Slot { int64_t N, K; int tokens, sms; bool found; W4DecodeShape d; };
+  constexpr int kSlots = 64;
+  static Slot slots[kSlots] = {};
+  static std::mutex mu;
+  Slot& slot = slots[((static_cast<uint64_t>(N) * 0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(K)) * 0x9E3779B97F4A7C15ull + static_cast<uint64_t>(tokens) * 0xC2B2AE3D27D4EB4Full) >> 58];
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (slot.tokens == tokens && slot.N == N && slot.K == K && slot.sms == sms) { *best = slot.d; return slot.found; }
+  }
+  Slot fresh = {N, K, tokens, sms, false, {}};
+  fresh.found = w4_decode_search(&fresh.d, tokens, 0, N, K, sms);
+  std::lock_guard<std::mutex> lock(mu);
+  slot = fresh;
+  *best = fresh.d;
+  return fresh.found;
 }
 
 msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, const uint8_t* q, int64_t q_rows, int64_t w_rows, int M, int64_t N,
