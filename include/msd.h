@@ -227,6 +227,11 @@ msd_status_t msd_gemm_w4a16(const void* x_bf16, const uint8_t* w_fp4, const uint
                             int64_t K, void* y, msd_out_t ytype, void* workspace, size_t workspace_bytes,
                             void* stream);
 
+/* How msd_gemm_w4a16 and msd_gemm_w4a16_prepared run a call of this shape (for tests; host arithmetic): schedule_host[0] the kernel (0 tiles
+ * of 128 tokens, 1 the same on CTA pairs, 2 few tokens), [1] weight rows per tile, [2] CTAs of a cluster (1: none), [3] K splits, [4]
+ * dynamic shared memory of a CTA in bytes. */
+msd_status_t msd_debug_gemm_w4a16_schedule(int64_t M, int64_t N, int64_t K, int32_t* schedule_host);
+
 /*
  * Grouped W4A16 MSD layer for mixture-of-experts blocks (Discussion, "Extension to MoE and Sparse
  * Architectures"; the decomposition works per 32-element block of an

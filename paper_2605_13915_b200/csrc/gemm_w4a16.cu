@@ -767,6 +767,7 @@ struct GemmW4Plan {
   W4DecodeShape d;
   int sf_tile_rows;             // weight rows per tile of the blocked scale layout (224 or 256; 128-row tiles use 256)
   int ksplit, kper, a_rows, nstages;
+  size_t smem;                  // dynamic shared memory of a CTA (the CTA-pair kernel's is its own)
   size_t off_q1, off_q2, off_sfa1, off_sfa2, off_sfb, off_part, bytes;
 };
 
@@ -785,6 +786,10 @@ static bool w4_use_pair(int64_t M, int64_t N, int64_t K) {
   // rounds x tile width of either kernel (a pair tile takes a pair as long as a 128 x 256 tile takes a CTA)
   const int64_t cost_pair = (pair_tiles + clusters - 1) / clusters * 256, cost_single = (single_tiles + sm_count() - 1) / sm_count() * 224;
   return 100 * cost_pair <= 110 * cost_single;
+}
+
+static size_t w4_pair_smem(int tile_n) {
+  return static_cast<size_t>(kW4PairStages) * (2 * kW4ABytes + (tile_n / 2) * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
 }
 
 // Weight rows per tile: MSD_W4_TILEN (224 or 256) if set; else 256 for the CTA-pair kernel (one accumulator) and 224 for
@@ -927,7 +932,9 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   // one token tile of fewer than 128 rows: only those rows are loaded and the stages are packed (more of them fit)
   pl.a_rows = pl.m_tiles == 1 ? static_cast<int>((M + 7) / 8 * 8) : kW4TileM;
   size_t stage_bytes;
-  w4_stages(pl.a_rows, tile_n, pl.cluster > 1 ? 0 : 8 * kW4StoreBytes, &pl.nstages, &stage_bytes);
+  const size_t store_bytes = pl.cluster > 1 ? 0 : 8 * kW4StoreBytes;
+  w4_stages(pl.a_rows, tile_n, store_bytes, &pl.nstages, &stage_bytes);
+  pl.smem = pl.few ? static_cast<size_t>(pl.d.smem) : pl.nstages * stage_bytes + store_bytes + 1024;
   size_t off = 0;
   if (pl.few) {                 // components and their scales as one stack of rows
     pl.off_q1 = off;   off = round_up(off + static_cast<size_t>(pl.d.Mp + M) * (K / 2), 1024);
@@ -1025,6 +1032,19 @@ msd_status_t msd_prepare_w4a16_scales(const uint8_t* w_e8m0, int32_t E, int64_t 
 size_t msd_gemm_w4a16_workspace_bytes(int64_t M, int64_t N, int64_t K) {
   if (M < 1 || N < 1 || K < 128 || K % 128 != 0) return 0;
   return msd::plan_w4(M, N, K).bytes;
+}
+
+msd_status_t msd_debug_gemm_w4a16_schedule(int64_t M, int64_t N, int64_t K, int32_t* schedule_host) {
+  if (!schedule_host) return MSD_ERR_NULL_POINTER;
+  if (M < 1 || N < 1 || K < 128 || K % 128 != 0 || N % 8 != 0 || M > (1 << 24) || N > (1 << 24) || K > (1 << 24)) return MSD_ERR_BAD_SHAPE;
+  const msd::GemmW4Plan pl = msd::plan_w4(M, N, K);
+  const bool pair = !pl.few && msd::w4_use_pair(M, N, K);
+  schedule_host[0] = pl.few ? 2 : (pair ? 1 : 0);
+  schedule_host[1] = pl.few ? pl.d.h : pl.tile_n;
+  schedule_host[2] = pl.few ? pl.d.S : (pair ? 2 : pl.cluster);
+  schedule_host[3] = pl.few ? pl.d.S : (pair ? 1 : pl.ksplit);
+  schedule_host[4] = static_cast<int32_t>(pair ? msd::w4_pair_smem(pl.tile_n) : pl.smem);
+  return MSD_OK;
 }
 
 msd_status_t msd_gemm_w4a16(const void* x_bf16, const uint8_t* w_fp4, const uint8_t* w_e8m0, int64_t M, int64_t N,
@@ -1126,7 +1146,7 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
     if (!encode_tmap_2d(&tmap_bh, CU_TENSOR_MAP_DATA_TYPE_UINT8, w_fp4, kb, N, kb, 128, static_cast<uint32_t>(pl.tile_n / 2),
                         CU_TENSOR_MAP_SWIZZLE_128B))
       return MSD_ERR_CUDA;
-    const size_t smem_pair = static_cast<size_t>(kW4PairStages) * (2 * kW4ABytes + (pl.tile_n / 2) * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
+    const size_t smem_pair = w4_pair_smem(pl.tile_n);
     static DeviceOnce once;
     if (!once([] {
           return cudaFuncSetAttribute(gemm_w4a16_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
@@ -1146,15 +1166,11 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
   p.ksplit = pl.ksplit; p.kper = pl.kper; p.part_rows = static_cast<int>(part_rows);
   p.a_rows = pl.a_rows; p.nstages = pl.nstages;
   if (pl.cluster > 1) {          // (its shared-memory limit was raised when the plan asked how many clusters fit)
-    int nstages;
-    size_t stage_bytes;
-    w4_stages(pl.a_rows, pl.tile_n, 0, &nstages, &stage_bytes);
-    if (launch_pdl_cluster(w4_cluster_kernel(pl.tile_n), dim3(pl.grid), dim3(kW4ThreadsSf), nstages * stage_bytes + 1024, s, pdl,
+    if (launch_pdl_cluster(w4_cluster_kernel(pl.tile_n), dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl,
                            static_cast<unsigned>(pl.cluster), tmap_a1, tmap_a2, tmap_b, tmap_y, p) != cudaSuccess)
       return MSD_ERR_CUDA;
     return MSD_OK;
   }
-  const size_t smem_bytes = static_cast<size_t>(pl.nstages) * (2 * pl.a_rows * 128 + pl.tile_n * 128 + kW4SfBytes) + 8 * kW4StoreBytes + 1024;
   static DeviceOnce once;
   if (!once([] {
         return cudaFuncSetAttribute(gemm_w4a16_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
@@ -1162,8 +1178,8 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
       }))
     return MSD_ERR_CUDA;
   const cudaError_t le = pl.tile_n == 256
-      ? launch_pdl(gemm_w4a16_kernel<256>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p)
-      : launch_pdl(gemm_w4a16_kernel<224>, dim3(pl.grid), dim3(kW4ThreadsSf), smem_bytes, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p);
+      ? launch_pdl(gemm_w4a16_kernel<256>, dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p)
+      : launch_pdl(gemm_w4a16_kernel<224>, dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p);
   if (le != cudaSuccess) return MSD_ERR_CUDA;
   if (split) {
     const msd_status_t rs = launch_ksplit_reduce(part, pl.ksplit, static_cast<int64_t>(part_rows) * N, M, N, y, static_cast<int>(ytype), s, pdl);

@@ -24,6 +24,12 @@ constexpr int kDecMaxStages = 16;
 constexpr int kDecMaxSets = 4;
 constexpr int kDecStoreBytes = 2 * 16 * 128 * 4;  // epilogue staging: two buffers of [16 tokens][128 rows] FP32
 constexpr int kDecSmem = 227 * 1024 - 2048;
+// Least shared memory of a CTA that waits for others (K split over a cluster).  Every CTA takes all of its SM's tensor memory, and the wait
+// for that has no limit: of two such CTAs on one SM the second would wait for the first to end, the first at a cluster barrier
+// for the peers of the second or for the second itself.  With more than half of an SM's 228 KB each (1 KB of it the system's) there is
+// only one of them, and none beside a CTA of the other kernels whose CTAs wait for one another, which take 160 KB and more.
+constexpr int kDecClusterSmem = 116 * 1024;
+static_assert(2 * (kDecClusterSmem + 1024) > 228 * 1024, "two CTAs of a cluster would fit one SM");
 constexpr int kDecTmemCols = 512;
 
 struct W4DecodeParams {
@@ -442,7 +448,7 @@ static bool w4_decode_attr() {
   });
 }
 
-// How many clusters of S CTAs of the kernel the device holds at once, one CTA per SM (0 on error).
+// How many clusters of S CTAs of the kernel the device holds at once, one CTA per SM as in every launch with clusters (0 on error).
 static int w4_decode_clusters(int S) {
   static std::mutex mu;
   static int cache[64][9] = {};
@@ -501,6 +507,7 @@ static bool w4_decode_layout(W4DecodeShape* d, int tokens, int groups, int64_t N
   d->epi_off = one ? slots : pipe;
   const int epi_end = d->epi_off + kDecStoreBytes;
   d->smem = (pipe > epi_end ? pipe : epi_end) + 1024;
+  if (S > 1 && d->smem < kDecClusterSmem) d->smem = kDecClusterSmem;
   return d->smem <= kDecSmem;
 }
 

@@ -1,0 +1,31 @@
+"""Host arithmetic of the W4A16 kernels' schedules: no GPU needed."""
+import pytest
+
+from paper_2605_13915_b200 import binding
+
+SM_SHARED, CTA_RESERVED = 228 * 1024, 1024        # shared memory of an SM, and what the system takes of it per CTA
+
+
+@pytest.fixture(autouse=True)
+def _options():
+    yield
+    binding.debug_reset_options()
+
+
+@pytest.mark.parametrize("M", [1, 16, 33, 128])
+@pytest.mark.parametrize("N,K", [(2048, 2048), (1000, 2176), (4096, 4096), (2048, 14336)])
+def test_few_token_clusters_have_their_sms_to_themselves(M, N, K):
+    """A CTA holds all tensor memory of its SM while it waits for the CTAs of its cluster, so two of them must not share an SM: each
+    asks for more than half of the shared memory, whatever its pipeline needs."""
+    seen = 0
+    for kw in (1, 2, 4):
+        for S in range(2, 9):
+            for h in (96, 128):
+                binding.debug_set_option("MSD_W4_DECODE", 100000 * kw + 1000 * S + h)
+                kernel, rows, cluster, splits, smem = binding.debug_gemm_w4a16_schedule(M, N, K)
+                if kernel != 2:
+                    continue                      # (a shape that does not fit)
+                assert (rows, cluster, splits) == (h, S, S)
+                assert 2 * (smem + CTA_RESERVED) > SM_SHARED, (kw, S, h, smem)
+                seen += 1
+    assert seen
