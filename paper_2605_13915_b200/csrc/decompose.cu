@@ -185,6 +185,9 @@ decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, i
       e1[so1] = static_cast<uint8_t>(a + 127);
       e2[so2] = static_cast<uint8_t>(bexp + 127);
     }
+    // A K that ends halfway through a 256-element block leaves it a group of four scales that the MMAs take with operands of zeros: they
+    // must be numbers (0xFF is NaN), whatever the workspace held.
+    if (sf_kgroups > (kblocks >> 2) && kb + 4 >= kblocks) e1[so1 + 512] = e2[so2 + 512] = 0;
     }
   }
 }

@@ -170,3 +170,24 @@ def test_few_token_kernel_in_every_shape(M, N, K, kw, S, h):
     binding.last_device_status()
     assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
     _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)
+
+
+@pytest.mark.parametrize("M,N,K,before", [(1, 264, 1152, 12), (16, 1000, 2176, 30), (33, 264, 3200, 60), (100, 1000, 3200, 150), (300, 264, 384, 500),
+                                          (520, 1032, 640, 800)])
+def test_padding_scales_in_a_used_workspace(M, N, K, before):
+    """K % 256 == 128: the MMAs take the second half of the last K block, which is empty, with whatever scales are there.  An earlier call
+    with more rows leaves 0xFF bytes in that place (-3.4375 is -3 and a residual of -7 / 16, the second code -6), NaN as E8M0
+    scales; the call after it has to give what it gives with a workspace of its own.  Few-token kernel, tiles with and without
+    clusters, CTA pairs."""
+    c = inputs.gemm_w4_case(M, N, K, seed=M + K)
+    x, w, e = bf16_dev(c.x), dev(c.w_fp4), dev(c.w_e8m0)
+    old = torch.full((before, K), -3.4375, dtype=torch.bfloat16, device="cuda")
+    assert bool((binding.decompose_mxfp4(old)[1] == 0xFF).all())
+    ws = binding.workspace(max(binding.gemm_w4a16_workspace_bytes(m, N, K) for m in (M, before)))
+    want = binding.gemm_w4a16(x, w, e, out_dtype=torch.float32)
+    binding.gemm_w4a16(old, w, e, out_dtype=torch.float32, ws=ws)
+    y = binding.gemm_w4a16(x, w, e, out_dtype=torch.float32, ws=ws)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert torch.equal(y, want)
+    _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)

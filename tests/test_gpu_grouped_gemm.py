@@ -131,3 +131,27 @@ def test_grouped_w4a16_with_prepared_scales(sizes, N, K):
     n = np.linalg.norm(ref, axis=-1, keepdims=True)
     assert np.all(np.abs(y.cpu().numpy() - ref) <= TOL * n + 1e-30)
     assert torch.equal(y, plain)
+
+
+def _w4_oracle(x, q, e, sizes):
+    ref = np.zeros((x.shape[0], q.shape[1]), np.float64)
+    off = 0
+    for g, m in enumerate(sizes):
+        if m:
+            ref[off:off + m] = oracle.gemm_w4a16(x[off:off + m], q[g], e[g], "f64")
+        off += m
+    return ref
+
+
+@pytest.mark.parametrize("sizes,N,K", [([3, 0, 16, 1], 448, 384), ([128, 5, 0, 64, 33], 1000, 1152), ([100, 128, 90, 77], 520, 640)])
+def test_grouped_w4a16_workspace_needs_no_initialisation(sizes, N, K):
+    """K % 256 == 128 and a workspace of 0xFF bytes, NaN as E8M0 scales of the empty half of the last K block."""
+    x, q, e = _case_w4(sizes, N, K, seed=9 + len(sizes))
+    xd, qd, ed = bf16_dev(x), dev(q), dev(e)
+    want = _w4_oracle(x, q, e, sizes)
+    ws = binding.workspace(int(binding.lib().msd_grouped_gemm_w4a16_workspace_bytes(len(sizes), N, K)))
+    ws.fill_(0xFF)
+    y = binding.grouped_gemm_w4a16(xd, qd, ed, sizes, out_dtype=torch.float32, ws=ws)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert np.all(np.abs(y.cpu().numpy() - want) <= TOL * np.linalg.norm(want, axis=-1, keepdims=True) + 1e-30)
