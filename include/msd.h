@@ -249,6 +249,10 @@ size_t msd_grouped_gemm_w4a16_workspace_bytes(int32_t E, int64_t N, int64_t K);
 msd_status_t msd_grouped_gemm_w4a16(const void* x_bf16, const uint8_t* w_fp4, const uint8_t* w_e8m0,
                                     const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, void* y,
                                     msd_out_t ytype, void* workspace, size_t workspace_bytes, void* stream);
+/* How the first launch of such a call runs (for tests; host arithmetic): schedule_host[0] the kernel (2 few tokens), [1] weight rows per
+ * tile, [2] stages of a CTA's pipeline, [3] the most stages that a CTA goes through, of all its tiles, [4] dynamic shared memory of a
+ * CTA in bytes. */
+msd_status_t msd_debug_grouped_gemm_w4a16_schedule(const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, int32_t* schedule_host);
 
 /*
  * Weight scales prepared once.  The block-scaled MMA (Sec. 3.2.1 / Sec. 3.8.3: two FP4 GEMMs with E8M0 block scales)

@@ -55,6 +55,7 @@ _SIGS = {
     "msd_gemm_w4a16_workspace_bytes": (_sz, [_i64, _i64, _i64]),
     "msd_gemm_w4a16": (C.c_int, [_vp, _vp, _vp, _i64, _i64, _i64, _vp, C.c_int, _vp, _sz, _vp]),
     "msd_debug_gemm_w4a16_schedule": (C.c_int, [_i64, _i64, _i64, C.POINTER(_i32)]),
+    "msd_debug_grouped_gemm_w4a16_schedule": (C.c_int, [C.POINTER(_i32), _i32, _i64, _i64, C.POINTER(_i32)]),
     "msd_w4a16_prepared_scales_bytes": (_sz, [_i32, _i64, _i64]),
     "msd_prepare_w4a16_scales": (C.c_int, [_vp, _i32, _i64, _i64, _vp, _vp]),
     "msd_gemm_w4a16_prepared": (C.c_int, [_vp, _vp, _vp, _i64, _i64, _i64, _vp, C.c_int, _vp, _sz, _vp]),
@@ -313,6 +314,13 @@ def debug_gemm_w4a16_schedule(M, N, K):
     """(kernel, weight rows per tile, CTAs of a cluster, K splits, shared memory of a CTA) of a W4A16 call, as msd.h says."""
     out = (_i32 * 5)()
     _check(lib().msd_debug_gemm_w4a16_schedule(M, N, K, out), "msd_debug_gemm_w4a16_schedule")
+    return tuple(out)
+
+
+def debug_grouped_gemm_w4a16_schedule(group_sizes, N, K):
+    """(kernel, weight rows per tile, pipeline stages, stages a CTA goes through, shared memory of a CTA) of a grouped W4A16 call."""
+    out, sizes = (_i32 * 5)(), (_i32 * len(group_sizes))(*[int(v) for v in group_sizes])
+    _check(lib().msd_debug_grouped_gemm_w4a16_schedule(sizes, len(group_sizes), N, K, out), "msd_debug_grouped_gemm_w4a16_schedule")
     return tuple(out)
 
 

@@ -1197,6 +1197,23 @@ size_t msd_grouped_gemm_w4a16_workspace_bytes(int32_t E, int64_t N, int64_t K) {
   return msd::plan_grouped_w4(E, N, K).bytes;
 }
 
+msd_status_t msd_debug_grouped_gemm_w4a16_schedule(const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, int32_t* schedule_host) {
+  using namespace msd;
+  if (!group_sizes_host || !schedule_host) return MSD_ERR_NULL_POINTER;
+  if (E < 1 || N < 1 || K < 128 || K % 128 != 0 || N % 8 != 0 || N > (1 << 24) || K > (1 << 24)) return MSD_ERR_BAD_SHAPE;
+  int largest = 0, nonempty = 0;
+  for (int e = 0; e < E; ++e) {
+    if (group_sizes_host[e] < 0 || group_sizes_host[e] > kW4TileM) return MSD_ERR_BAD_SHAPE;
+    if (group_sizes_host[e] > largest) largest = group_sizes_host[e];
+    nonempty += group_sizes_host[e] > 0 ? 1 : 0;
+  }
+  if (largest == 0) return MSD_ERR_BAD_SHAPE;
+  W4DecodeShape d;
+  if (!w4_decode_shape(&d, largest, nonempty < kMaxRowGroups ? nonempty : kMaxRowGroups, N, K)) return MSD_ERR_UNSUPPORTED;
+  schedule_host[0] = 2; schedule_host[1] = d.h; schedule_host[2] = d.nstages; schedule_host[3] = d.steps; schedule_host[4] = d.smem;
+  return MSD_OK;
+}
+
 msd_status_t msd_grouped_gemm_w4a16(const void* x_bf16, const uint8_t* w_fp4, const uint8_t* w_e8m0,
                                     const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, void* y,
                                     msd_out_t ytype, void* workspace, size_t workspace_bytes, void* stream) {

@@ -500,7 +500,8 @@ static bool w4_decode_layout(W4DecodeShape* d, int tokens, int groups, int64_t N
   const int most = one ? d->kper : kDecMaxStages;
   if (n > most) n = most;
   if (n > kDecMaxStages) n = kDecMaxStages;
-  if (n < 1 || (n < 2 && d->kper > 1)) return false;
+  d->steps = d->kper * ((d->items * S + d->grid - 1) / d->grid);
+  if (n < 1 || (n < 2 && d->steps > 1)) return false;          // (a stage of the next item is asked for while this one's is multiplied)
   d->nstages = n;
   const int G = (tokens + 3) / 4, slots = S > 1 ? S * ((G + S - 1) / S) * 2048 : 0;
   const int pipe = n * d->stage_bytes + pad;
@@ -531,7 +532,7 @@ static bool w4_decode_search(W4DecodeShape* best, int tokens, int groups, int64_
           float us = 0.35f + 0.2f * static_cast<float>(kw);
           us = fmaxf(us, static_cast<float>(d.stage_bytes) / 60.0e3f);
           us = fmaxf(us, 136.0f * static_cast<float>(h * kw) * static_cast<float>(ctas) / 6.3e6f);
-          return d.nstages < 3 && d.kper > d.nstages ? 1.2f * us : us;
+          return d.nstages < 3 && d.steps > d.nstages ? 1.2f * us : us;
         };
         float c = static_cast<float>(d.kper) * (static_cast<float>(full) * stage_us(d.grid) + (rest ? stage_us(rest) : 0.0f));
         if (S > 1) c += 1.0f + static_cast<float>(tokens * (S - 1)) / static_cast<float>(32 * S);

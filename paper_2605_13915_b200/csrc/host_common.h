@@ -162,6 +162,7 @@ msd_status_t launch_decompose_mxfp4(const void* x_bf16, int64_t M, int64_t K, in
 struct W4DecodeShape {
   int h, kw, S;                        // weight rows per band, 256-element K blocks per stage, CTAs (K splits) per band
   int Mp, NB, nsfx, kblocks, ksteps, kper, bands, items, grid;
+  int steps;                           // stages a CTA goes through, of all its items
   int x_off, sf_off, stage_bytes, nstages, set_cols, nsets, sf_col, nacc, epi_off, smem;
 };
 // (groups: matrices of a grouped launch, 0 for an ungrouped call)

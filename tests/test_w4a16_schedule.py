@@ -29,3 +29,12 @@ def test_few_token_clusters_have_their_sms_to_themselves(M, N, K):
                 assert 2 * (smem + CTA_RESERVED) > SM_SHARED, (kw, S, h, smem)
                 seen += 1
     assert seen
+
+
+@pytest.mark.parametrize("tokens", [1, 16, 32, 64, 96, 128])
+@pytest.mark.parametrize("groups", [1, 8, 23, 64])
+def test_grouped_pipelines_have_two_stages(groups, tokens):
+    """A CTA that goes through several stages, of one tile or of several, needs room for two: the next is loaded while one is multiplied."""
+    for N, K in [(4096, 1024), (5632, 896), (2048, 512), (7168, 2048), (1000, 128), (2048, 7168)]:
+        _, _, stages, steps, _ = binding.debug_grouped_gemm_w4a16_schedule([tokens] * groups, N, K)
+        assert steps >= 1 and stages >= min(2, steps), (N, K, stages, steps)
