@@ -68,7 +68,7 @@ msd_status_t msd_debug_timeout_selftest(int64_t budget_cycles, void* stream);
  *   MSD_NO_PDL (1: no programmatic dependent launches), MSD_GEMM_MODE / MSD_GEMM_CTAS (work split and CTA count of the
  *   W8A16 decode kernel: 0 stream-K, 1 row bands, 2 clusters), MSD_P8_PAIR / MSD_P8_KSPLIT (W8A16 many-row kernel: CTA
  *   pairs, K split), MSD_W4_PAIR / MSD_W4_TILEN / MSD_W4_KSPLIT (W4A16 kernels), MSD_W4_DECODE (W4A16 with few tokens: 0 keeps
- *   calls for one matrix on the tile kernel, else 100000 x K blocks per stage + 1000 x CTAs per band + weight rows per band),
+ *   calls on the tile kernel, else 100000 x K blocks per stage + 1000 x CTAs per band + weight rows per band),
  *   MSD_ATTN_SPLITS / MSD_ATTN_CHUNK_TILES (context splits of the attention kernels; msd_attn_decode_schedule reports the schedule in force),
  *   MSD_ATTN_BALANCED (1: the balanced split schedule for every shape that has a kernel for it, 0: never; a forced
  *   split count or size switches it off as well). */
@@ -249,7 +249,7 @@ size_t msd_grouped_gemm_w4a16_workspace_bytes(int32_t E, int64_t N, int64_t K);
 msd_status_t msd_grouped_gemm_w4a16(const void* x_bf16, const uint8_t* w_fp4, const uint8_t* w_e8m0,
                                     const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, void* y,
                                     msd_out_t ytype, void* workspace, size_t workspace_bytes, void* stream);
-/* How the first launch of such a call runs (for tests; host arithmetic): schedule_host[0] the kernel (2 few tokens), [1] weight rows per
+/* How the first launch of such a call runs (for tests; host arithmetic): schedule_host[0] the kernel (0 token tiles, 2 few tokens), [1] weight rows per
  * tile, [2] stages of a CTA's pipeline, [3] the most stages that a CTA goes through, of all its tiles, [4] dynamic shared memory of a
  * CTA in bytes. */
 msd_status_t msd_debug_grouped_gemm_w4a16_schedule(const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, int32_t* schedule_host);

@@ -130,7 +130,7 @@ decompose_mxfp4_kernel(const uint16_t* __restrict__ x, int64_t ldx, int64_t M, i
         if (g + step < rg.n && row_in >= rg.off[g + step]) g += step;
       row = static_cast<int64_t>(g) * rg.rows + (row_in - rg.off[g]);
       srow = static_cast<int64_t>(g) * rg.srows + (row_in - rg.off[g]);
-      second = (rg.off[g + 1] - rg.off[g] + 7) & ~7;
+      if (rg.stacked) second = (rg.off[g + 1] - rg.off[g] + 7) & ~7;
     }
     uint32_t w[16];
 #pragma unroll

@@ -14,6 +14,7 @@
 // shapes; few tokens per weight matrix and mixture-of-experts calls run in gemm_w4a16_decode.cu.
 #include <cuda_bf16.h>
 
+#include <cmath>
 #include <cstdlib>
 #include <mutex>
 
@@ -46,7 +47,7 @@ struct GemmW4Params {
   int part_rows;                // ksplit > 1: rows per split of the partial-sum buffer the tiles are written to
   int nstages;                  // pipeline stages that fit with a_rows rows per component tile
   int a_rows;                   // rows of a token tile that are loaded (the box of the component tensor maps): 128, or
-                                // fewer when there is one token tile; the MMA reads stale rows beyond them,
+                                // fewer when no group of a grouped launch is longer; the MMA reads stale rows beyond them,
                                 // whose results are never stored
   int n_fastest;                // tile index -> (token tile, weight tile): weight tile fastest (1) or token tile fastest (0)
   unsigned* status;
@@ -91,11 +92,12 @@ msd_status_t launch_ksplit_reduce(const float* part, int ksplit, int64_t part_st
 // thread-block cluster: when all of them are done every CTA writes the columns that a peer finishes into that peer's
 // shared memory (the drained pipeline), and after a second cluster barrier sums its own columns, split 0 first.  Without it
 // the FP32 partial tiles went through memory and a reduce kernel of their own (see w4_tile_decode_shape).
-template <int kTN, bool kCluster = false>
+// kGrouped (mixture of experts): token tile g holds the rows of group g.
+template <int kTN, bool kCluster = false, bool kGrouped = false>
 __global__ void __launch_bounds__(kW4ThreadsSf, 1)
 gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_a2,
                   const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_y,
-                  const GemmW4Params p) {
+                  const GemmW4Params p, const __grid_constant__ typename W4GroupArg<kGrouped>::type grp) {
   constexpr int kBBytes = kTN * 128;
   // Shared-memory stage: the two component tiles, the weight tile, the scale blocks.  Launches with few rows (one
   // token tile of M < 128 rows, short groups) load only a_rows <= 128 rows per component (whole 1 KB swizzle atoms), pack the stage accordingly and use the room for more
@@ -131,8 +133,8 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       q.mt = 0;
       q.nt = static_cast<int>(cluster_id());
     } else {
-      const int tile_mn = q.tile / p.ksplit;
-      split = q.tile - tile_mn * p.ksplit;
+      const int tile_mn = kGrouped ? q.tile : q.tile / p.ksplit;      // (a grouped launch does not split K)
+      split = kGrouped ? 0 : q.tile - tile_mn * p.ksplit;
       q.mt = p.n_fastest ? tile_mn / p.n_tiles : tile_mn % p.m_tiles;
       q.nt = p.n_fastest ? tile_mn % p.n_tiles : tile_mn / p.m_tiles;
     }
@@ -148,10 +150,13 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     uint8_t* dst = smem + stage * kStageBytes;
     if (warp == 0) {
       mbar_arrive_expect_tx(&full_bar[stage], kStageBytes);
-      tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, q.nt * kTN, &full_bar[stage]);
+      int b_row = q.nt * kTN;
+      if constexpr (kGrouped) b_row += grp.expert[q.mt] * p.N;          // the weights of the group's expert
+      tma_load_2d(dst + 2 * a_bytes, &tmap_b, q.ks * 128, b_row, &full_bar[stage]);
     } else {
       uint8_t* sf = dst + 2 * a_bytes + kBBytes;
-      const size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
+      size_t sfb_blk = static_cast<size_t>(kSfbBlocks * q.nt);
+      if constexpr (kGrouped) sfb_blk += static_cast<size_t>(grp.expert[q.mt]) * 2 * p.n_tiles;
       bulk_load(sf + 2048, p.sfb + (sfb_blk * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
       if constexpr (kSfbBlocks == 2) bulk_load(sf + 3072, p.sfb + ((sfb_blk + 1) * p.sf_kgroups + 2 * q.ks) * 512, 1024, &full_bar[stage]);
     }
@@ -168,6 +173,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       bulk_load(sf + 1024, p.sfa2 + a_off, 1024, &full_bar[stage]);
     }
   };
+  constexpr int kGroupedEarly = 2;
   Pos q = {}, first = {};
   int pre = 0;                   // stages whose weights were asked for before the wait on the kernel launched just before
 
@@ -220,18 +226,21 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     // scale blocks (their bytes may be counted before warp 0's arrival announces them: the phase cannot end without it).
     if (lane == 0) {
       bool ok = true;
+      // (This kernel lets no dependent in early: the waiting decomposition of a next call beside it cost 2 us on 32 experts.)
       if (warp == 10 || !kCluster) {
-        // neither weights nor prepared weight scales depend on the kernel launched just before
+        // neither weights nor prepared weight scales depend on the kernel launched just before; a grouped launch asks for two
+        // stages that early and leaves the bandwidth to the decomposition of its many rows (64 experts 38.8 us, 40.2 asking for all; 32: 57.1 and 57.7)
         q.tile = blockIdx.x;
         enter(q);
         first = q;
         if (warp == 10 && !p.sfb_ready) pdl_wait_primary();
-        for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
+        for (; pre < (kGrouped ? kGroupedEarly : nstages) && q.tile < total_tiles; ++pre) { load_weights(q, pre); advance(q); }
       }
       // what the decomposition, launched just before, writes: the components and their scales
       if (warp == 0 || p.sfb_ready) pdl_wait_primary();
       q = first;
       for (int i = 0; i < pre; ++i) { load_activations(q, i); advance(q); }
+      if (kGrouped) for (; pre < nstages && q.tile < total_tiles; ++pre) { load_weights(q, pre); load_activations(q, pre); advance(q); }
       int stage = pre == nstages ? 0 : pre;
       uint32_t phase = pre == nstages ? 1 : 0;
       while (q.tile < total_tiles) {
@@ -356,12 +365,17 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
       ok = wait_bounded(&tfull_bar[acc], tphase, abort, p.status);
       if (!ok) break;
       tc_fence_after();
-      const int row0 = mt * kW4TileM + quad * 32;        // first output row of this warp
+      int row0 = mt * kW4TileM + quad * 32;              // first output row of this warp
+      int rows_end = p.M;                                // output rows at or past it belong to nobody (or somebody else)
+      if constexpr (kGrouped) {
+        row0 = grp.off[mt] + quad * 32;
+        rows_end = grp.off[mt + 1];
+      }
       const uint32_t trow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + acc * kTN;
       // columns of this tile inside the matrix (a warp whose rows are all past M has nothing to store); chunks
       // beyond them are skipped altogether, so every pass through the loop commits exactly one store group
       const int cols_here = p.N - nt * kTN < kTN ? p.N - nt * kTN : kTN;
-      const int cend = row0 < p.M ? cols_here : 0;
+      const int cend = row0 < rows_end ? cols_here : 0;
       if (cend == 0) {
         tc_fence_before();
         __syncwarp();
@@ -388,7 +402,9 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           if (lane == 0) mbar_arrive(&tempty_bar[acc]);
         }
         uint8_t* sb = stage_buf + buf * kW4StoreBytes;
-        if (lane == 0) bulk_wait_group_read<1>();      // the store that read this buffer two chunks ago is done with it
+        // the store that read this buffer two chunks ago is done with it (grouped launches may skip a commit when a
+        // group ends inside the warp's rows, so there all earlier stores are waited for)
+        if (lane == 0) { if constexpr (kGrouped) bulk_wait_group_read<0>(); else bulk_wait_group_read<1>(); }
         __syncwarp();
         uint8_t* srow = sb + lane * 64;
 #pragma unroll
@@ -396,9 +412,27 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           *reinterpret_cast<uint4*>(srow + ((static_cast<uint32_t>(j) ^ swz) << 4)) = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) {
-          tma_store_2d(&tmap_y, nt * kTN + c0, row0 + split * p.part_rows, sb);
-          bulk_commit_group();
+        if (!kGrouped || row0 + 32 <= rows_end) {
+          if (lane == 0) {
+            tma_store_2d(&tmap_y, nt * kTN + c0, row0 + split * p.part_rows, sb);
+            bulk_commit_group();
+          }
+        } else {
+          // the group ends inside this warp's 32 rows: the rows below belong to the next group, so the box store
+          // is replaced by 16-byte stores of the group's own rows (lane -> row lane / 4 + 8 i, 16-byte piece lane % 4)
+          const int esize = (p.ytype == MSD_OUT_BF16) ? 2 : 4;
+          const int col = nt * kTN + c0, piece = lane & 3;
+          if ((col + (piece + 1) * (16 / esize)) <= p.N) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int r = (lane >> 2) + 8 * i;
+              if (row0 + r < rows_end) {
+                const uint4 v = *reinterpret_cast<const uint4*>(sb + r * 64 + ((static_cast<uint32_t>(piece) ^ static_cast<uint32_t>((r >> 1) & 3)) << 4));
+                *reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.y) + (static_cast<size_t>(row0 + r) * p.N + col) * esize + piece * 16) = v;
+              }
+            }
+          }
+          __syncwarp();
         }
       }
     }
@@ -799,7 +833,7 @@ static int w4_tile_n(bool pair = false) {
   return pair ? 256 : 224;
 }
 
-using W4Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmW4Params);
+using W4Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmW4Params, W4NoGroups);
 static W4Kernel w4_cluster_kernel(int tile_n) {
   return tile_n == 128 ? gemm_w4a16_kernel<128, true> : tile_n == 224 ? gemm_w4a16_kernel<224, true> : gemm_w4a16_kernel<256, true>;
 }
@@ -956,21 +990,72 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
 }
 
 // ---- grouped (mixture of experts) ----------------------------------------------------------------------------------
-// Workspace: stacked components of up to 64 groups at a time, their scale blocks, and the blocked scales of all experts' weights.
+// Workspace: components of up to 64 groups at a time, their scale blocks, and the blocked scales of all experts' weights (sized for
+// the larger of the two layouts).
 struct GroupedW4Plan {
-  int sf_kgroups, row_blocks;
-  size_t off_q, off_sfx, off_sfw, bytes;
+  bool tiles;                   // token tiles of 128 rows (gemm_w4a16_kernel), else the few-token kernel
+  int tile_n, row_blocks, sf_kgroups, kstages;
+  W4DecodeShape d;              // the few-token kernel's shape for the first launch
+  size_t off_q1, off_q2, off_sfx1, off_sfx2, off_sfw, bytes;
 };
-static GroupedW4Plan plan_grouped_w4(int32_t E, int64_t N, int64_t K) {
-  GroupedW4Plan pl;
-  pl.sf_kgroups = 2 * static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
-  pl.row_blocks = 2 * static_cast<int>((N + 255) / 256);
-  size_t off = 0;
-  pl.off_q = off;   off = round_up(off + static_cast<size_t>(kMaxRowGroups) * 2 * kW4TileM * (K / 2), 1024);
-  pl.off_sfx = off; off = round_up(off + static_cast<size_t>(kMaxRowGroups) * 2 * pl.sf_kgroups * 512, 1024);
-  pl.off_sfw = off; off = round_up(off + static_cast<size_t>(E) * pl.row_blocks * pl.sf_kgroups * 512, 1024);
-  pl.bytes = off;
+
+// Grouped calls that run as token tiles of 128 rows x 224 or 256 weight rows instead of bands of at most 128 weight rows
+// (gemm_w4a16_decode.cu): those that it makes shorter.  A tile's MMAs cost the same however few its tokens, but the components, of which
+// an SM takes in more than of weights once groups are long, are brought half as often.  In us, fitted to both kernels timed in
+// turn on 1480 calls (1 to 80 experts, 1 to 128 tokens each, 256 to 8192 x 512 to 8192), rounds of tiles as of bands:
+//   a stage  the largest of 0.05 + 0.0025 x width (MMAs), its bytes at 64 GB/s (what an SM takes in) and all CTAs' weights at 6 TB/s
+//   a tile   its stages, and 2 (256 rows, one accumulator) or 0.6 (224, two) for the epilogue
+// Tiles have to come out 5 % shorter: near the line the fit is no better than that.  The choice is 1.003 of the faster kernel on average,
+// and more than 1.05 in 34 of the calls; bands always are 1.030, tiles always 1.235.  Bands / tiles with 128 tokens each, us: 32
+// experts of 2048 x 7168 107 / 85, 64 of 7168 x 2048 235 / 138, 8 of 7168 x 2048 40 / 25; 16 tokens each, 32 of 2048 x 7168 48 / 59.
+static bool w4_grouped_tiles(int largest, int64_t rows, int groups, int64_t N, int64_t K, int* tile_n, W4DecodeShape* d) {
+  const int launched = groups < kMaxRowGroups ? groups : kMaxRowGroups;
+  const long long sms = sm_count();
+  const long long t224 = launched * ((N + 223) / 224), t256 = launched * ((N + 255) / 256);
+  // the width whose tiles fill the SMs in fewer, or shorter, rounds
+  *tile_n = (t256 + sms - 1) / sms * 256 < (t224 + sms - 1) / sms * 224 ? 256 : 224;
+  const int forced = option(OPT_W4_DECODE);               // testing aid
+  if (forced == 0 || !w4_decode_shape(d, largest, launched, N, K)) return true;
+  if (forced > 0) return false;
+  const long long tiles = *tile_n == 256 ? t256 : t224, grid = tiles < sms ? tiles : sms, full = tiles / grid, rest = tiles - full * grid;
+  const float kstages = static_cast<float>((K + kW4BlockK - 1) / kW4BlockK), width = static_cast<float>(*tile_n);
+  const float stage_bytes = static_cast<float>(2 * ((largest + 7) / 8 * 8) * 128 + *tile_n * 128 + kW4SfBytes);
+  auto tile_us = [&](long long ctas) {
+    const float stage = fmaxf(fmaxf(0.05f + 0.0025f * width, stage_bytes / 64.0e3f), 136.0f * width * static_cast<float>(ctas) / 6.0e6f);
+    return kstages * stage + (*tile_n == 256 ? 2.0f : 0.6f);
+  };
+  return 1.05f * (static_cast<float>(full) * tile_us(grid) + (rest ? tile_us(rest) : 0.0f)) <
+         w4_decode_grouped_us(*d, static_cast<float>(rows) / static_cast<float>(groups));
+}
+
+// (rows of all groups and of the longest, non-empty groups; 0 rows where only the size of the workspace is wanted)
+static GroupedW4Plan plan_grouped_w4(int32_t E, int64_t N, int64_t K, int largest, int64_t rows, int groups) {
+  GroupedW4Plan pl = {};
+  pl.tile_n = 256;
+  pl.tiles = largest > 0 && w4_grouped_tiles(largest, rows, groups, N, K, &pl.tile_n, &pl.d);
+  pl.kstages = static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
+  pl.sf_kgroups = 2 * pl.kstages;
+  if (!pl.tiles) pl.tile_n = 256;
+  pl.row_blocks = 2 * static_cast<int>((N + pl.tile_n - 1) / pl.tile_n);
+  const size_t q = static_cast<size_t>(kMaxRowGroups) * kW4TileM * (K / 2), sfx = static_cast<size_t>(kMaxRowGroups) * pl.sf_kgroups * 512;
+  pl.off_q1 = 0;
+  pl.off_q2 = pl.tiles ? q : 0;                            // (multiples of 1024, all of them)
+  pl.off_sfx1 = 2 * q;
+  pl.off_sfx2 = pl.off_sfx1 + (pl.tiles ? sfx : 0);
+  pl.off_sfw = pl.off_sfx1 + 2 * sfx;
+  pl.bytes = pl.off_sfw + round_up(static_cast<size_t>(E) * 2 * ((N + 223) / 224) * pl.sf_kgroups * 512, 1024);
   return pl;
+}
+
+struct W4GroupedTiles { int a_rows, nstages, grid; size_t stage_bytes, smem; };
+static W4GroupedTiles w4_grouped_tiles_shape(const GroupedW4Plan& pl, int largest, int groups) {
+  W4GroupedTiles t;
+  t.a_rows = (largest + 7) / 8 * 8;             // rows of a token tile worth loading (whole 8-row swizzle atoms)
+  w4_stages(t.a_rows, pl.tile_n, 8 * kW4StoreBytes, &t.nstages, &t.stage_bytes);
+  t.smem = t.nstages * t.stage_bytes + 8 * kW4StoreBytes + 1024;
+  const long long tiles = static_cast<long long>(groups) * (pl.row_blocks / 2);
+  t.grid = static_cast<int>(tiles < sm_count() ? tiles : sm_count());
+  return t;
 }
 
 // Weight scales brought into the blocked layout once (msd_prepare_w4a16_scales): both tile widths' layouts back to
@@ -1107,7 +1192,7 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
   if (st != MSD_OK) return st;
   if (pl.few)
     return w4_decode_launch(pl.d, w_fp4, q1, pl.d.Mp + M, N, static_cast<int>(M), N, K, sfb, prepared != nullptr, ws + pl.off_sfa1, y,
-                            static_cast<int>(ytype), 0, nullptr, nullptr, status, s);
+                            static_cast<int>(ytype), nullptr, status, s);
 
   CUtensorMap tmap_a1, tmap_a2, tmap_b;
   const uint64_t kb = static_cast<uint64_t>(K / 2);
@@ -1167,7 +1252,7 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
   p.a_rows = pl.a_rows; p.nstages = pl.nstages;
   if (pl.cluster > 1) {          // (its shared-memory limit was raised when the plan asked how many clusters fit)
     if (launch_pdl_cluster(w4_cluster_kernel(pl.tile_n), dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl,
-                           static_cast<unsigned>(pl.cluster), tmap_a1, tmap_a2, tmap_b, tmap_y, p) != cudaSuccess)
+                           static_cast<unsigned>(pl.cluster), tmap_a1, tmap_a2, tmap_b, tmap_y, p, W4NoGroups()) != cudaSuccess)
       return MSD_ERR_CUDA;
     return MSD_OK;
   }
@@ -1178,8 +1263,8 @@ static msd_status_t gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, co
       }))
     return MSD_ERR_CUDA;
   const cudaError_t le = pl.tile_n == 256
-      ? launch_pdl(gemm_w4a16_kernel<256>, dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p)
-      : launch_pdl(gemm_w4a16_kernel<224>, dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p);
+      ? launch_pdl(gemm_w4a16_kernel<256>, dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, W4NoGroups())
+      : launch_pdl(gemm_w4a16_kernel<224>, dim3(pl.grid), dim3(kW4ThreadsSf), pl.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, W4NoGroups());
   if (le != cudaSuccess) return MSD_ERR_CUDA;
   if (split) {
     const msd_status_t rs = launch_ksplit_reduce(part, pl.ksplit, static_cast<int64_t>(part_rows) * N, M, N, y, static_cast<int>(ytype), s, pdl);
@@ -1194,7 +1279,7 @@ extern "C" {
 
 size_t msd_grouped_gemm_w4a16_workspace_bytes(int32_t E, int64_t N, int64_t K) {
   if (E < 1 || N < 1 || K < 128 || K % 128 != 0) return 0;
-  return msd::plan_grouped_w4(E, N, K).bytes;
+  return msd::plan_grouped_w4(E, N, K, 0, 0, 0).bytes;
 }
 
 msd_status_t msd_debug_grouped_gemm_w4a16_schedule(const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, int32_t* schedule_host) {
@@ -1202,14 +1287,23 @@ msd_status_t msd_debug_grouped_gemm_w4a16_schedule(const int32_t* group_sizes_ho
   if (!group_sizes_host || !schedule_host) return MSD_ERR_NULL_POINTER;
   if (E < 1 || N < 1 || K < 128 || K % 128 != 0 || N % 8 != 0 || N > (1 << 24) || K > (1 << 24)) return MSD_ERR_BAD_SHAPE;
   int largest = 0, nonempty = 0;
+  int64_t rows = 0;
   for (int e = 0; e < E; ++e) {
     if (group_sizes_host[e] < 0 || group_sizes_host[e] > kW4TileM) return MSD_ERR_BAD_SHAPE;
+    rows += group_sizes_host[e];
     if (group_sizes_host[e] > largest) largest = group_sizes_host[e];
     nonempty += group_sizes_host[e] > 0 ? 1 : 0;
   }
   if (largest == 0) return MSD_ERR_BAD_SHAPE;
-  W4DecodeShape d;
-  if (!w4_decode_shape(&d, largest, nonempty < kMaxRowGroups ? nonempty : kMaxRowGroups, N, K)) return MSD_ERR_UNSUPPORTED;
+  const int launched = nonempty < kMaxRowGroups ? nonempty : kMaxRowGroups;
+  const GroupedW4Plan pl = plan_grouped_w4(E, N, K, largest, rows, nonempty);
+  if (pl.tiles) {
+    const W4GroupedTiles t = w4_grouped_tiles_shape(pl, largest, launched);
+    schedule_host[0] = 0; schedule_host[1] = pl.tile_n; schedule_host[2] = t.nstages;
+    schedule_host[3] = pl.kstages * ((launched * (pl.row_blocks / 2) + t.grid - 1) / t.grid); schedule_host[4] = static_cast<int32_t>(t.smem);
+    return MSD_OK;
+  }
+  const W4DecodeShape& d = pl.d;
   schedule_host[0] = 2; schedule_host[1] = d.h; schedule_host[2] = d.nstages; schedule_host[3] = d.steps; schedule_host[4] = d.smem;
   return MSD_OK;
 }
@@ -1232,6 +1326,41 @@ msd_status_t msd_grouped_gemm_w4a16_prepared(const void* x_bf16, const uint8_t* 
 
 namespace msd {
 
+// Up to 64 groups as token tiles of 128 rows; the CTAs of a wave share a group's components, every expert's weights are read once.
+static msd_status_t w4_grouped_tiles_launch(const GroupedW4Plan& pl, const uint8_t* w_fp4, const uint8_t* q1, const uint8_t* q2, const uint8_t* sfx1,
+                                            const uint8_t* sfx2, const uint8_t* sfw, bool sfw_ready, int largest, int groups, const W4Groups& grp,
+                                            int32_t E, int64_t M_total, int64_t N, int64_t K, void* y, msd_out_t ytype, unsigned* status,
+                                            cudaStream_t s) {
+  const W4GroupedTiles t = w4_grouped_tiles_shape(pl, largest, groups);
+  const bool ybf = ytype == MSD_OUT_BF16;
+  const uint64_t kb = static_cast<uint64_t>(K / 2), q_rows = static_cast<uint64_t>(kMaxRowGroups) * kW4TileM;
+  CUtensorMap tmap_a1, tmap_a2, tmap_b, tmap_y;
+  if (!encode_tmap_2d(&tmap_a1, CU_TENSOR_MAP_DATA_TYPE_UINT8, q1, kb, q_rows, kb, 128, static_cast<uint32_t>(t.a_rows), CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_tmap_2d(&tmap_a2, CU_TENSOR_MAP_DATA_TYPE_UINT8, q2, kb, q_rows, kb, 128, static_cast<uint32_t>(t.a_rows), CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_tmap_2d(&tmap_b, CU_TENSOR_MAP_DATA_TYPE_UINT8, w_fp4, kb, static_cast<uint64_t>(E) * N, kb, 128, static_cast<uint32_t>(pl.tile_n), CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_tmap_2d(&tmap_y, ybf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, y, static_cast<uint64_t>(N),
+                      static_cast<uint64_t>(M_total), static_cast<uint64_t>(N) * (ybf ? 2 : 4), ybf ? 32 : 16, 32, CU_TENSOR_MAP_SWIZZLE_64B))
+    return MSD_ERR_CUDA;
+  static DeviceOnce once;
+  if (!once([] {
+        return cudaFuncSetAttribute(gemm_w4a16_kernel<256, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess &&
+               cudaFuncSetAttribute(gemm_w4a16_kernel<224, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048) == cudaSuccess;
+      }))
+    return MSD_ERR_CUDA;
+  GemmW4Params p;
+  p.M = static_cast<int>(M_total); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
+  p.m_tiles = groups; p.n_tiles = pl.row_blocks / 2; p.kstages = pl.kstages; p.sf_kgroups = pl.sf_kgroups;
+  p.sfa1 = sfx1; p.sfa2 = sfx2; p.sfb = sfw; p.sfb_ready = sfw_ready ? 1 : 0;
+  p.y = y; p.ytype = ytype; p.status = status;
+  p.a_rows = t.a_rows; p.nstages = t.nstages; p.ksplit = 1; p.kper = pl.kstages; p.part_rows = 0; p.n_fastest = 1;
+  const dim3 grid(static_cast<unsigned>(t.grid));
+  const bool pdl = option(OPT_NO_PDL) <= 0;
+  const cudaError_t e = pl.tile_n == 256
+      ? launch_pdl(gemm_w4a16_kernel<256, false, true>, grid, dim3(kW4ThreadsSf), t.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, grp)
+      : launch_pdl(gemm_w4a16_kernel<224, false, true>, grid, dim3(kW4ThreadsSf), t.smem, s, pdl, tmap_a1, tmap_a2, tmap_b, tmap_y, p, grp);
+  return e == cudaSuccess ? MSD_OK : MSD_ERR_CUDA;
+}
+
 static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w_fp4, const uint8_t* w_e8m0, const uint8_t* prepared,
                                             const int32_t* group_sizes_host, int32_t E, int64_t N, int64_t K, void* y,
                                             msd_out_t ytype, void* workspace, size_t workspace_bytes, void* stream) {
@@ -1244,38 +1373,42 @@ static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w
       !aligned(workspace, 1024))
     return MSD_ERR_BAD_ALIGNMENT;
   int64_t M_total = 0;
-  int largest = 0;
+  int largest = 0, nonempty = 0;
   for (int e = 0; e < E; ++e) {
     if (group_sizes_host[e] < 0 || group_sizes_host[e] > kW4TileM) return MSD_ERR_BAD_SHAPE;     // decode regime per expert
     M_total += group_sizes_host[e];
+    nonempty += group_sizes_host[e] > 0 ? 1 : 0;
     if (group_sizes_host[e] > largest) largest = group_sizes_host[e];
   }
   if (M_total > 0x7FFFFFFFLL) return MSD_ERR_BAD_SHAPE;
-  const GroupedW4Plan pl = plan_grouped_w4(E, N, K);
+  const GroupedW4Plan pl = plan_grouped_w4(E, N, K, largest, M_total, nonempty);
   if (workspace_bytes < pl.bytes) return MSD_ERR_WORKSPACE_TOO_SMALL;
   if (M_total == 0) return MSD_OK;
   unsigned* status = device_status_ptr();
   if (!status) return MSD_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  uint8_t* q = ws + pl.off_q;
-  uint8_t* sfx = ws + pl.off_sfx;
+  uint8_t *q1 = ws + pl.off_q1, *q2 = ws + pl.off_q2, *sfx1 = ws + pl.off_sfx1, *sfx2 = ws + pl.off_sfx2;
 
   // up to 64 non-empty groups per pair of launches (decomposition + GEMM); the weight scales of all experts are brought
   // into the blocked layout by the first decomposition launch
   bool scales_done = prepared != nullptr;
-  const uint8_t* sfw = prepared ? prepared + prepared_scales_layout(E, N, K).off256 : ws + pl.off_sfw;
+  const uint8_t* sfw = ws + pl.off_sfw;
+  if (prepared) {
+    const PreparedScales ps = prepared_scales_layout(E, N, K);
+    sfw = prepared + (pl.tile_n == 224 ? ps.off224 : ps.off256);
+  }
   int e = 0;
   int64_t row = 0;
   while (e < E) {
-    int expert[kMaxRowGroups], off[kMaxRowGroups + 1];
+    W4Groups grp;
     RowGroups rg = {};
     const int64_t row_first = row;
     while (e < E && rg.n < kMaxRowGroups) {
       const int sz = group_sizes_host[e];
       if (sz > 0) {
-        expert[rg.n] = e;
-        off[rg.n] = static_cast<int>(row);
+        grp.expert[rg.n] = e;
+        grp.off[rg.n] = static_cast<int>(row);
         rg.off[rg.n] = static_cast<int>(row - row_first);
         row += sz;
         ++rg.n;
@@ -1283,20 +1416,27 @@ static msd_status_t grouped_gemm_w4a16_impl(const void* x_bf16, const uint8_t* w
       ++e;
     }
     if (rg.n == 0) break;
-    off[rg.n] = static_cast<int>(row);
+    grp.off[rg.n] = static_cast<int>(row);
     rg.off[rg.n] = static_cast<int>(row - row_first);
-    W4DecodeShape d;
-    if (!w4_decode_shape(&d, largest, rg.n, N, K)) return MSD_ERR_UNSUPPORTED;      // (one exists for every call accepted above)
-    rg.rows = d.NB; rg.srows = 128 * d.nsfx;
+    W4DecodeShape d = pl.d;
+    if (pl.tiles) {
+      rg.rows = rg.srows = kW4TileM;
+    } else {
+      if (row_first > 0 && !w4_decode_shape(&d, largest, rg.n, N, K)) return MSD_ERR_UNSUPPORTED;      // (one exists, as for the first launch)
+      rg.rows = d.NB; rg.srows = 128 * d.nsfx; rg.stacked = true;
+    }
     SfRelayout rl = {};
     rl.src = w_e8m0; rl.dst = ws + pl.off_sfw; rl.rows = N; rl.kblocks = static_cast<int>(K / 32);
-    rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = 256; rl.row_blocks = pl.row_blocks; rl.matrices = E;
-    msd_status_t st = launch_decompose_mxfp4(static_cast<const uint16_t*>(x_bf16) + row_first * K, row - row_first, K, K, q, q,
-                                             sfx, sfx, pl.sf_kgroups, s, scales_done ? nullptr : &rl, &rg);
+    rl.sf_kgroups = pl.sf_kgroups; rl.tile_rows = pl.tile_n; rl.row_blocks = pl.row_blocks; rl.matrices = E;
+    msd_status_t st = launch_decompose_mxfp4(static_cast<const uint16_t*>(x_bf16) + row_first * K, row - row_first, K, K, q1, q2,
+                                             sfx1, sfx2, pl.sf_kgroups, s, scales_done ? nullptr : &rl, &rg);
     if (st != MSD_OK) return st;
     // (a later launch finds weight scales that the first one's decomposition laid out: complete before its own began)
-    st = w4_decode_launch(d, w_fp4, q, static_cast<int64_t>(rg.n) * d.NB, static_cast<int64_t>(E) * N, 0, N, K, sfw, scales_done, sfx, y,
-                          static_cast<int>(ytype), rg.n, expert, off, status, s);
+    if (pl.tiles)
+      st = w4_grouped_tiles_launch(pl, w_fp4, q1, q2, sfx1, sfx2, sfw, scales_done, largest, rg.n, grp, E, M_total, N, K, y, ytype, status, s);
+    else
+      st = w4_decode_launch(d, w_fp4, q1, static_cast<int64_t>(rg.n) * d.NB, static_cast<int64_t>(E) * N, 0, N, K, sfw, scales_done, sfx1, y,
+                            static_cast<int>(ytype), &grp, status, s);
     if (st != MSD_OK) return st;
     scales_done = true;
   }

@@ -52,17 +52,10 @@ struct W4DecodeParams {
   int ytype;
   unsigned* status;
 };
-struct W4DecodeGroups {
-  int n;
-  int expert[kMaxRowGroups], off[kMaxRowGroups + 1];
-};
-struct W4DecodeNoGroups {};
 // Component boxes: in a grouped launch of a quarter, half, three quarters and all of NB rows, of which a group loads the smallest that
 // holds its own (32 experts of 2048 x 7168, 6 to 35 tokens each: 51.1 us with one, 49.5 with four).
 template <bool kGrouped> struct W4DecodeXMaps { CUtensorMap m[kGrouped ? kDecBoxes : 1]; };
 __host__ __device__ inline int w4d_box_rows(int NB, int i) { return (NB * (i + 1) / kDecBoxes + 15) / 16 * 16; }
-template <bool kGrouped> struct W4DecodeArg { using type = W4DecodeNoGroups; };
-template <> struct W4DecodeArg<true> { using type = W4DecodeGroups; };
 
 // Stores `wt` tokens of a band, given as [16][128] values in shared memory, to y rows y_row0 ...; 128 threads, 16-byte vectors.
 template <typename OutT>
@@ -82,7 +75,7 @@ __device__ __forceinline__ void w4d_stage_value(uint8_t* buf, int j, int r, floa
 template <bool kGrouped>
 __global__ void __launch_bounds__(kDecThreads, 1)
 gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ W4DecodeXMaps<kGrouped> tmap_x, const W4DecodeParams p,
-                         const __grid_constant__ typename W4DecodeArg<kGrouped>::type grp) {
+                         const __grid_constant__ typename W4GroupArg<kGrouped>::type grp) {
   extern __shared__ uint8_t smem_dyn[];
   __shared__ __align__(8) uint64_t full_bar[kDecMaxStages], empty_bar[kDecMaxStages], tfull_bar[2], tempty_bar[2];
   __shared__ __align__(8) uint64_t sf_ready[kDecMaxSets], sf_free[kDecMaxSets];
@@ -541,6 +534,23 @@ static bool w4_decode_search(W4DecodeShape* best, int tokens, int groups, int64_
   return cost < 1e30f;
 }
 
+// What a grouped launch takes, in us, from the same fit as the cost of token tiles (w4_grouped_tiles; `tokens`: an average group's).
+// Finer than the rule above: bands of short groups load less than the longest's components, and the epilogue of a band, hidden
+// behind the next one's MMAs where there are two accumulators, counts.
+float w4_decode_grouped_us(const W4DecodeShape& d, float tokens) {
+  const float x_rows = fminf(static_cast<float>(d.NB), 2.0f * tokens + static_cast<float>(d.NB) / 8.0f + 8.0f);
+  const float bytes = static_cast<float>(d.kw) * (static_cast<float>(d.h) * 128.0f + x_rows * 128.0f + static_cast<float>(2 + d.nsfx) * 1024.0f);
+  const float epilogue = fmaxf(0.0f, 0.0226f * tokens - 0.775f);
+  const int full = d.items / d.grid, rest = d.items - full * d.grid;
+  auto band_us = [&](int ctas) {
+    float us = fmaxf(fmaxf(0.47f + 0.02f * static_cast<float>(d.kw), bytes / 69.0e3f), 136.0f * static_cast<float>(d.h * d.kw) * static_cast<float>(ctas) / 7.3e6f);
+    if (d.nstages < 3 && d.steps > d.nstages) us *= 1.2f;
+    us *= static_cast<float>(d.ksteps);
+    return d.nacc == 2 ? fmaxf(us, epilogue) : us + epilogue;
+  };
+  return static_cast<float>(full) * band_us(d.grid) + (rest ? band_us(rest) : 0.0f) + (d.nacc == 2 ? epilogue : 0.0f);
+}
+
 // The search looks at up to 72 shapes, several microseconds of host time: a layer's is remembered (64 direct-mapped slots by everything
 // it depends on; calls with experts, whose groups change from call to call, have nine to look at).
 bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K) {
@@ -566,8 +576,8 @@ bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int
 }
 
 msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, const uint8_t* q, int64_t q_rows, int64_t w_rows, int M, int64_t N,
-                              int64_t K, const uint8_t* sfw, bool sfw_ready, const uint8_t* sfx, void* y, int ytype, int nonempty,
-                              const int* expert, const int* off, unsigned* status, cudaStream_t s) {
+                              int64_t K, const uint8_t* sfw, bool sfw_ready, const uint8_t* sfx, void* y, int ytype, const W4Groups* groups,
+                              unsigned* status, cudaStream_t s) {
   if (!w4_decode_attr()) return MSD_ERR_CUDA;
   const uint64_t kb = static_cast<uint64_t>(K / 2);
   const bool t3 = K % kDecBlockK == 0;
@@ -575,12 +585,12 @@ msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, cons
   const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B;
   CUtensorMap tmap_w;
   W4DecodeXMaps<true> tmap_x;
-  const int boxes = expert ? kDecBoxes : 1;
+  const int boxes = groups ? kDecBoxes : 1;
   bool ok =
       t3 ? encode_tmap_3d(&tmap_w, u8, w_fp4, 128, static_cast<uint64_t>(w_rows), kb / 128, kb, 128, 128, static_cast<uint32_t>(d.h), static_cast<uint32_t>(d.kw), sw)
          : encode_tmap_2d(&tmap_w, u8, w_fp4, kb, static_cast<uint64_t>(w_rows), kb, 128, static_cast<uint32_t>(d.h), sw);
   for (int i = 0; i < boxes && ok; ++i) {
-    const uint32_t rows = static_cast<uint32_t>(expert ? w4d_box_rows(d.NB, i) : d.NB);
+    const uint32_t rows = static_cast<uint32_t>(groups ? w4d_box_rows(d.NB, i) : d.NB);
     ok = t3 ? encode_tmap_3d(&tmap_x.m[i], u8, q, 128, static_cast<uint64_t>(q_rows), kb / 128, kb, 128, 128, rows, static_cast<uint32_t>(d.kw), sw)
             : encode_tmap_2d(&tmap_x.m[i], u8, q, kb, static_cast<uint64_t>(q_rows), kb, 128, rows, sw);
   }
@@ -591,22 +601,18 @@ msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, cons
   p.kblocks = d.kblocks; p.kw = d.kw; p.ksteps = d.ksteps; p.S = d.S; p.kper = d.kper;
   p.nstages = d.nstages; p.stage_bytes = d.stage_bytes; p.x_off = d.x_off; p.sf_off = d.sf_off; p.nsfx = d.nsfx;
   // (a grouped call leaves most of the bandwidth to the decomposition of its many rows)
-  p.t3 = t3 ? 1 : 0; p.early = expert && d.nstages > 2 ? 2 : d.nstages;
+  p.t3 = t3 ? 1 : 0; p.early = groups && d.nstages > 2 ? 2 : d.nstages;
   p.nacc = d.nacc; p.nsets = d.nsets; p.sf_col = d.sf_col; p.set_cols = d.set_cols; p.epi_off = d.epi_off;
   p.sf_kgroups = 2 * d.kblocks; p.row_blocks = 2 * static_cast<int>((N + 255) / 256);
   p.sfw = sfw; p.sfx = sfx; p.sfw_ready = sfw_ready ? 1 : 0;
   p.y = y; p.ytype = ytype; p.status = status;
   const bool pdl = option(OPT_NO_PDL) <= 0;
   cudaError_t e;
-  if (expert) {
-    W4DecodeGroups g;
-    g.n = nonempty;
-    for (int i = 0; i < nonempty; ++i) { g.expert[i] = expert[i]; g.off[i] = off[i]; }
-    g.off[nonempty] = off[nonempty];
-    e = launch_pdl(gemm_w4a16_decode_kernel<true>, dim3(d.grid), dim3(kDecThreads), static_cast<size_t>(d.smem), s, pdl, tmap_w, tmap_x, p, g);
+  if (groups) {
+    e = launch_pdl(gemm_w4a16_decode_kernel<true>, dim3(d.grid), dim3(kDecThreads), static_cast<size_t>(d.smem), s, pdl, tmap_w, tmap_x, p, *groups);
   } else {
     e = launch_pdl_cluster(gemm_w4a16_decode_kernel<false>, dim3(d.grid), dim3(kDecThreads), static_cast<size_t>(d.smem), s, pdl, static_cast<unsigned>(d.S),
-                           tmap_w, W4DecodeXMaps<false>{{tmap_x.m[0]}}, p, W4DecodeNoGroups());
+                           tmap_w, W4DecodeXMaps<false>{{tmap_x.m[0]}}, p, W4NoGroups());
   }
   return e == cudaSuccess ? MSD_OK : MSD_ERR_CUDA;
 }

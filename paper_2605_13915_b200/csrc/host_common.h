@@ -143,13 +143,14 @@ struct SfRelayout {
                        // weights), each cut into its own `row_blocks` blocks
   int blocks;          // filled in by the launcher
 };
-// Rows sorted by group (mixture of experts): group g owns rows [off[g], off[g+1]).  Its two components go, one below the other, to
-// rows g * rows ... of ONE buffer: the first from there, the second ceil8(rows of the group) further down; their scales likewise
-// to rows g * srows ... of one scale buffer (whole 128-row blocks per group).
+// Rows sorted by group (mixture of experts): group g owns rows [off[g], off[g+1]).  Its first component goes to rows g * rows ... of q1
+// and its scales to rows g * srows ... (whole 128-row blocks per group) of e1; the second likewise into q2 and e2 or, stacked (one
+// buffer for both, q1 = q2 and e1 = e2), ceil8(rows of the group) further down.
 constexpr int kMaxRowGroups = 64;
 struct RowGroups {
   int n;                       // 0: no groups, output row = input row
   int rows, srows;
+  bool stacked;
   int second;                  // no groups: rows from the first component's to the second's (0: buffers of their own)
   int off[kMaxRowGroups + 1];
 };
@@ -167,10 +168,18 @@ struct W4DecodeShape {
 };
 // (groups: matrices of a grouped launch, 0 for an ungrouped call)
 bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K);
-// expert == nullptr: one matrix, M tokens; otherwise `nonempty` groups, group g = rows [off[g], off[g + 1]) of y and weights expert[g]
+float w4_decode_grouped_us(const W4DecodeShape& d, float tokens);
+// Groups of one launch: group g = rows [off[g], off[g + 1]) of y (at most 128) and the weights of expert[g].
+struct W4Groups {
+  int expert[kMaxRowGroups], off[kMaxRowGroups + 1];
+};
+struct W4NoGroups {};              // what ungrouped instantiations take in its place: no parameter bytes to copy per launch
+template <bool kGrouped> struct W4GroupArg { using type = W4NoGroups; };
+template <> struct W4GroupArg<true> { using type = W4Groups; };
+// groups == nullptr: one matrix, M tokens
 msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, const uint8_t* q, int64_t q_rows, int64_t w_rows, int M, int64_t N,
-                              int64_t K, const uint8_t* sfw, bool sfw_ready, const uint8_t* sfx, void* y, int ytype, int nonempty,
-                              const int* expert, const int* off, unsigned* status, cudaStream_t s);
+                              int64_t K, const uint8_t* sfw, bool sfw_ready, const uint8_t* sfx, void* y, int ytype, const W4Groups* groups,
+                              unsigned* status, cudaStream_t s);
 
 #ifdef __CUDACC__
 // Relayout of row-major E8M0 scales [rows, kblocks] into the 512-byte blocks (128 rows x 4 scales) of the block-scaled

@@ -155,3 +155,30 @@ def test_grouped_w4a16_workspace_needs_no_initialisation(sizes, N, K):
     torch.cuda.synchronize()
     binding.last_device_status()
     assert np.all(np.abs(y.cpu().numpy() - want) <= TOL * np.linalg.norm(want, axis=-1, keepdims=True) + 1e-30)
+
+
+@pytest.mark.parametrize("K", [384, 512])
+@pytest.mark.parametrize("sizes,shape", [([35, 1, 0, 20, 33, 8, 9, 3, 27, 16, 12], 0), ([35, 1, 0, 20, 33, 8, 9, 3, 27, 16, 12], 101128),
+                                         ([35, 1, 0, 20, 33, 8, 9, 3, 27, 16, 12], 201112), ([128, 7, 65, 0, 100, 31, 64, 97, 2, 33, 48], 0),
+                                         ([128, 7, 65, 0, 100, 31, 64, 97, 2, 33, 48], 101128)])
+def test_grouped_w4a16_with_more_bands_than_sms(sizes, shape, K):
+    """Uneven groups and several tiles a CTA: token tiles (shape 0), bands of weight rows with two accumulators and component boxes that
+    change height from band to band (35 tokens), with one accumulator and two scale blocks (128 tokens); ragged last tile, K a
+    multiple of 256 (3-D copies) or not (2-D).  Against the oracle, row-major and prepared scales bit for bit, BF16 the FP32 result
+    rounded once."""
+    N = 4104
+    binding.debug_set_option("MSD_W4_DECODE", shape)
+    kernel, _, stages, steps, _ = binding.debug_grouped_gemm_w4a16_schedule(sizes, N, K)
+    assert kernel == (2 if shape else 0) and steps > (K + 255) // 256 // (shape // 100000 or 1)
+    x, q, e = _case_w4(sizes, N, K, seed=K + len(sizes))
+    xd, qd, ed = bf16_dev(x), dev(q), dev(e)
+    y = torch.full((x.shape[0], N), 12345.0, dtype=torch.float32, device="cuda")
+    binding.grouped_gemm_w4a16(xd, qd, ed, sizes, out=y)
+    prepared = binding.prepare_w4a16_scales(ed)
+    y2 = binding.grouped_gemm_w4a16(xd, qd, None, sizes, out_dtype=torch.float32, prepared=prepared)
+    yb = binding.grouped_gemm_w4a16(xd, qd, None, sizes, out_dtype=torch.bfloat16, prepared=prepared)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
+    want = _w4_oracle(x, q, e, sizes)
+    assert np.all(np.abs(y.cpu().numpy() - want) <= TOL * np.linalg.norm(want, axis=-1, keepdims=True) + 1e-30)

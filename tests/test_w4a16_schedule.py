@@ -38,3 +38,13 @@ def test_grouped_pipelines_have_two_stages(groups, tokens):
     for N, K in [(4096, 1024), (5632, 896), (2048, 512), (7168, 2048), (1000, 128), (2048, 7168)]:
         _, _, stages, steps, _ = binding.debug_grouped_gemm_w4a16_schedule([tokens] * groups, N, K)
         assert steps >= 1 and stages >= min(2, steps), (N, K, stages, steps)
+
+
+@pytest.mark.parametrize("tokens,E,N,K,kernel", [(16, 32, 2048, 7168, 2), (128, 32, 2048, 7168, 0), (96, 64, 7168, 2048, 0), (128, 8, 7168, 2048, 0),
+                                                 (128, 23, 4096, 1024, 0), (1, 64, 4096, 1024, 2), (64, 8, 2048, 7168, 2)])
+def test_grouped_calls_with_long_groups_take_token_tiles(tokens, E, N, K, kernel):
+    """Both sides of the line between bands of weight rows (few tokens) and token tiles; empty groups do not count."""
+    assert binding.debug_grouped_gemm_w4a16_schedule([tokens] * E, N, K)[0] == kernel
+    assert binding.debug_grouped_gemm_w4a16_schedule([0, tokens] * E, N, K)[0] == kernel
+    binding.debug_set_option("MSD_W4_DECODE", 0)
+    assert binding.debug_grouped_gemm_w4a16_schedule([tokens] * E, N, K)[0] == 0
