@@ -989,6 +989,24 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   return pl;
 }
 
+// What a caller is asked for: enough for calls with fewer tokens too.  Those may run in another kernel, with the other layout of the
+// weight scales or with the components stacked, and need more than the call itself.  (Partial sums in memory are counted for this M only.)
+static size_t w4_workspace_bytes(int64_t M, int64_t N, int64_t K) {
+  const GemmW4Plan pl = plan_w4(M, N, K);
+  const size_t block = static_cast<size_t>(pl.sf_kgroups) * 512;
+  auto scales = [&](int64_t tile_rows) { return round_up(static_cast<size_t>(2 * ((N + tile_rows - 1) / tile_rows)) * block, 1024); };
+  const size_t widest = scales(224) > scales(256) ? scales(224) : scales(256);
+  size_t bytes = pl.few ? pl.bytes : pl.bytes - scales(pl.sf_tile_rows) + widest;
+  if (M <= kW4TileM) {
+    const int64_t Mp = (M + 7) / 8 * 8;
+    const size_t stacked = round_up(static_cast<size_t>(Mp + M) * (K / 2), 1024) + round_up((2 * Mp > 128 ? 2 : 1) * block, 1024) + scales(256);
+    const size_t tiles = 2 * (round_up(static_cast<size_t>(M) * (K / 2), 1024) + round_up(block, 1024)) + widest;
+    if (stacked > bytes) bytes = stacked;
+    if (tiles > bytes) bytes = tiles;
+  }
+  return bytes;
+}
+
 // ---- grouped (mixture of experts) ----------------------------------------------------------------------------------
 // Workspace: components of up to 64 groups at a time, their scale blocks, and the blocked scales of all experts' weights (sized for
 // the larger of the two layouts).
@@ -1116,7 +1134,7 @@ msd_status_t msd_prepare_w4a16_scales(const uint8_t* w_e8m0, int32_t E, int64_t 
 
 size_t msd_gemm_w4a16_workspace_bytes(int64_t M, int64_t N, int64_t K) {
   if (M < 1 || N < 1 || K < 128 || K % 128 != 0) return 0;
-  return msd::plan_w4(M, N, K).bytes;
+  return msd::w4_workspace_bytes(M, N, K);
 }
 
 msd_status_t msd_debug_gemm_w4a16_schedule(int64_t M, int64_t N, int64_t K, int32_t* schedule_host) {

@@ -191,3 +191,10 @@ def test_padding_scales_in_a_used_workspace(M, N, K, before):
     binding.last_device_status()
     assert torch.equal(y, want)
     _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)
+
+
+@pytest.mark.parametrize("N,K", [(5760, 9984), (8192, 2048), (8192, 2176), (14336, 4096), (520, 1024)])
+def test_workspace_for_many_tokens_serves_fewer(N, K):
+    """The kernel changes with the token count; a workspace asked for at one count is enough at every smaller one."""
+    sizes = [binding.gemm_w4a16_workspace_bytes(M, N, K) for M in range(1, 129)]
+    assert sizes == sorted(sizes)
