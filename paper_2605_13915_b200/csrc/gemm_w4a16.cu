@@ -915,15 +915,63 @@ static void w4_tile_decode_shape(int64_t M, int64_t N, int kstages, int* tile_n,
   }
 }
 
-// Calls of at most 128 tokens that the kernel of gemm_w4a16_decode.cu takes: all where it leaves K whole, and up to 32 tokens where it
-// splits it (then the sums exchanged and the components each CTA loads grow with the tokens, and tiles of 128 tokens x 128 to 256
-// weight rows with half as many CTAs per row cost less: 4096 x 14336, 16 tokens 12.7 us here and 15.1 there, 61 tokens 16.5
-// and 15.0; 2560 x 9984, 29 tokens 10.7 and 12.0; K whole, 14336 x 4096, 61 tokens 12.5 and 14.4, 128 tokens 15.4 and 16.0).
-// One weight tile with so long a K that eight CTAs are too few for it is split through memory.
-static bool w4_decode_takes(W4DecodeShape* d, int64_t M, int64_t N, int64_t K, int kstages) {
-  const int forced = option(OPT_W4_DECODE);          // testing aid: 0 never, a shape wherever it fits
-  if (M > kW4TileM || forced == 0 || (N <= 224 && kstages > 28)) return false;
-  return w4_decode_shape(d, static_cast<int>(M), 0, N, K) && (forced > 0 || d->S == 1 || M <= 32);
+// K splits through memory of `tiles` output tiles: about one work item per SM, each at least four stages long.
+static int w4_memory_split(long long tiles, int kstages) {
+  const int want = 2 * tiles <= sm_count() ? static_cast<int>(sm_count() / tiles) : 1;
+  return want > kstages / 4 ? kstages / 4 : want;
+}
+
+// Calls of at most 128 tokens: the kernel of gemm_w4a16_decode.cu or tiles, whichever costs less.  In us, fitted to 594 calls timed with
+// both (1 to 128 tokens, most above 16, 256 to 20480 x 512 to 16384), tiles
+//   a stage  the larger of 0.0044 x width - 0.22 (MMAs) and all CTAs' weights at 4.6 TB/s
+//   a call   its rounds of stages, 0.0022 x tokens, and with a cluster of S 0.00021 x tokens x width x (S - 1) / S + 0.36 S for the exchange
+// and bands as in w4_decode_us.  The choice is 1.003 of the faster one on average, bands always 1.018, tiles always 1.117.  Tiles win with 60
+// tokens and more where bands need a second round or the components outweigh the weights, us bands / tiles: 76 tokens, 9984 x 12416 29.1 /
+// 21.8; 95, 19288 x 7040 32.9 / 25.6; 121, 3392 x 1536 9.8 / 8.7.  Bands with K split over a cluster are left to 32 tokens at most (4096 x 14336,
+// 16 tokens 12.7 and 15.1, 61 tokens 16.5 and 15.0).  One weight tile with so long a K that eight CTAs are too few for it is split through
+// memory; nothing else goes there from bands.
+struct W4Small {
+  int64_t N, K;
+  int M, device;
+  bool few;
+  W4DecodeShape d;              // few
+  int tile_n, cluster;          // otherwise
+};
+static void w4_few_or_tiles(W4Small* c, int tile_n) {
+  const int kstages = static_cast<int>((c->K + kW4BlockK - 1) / kW4BlockK), forced = option(OPT_W4_DECODE);     // testing aid: 0 never, a shape wherever it fits
+  c->tile_n = tile_n;
+  w4_tile_decode_shape(c->M, c->N, kstages, &c->tile_n, &c->cluster);
+  c->few = forced != 0 && !(c->N <= 224 && kstages > 28) && w4_decode_shape(&c->d, c->M, 0, c->N, c->K);
+  if (!c->few || forced > 0) return;
+  if (c->d.S > 1 && c->M > 32) { c->few = false; return; }
+  const long long tiles = (c->N + c->tile_n - 1) / c->tile_n;
+  if (c->cluster == 1 && w4_memory_split(tiles, kstages) > 1) return;
+  const float width = static_cast<float>(c->tile_n), tokens = static_cast<float>(c->M), S = static_cast<float>(c->cluster);
+  const long long items = tiles * c->cluster, grid = items < sm_count() ? items : sm_count(), full = items / grid, rest = items - full * grid;
+  auto stage_us = [&](long long ctas) { return fmaxf(0.0044f * width - 0.22f, 136.0f * width * static_cast<float>(ctas) / 4.6e6f); };
+  float us = static_cast<float>((kstages + c->cluster - 1) / c->cluster) * (static_cast<float>(full) * stage_us(grid) + (rest ? stage_us(rest) : 0.0f)) + 0.0022f * tokens;
+  if (c->cluster > 1) us += 2.1e-4f * tokens * width * (S - 1.0f) / S + 0.36f * S;
+  c->few = w4_decode_us(c->d, tokens) <= us + 0.2f;
+}
+
+// The choice looks at some hundred shapes, microseconds of host time: a layer's is remembered (64 direct-mapped slots by everything it
+// depends on).
+static W4Small w4_small_plan(int64_t M, int64_t N, int64_t K, int tile_n) {
+  W4Small c = {};
+  c.N = N; c.K = K; c.M = static_cast<int>(M);
+  if (cudaGetDevice(&c.device) != cudaSuccess) c.device = -1;
+  if (option(OPT_W4_DECODE) >= 0) { w4_few_or_tiles(&c, tile_n); return c; }
+  constexpr int kSlots = 64;
+  static W4Small slots[kSlots] = {};
+  static std::mutex mu;
+  W4Small& slot = slots[((static_cast<uint64_t>(N) * 0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(K)) * 0x9E3779B97F4A7C15ull + static_cast<uint64_t>(M) * 0xC2B2AE3D27D4EB4Full) >> 58];
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (slot.M == c.M && slot.N == N && slot.K == K && slot.device == c.device) return slot;
+  }
+  w4_few_or_tiles(&c, tile_n);
+  std::lock_guard<std::mutex> lock(mu);
+  return slot = c;
 }
 
 static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
@@ -933,8 +981,10 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   pl.few = false;
   pl.kstages = static_cast<int>((K + kW4BlockK - 1) / kW4BlockK);
   if (M <= kW4TileM && option(OPT_W4_TILEN) < 0 && option(OPT_W4_KSPLIT) < 0 && option(OPT_W4_PAIR) < 0) {
-    pl.few = w4_decode_takes(&pl.d, M, N, K, pl.kstages);
-    if (!pl.few) w4_tile_decode_shape(M, N, pl.kstages, &tile_n, &pl.cluster);
+    const W4Small c = w4_small_plan(M, N, K, tile_n);
+    pl.few = c.few;
+    if (c.few) pl.d = c.d;
+    else { tile_n = c.tile_n; pl.cluster = c.cluster; }
   }
   pl.sf_tile_rows = tile_n == 224 && !pl.few ? 224 : 256;
   pl.tile_n = tile_n;
@@ -948,7 +998,7 @@ static GemmW4Plan plan_w4(int64_t M, int64_t N, int64_t K) {
   pl.kper = pl.kstages;
   {
     const int forced = option(OPT_W4_KSPLIT);     // testing aid
-    int want = forced >= 0 ? forced : (2 * tiles <= sm_count() ? sm_count() / tiles : 1);
+    int want = forced >= 0 ? forced : w4_memory_split(tiles, pl.kstages);
     if (want > pl.kstages / 4) want = pl.kstages / 4;
     if (want > 1) {
       pl.kper = (pl.kstages + want - 1) / want;

@@ -551,28 +551,25 @@ float w4_decode_grouped_us(const W4DecodeShape& d, float tokens) {
   return static_cast<float>(full) * band_us(d.grid) + (rest ? band_us(rest) : 0.0f) + (d.nacc == 2 ? epilogue : 0.0f);
 }
 
-// The search looks at up to 72 shapes, several microseconds of host time: a layer's is remembered (64 direct-mapped slots by everything
-// it depends on; calls with experts, whose groups change from call to call, have nine to look at).
+// The same for a call with one matrix, as far as it differs: weights come in one burst, not as a steady stream, and a cluster's exchange
+// counts (see w4_few_or_tiles).
+float w4_decode_us(const W4DecodeShape& d, float tokens) {
+  const float epilogue = fmaxf(0.0f, 0.0162f * tokens - 0.52f);
+  auto stages_us = [&](int ctas) {
+    float us = fmaxf(fmaxf(0.52f, static_cast<float>(d.stage_bytes) / 85.0e3f), 136.0f * static_cast<float>(d.h * d.kw) * static_cast<float>(ctas) / 6.15e6f);
+    if (d.nstages < 3 && d.steps > d.nstages) us *= 1.2f;
+    return static_cast<float>(d.kper) * us;
+  };
+  if (d.S > 1) return stages_us(d.grid) + 0.8f + 0.081f * tokens * static_cast<float>(d.S - 1) / static_cast<float>(d.S);
+  const int full = d.items / d.grid, rest = d.items - full * d.grid;
+  auto band_us = [&](int ctas) { return d.nacc == 2 ? fmaxf(stages_us(ctas), epilogue) : stages_us(ctas) + epilogue; };
+  return static_cast<float>(full) * band_us(d.grid) + (rest ? band_us(rest) : 0.0f) + (d.nacc == 2 ? epilogue : 0.0f);
+}
+
 bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K) {
   if (const int forced = option(OPT_W4_DECODE); forced > 0)
     return w4_decode_layout(best, tokens, groups, N, K, forced % 1000, forced / 100000, forced / 1000 % 100);
-  const int sms = sm_count();
-  if (groups > 0) return w4_decode_search(best, tokens, groups, N, K, sms);
-  struct Slot { int64_t N, K; int tokens, sms; bool found; W4DecodeShape d; };
-  constexpr int kSlots = 64;
-  static Slot slots[kSlots] = {};
-  static std::mutex mu;
-  Slot& slot = slots[((static_cast<uint64_t>(N) * 0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(K)) * 0x9E3779B97F4A7C15ull + static_cast<uint64_t>(tokens) * 0xC2B2AE3D27D4EB4Full) >> 58];
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (slot.tokens == tokens && slot.N == N && slot.K == K && slot.sms == sms) { *best = slot.d; return slot.found; }
-  }
-  Slot fresh = {N, K, tokens, sms, false, {}};
-  fresh.found = w4_decode_search(&fresh.d, tokens, 0, N, K, sms);
-  std::lock_guard<std::mutex> lock(mu);
-  slot = fresh;
-  *best = fresh.d;
-  return fresh.found;
+  return w4_decode_search(best, tokens, groups, N, K, sm_count());
 }
 
 msd_status_t w4_decode_launch(const W4DecodeShape& d, const uint8_t* w_fp4, const uint8_t* q, int64_t q_rows, int64_t w_rows, int M, int64_t N,

@@ -169,6 +169,7 @@ struct W4DecodeShape {
 // (groups: matrices of a grouped launch, 0 for an ungrouped call)
 bool w4_decode_shape(W4DecodeShape* best, int tokens, int groups, int64_t N, int64_t K);
 float w4_decode_grouped_us(const W4DecodeShape& d, float tokens);
+float w4_decode_us(const W4DecodeShape& d, float tokens);
 // Groups of one launch: group g = rows [off[g], off[g + 1]) of y (at most 128) and the weights of expert[g].
 struct W4Groups {
   int expert[kMaxRowGroups], off[kMaxRowGroups + 1];

@@ -133,9 +133,8 @@ def test_prepared_weight_scales(M, N, K, pair, tile):
 @pytest.mark.parametrize("M,N,K", [(1, 4096, 2048), (16, 4088, 14336), (33, 1000, 1280), (61, 14336, 1024), (128, 2056, 4096),
                                    (8, 8, 4096), (100, 136, 8192), (17, 16776, 1152), (4, 8248, 4096), (125, 15904, 1280), (5, 16, 7424)])
 def test_decode_k_split_as_a_cluster(M, N, K):
-    """One token tile with the K splits of a weight tile as the CTAs of a cluster: every tile width, ragged last tiles (one 8-column
-    piece among them), uneven last splits, one row to a full tile, and the shapes left whole or split through memory beside
-    them; row-major and prepared scales give the same bits, FP32 against the oracle, BF16 the FP32 result rounded once.  Partial
+    """Layers of at most 128 tokens in the kernel they are given (token tiles or bands of weight rows; K whole, split over a cluster or
+    through memory): ragged last tiles (one 8-column piece among them), uneven last splits, one row to a full tile; row-major and prepared scales give the same bits, FP32 against the oracle, BF16 the FP32 result rounded once.  Partial
     tiles in memory show in the workspace: a single weight tile with a long K has them, a shape with clusters does not."""
     up, groups = lambda v: (v + 1023) // 1024 * 1024, 2 * ((K + 255) // 256)
     no_partial = 2 * up(M * K // 2) + 2 * up(512 * groups) + up(2 * ((N + 223) // 224) * groups * 512)
@@ -198,3 +197,23 @@ def test_workspace_for_many_tokens_serves_fewer(N, K):
     """The kernel changes with the token count; a workspace asked for at one count is enough at every smaller one."""
     sizes = [binding.gemm_w4a16_workspace_bytes(M, N, K) for M in range(1, 129)]
     assert sizes == sorted(sizes)
+
+
+@pytest.mark.parametrize("M,N,K,width", [(1, 264, 4096, 128), (33, 264, 1280, 128), (128, 2056, 4096, 128), (33, 5776, 4096, 224), (8, 10248, 1024, 224),
+                                         (33, 5880, 5120, 256), (8, 10248, 2176, 256)])
+def test_token_tiles_with_k_split_over_a_cluster(M, N, K, width):
+    """The tile kernel's cluster form at every width, few-token kernel switched off: against the oracle, row-major and prepared scales
+    bit for bit, BF16 the FP32 result rounded once.  No CTA of a cluster shares its SM."""
+    binding.debug_set_option("MSD_W4_DECODE", 0)
+    kernel, rows, cluster, splits, smem = binding.debug_gemm_w4a16_schedule(M, N, K)
+    assert (kernel, rows) == (0, width) and cluster == splits > 1 and 2 * (smem + 1024) > 228 * 1024
+    c = inputs.gemm_w4_case(M, N, K, seed=M + N)
+    x, w, e = bf16_dev(c.x), dev(c.w_fp4), dev(c.w_e8m0)
+    y = binding.gemm_w4a16(x, w, e, out_dtype=torch.float32)
+    prep = binding.prepare_w4a16_scales(e)
+    y2 = binding.gemm_w4a16(x, w, None, out_dtype=torch.float32, prepared=prep)
+    yb = binding.gemm_w4a16(x, w, None, out_dtype=torch.bfloat16, prepared=prep)
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
+    _close(y.cpu().numpy().astype(np.float64), oracle.gemm_w4a16(c.x, c.w_fp4, c.w_e8m0, "f64"), False)

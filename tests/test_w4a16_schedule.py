@@ -48,3 +48,11 @@ def test_grouped_calls_with_long_groups_take_token_tiles(tokens, E, N, K, kernel
     assert binding.debug_grouped_gemm_w4a16_schedule([0, tokens] * E, N, K)[0] == kernel
     binding.debug_set_option("MSD_W4_DECODE", 0)
     assert binding.debug_grouped_gemm_w4a16_schedule([tokens] * E, N, K)[0] == 0
+
+
+@pytest.mark.parametrize("M,N,K,kernel", [(95, 19288, 7040, 0), (79, 19712, 2432, 0), (16, 19288, 7040, 2), (1, 4096, 14336, 2), (64, 14336, 4096, 2)])
+def test_layers_take_the_shorter_kernel(M, N, K, kernel):
+    """Both sides of the line between bands of weight rows and token tiles, on shapes whose K neither of them splits; the same when the
+    choice is remembered."""
+    for _ in range(2):
+        assert binding.debug_gemm_w4a16_schedule(M, N, K)[0] == kernel
