@@ -64,7 +64,8 @@ msd_status_t msd_debug_timeout_selftest(int64_t budget_cycles, void* stream);
 
 /* Testing and diagnostic switches.  Each is read from the environment variable of the same name once, when the first
  * call needs one; msd_debug_set_option overrides it afterwards (value -1 = unset), msd_debug_reset_options returns to
- * what the environment says.  Unknown names: MSD_ERR_UNSUPPORTED.  None of them changes results.
+ * what the environment says.  Unknown names: MSD_ERR_UNSUPPORTED.  They choose kernels and splits: INT8 layers keep their results, FP32 sums
+ * (W4A16) and running maxima (attention) may round elsewhere.
  *   MSD_NO_PDL (1: no programmatic dependent launches), MSD_GEMM_MODE / MSD_GEMM_CTAS (work split and CTA count of the
  *   W8A16 decode kernel: 0 stream-K, 1 row bands, 2 clusters), MSD_P8_PAIR / MSD_P8_KSPLIT (W8A16 many-row kernel: CTA
  *   pairs, K split), MSD_W4_PAIR / MSD_W4_TILEN / MSD_W4_KSPLIT (W4A16 kernels), MSD_W4_DECODE (W4A16 with few tokens: 0 keeps
@@ -241,8 +242,7 @@ msd_status_t msd_debug_gemm_w4a16_schedule(int64_t M, int64_t N, int64_t K, int3
  *   x_bf16 [M_total, K] (device), w_fp4 [E, N, K/2], w_e8m0 [E, N, K/32], y [M_total, N] (device);
  *   group_sizes_host [E] INT32 in HOST memory, each 0..128 (decode regime per expert), M_total = their sum.
  * Empty groups are skipped (their weights are not read).  Per 64 non-empty groups one decomposition launch (the first
- * also brings every expert's weight scales into the blocked layout) and one GEMM launch in which group g is token tile
- * g.  K % 128 == 0, N % 8 == 0, E * N < 2^31; x, w_fp4, y 16-byte aligned, w_e8m0 4-byte aligned.
+ * also brings every expert's weight scales into the blocked layout) and one GEMM launch.  K % 128 == 0, N % 8 == 0, E * N < 2^31; x, w_fp4, y 16-byte aligned, w_e8m0 4-byte aligned.
  * workspace: >= msd_grouped_gemm_w4a16_workspace_bytes(E, N, K), 1024-byte aligned; no initialisation needed.
  */
 size_t msd_grouped_gemm_w4a16_workspace_bytes(int32_t E, int64_t N, int64_t K);

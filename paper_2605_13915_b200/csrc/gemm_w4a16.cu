@@ -11,7 +11,8 @@
 //
 // Warps: 0 = operand producer, 1 = MMA issuer + TMEM owner, 2..5 = epilogue (TMEM -> BF16/FP32 -> swizzled staging
 // buffer -> TMA store), 6..9 = scale warps, 10 = scale producer.  gemm_w4a16_pair_kernel is the cta_group::2 variant for prefill
-// shapes; few tokens per weight matrix and mixture-of-experts calls run in gemm_w4a16_decode.cu.
+// shapes; calls with few tokens per weight matrix, with or without experts, run in gemm_w4a16_decode.cu where that is shorter
+// (w4_few_or_tiles, w4_grouped_tiles).
 #include <cuda_bf16.h>
 
 #include <cmath>

@@ -6,7 +6,8 @@
 //
 // Bound: HBM for experts (32 of 2048 x 7168, 512 tokens: 53 us, 4.8 TB/s), the chain of two kernels for single layers (16 tokens, 4096 x 14336
 // and back: 11.2 and 12.6 us for 31 MB each).  With tiles of 128 token rows, padded and once per component, a 256 x 256 weight stage
-// took 0.65 us of tensor time where HBM needs 0.8 for all SMs: 68 and 32 us for the two.
+// took 0.65 us of tensor time where HBM needs 0.8 for all SMs: 68 and 32 us for the two.  With about 64 tokens and more the components,
+// brought once per band, outweigh the weights and those tiles are the shorter way again.
 #include <cuda_bf16.h>
 
 #include <cmath>

@@ -86,9 +86,9 @@ def _case_w4(sizes, N, K, seed):
 @pytest.mark.parametrize("sizes,N,K", [([3, 0, 16, 1], 448, 512), ([128, 5, 0, 0, 64, 33, 9, 2], 1000, 1024),
                                        ([1] * 70 + [0] * 10 + [4] * 5, 232, 256), ([0, 0, 11], 2048, 4096)])
 def test_grouped_w4a16_matches_per_expert_oracle(sizes, N, K):
-    """Grouped W4A16 (MXFP4 weights per expert) against the oracle run expert by expert: uneven groups whose end falls
-    inside a warp's 32 output rows (masked stores) and on their boundary (box stores), empty experts, more than 64
-    non-empty groups (two launches), ragged last weight tile; FP32 and BF16 outputs; the workspace is reused."""
+    """Grouped W4A16 (MXFP4 weights per expert) against the oracle run expert by expert, in the kernel that the call is given:
+    uneven groups of 1 to 128 tokens, empty experts, more than 64 non-empty groups (two launches), ragged last weight
+    tile; FP32 and BF16 outputs; the workspace is reused."""
     x, q, e = _case_w4(sizes, N, K, seed=len(sizes) + N)
     ref = np.zeros((x.shape[0], N), np.float64)
     off = 0
@@ -180,5 +180,20 @@ def test_grouped_w4a16_with_more_bands_than_sms(sizes, shape, K):
     torch.cuda.synchronize()
     binding.last_device_status()
     assert torch.equal(y, y2) and torch.equal(yb, y.to(torch.bfloat16))
+    want = _w4_oracle(x, q, e, sizes)
+    assert np.all(np.abs(y.cpu().numpy() - want) <= TOL * np.linalg.norm(want, axis=-1, keepdims=True) + 1e-30)
+
+
+def test_grouped_w4a16_token_tiles_in_two_launches():
+    """More than 64 groups as token tiles: the second launch takes weight scales that the first one's decomposition laid out."""
+    sizes, N, K = [1, 0, 4] * 40 + [128, 3], 232, 384
+    binding.debug_set_option("MSD_W4_DECODE", 0)
+    x, q, e = _case_w4(sizes, N, K, seed=77)
+    xd, qd, ed = bf16_dev(x), dev(q), dev(e)
+    y = binding.grouped_gemm_w4a16(xd, qd, ed, sizes, out_dtype=torch.float32)
+    y2 = binding.grouped_gemm_w4a16(xd, qd, None, sizes, out_dtype=torch.float32, prepared=binding.prepare_w4a16_scales(ed))
+    torch.cuda.synchronize()
+    binding.last_device_status()
+    assert torch.equal(y, y2)
     want = _w4_oracle(x, q, e, sizes)
     assert np.all(np.abs(y.cpu().numpy() - want) <= TOL * np.linalg.norm(want, axis=-1, keepdims=True) + 1e-30)
